@@ -620,46 +620,64 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
     }
 }
 
-// State after a T-token prompt.  One block per (b,h); the cache was zero-filled beforehand.
-template <typename T>
-__global__ void cache_init_kernel(unsigned char* __restrict__ cache, CacheLayout L, const T* __restrict__ k,
-                                  const T* __restrict__ v, const float* __restrict__ z, const int32_t* __restrict__ idx,
-                                  const int32_t* __restrict__ cnt, int Tlen, int D, int W, int R, int half)
+// State after a T-token prompt.  Bound by memory: every byte of the cache is written exactly once (the rows nothing fills,
+// the tail's padding and the header as zeros, so no fill pass comes before), every window and retained row is read once, in
+// 16-byte pieces.  Block (part, (b,h)) writes IROWS rows of the head's block with their logits; a block per head with two
+// divisions per element took 248 + 17 us for 256 heads of 1,280 rows (d = 64), this takes 28.
+constexpr int IROWS = 64;
+__global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restrict__ cache, CacheLayout L, const uint4* __restrict__ k,
+                                                         const uint4* __restrict__ v, const float* __restrict__ z,
+                                                         const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, int Tlen,
+                                                         int pshift, int W, int R, int half)
 {
-    const int bh = blockIdx.x;
+    __shared__ int s_pos[IROWS];                               // token of each row of this part, -1: none
+    pdl_launch_dependents();
+    pdl_wait();
+    const int bh = blockIdx.y, tid = threadIdx.x;
     unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
-    T* Kc = reinterpret_cast<T*>(blk + L.off_k);
-    T* Vc = reinterpret_cast<T*>(blk + L.off_v);
-    float* zc = reinterpret_cast<float*>(blk + L.off_z);
-    int32_t* pidx = reinterpret_cast<int32_t*>(blk + L.off_pidx);
-    int32_t* meta = reinterpret_cast<int32_t*>(blk + L.off_meta);
     const int n_ret = Tlen > 0 && R > 0 ? cnt[bh] : 0;
     const int lo = Tlen - W > 0 ? Tlen - W : 0;
-    const int nwin = Tlen - lo;
-    for (int e = threadIdx.x; e < (nwin + n_ret) * D; e += blockDim.x) {
-        const int a = e / D, c = e % D;
-        const int pos = a < nwin ? lo + a : idx[(size_t)bh * R + (a - nwin)];
-        const int row = a < nwin ? pos % W : W + (a - nwin);
-        const int cdst = L.swz ? ((((c >> 3) ^ (row & 7)) << 3) | (c & 7)) : c;   // swizzled layout: chunk c/8 moves
-        Kc[(size_t)row * D + cdst] = k[((size_t)bh * Tlen + pos) * D + c];
-        Vc[(size_t)row * D + cdst] = v[((size_t)bh * Tlen + pos) * D + c];
-    }
-    for (int a = threadIdx.x; a < W + R; a += blockDim.x) {
-        float zz = -INFINITY;
+    const int row0 = blockIdx.x * IROWS, n_rows = min(IROWS, L.rows_alloc - row0);
+    if (tid < n_rows) {
+        const int a = row0 + tid;
+        int pos = -1;
         if (a < W) {
             // slot a holds the newest position congruent to a (mod W), if any
-            if (a < nwin || Tlen >= W) {
-                int pos = lo + ((a - lo % W) + W) % W;
-                if (pos < Tlen && pos <= Tlen - 1 - half) zz = z[(size_t)bh * Tlen + pos];
-            }
+            pos = lo + (a - lo % W + W) % W;
+            if (pos >= Tlen) pos = -1;
         } else if (a - W < n_ret) {
-            const int pos = idx[(size_t)bh * R + (a - W)];
-            zz = z[(size_t)bh * Tlen + pos];
-            pidx[a - W] = pos;
+            pos = idx[(size_t)bh * R + (a - W)];
         }
-        zc[a] = zz;
+        s_pos[tid] = pos;
+        if (a < W + R) {
+            const bool scored = pos >= 0 && (a >= W || pos <= Tlen - 1 - half);
+            reinterpret_cast<float*>(blk + L.off_z)[a] = scored ? z[(size_t)bh * Tlen + pos] : -INFINITY;
+            if (a >= W) reinterpret_cast<int32_t*>(blk + L.off_pidx)[a - W] = pos < 0 ? 0 : pos;
+        }
     }
-    if (threadIdx.x == 0) { meta[0] = Tlen; meta[1] = n_ret; meta[2] = 0; meta[3] = 0; }
+    if (blockIdx.x == 0) {                                     // counters and padding; the header
+        uint32_t* tail = reinterpret_cast<uint32_t*>(blk + L.off_meta);
+        const int n_tail = (int)((L.stride - L.off_meta) / 4);
+        for (int e = tid; e < n_tail; e += 256) tail[e] = e == 0 ? (uint32_t)Tlen : e == 1 ? (uint32_t)n_ret : 0u;
+        if (bh == 0 && tid < (int)(L.header / 4)) reinterpret_cast<uint32_t*>(cache)[tid] = 0u;
+    }
+    __syncthreads();
+    uint4* Kc = reinterpret_cast<uint4*>(blk + L.off_k);
+    uint4* Vc = reinterpret_cast<uint4*>(blk + L.off_v);
+    const size_t src0 = (size_t)bh * Tlen;
+    const int n = n_rows << pshift, pmask = (1 << pshift) - 1;
+#pragma unroll 4
+    for (int e = tid; e < n; e += 256) {
+        const int r = e >> pshift, c = e & pmask, row = row0 + r, pos = s_pos[r];
+        uint4 kx = make_uint4(0, 0, 0, 0), vx = kx;
+        if (pos >= 0) {
+            kx = k[((src0 + pos) << pshift) + c];
+            vx = v[((src0 + pos) << pshift) + c];
+        }
+        const size_t d = ((size_t)row << pshift) + cache_chunk_pos(L, row, c);
+        Kc[d] = kx;
+        Vc[d] = vx;
+    }
 }
 
 }  // namespace
@@ -670,17 +688,9 @@ int launch_cache_init(const Params& p, const void* k, const void* v, const float
                       const int32_t* cnt, void* cache, cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    const size_t bytes = L.header + (size_t)p.B * p.H * L.stride;
-    cudaError_t e = cudaMemsetAsync(cache, 0, bytes, st);
-    if (e != cudaSuccess) return LTE_ERR_CUDA;
-    if (p.dtype == LTE_BF16)
-        cache_init_kernel<__nv_bfloat16><<<p.B * p.H, 256, 0, st>>>((unsigned char*)cache, L, (const __nv_bfloat16*)k,
-                                                                    (const __nv_bfloat16*)v, z, idx, cnt, p.T, p.d, p.W,
-                                                                    p.R, p.half);
-    else
-        cache_init_kernel<float><<<p.B * p.H, 256, 0, st>>>((unsigned char*)cache, L, (const float*)k, (const float*)v, z,
-                                                            idx, cnt, p.T, p.d, p.W, p.R, p.half);
-    return cuda_status(cudaGetLastError());
+    const dim3 grid((L.rows_alloc + IROWS - 1) / IROWS, p.B * p.H);
+    return cuda_status(launch_pdl(cache_init_kernel, grid, dim3(256), 0, st, (unsigned char*)cache, L, (const uint4*)k, (const uint4*)v, z,
+                                  idx, cnt, p.T, piece_shift(L, p.d), p.W, p.R, p.half));
 }
 
 // ---- lazy scoring of the ring for scorers that do not run inside the step (the three-layer stack) -------------------
@@ -691,46 +701,70 @@ int launch_cache_init(const Params& p, const void* k, const void* v, const float
 // With rotary tables (cos, sin [rope_len, D/2], half-split pairing: channels c and c + D/2 form a pair) the keys are
 // rotated back to their un-rotated form on the way: the scorer consumes keys as they were before the position embedding,
 // the cache holds them after it (Section 3.1.3, lazy scoring paragraph).  Row r is the token at position base + r.
+// Bound by memory: a thread moves the two 16-byte pieces that hold a pair's channels, of the key and of the value, so every
+// byte is read and written once; blocks of LROWS rows (a block per head with two divisions per element took 154 us for 256
+// heads of 768 rows, d = 64, this takes 14).
+constexpr int LROWS = 64;
 template <typename T>
-__global__ void ring_linearize_kernel(const unsigned char* __restrict__ cache, CacheLayout L, T* __restrict__ klin,
-                                      T* __restrict__ vlin, int D, int W, const float* __restrict__ rope_cos,
-                                      const float* __restrict__ rope_sin, int rope_len)
+__global__ void __launch_bounds__(256) ring_linearize_kernel(const unsigned char* __restrict__ cache, CacheLayout L, uint4* __restrict__ klin,
+                                                             uint4* __restrict__ vlin, int pshift, int W, const float* __restrict__ rope_cos,
+                                                             const float* __restrict__ rope_sin, int rope_len)
 {
-    const int bh = blockIdx.x;
+    constexpr int EPV = V16<T>::N;
+    pdl_launch_dependents();
+    pdl_wait();
+    const int bh = blockIdx.y;
     const unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
-    const T* Kc = reinterpret_cast<const T*>(blk + L.off_k);
-    const T* Vc = reinterpret_cast<const T*>(blk + L.off_v);
+    const uint4* Kc = reinterpret_cast<const uint4*>(blk + L.off_k);
+    const uint4* Vc = reinterpret_cast<const uint4*>(blk + L.off_v);
     const int n = reinterpret_cast<const int32_t*>(blk + L.off_meta)[0];
     const int base = n > W ? n - W : 0, n_eff = n < W ? n : W;
-    for (int e = threadIdx.x; e < W * D; e += blockDim.x) {
-        const int r = e / D, c = e % D;
-        T kx = from_f<T>(0.f), vx = from_f<T>(0.f);
+    const int r0 = blockIdx.x * LROWS, n_rows = min(LROWS, W - r0);
+    const int hshift = pshift - 1, hp = 1 << hshift;           // pieces of half a row
+    const int slot0 = (base + r0) % W;
+    for (int e = threadIdx.x; e < n_rows << hshift; e += 256) {
+        const int r = r0 + (e >> hshift), c = e & (hp - 1);
+        uint4 k1 = make_uint4(0, 0, 0, 0), k2 = k1, v1 = k1, v2 = k1;
         if (r < n_eff) {
-            const int row = (base + r) % W;
-            const int cs = L.swz ? ((((c >> 3) ^ (row & 7)) << 3) | (c & 7)) : c;
-            kx = Kc[(size_t)row * D + cs]; vx = Vc[(size_t)row * D + cs];
+            int row = slot0 + (r - r0);
+            if (row >= W) row -= W;
+            const size_t rb = (size_t)row << pshift;
+            const int c1 = cache_chunk_pos(L, row, c), c2 = cache_chunk_pos(L, row, c + hp);
+            k1 = Kc[rb + c1]; k2 = Kc[rb + c2]; v1 = Vc[rb + c1]; v2 = Vc[rb + c2];
             if (rope_cos) {
-                const int pos = base + r, hd = D / 2;
+                const int pos = base + r;
                 if (pos < rope_len) {
-                    const int cp = c < hd ? c + hd : c - hd;       // the channel this one is paired with
-                    const int cps = L.swz ? ((((cp >> 3) ^ (row & 7)) << 3) | (cp & 7)) : cp;
-                    const float co = rope_cos[(size_t)pos * hd + (c % hd)], si = rope_sin[(size_t)pos * hd + (c % hd)];
-                    const float a = to_f(kx), b = to_f(Kc[(size_t)row * D + cps]);
-                    // inverse rotation: (x1, x2) -> (x1 cos + x2 sin, x2 cos - x1 sin)
-                    kx = from_f<T>(c < hd ? a * co + b * si : a * co - b * si);
+                    const size_t tb = ((size_t)pos << hshift) * EPV + (size_t)c * EPV;
+                    float a[EPV], b[EPV];
+                    unpack<T>(k1, a); unpack<T>(k2, b);
+                    T o1[EPV], o2[EPV];
+#pragma unroll
+                    for (int i = 0; i < EPV; i += 4) {
+                        const float4 co = *reinterpret_cast<const float4*>(rope_cos + tb + i), si = *reinterpret_cast<const float4*>(rope_sin + tb + i);
+                        const float cf[4] = {co.x, co.y, co.z, co.w}, sf[4] = {si.x, si.y, si.z, si.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {          // inverse rotation: (x1, x2) -> (x1 cos + x2 sin, x2 cos - x1 sin)
+                            o1[i + j] = from_f<T>(a[i + j] * cf[j] + b[i + j] * sf[j]);
+                            o2[i + j] = from_f<T>(b[i + j] * cf[j] - a[i + j] * sf[j]);
+                        }
+                    }
+                    memcpy(&k1, o1, 16); memcpy(&k2, o2, 16);
                 } else if (c == 0) {
-                    atomicExch(&g_decode_status.code, 32);              // the tables do not reach this position: key left rotated
+                    atomicExch(&g_decode_status.code, 32);     // the tables do not reach this position: key left rotated
                 }
             }
         }
-        klin[((size_t)bh * W + r) * D + c] = kx;
-        vlin[((size_t)bh * W + r) * D + c] = vx;
+        const size_t d = (((size_t)bh * W + r) << pshift) + c;
+        klin[d] = k1; klin[d + hp] = k2;
+        vlin[d] = v1; vlin[d + hp] = v2;
     }
 }
 
 __global__ void ring_scatter_z_kernel(unsigned char* __restrict__ cache, CacheLayout L, const float* __restrict__ zlin, int W,
                                       int half)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     const int bh = blockIdx.x;
     unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
     float* zc = reinterpret_cast<float*>(blk + L.off_z);
@@ -744,20 +778,16 @@ int launch_ring_linearize(const Params& p, const void* cache, void* klin, void* 
                           int rope_len, cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    if (p.dtype == LTE_BF16)
-        ring_linearize_kernel<__nv_bfloat16><<<p.B * p.H, 256, 0, st>>>((const unsigned char*)cache, L, (__nv_bfloat16*)klin,
-                                                                        (__nv_bfloat16*)vlin, p.d, p.W, rope_cos, rope_sin, rope_len);
-    else
-        ring_linearize_kernel<float><<<p.B * p.H, 256, 0, st>>>((const unsigned char*)cache, L, (float*)klin, (float*)vlin, p.d, p.W,
-                                                                rope_cos, rope_sin, rope_len);
-    return cuda_status(cudaGetLastError());
+    const dim3 grid((p.W + LROWS - 1) / LROWS, p.B * p.H);
+    auto kern = p.dtype == LTE_BF16 ? ring_linearize_kernel<__nv_bfloat16> : ring_linearize_kernel<float>;
+    return cuda_status(launch_pdl(kern, grid, dim3(256), 0, st, (const unsigned char*)cache, L, (uint4*)klin, (uint4*)vlin, piece_shift(L, p.d),
+                                  p.W, rope_cos, rope_sin, rope_len));
 }
 
 int launch_ring_scatter_z(const Params& p, void* cache, const float* zlin, cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    ring_scatter_z_kernel<<<p.B * p.H, 128, 0, st>>>((unsigned char*)cache, L, zlin, p.W, p.half);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(ring_scatter_z_kernel, dim3(p.B * p.H), dim3(128), 0, st, (unsigned char*)cache, L, zlin, p.W, p.half));
 }
 
 // ---- grouped-query attention -----------------------------------------------------------------------------------------
