@@ -1,4 +1,4 @@
-"""Build ``liblte.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Build ``liblte.so`` (the C-ABI CUDA library, nvcc for sm_100a) and ``_binding.so`` (its Python binding, g++) in-tree.
 
 Usage: ``python -m paper_2510_20787_b200.build [--force] [--verbose]``.
 Object files are cached per source under ``csrc/build`` and rebuilt when the source or a header is newer.
@@ -8,11 +8,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "liblte.so")
+BINDING = os.path.join(HERE, "_binding.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -23,6 +25,29 @@ def _newer(target, deps):
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_binding(force=False, verbose=False):
+    """The CPython module over ``liblte.so``: needs torch's headers and libraries, no CUDA compiler."""
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and not _newer(BINDING, [src, LIB, os.path.join(INCLUDE, "lte.h")]):
+        return BINDING
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    cmd = (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), src, "-o", tmp]
+           + ["-I" + d for d in (INCLUDE, sysconfig.get_paths()["include"])]
+           + ["-isystem" + d for d in (os.path.join(troot, "include"), os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+                                       os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"))]
+           + ["-L" + os.path.join(troot, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+              "-L" + HERE, "-l:liblte.so", "-Wl,-rpath,$ORIGIN"])
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+    if r.returncode:
+        raise RuntimeError("g++ failed for binding.cpp")
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 def build(force=False, verbose=False):
@@ -53,6 +78,7 @@ def build(force=False, verbose=False):
         tmp = LIB + ".tmp.%d" % os.getpid()
         subprocess.check_call([NVCC, "-shared", "-o", tmp] + objs + ["-lcudart"])
         os.replace(tmp, LIB)
+    build_binding(force, verbose)
     return LIB
 
 

@@ -2,8 +2,9 @@
 
 Every function takes CUDA ``torch`` tensors (device memory and the current stream are all PyTorch
 is used for), checks dtype / contiguity, and passes raw pointers to the entry point of the same name
-declared in ``include/lte.h``.  There is no fallback: if the library is missing or a call fails, an
-exception is raised.
+declared in ``include/lte.h``.  The calls that take tensors do this in the native module ``_binding``
+(``csrc/binding.cpp``), because a small call is bound by the host; ``lib()`` is the plain ctypes handle.
+There is no fallback: if the library is missing or a call fails, an exception is raised.
 """
 import ctypes
 import os
@@ -13,11 +14,13 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblte.so")
 _lib = None
+_native = None
 
 F32, BF16 = 0, 1
 OP_SCORES, OP_SELECT, OP_PREFILL, OP_DECODE, OP_BWD, OP_CHUNK, OP_STATS, OP_CHUNK_STREAM = range(8)
 CHUNK_STREAMING = 1
 BWD_CNN_INPUT_GRAD = 1
+RULE_LEARNED, RULE_UNIFORM, RULE_ACCUM_ATTN = 0, 1, 2
 
 EXPORTS = ["lte_device_status", "lte_workspace_bytes", "lte_strerror", "lte_scores", "lte_select", "lte_cache_score", "lte_attn_prefill",
            "lte_cache_bytes", "lte_cache_init", "lte_attn_decode", "lte_attn_prefill_chunk", "lte_attn_bwd", "lte_attn_bwd_static",
@@ -122,17 +125,14 @@ def conv_stack(wl, wout, bl=None, bout=None):
     return c
 
 
-def _ptr(t, dtype=None):
-    if t is None:
-        return None
-    assert t.is_cuda and t.is_contiguous(), "tensors must be contiguous CUDA tensors"
-    if dtype is not None:
-        assert t.dtype == dtype, "expected %s, got %s" % (dtype, t.dtype)
-    return t.data_ptr()
-
-
-def _stream():
-    return torch.cuda.current_stream().cuda_stream
+def _load():
+    """The native module (it links against ``liblte.so``, both built by ``python -m paper_2510_20787_b200.build``)."""
+    global _native
+    lib()
+    from . import _binding
+    _binding.set_error(LteError)
+    _native = _binding
+    return _binding
 
 
 def _check(fn, status):
@@ -152,70 +152,31 @@ def lte_workspace_bytes(op, s, c=None):
 def lte_scores(s, c, k, v, z=None, r=None, ws=None):
     """k, v [B,H,T,d] -> z [B,H,T] fp32 (and r = sigmoid(z) if a tensor is given).  ws: a uint8 workspace tensor of
     lte_workspace_bytes(OP_SCORES, s, c) bytes (allocated here when None and the call wants one; False = none)."""
-    if z is None:
-        z = torch.empty((s.B, s.H, s.T), dtype=torch.float32, device=k.device)
-    if ws is None:
-        n = lte_workspace_bytes(OP_SCORES, s, c)
-        ws = torch.empty(n, dtype=torch.uint8, device=k.device) if n > 0 else False
-    wp, wn = (None, 0) if ws is False else (_ptr(ws, torch.uint8), ws.numel())
-    _check("lte_scores", lib().lte_scores(ctypes.addressof(s), ctypes.addressof(c), _ptr(k), _ptr(v),
-                                          _ptr(z, torch.float32), _ptr(r, torch.float32), wp, wn, _stream()))
-    return z
+    return (_native or _load()).scores(s, c, k, v, z, r, ws)
 
 
 def lte_select(s, z, idx=None, cnt=None, ncand=None):
     """z [B,H,T] fp32 -> idx [B,H,R] int32 ascending (-1 unused), cnt [B,H] int32."""
-    dev = z.device
-    if idx is None:
-        idx = torch.empty((s.B, s.H, s.R), dtype=torch.int32, device=dev)
-    if cnt is None:
-        cnt = torch.empty((s.B, s.H), dtype=torch.int32, device=dev)
-    _check("lte_select", lib().lte_select(ctypes.addressof(s), _ptr(z, torch.float32), _ptr(idx, torch.int32),
-                                          _ptr(cnt, torch.int32), _ptr(ncand, torch.int32), None, 0, _stream()))
-    return idx, cnt
-
-
-RULE_LEARNED, RULE_UNIFORM, RULE_ACCUM_ATTN = 0, 1, 2
+    return (_native or _load()).select_rule(s, RULE_LEARNED, z, idx, cnt, ncand, z)
 
 
 def lte_select_rule(s, rule, score=None, idx=None, cnt=None, ncand=None, device=None):
     """lte_select under one of the rules: RULE_LEARNED (score = z), RULE_UNIFORM (no score), RULE_ACCUM_ATTN (score = the
     accumulated attention of lte_attn_colsum)."""
-    dev = score.device if score is not None else (device or torch.device("cuda"))
-    if idx is None:
-        idx = torch.empty((s.B, s.H, s.R), dtype=torch.int32, device=dev)
-    if cnt is None:
-        cnt = torch.empty((s.B, s.H), dtype=torch.int32, device=dev)
-    _check("lte_select_rule", lib().lte_select_rule(ctypes.addressof(s), int(rule), _ptr(score, torch.float32), _ptr(idx, torch.int32),
-                                                    _ptr(cnt, torch.int32), _ptr(ncand, torch.int32), None, 0, _stream()))
-    return idx, cnt
+    like = score if score is not None else torch.empty((), device=device or torch.device("cuda"))
+    return (_native or _load()).select_rule(s, int(rule), score, idx, cnt, ncand, like)
 
 
 def lte_attn_colsum(s, q, k, lse, idx, cnt, a=None):
     """Accumulated attention a [B,H,T] fp32 of every key under the attention lte_attn_prefill ran with this list."""
-    if a is None:
-        a = torch.empty((s.B, s.H, s.T), dtype=torch.float32, device=q.device)
-    _check("lte_attn_colsum", lib().lte_attn_colsum(ctypes.addressof(s), _ptr(q), _ptr(k), _ptr(lse, torch.float32),
-                                                    _ptr(idx, torch.int32), _ptr(cnt, torch.int32), _ptr(a, torch.float32), _stream()))
-    return a
+    return (_native or _load()).attn_colsum(s, q, k, lse, idx, cnt, a)
 
 
 def lte_attn_prefill(s, q, k, v, idx, cnt, o=None, lse=None, ws=None):
     """q [B,H*group,T,d], k, v [B,H,T,d], retained list -> o [B,H*group,T,d], lse [B,H*group,T] fp32.
     ws: uint8 tensor of lte_workspace_bytes(OP_PREFILL, s) bytes (the retained rows are compacted into it and fetched
     as tiles), allocated here when None; False: no workspace (the kernels gather the retained rows themselves)."""
-    if o is None:
-        o = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((s.B, s.H * max(s.group, 1), s.T), dtype=torch.float32, device=q.device)
-    if ws is None:
-        need = lte_workspace_bytes(OP_PREFILL, s, None)
-        ws = torch.empty(need, dtype=torch.uint8, device=q.device) if need > 0 else False
-    wp, wn = (None, 0) if ws is False else (_ptr(ws), ws.numel())
-    _check("lte_attn_prefill", lib().lte_attn_prefill(ctypes.addressof(s), _ptr(q), _ptr(k), _ptr(v),
-                                                      _ptr(idx, torch.int32), _ptr(cnt, torch.int32), _ptr(o),
-                                                      _ptr(lse, torch.float32), wp, wn, _stream()))
-    return o, lse
+    return (_native or _load()).attn_prefill(s, q, k, v, idx, cnt, o, lse, ws)
 
 
 def lte_cache_bytes(s):
@@ -225,24 +186,14 @@ def lte_cache_bytes(s):
 def lte_cache_init(s, c, k=None, v=None, z=None, idx=None, cnt=None, cache=None):
     """Decode cache holding the state after the T-token prompt (T = 0: empty cache)."""
     if cache is None:
-        dev = k.device if k is not None else torch.device("cuda")
-        cache = torch.empty(lte_cache_bytes(s), dtype=torch.uint8, device=dev)
-    _check("lte_cache_init", lib().lte_cache_init(ctypes.addressof(s), ctypes.addressof(c), _ptr(k), _ptr(v),
-                                                  _ptr(z), _ptr(idx), _ptr(cnt), _ptr(cache), _stream()))
-    return cache
+        cache = torch.empty(lte_cache_bytes(s), dtype=torch.uint8, device=k.device if k is not None else torch.device("cuda"))
+    return (_native or _load()).cache_init(s, c, k, v, z, idx, cnt, cache)
 
 
 def lte_attn_decode(s, c, cache, q1, k1, v1, o1=None, lse1=None):
     """One decode step: q1 [B,H*group,d], k1, v1 [B,H,d] -> o1 [B,H*group,d], lse1 [B,H*group]; the cache is
     updated in place."""
-    if o1 is None:
-        o1 = torch.empty_like(q1)
-    if lse1 is None:
-        lse1 = torch.empty((s.B, s.H * max(s.group, 1)), dtype=torch.float32, device=q1.device)
-    _check("lte_attn_decode", lib().lte_attn_decode(ctypes.addressof(s), ctypes.addressof(c), _ptr(cache),
-                                                    _ptr(q1), _ptr(k1), _ptr(v1), _ptr(o1),
-                                                    _ptr(lse1, torch.float32), _stream()))
-    return o1, lse1
+    return (_native or _load()).attn_decode(s, c, cache, q1, k1, v1, o1, lse1)
 
 
 def lte_attn_prefill_chunk(s, c, cache, n_past, q, k, v, o=None, lse=None, ws=None, streaming=False):
@@ -250,17 +201,7 @@ def lte_attn_prefill_chunk(s, c, cache, n_past, q, k, v, o=None, lse=None, ws=No
     tokens) -> o, lse of the chunk's queries; the cache is advanced to n_past + T tokens in place.  ws: uint8 tensor of
     lte_workspace_bytes(OP_CHUNK or OP_CHUNK_STREAM, s, c) bytes, allocated here when None.  streaming=True: the
     token-by-token reading (what decode steps compute, also where the cap binds)."""
-    if o is None:
-        o = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((s.B, s.H * max(s.group, 1), s.T), dtype=torch.float32, device=q.device)
-    if ws is None:
-        ws = torch.empty(max(lte_workspace_bytes(OP_CHUNK_STREAM if streaming else OP_CHUNK, s, c), 256), dtype=torch.uint8, device=q.device)
-    _check("lte_attn_prefill_chunk", lib().lte_attn_prefill_chunk_ex(ctypes.addressof(s), ctypes.addressof(c), _ptr(cache),
-                                                                     ctypes.c_int32(int(n_past)), _ptr(q), _ptr(k), _ptr(v),
-                                                                     _ptr(o), _ptr(lse, torch.float32), CHUNK_STREAMING if streaming else 0,
-                                                                     _ptr(ws), ws.numel(), _stream()))
-    return o, lse
+    return (_native or _load()).attn_prefill_chunk(s, c, cache, int(n_past), q, k, v, o, lse, ws, CHUNK_STREAMING if streaming else 0)
 
 
 class LteLambdaCfg(ctypes.Structure):
@@ -270,13 +211,7 @@ class LteLambdaCfg(ctypes.Structure):
 
 def lte_sparsity_stats(s, z, lam=None, ws=None):
     """Eq. 7 statistics: z [B,H,T] -> count [H] (batch mean of tokens above the threshold), penalty [1]."""
-    count = torch.empty((s.H,), dtype=torch.float32, device=z.device)
-    penalty = torch.empty((1,), dtype=torch.float32, device=z.device)
-    if ws is None:
-        ws = torch.empty(max(lte_workspace_bytes(OP_STATS, s, None), 256), dtype=torch.uint8, device=z.device)
-    _check("lte_sparsity_stats", lib().lte_sparsity_stats(ctypes.addressof(s), _ptr(z, torch.float32), _ptr(lam, torch.float32),
-                                                          _ptr(count), _ptr(penalty), _ptr(ws), ws.numel(), _stream()))
-    return count, penalty
+    return (_native or _load()).sparsity_stats(s, z, lam, ws)
 
 
 def lte_lambda_update(lam, cbar, count, step, cfg=None, group=None):
@@ -296,42 +231,19 @@ def lte_lambda_update(lam, cbar, count, step, cfg=None, group=None):
 def lte_cache_score(s, c, cache, ws=None):
     """Three-layer stack only: score the ring tokens whose receptive field is complete (call at least every W - 13
     decode steps).  ws: uint8 tensor of lte_workspace_bytes(OP_DECODE, s, c) bytes, allocated here when None."""
-    if ws is None:
-        ws = torch.empty(max(lte_workspace_bytes(OP_DECODE, s, c), 256), dtype=torch.uint8, device=cache.device)
-    _check("lte_cache_score", lib().lte_cache_score(ctypes.addressof(s), ctypes.addressof(c), _ptr(cache), _ptr(ws),
-                                                    ws.numel(), _stream()))
+    (_native or _load()).cache_score(s, c, cache, None, None, ws)
 
 
 def lte_cache_score_unrope(s, c, cache, rope_cos, rope_sin, ws=None):
     """lte_cache_score for a cache that holds rotated keys: rope_cos, rope_sin [positions, d/2] fp32 on the device."""
-    if ws is None:
-        ws = torch.empty(max(lte_workspace_bytes(OP_DECODE, s, c), 256), dtype=torch.uint8, device=cache.device)
-    _check("lte_cache_score_unrope", lib().lte_cache_score_unrope(ctypes.addressof(s), ctypes.addressof(c), _ptr(cache),
-                                                                  _ptr(rope_cos, torch.float32), _ptr(rope_sin, torch.float32),
-                                                                  int(rope_cos.shape[0]), _ptr(ws), ws.numel(), _stream()))
+    (_native or _load()).cache_score(s, c, cache, rope_cos, rope_sin, ws)
 
 
 def lte_attn_bwd(s, c, q, k, v, o, lse, dO, z, idx, cnt, lam=None, flags=BWD_CNN_INPUT_GRAD, want_dbias=True,
                  ws=None):
     """Backward with the straight-through surrogate -> dq, dk, dv, dw [H,K,2d], dbias [H] (or None).  With the
     three-layer stack (conv_stack) dw and dbias are flat, packed like the parameters: use unpack_stack_grads."""
-    dq, dk, dv = torch.empty_like(q), torch.empty_like(k), torch.empty_like(v)
-    if c.n_layers == 3:
-        d = s.d
-        dw = torch.empty((s.H * (d * 3 * 2 * d + (d // 2) * 3 * d + (d // 4) * 3 * (d // 2) + d // 4),), dtype=torch.float32, device=q.device)
-        db = torch.empty((s.H * (d + d // 2 + d // 4 + 1),), dtype=torch.float32, device=q.device) if want_dbias else None
-    else:
-        dw = torch.empty((s.H, c.kernel, 2 * s.d), dtype=torch.float32, device=q.device)
-        db = torch.empty((s.H,), dtype=torch.float32, device=q.device) if want_dbias else None
-    need = lte_workspace_bytes(OP_BWD, s, c)
-    if ws is None:
-        ws = torch.empty(max(need, 16), dtype=torch.uint8, device=q.device)
-    _check("lte_attn_bwd", lib().lte_attn_bwd(
-        ctypes.addressof(s), ctypes.addressof(c), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse, torch.float32),
-        _ptr(dO), _ptr(z, torch.float32), _ptr(idx, torch.int32), _ptr(cnt, torch.int32),
-        _ptr(lam, torch.float32), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dw), _ptr(db), flags, _ptr(ws),
-        ws.numel(), _stream()))
-    return dq, dk, dv, dw, db
+    return (_native or _load()).attn_bwd(s, c, q, k, v, o, lse, dO, z, idx, cnt, lam, flags, bool(want_dbias), ws, None, False)
 
 
 def unpack_stack_grads(H, d, dw, db=None):
@@ -356,13 +268,4 @@ def lte_attn_bwd_static(s, c, q, k, v, o, lse, dO, z, idx, cnt, lam=None, flags=
     allocate device memory.  ``outs`` = (dq, dk, dv, dw, dbias) preallocated by the caller makes the whole call
     allocation-free; when omitted they are created here for convenience.  Shapes needing more scratch than
     STATIC_SCRATCH_BYTES raise LteError (status -3)."""
-    if outs is None:
-        outs = (torch.empty_like(q), torch.empty_like(k), torch.empty_like(v),
-                torch.empty((s.H, c.kernel, 2 * s.d), dtype=torch.float32, device=q.device),
-                torch.empty((s.H,), dtype=torch.float32, device=q.device))
-    dq, dk, dv, dw, db = outs
-    _check("lte_attn_bwd_static", lib().lte_attn_bwd_static(
-        ctypes.addressof(s), ctypes.addressof(c), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse, torch.float32),
-        _ptr(dO), _ptr(z, torch.float32), _ptr(idx, torch.int32), _ptr(cnt, torch.int32),
-        _ptr(lam, torch.float32), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dw), _ptr(db), flags, _stream()))
-    return dq, dk, dv, dw, db
+    return (_native or _load()).attn_bwd(s, c, q, k, v, o, lse, dO, z, idx, cnt, lam, flags, True, None, None if outs is None else tuple(outs), True)
