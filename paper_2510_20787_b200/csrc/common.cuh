@@ -131,6 +131,8 @@ int launch_sparsity_stats(const Params& p, const float* z, const float* lambda, 
                           cudaStream_t st);
 int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k1, const void* v1, void* o1,
                      float* lse1, cudaStream_t st);
+int launch_decode_mma(const Params& p, void* cache, const void* q1, const void* k1, const void* v1, void* o1, float* lse1,
+                      cudaStream_t st);
 int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, const void* v1, void* o1,
                   float* lse1, cudaStream_t st);
 size_t bwd_workspace_bytes(const Params& p, uint32_t flags);

@@ -1,5 +1,5 @@
-// Decode step over the constant-size per-head cache (Fig. 3; Section 3.1.3, decoding paragraph),
-// plus the kernel that builds the cache after a prompt.
+// Decode step over the constant-size per-head cache (Fig. 3; Section 3.1.3, decoding paragraph) for fp32 caches (bf16:
+// decode_mma.cu and decode_tc.cu), plus the kernel that builds the cache after a prompt.
 //
 // One block per (b,h).  All key/value traffic is issued up front as 128-bit coalesced loads of the
 // OLD cache rows (their addresses depend on nothing but the layout), while one warp reads the head's
@@ -815,8 +815,6 @@ __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ c
     int32_t* meta = reinterpret_cast<int32_t*>(blk + L.off_meta);
     const int n = meta[0], cnt_old = meta[1];
     const int slot = n % W, p = n - W, half = K / 2;
-    // element ch of row r (the swizzled layout permutes the 16-byte pieces of a row)
-    auto pos_of = [&](int r, int ch) { return L.swz ? ((((ch >> 3) ^ (r & 7)) << 3) | (ch & 7)) : ch; };
 
     // ---- the token leaving the window is offered to the pool (same rule as the step kernels) ----
     int dst = -1, cnt_new = cnt_old;
@@ -866,7 +864,7 @@ __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ c
                     const float wk = cw[((size_t)h * K + t) * 2 * D + ch], wv = cw[((size_t)h * K + t) * 2 * D + D + ch];
                     float kx, vx;
                     if (pos == n) { kx = to_f(k1[(size_t)bh * D + ch]); vx = to_f(v1[(size_t)bh * D + ch]); }
-                    else { const int r = pos % W; kx = to_f(Kc[(size_t)r * D + pos_of(r, ch)]); vx = to_f(Vc[(size_t)r * D + pos_of(r, ch)]); }
+                    else { const int r = pos % W; kx = to_f(Kc[(size_t)r * D + ch]); vx = to_f(Vc[(size_t)r * D + ch]); }
                     a += wk * kx + wv * vx;
                 }
             }
@@ -877,17 +875,17 @@ __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ c
     // ---- moves: the popped row into its pool row, the new key/value into the ring slot ----
     uint4 mv = make_uint4(0, 0, 0, 0), nw = mv;
     const bool mover = tid < 2 * PIECES;
-    const int pc = tid % PIECES;                               // logical 16-byte piece of the row
+    const int pc = tid % PIECES;                               // 16-byte piece of the row
     if (mover) {
         const uint4* src = reinterpret_cast<const uint4*>(tid < PIECES ? Kc : Vc);
-        mv = src[(size_t)slot * PIECES + (L.swz ? (pc ^ (slot & 7)) : pc)];
+        mv = src[(size_t)slot * PIECES + pc];
         nw = reinterpret_cast<const uint4*>((tid < PIECES ? k1 : v1) + (size_t)bh * D)[pc];
     }
     __syncthreads();                                           // the ring rows the taps read are still the old ones up to here
     if (mover) {
         uint4* dstp = reinterpret_cast<uint4*>(tid < PIECES ? Kc : Vc);
-        if (dst >= 0) dstp[(size_t)(W + dst) * PIECES + (L.swz ? (pc ^ ((W + dst) & 7)) : pc)] = mv;
-        dstp[(size_t)slot * PIECES + (L.swz ? (pc ^ (slot & 7)) : pc)] = nw;
+        if (dst >= 0) dstp[(size_t)(W + dst) * PIECES + pc] = mv;
+        dstp[(size_t)slot * PIECES + pc] = nw;
     }
     if (tid == 0) {
         if (dst >= 0) { zc[W + dst] = zp; pidx[dst] = p; }
@@ -951,11 +949,10 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
     const int a_lo = min(rank * share, rows_all), rows = min(a_lo + share, rows_all) - a_lo;   // this block's rows: a_lo + [0, rows)
     float* s_log = att_sm;
     float* s_out = att_sm + (size_t)ATT_Q * rows;
-    // this thread's piece of list entry a: cache row (ring rows first, then pool rows) and the piece's place in it (the
-    // swizzled layout permutes the pieces of a row)
+    // this thread's piece of list entry a (ring rows first, then pool rows)
     auto piece_of = [&](int a) {
         const int r = a_lo + a < n_ring ? a_lo + a : W + (a_lo + a - n_ring);
-        return (size_t)r * LPR + (L.swz ? (seg ^ (r & 7)) : seg);
+        return (size_t)r * LPR + seg;
     };
     for (int g0 = g_first; g0 < G; g0 += ATT_Q) {
         const int nq = G - g0 < ATT_Q ? G - g0 : ATT_Q;
@@ -1110,9 +1107,7 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
 static int launch_decode_step(const Params& p, void* cache, const void* q1, const void* k1, const void* v1, void* o1, float* lse1,
                               cudaStream_t st)
 {
-    if (p.W + p.R > MAX_ROWS) return LTE_ERR_UNSUPPORTED;
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    if (L.swz) return launch_decode_tc(p, cache, q1, k1, v1, o1, lse1, st);   // bf16, d = 64, W+R <= 256: tensor-core kernel
     const BulkSmem bp = bulk_smem_plan(L, p.W, p.R);
     const size_t bulk_smem = bp.total;
     const bool bulk = bulk_smem <= 73 * 1024 && p.K <= 2 * (DT / 32);   // three blocks per SM still fit
@@ -1132,20 +1127,11 @@ static int launch_decode_step(const Params& p, void* cache, const void* q1, cons
             p.zthr, p.scale, p.G);                                                                                     \
     } while (0)
     if (bulk) {
-        if (p.dtype == LTE_BF16) {
-            switch (p.d) {
-                case 32: LTE_BULK(__nv_bfloat16, 32); break;
-                case 64: LTE_BULK(__nv_bfloat16, 64); break;
-                case 128: LTE_BULK(__nv_bfloat16, 128); break;
-                default: return LTE_ERR_UNSUPPORTED;
-            }
-        } else {
-            switch (p.d) {
-                case 32: LTE_BULK(float, 32); break;
-                case 64: LTE_BULK(float, 64); break;
-                case 128: LTE_BULK(float, 128); break;
-                default: return LTE_ERR_UNSUPPORTED;
-            }
+        switch (p.d) {
+            case 32: LTE_BULK(float, 32); break;
+            case 64: LTE_BULK(float, 64); break;
+            case 128: LTE_BULK(float, 128); break;
+            default: return LTE_ERR_UNSUPPORTED;
         }
         return cuda_status(cudaGetLastError());
     }
@@ -1154,20 +1140,11 @@ static int launch_decode_step(const Params& p, void* cache, const void* q1, cons
     decode_kernel<T, D><<<p.B * p.H, DT, 0, st>>>((unsigned char*)cache, L, (const T*)q1, (const T*)k1, (const T*)v1, \
                                                   (T*)o1, lse1, p.w, p.bias, p.H, p.W, p.R, p.sink, p.K, p.zthr,   \
                                                   p.scale, p.G)
-    if (p.dtype == LTE_BF16) {
-        switch (p.d) {
-            case 32: LTE_GO(__nv_bfloat16, 32); break;
-            case 64: LTE_GO(__nv_bfloat16, 64); break;
-            case 128: LTE_GO(__nv_bfloat16, 128); break;
-            default: return LTE_ERR_UNSUPPORTED;
-        }
-    } else {
-        switch (p.d) {
-            case 32: LTE_GO(float, 32); break;
-            case 64: LTE_GO(float, 64); break;
-            case 128: LTE_GO(float, 128); break;
-            default: return LTE_ERR_UNSUPPORTED;
-        }
+    switch (p.d) {
+        case 32: LTE_GO(float, 32); break;
+        case 64: LTE_GO(float, 64); break;
+        case 128: LTE_GO(float, 128); break;
+        default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_GO
     return cuda_status(cudaGetLastError());
@@ -1178,9 +1155,15 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
 {
     Params ps = p;
     if (p.stack) ps.K = 0;                               // the stack is scored outside the step (lte_cache_score)
+    if (p.W + p.R > MAX_ROWS) return LTE_ERR_UNSUPPORTED;
+    if (p.dtype == LTE_BF16) {
+        // one query head and a block of 256 rows that is a tcgen05 operand as it stands: 29 us at 2,048 heads, where the other
+        // kernel takes 35; everything else in bf16 goes through mma.sync
+        if (p.G <= 1 && cache_layout(p.d, p.W, p.R, p.dtype).swz) return launch_decode_tc(ps, cache, q1, k1, v1, o1, lse1, st);
+        return launch_decode_mma(ps, cache, q1, k1, v1, o1, lse1, st);
+    }
     if (p.G <= 1) return launch_decode_step(ps, cache, q1, k1, v1, o1, lse1, st);
     // grouped queries: one kernel updates the head's cache block and then serves all query heads of the group from it
-    if (p.W + p.R > MAX_ROWS) return LTE_ERR_UNSUPPORTED;
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
     const size_t att_smem = sizeof(float) * ((size_t)ATT_Q * (p.W + p.R) + (size_t)(DT / 32) * ATT_Q * p.d);
     // blocks per key/value head (a cluster): more than one only while there are fewer blocks than SMs and a share keeps 256 rows
@@ -1205,20 +1188,11 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
                                p.W, p.G, p.scale, 0, (const T*)k1, (const T*)v1, p.w, p.bias, p.H, p.R, p.sink, ps.K,    \
                                p.zthr) != cudaSuccess) return LTE_ERR_CUDA;                                             \
     } while (0)
-    if (p.dtype == LTE_BF16) {
-        switch (p.d) {
-            case 32: LTE_ATT(__nv_bfloat16, 32); break;
-            case 64: LTE_ATT(__nv_bfloat16, 64); break;
-            case 128: LTE_ATT(__nv_bfloat16, 128); break;
-            default: return LTE_ERR_UNSUPPORTED;
-        }
-    } else {
-        switch (p.d) {
-            case 32: LTE_ATT(float, 32); break;
-            case 64: LTE_ATT(float, 64); break;
-            case 128: LTE_ATT(float, 128); break;
-            default: return LTE_ERR_UNSUPPORTED;
-        }
+    switch (p.d) {
+        case 32: LTE_ATT(float, 32); break;
+        case 64: LTE_ATT(float, 64); break;
+        case 128: LTE_ATT(float, 128); break;
+        default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_ATT
     return cuda_status(cudaGetLastError());
