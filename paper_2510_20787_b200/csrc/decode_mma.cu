@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
     constexpr int SPLIT = NW == max_warps(D) ? MAX_SPLIT : 1;  // (only the largest blocks come in clusters)
     __shared__ float s_in[2][SPLIT > 1 ? MQ * D : 1];
     __shared__ __align__(16) float s_ml[2][SPLIT][MQ][2];  // the cluster's shares of this block's output elements (by pass parity)
-    __shared__ float s_tap[kMaxTaps], s_wz[NW];
+    __shared__ float s_tap[kMaxTaps];
+    __shared__ uint32_t s_wkey[NW];
     __shared__ int s_wpos[NW], s_wslot[NW];
     cg::cluster_group cluster = cg::this_cluster();
     const int nsplit = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
@@ -147,10 +148,11 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
     };
     load_q(0);
     // the pool's logits and positions, before it is known whether the decision needs them
-    float pz[2];
-    int pp[2];
+    constexpr int PRE = NT < 256 ? 4 : 2;
+    float pz[PRE];
+    int pp[PRE];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < PRE; ++u) {
         const int m = tid + u * NT;
         pz[u] = m < R ? zc[W + m] : INFINITY;
         pp[u] = m < R ? pidx[m] : -1;
@@ -198,32 +200,30 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
         if (cnt_old < R) { dst = cnt_old; cnt_new = cnt_old + 1; }
         else if (p >= sink) {
             // worst entry: lowest logit, the youngest among equals, never a sink entry
-            float wz = INFINITY; int wpos = -1, wslot = -1;
+            uint32_t key = 0xffffffffu;                        // (order_key of a number; -0 counts as 0)
+            int wpos = -1, wslot = -1;
+            auto offer = [&](float z, int pos, int m) {
+                const uint32_t k = order_key(z + 0.f);
+                if (m < cnt_old && pos >= sink && (k < key || (k == key && pos > wpos))) { key = k; wpos = pos; wslot = m; }
+            };
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int m = tid + u * NT;
-                if (m < cnt_old && pp[u] >= sink && (pz[u] < wz || (pz[u] == wz && pp[u] > wpos))) { wz = pz[u]; wpos = pp[u]; wslot = m; }
+            for (int u = 0; u < PRE; ++u) offer(pz[u], pp[u], tid + u * NT);
+            for (int m = tid + PRE * NT; m < cnt_old; m += NT) offer(zc[W + m], pidx[m], m);
+            auto worst = [&]() {                               // over the warp; every lane then has it
+                const uint32_t kmin = __reduce_min_sync(0xffffffffu, key);
+                const int pmax = __reduce_max_sync(0xffffffffu, key == kmin ? wpos : -1);
+                const unsigned who = __ballot_sync(0xffffffffu, key == kmin && wpos == pmax);
+                wslot = __shfl_sync(0xffffffffu, wslot, __ffs(who) - 1);
+                key = kmin; wpos = pmax;
+            };
+            worst();
+            if (NW > 1) {
+                if (lane == 0) { s_wkey[wid] = key; s_wpos[wid] = wpos; s_wslot[wid] = wslot; }
+                __syncthreads();
+                key = lane < NW ? s_wkey[lane] : 0xffffffffu; wpos = lane < NW ? s_wpos[lane] : -1; wslot = lane < NW ? s_wslot[lane] : -1;
+                worst();
             }
-            for (int m = tid + 2 * NT; m < cnt_old; m += NT) {
-                const int pos = pidx[m];
-                const float zm = zc[W + m];
-                if (pos >= sink && (zm < wz || (zm == wz && pos > wpos))) { wz = zm; wpos = pos; wslot = m; }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float oz = __shfl_xor_sync(0xffffffffu, wz, o);
-                const int op = __shfl_xor_sync(0xffffffffu, wpos, o), os = __shfl_xor_sync(0xffffffffu, wslot, o);
-                if (os >= 0 && (wslot < 0 || oz < wz || (oz == wz && op > wpos))) { wz = oz; wpos = op; wslot = os; }
-            }
-            if (lane == 0) { s_wz[wid] = wz; s_wpos[wid] = wpos; s_wslot[wid] = wslot; }
-            __syncthreads();
-            wz = s_wz[0]; wpos = s_wpos[0]; wslot = s_wslot[0];
-#pragma unroll
-            for (int w2 = 1; w2 < NW; ++w2) {
-                const float oz = s_wz[w2]; const int op = s_wpos[w2], os = s_wslot[w2];
-                if (os >= 0 && (wslot < 0 || oz < wz || (oz == wz && op > wpos))) { wz = oz; wpos = op; wslot = os; }
-            }
-            if (wslot >= 0 && zp > wz) dst = wslot;
+            if (wslot >= 0 && order_key(zp + 0.f) > key) dst = wslot;
         }
     }
     const int masked_ring = p >= 0 && dst < 0 ? slot : -2;     // the popped row counts iff the pool takes it ...
