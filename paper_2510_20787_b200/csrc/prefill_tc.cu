@@ -1,140 +1,172 @@
-// Prefill attention on the 5th-generation tensor cores (Section 3.1.3, "Cached prefilling and decoding").
+// Prefill attention on the 5th-generation tensor cores for bf16, d = 64 and d = 32 (Section 3.1.3, "Cached prefilling and
+// decoding").
 //
-// Persistent CTAs (two per SM): each walks work items, an item being one 128-query tile of one (b,h), so that the
-// loads of the next item are in flight while the current one is finished (a CTA per item spent a third of its life
-// waiting for its first tiles).  Four softmax warps, one MMA-issue warp and one load warp.  Key/value tiles of 64
-// rows come from two sources, as in the paper's two-stage loop: (1) the contiguous window span, staged by TMA
-// (cp.async.bulk.tensor, 128-byte swizzle); (2) the retained rows already out of the tile's window, gathered
-// row by row with cp.async into the same swizzled layout (idx is ascending, so the entries a query may see are
-// a prefix of the list and every mask is a column range).  Per tile:
-//   S = Q K^T      tcgen05.mma (kind::f16, bf16 in, fp32 out) into one of two TMEM buffers, so the next two
-//                  S tiles are computed while the softmax of the current one runs
-//   softmax        thread r owns query row r = TMEM lane r: tcgen05.ld, range mask (whole 32-column chunks are
-//                  skipped or taken unmasked when the warp's rows allow it), running max / sum in fp32 (exp2 with
-//                  the scale folded in), P written as bf16 back into TMEM over the S buffer it came from
-//   O += P V       tcgen05.mma with P as the TMEM A operand and V as an MN-major shared-memory operand,
-//                  accumulated in TMEM; the accumulator is rescaled
-//                  in place only when a row's maximum grows by more than 2^8 (lazy rescale)
-// Tiles are numbered through all items of a CTA (g); stage, buffer and barrier phase of a tile follow from g alone.
-// Every mbarrier wait is bounded; a wait that runs out records a status word and the kernel still terminates.
+// Bound by the instruction stream of the softmax warps (no pipe is full: exponential unit 50 %, issue 46 %, tensor pipe 28 %),
+// so work is paid once per 128 keys, spread over 16 warps per SM, and nothing waits that need not:
+//   work      Two CTAs per SM; an item is a 128-query tile of one head.  Key/value tiles of 128 rows come by TMA, first the window
+//             span, then the head's retained rows that any of the item's rows may see (compacted beforehand where the caller
+//             brought a workspace; otherwise the load warp gathers them row by row into the same swizzled layout).  Eight softmax
+//             warps (two threads per row, 64 columns each), one warp issuing the products, one issuing the loads.
+//   S(g) = Q K^T    one buffer: the softmax has taken all of S(g) when half of its exponentials are done, and S(g+1) is computed
+//             under the other half (P has columns of its own, so nothing else holds the buffer).  TMEM: S [0,128), P [128,192),
+//             O [192,256)
+//   softmax   mask from positions (32-column chunks are skipped or taken unmasked where the warp's rows allow); the row maximum
+//             of the two halves is exchanged through shared memory; the reference follows it only when it grew by 2^8 (lazy
+//             rescale); exp2 with the scale folded in; P as bf16 into TMEM
+//   O += P V  P as the TMEM A operand, V as the MN-major shared-memory operand; O is read and stored under the next item's first tile
+// How many retained entries a row sees: the load warp finds an item's place in the list (a 32-way search) and hands out, one
+// item ahead, a bit map of the entries that fall between the limits of the item's first and last row.
+// Tiles are numbered through all items of a CTA (g); stage, buffer and barrier phase follow from that number, and the loads
+// and products of the next item run under the current one.  Every mbarrier wait is bounded; one that runs out records a
+// status word and the kernel still terminates.
+//
+// Measured (B200, the call with a workspace): 1,024 query heads x 4,096, W = 768, R = 512 half used: 1.43 ms (601 TFLOP/s), before
+// 2.10; 64 heads x 4,096, W = R = 128: 51 us, before 66.  The steps, at an eighth of the first shape: four warps with 64-key
+// tiles 275 us; one thread per row, 128-key tiles 242; two threads per row 223; dynamic items 203; O stored under the next item
+// 190.  Tried there and slower: rolled 32-column loops (214), column bounds carried from tile to tile and a vote in place of the
+// exchange of maxima (209), one thread per row with dynamic items (213), the two streams of an SM taking turns at the
+// exponential unit (328), a quarter of the exponentials as polynomials on the multiply-add pipe (207).
+//
+// d = 32 runs the same kernel: the tensor maps describe 32-column rows with a 64-column box, the copy engine fills the upper
+// half of every tile row with zeros, and only the first 32 output columns are stored.
 #include "tc_common.cuh"
 
 namespace lte {
 
 __device__ StatusWord g_prefill_status = LTE_STATUS_INIT;         // 0 = fine; otherwise the code of the wait that gave up
 
-// -DLTE_PROFILE: cycle counters of the row threads' phases (lane 0 of warp 0 of every CTA), added up over all CTAs;
-// PP(c) charges the time since the previous mark to phase c.  The product build does not define it.
-#ifdef LTE_PROFILE
-__device__ unsigned long long g_pprof[16];
-__device__ unsigned long long g_pprof_cta[1024 * 2];           // per CTA: globaltimer at kernel entry and at the end of the row loop
-#define PP_DECL long long pp_t = clock64(); long long pp_a[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0}
-#define PP(c) do { const long long pp_n = clock64(); pp_a[c] += pp_n - pp_t; pp_t = pp_n; } while (0)
-#define PP_COUNT(c, n) do { pp_a[c] += (n); } while (0)
-#define PP_FLUSH() do { if (warp == 0 && lane == 0) { _Pragma("unroll") for (int pp_i = 0; pp_i < 16; ++pp_i) atomicAdd(&g_pprof[pp_i], (unsigned long long)pp_a[pp_i]); \
-    unsigned long long gt; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(gt)); if (blockIdx.x < 1024) g_pprof_cta[blockIdx.x * 2 + 1] = gt; } } while (0)
-#else
-#define PP_DECL
-#define PP(c)
-#define PP_COUNT(c, n)
-#define PP_FLUSH()
-#endif
-
 namespace {
 
-constexpr int BM = 128, BN = 64, NTHREADS = 192;
+constexpr int BM = 128, BN = 128, D = 64, NTHREADS = 320;         // warps 0-7 softmax, 8 products, 9 loads
 using namespace tc;
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_prefill_status); }
 
-template <int D> struct Smem {
-    static constexpr int SUB = D / 64;                        // 64-column (128-byte) sub-tiles per row
-    static constexpr int KST = 3;                             // key stages
-    static constexpr int VST = D == 64 ? 3 : 2;               // value stages
-    static constexpr int QTILE = BM * D * 2;                  // [128][D] bf16
-    static constexpr int KVTILE = BN * D * 2;                 // [64][D] bf16
-    static constexpr int OFF_Q = 0;
-    static constexpr int OFF_K = QTILE;
-    static constexpr int OFF_V = OFF_K + KST * KVTILE;
-    // d = 64: the row sums are taken by the tensor core as well: PV gets 16 extra B columns of ones, so column D of
-    // the accumulator is sum_j P_ij of exactly the (bf16-rounded) probabilities the product used.  The ones live in one
-    // more 64-column group, LBO away from the value tile.
-    static constexpr bool ONES = D == 64;
-    static constexpr int OFF_ONES = OFF_V + VST * KVTILE;     // [64][64] bf16 ones (8 KB), d = 64 only
-    static constexpr int OFF_BAR = OFF_ONES + (ONES ? BN * 128 : 0);   // mbarriers, tmem slot
-    static constexpr int OFF_LV = OFF_BAR + 256;              // STREAM: the leave times of a retained tile, [4 warps][64]
-    static constexpr int BYTES = OFF_LV + 4 * 64 * 4;
-    static constexpr uint32_t TMEM_COLS = 256;                // S0: [0,64)  S1: [64,128)  O: [128, 128+D) (+16 row-sum columns)
+template <bool STREAM> struct Smem {
+    static constexpr int TILE = 128 * D * 2;                  // [128][64] bf16: Q, K and V tiles alike
+    static constexpr int QST = 2, KST = 2, VST = 2;
+    static constexpr int OFF_Q = 0, OFF_K = QST * TILE, OFF_V = OFF_K + KST * TILE;
+    static constexpr int OFF_BAR = OFF_V + VST * TILE;
+    static constexpr int OFF_INFO = OFF_BAR + 256;            // ring of four items' Info
+    static constexpr int OFF_X = OFF_INFO + 4 * 64;           // row maxima on their way to the other half (by tile parity), [2][2][128]
+    static constexpr int OFF_L = OFF_X + 2 * 2 * BM * 4;      // row sums of the two halves (by item parity), [2][2][128]
+    static constexpr int OFF_LV = OFF_L + 2 * 2 * BM * 4;     // STREAM: the leave times of a retained tile, [8 warps][64]
+    static constexpr int BYTES = OFF_LV + (STREAM ? 8 * 64 * 4 : 0);
 };
+constexpr uint32_t TMEM_COLS = 256, S_COL = 0, P_COL = 128, O_COL = 192;
 
-// One work item: a 128-query tile of one (b,h).
-struct Item {
-    int bh, bhk, i0, i_hi, j_start, n_win;              // bh: query head (b, h, g); bhk: its key/value head (b, h)
-};
-// Items are numbered from the last query tile of every (b,h) down to the first: later query tiles see more retained
-// rows and cost more, and a CTA takes items n, n + grid, n + 2 grid, ... so every CTA gets one item of each cost band
-// (largest first), which balances the static schedule.
-__device__ __forceinline__ Item decode_item(int item, int n_qt, int n_bh, int Tlen, int W, int G, int qoff)
+// An item: a 128-query tile of one (b,h).  Items are numbered from the last query tile of every head down to the first: later
+// tiles see more retained rows and cost more.  The grid has a block per item, but a block that has run out of work takes the
+// next block that has not started (cluster launch control) instead of leaving, so items are handed out in order, largest
+// first, to whoever is free: dealt out beforehand, the blocks finished up to 30 % apart (159 to 219 us).
+struct Item { int bh, bhk, i0, j_start, n_win, n_tiles, item; };   // bh: query head (b, h, g); bhk: its key/value head (b, h)
+struct Args { int n_items, n_qt, n_bh, Tlen, W, G, qoff; };
+// What the load warp tells the others about an item.  Row x of the item (0 .. 127) sees before[x / 32] entries and those of
+// bits[x / 32] below bit x % 32.
+struct Info { uint32_t before[4], bits[4]; int n_tiles, item; };   // item = -1: there is none
+
+__device__ __forceinline__ Item item_of(const Args& a, int item)
 {
     Item it;
-    const int r = item / n_bh;
-    it.bh = item - r * n_bh;
-    it.bhk = it.bh / G;                                 // the G query heads of a key/value head are adjacent
-    it.i0 = qoff + (n_qt - 1 - r) * BM;                 // positions; the query tensors start at position qoff
-    it.i_hi = min(it.i0 + BM - 1, Tlen - 1);
-    it.j_start = max(it.i0 - W + 1, 0);
-    it.n_win = (it.i_hi - it.j_start + 1 + BN - 1) / BN;
+    const int r = item / a.n_bh;
+    it.item = item;
+    it.bh = item - r * a.n_bh;
+    it.bhk = it.bh / a.G;
+    it.i0 = a.qoff + (a.n_qt - 1 - r) * BM;                    // positions; the query tensors start at position qoff
+    const int i_hi = min(it.i0 + BM - 1, a.Tlen - 1);
+    it.j_start = max(it.i0 - a.W + 1, 0);
+    it.n_win = (i_hi - it.j_start + BN) / BN;
+    it.n_tiles = it.n_win;                                     // until the item's Info is there
     return it;
 }
-// Entries of the ascending list id[0, n) that are <= lim (whole warp).
-__device__ __forceinline__ int count_le(const int32_t* id, int n, int lim, int lane)
+// The item's Info from the head's ascending list id[0, n) (whole warp).
+__device__ __forceinline__ Info make_info(const Args& a, const Item& it, const int32_t* id, int n, int lane)
 {
-    int c = 0;
-    for (int e0 = 0; e0 < n; e0 += 32) {
-        const int e = e0 + lane < n ? id[e0 + lane] : 0x7fffffff;
-        const unsigned bal = __ballot_sync(0xffffffffu, e <= lim);
-        c += __popc(bal);
-        if (bal != 0xffffffffu) break;
+    Info f;
+    const int last = min(it.i0 + BM - 1, a.Tlen - 1) - it.i0, lim0 = it.i0 - a.W;   // rows 0 .. last see positions <= lim0 .. lim0 + last
+    int lo = 0, hi = lim0 + last < 0 ? 0 : n;                  // entries <= lim0: in [lo, hi]
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step - 1;
+        const int c = __popc(__ballot_sync(0xffffffffu, at < hi && id[min(at, n - 1)] <= lim0));
+        lo += c * step;
+        if (step == 1) break;
+        hi = min(hi, lo + step - 1);
     }
-    return c;
+    lo = min(lo, n);
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {                              // at most 127 entries lie in (lim0, lim0 + 127]
+        const int e = lo + u * 32 + lane, x = e < n && lim0 + last >= 0 ? id[e] - lim0 - 1 : BM;
+        const uint32_t bit = x >= 0 && x < last ? 1u << (x & 31) : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] |= (x >> 5) == k ? bit : 0u;
+    }
+    uint32_t sum = (uint32_t)lo;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        f.bits[k] = __reduce_or_sync(0xffffffffu, w[k]);
+        f.before[k] = sum;
+        sum += __popc(f.bits[k]);
+    }
+    f.n_tiles = it.n_win + ((int)sum + BN - 1) / BN;
+    return f;
 }
 
-// Warps 0-3 (128 threads): softmax (thread r owns query row r) and the cp.async gathers of retained rows.
-// Warp 4, one lane: every tcgen05.mma.  Warp 5, one lane: the TMA loads of Q and of the window tiles (a single
-// lane doing both was the bottleneck: its dependent instruction stream took longer per tile than the softmax).
-// They meet on mbarriers (g = the tile's number within the CTA, it = the item's):
-//   bar_q                    Q of item `it` has landed (TMA)                          phase it
-//   bar_qf    (commit)       the last S product of item `it` has completed            phase it     MMA -> load
-//   bar_of    (4 arrivals)   O of item `it` has been read out of TMEM                 phase it     softmax -> MMA
-//   bar_s[b]  (commit)       S(g) is in TMEM buffer b = g & 1                         phase g >> 1 MMA -> softmax
-//   bar_p     (4 arrivals)   P(g) is in TMEM, over S(g)                               phase g      softmax -> MMA
-//   bar_pv    (commit)       PV(g) has completed                                      phase g      MMA -> softmax
-//   bar_g[b]  (4 arrivals)   gathers issued before the top of tile g have landed      phase g >> 1 softmax -> MMA
-//   bar_k[s], bar_v[s]       TMA transaction barriers of the window tiles (one phase per TMA use of the stage)
-//   bar_kf[s], bar_vf[s]     (commit) the MMA that read the stage's tile g has completed   phase g / stages   MMA -> load
-// S(g+1) and S(g+2) are computed while the softmax of tile g runs; loads run two to three tiles ahead, across items.
-// COMPACT: the retained rows were copied into contiguous tensors [B*H][R][d] beforehand (tmKc, tmVc), so retained tiles are
-// TMA boxes like the window tiles and the softmax warps gather nothing (a compile-time variant: the gather code costs the
-// softmax loop instruction-cache room even where it does not run).
-// STREAM (with COMPACT): the list is every entry that is retained at some query of a chunk, and entry e is gone from query
-// leave[e] on (the streaming reading of a chunk): retained tiles take one more mask, leave > query position.
-template <int D, bool COMPACT, bool STREAM>
+// Walks a CTA's tiles in order: tile t of its n-th item is tile g.
+struct Cursor {
+    Item it;
+    int n = 0, t = 0;
+    uint32_t g = 0;
+    bool live = true;
+    __device__ __forceinline__ void advance() { ++g; if (++t == it.n_tiles) { t = 0; ++n; } }
+};
+// Asks for a block of this grid that has not started (the answer, 16 bytes, arrives on the barrier).
+__device__ __forceinline__ void ask_for_block(uint32_t answer, uint32_t bar) {
+    mbar_expect_tx(bar, 16);
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
+}
+__device__ __forceinline__ int block_from(uint32_t answer) {   // its index, or -1
+    uint32_t ok, x;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tld.shared.b128 h, [%2];\n\tclusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, _, _, _}, h;\n\t}"
+                 : "=r"(ok), "=r"(x) : "r"(answer) : "memory");
+    return ok ? (int)x : -1;
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                   "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory");
+}
+
+// Barriers (g = tile number, n = item number within the CTA):
+//   bar_q[b], bar_qf[b]   Q of item n has landed in buffer b = n & 1 (TMA) / the item's last S is complete (commit)    phase n >> 1
+//   bar_k[s], bar_v[s]    TMA of tile g into stage s = g % stages                                                       phase g / stages
+//   bar_kf[s], bar_vf[s]  (commit) the product that read the stage's tile is complete                                   phase g / stages
+//   bar_s    (commit)     S(g) is in TMEM                   bar_sf (8 arrivals)  S(g) is in registers                   phase g
+//   bar_p    (8 arrivals) P(g) is in TMEM, and PV(g-1) has been awaited               bar_pv (commit)  PV(g) is complete  phase g
+//   bar_of   (8 arrivals) O of item n has been read out                                                                phase n
+//   bar_i[n & 3]          Info of item n is in the ring (1 arrival): a slot is written again only after the last S of item n + 2
+//                         is complete, by when every warp is past item n                                       phase n >> 2
+//   bar_c                 the answer to the n-th request for a block                                           phase n
+//   GATHER: bar_gk[s], bar_gv[s] (32 arrivals, by cp.async completion) a gathered tile is in stage s; the TMA barriers then only
+//           count the window tiles (their phases are followed by toggling)
+// STREAM: the list is every entry that is retained at some query of a chunk, and entry e is gone from query leave[e] on (the
+// streaming reading of a chunk): retained tiles take one more mask, leave > query position.
+template <bool GATHER, bool STREAM>
 __global__ void __launch_bounds__(NTHREADS, 2)
-prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                  const __grid_constant__ CUtensorMap tmV,
-                  const __grid_constant__ CUtensorMap tmKc, const __grid_constant__ CUtensorMap tmVc,
-                  const __nv_bfloat16* __restrict__ kg,
-                  const __nv_bfloat16* __restrict__ vg, __nv_bfloat16* __restrict__ og, const int32_t* __restrict__ idx,
-                  const int32_t* __restrict__ cnt, const int32_t* __restrict__ leave, float* __restrict__ lse, int Tlen,
-                  int W, int R, float scale, int n_qt, int n_bh, int G, int qoff, int dg)
+prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                  const __grid_constant__ CUtensorMap tmKc, const __grid_constant__ CUtensorMap tmVc, const Args args,
+                  const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* __restrict__ vg, const int32_t* __restrict__ idx,
+                  const int32_t* __restrict__ cnt, __nv_bfloat16* __restrict__ og, float* __restrict__ lse,
+                  const int32_t* __restrict__ leave, int R, float scale, int dg)
 {
-    const int n_items = n_qt * n_bh;
-#ifdef LTE_PROFILE
-    if (threadIdx.x == 0 && blockIdx.x < 1024) { unsigned long long gt; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(gt)); g_pprof_cta[blockIdx.x * 2] = gt; }
-#endif
-    using S = Smem<D>;
-    constexpr int SUB = S::SUB, KST = S::KST, VST = S::VST;
-    constexpr uint32_t TMEM_COLS = S::TMEM_COLS;
-    constexpr uint32_t O_COL = 2 * BN;
+    using S = Smem<STREAM>;
+    constexpr int KST = S::KST, VST = S::VST, TILE = S::TILE;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if ((base & 1023u) != 0) {                                 // the swizzled tiles need 1024-byte alignment
@@ -142,41 +174,28 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         return;
     }
     const uint32_t sQ = base + S::OFF_Q, sK = base + S::OFF_K, sV = base + S::OFF_V;
-    const uint32_t bar_q = base + S::OFF_BAR;
-    const uint32_t bar_k0 = bar_q + 8;                         // 3 slots
-    const uint32_t bar_v0 = bar_q + 32;                        // 3 slots
-    const uint32_t bar_s0 = bar_q + 56;                        // 2 slots
-    const uint32_t bar_g0 = bar_q + 72;                        // 2 slots
-    const uint32_t bar_p = bar_q + 88, bar_pv = bar_q + 96;
-    const uint32_t bar_kf0 = bar_q + 104;                      // 3 slots: K stage free
-    const uint32_t bar_vf0 = bar_q + 128;                      // 3 slots: V stage free
-    const uint32_t bar_qf = bar_q + 152, bar_of = bar_q + 160;
-    const uint32_t tmem_slot = bar_q + 168;
-    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + S::OFF_BAR + 168);
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t bar_q = base + S::OFF_BAR, bar_qf = bar_q + 16, bar_k = bar_q + 32, bar_kf = bar_q + 48, bar_v = bar_q + 64, bar_vf = bar_q + 80;
+    const uint32_t bar_s = bar_q + 96, bar_sf = bar_q + 104, bar_p = bar_q + 112, bar_pv = bar_q + 120, bar_of = bar_q + 128, bar_c = bar_q + 136;
+    const uint32_t bar_i = bar_q + 144, bar_gk = bar_q + 176, bar_gv = bar_q + 192, tmem_slot = bar_q + 208, answer = bar_q + 224;   // (answer: 16 bytes)
+    auto slot = [&](int n) { return reinterpret_cast<volatile Info*>(smem_raw + S::OFF_INFO + (n & 3) * 64); };
+    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + S::OFF_BAR + 208);
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (so the compiler knows warp is uniform)
 
     if (tid == 0) {
-        mbar_init(bar_q, 1);
 #pragma unroll
-        for (int s2 = 0; s2 < 3; ++s2) {
-            mbar_init(bar_k0 + 8 * s2, 1); mbar_init(bar_v0 + 8 * s2, 1);
-            mbar_init(bar_kf0 + 8 * s2, 1); mbar_init(bar_vf0 + 8 * s2, 1);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(bar_q + 8 * s, 1); mbar_init(bar_qf + 8 * s, 1);
+            mbar_init(bar_k + 8 * s, 1); mbar_init(bar_kf + 8 * s, 1);
+            mbar_init(bar_v + 8 * s, 1); mbar_init(bar_vf + 8 * s, 1);
+            mbar_init(bar_gk + 8 * s, 32); mbar_init(bar_gv + 8 * s, 32);
         }
-        mbar_init(bar_s0, 1); mbar_init(bar_s0 + 8, 1);
-        // the softmax warps arrive once per warp (lane 0, after __syncwarp): 128 arrivals on one barrier word serialise
-        mbar_init(bar_g0, 4); mbar_init(bar_g0 + 8, 4);
-        mbar_init(bar_p, 4); mbar_init(bar_pv, 1);
-        mbar_init(bar_qf, 1); mbar_init(bar_of, 4);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) mbar_init(bar_i + 8 * s, 1);
+        mbar_init(bar_c, 1);
+        mbar_init(bar_s, 1); mbar_init(bar_sf, 8); mbar_init(bar_p, 8); mbar_init(bar_pv, 1); mbar_init(bar_of, 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) tmem_alloc(tmem_slot, TMEM_COLS);
-    if (S::ONES && tid < 128) {                                // 8 KB of bf16 1.0: 64 bytes per thread, once per CTA
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + S::OFF_ONES + tid * 64 + u * 16), "r"(0x3F803F80u) : "memory");
-        fence_proxy_async();
-    }
+    if (warp == 8) tmem_alloc(tmem_slot, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -184,527 +203,424 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     pdl_launch_dependents();
     pdl_wait();                                                // everything above ran beside the previous kernel's tail
 
-    if (warp == 5) {
-        // ================================= load warp (lane 0 issues) ========================================
-        uint32_t g = 0;                                        // tiles of the items before this one
-        int it = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
-            const Item w = decode_item(item, n_qt, n_bh, Tlen, W, G, qoff);
-            if (lane == 0) {
-                // Q: its buffer is free once the previous item's last S product has completed
-                if (it > 0) mbar_wait(bar_qf, (it - 1) & 1, 12);
-                mbar_expect_tx(bar_q, S::QTILE);
+    if (warp == 9) {
+        // ================================= load warp ========================================================
+        // Keys run one tile ahead of values: K(g+1) is wanted at the start of softmax g, V(g) at its end.  The whole warp walks
+        // the loop, lane 0 issues the copies.
+        Cursor ck, cv;
+        int pos_k[4], pos_v[4];                                // GATHER: positions of the rows of the key cursor's tile, of the tile before it
+        auto fetch_positions = [&]() {                         // (of a retained tile)
+            const int e0 = (ck.t - ck.it.n_win) * BN, n = cnt[ck.it.bhk];
+            const int32_t* id = idx + (size_t)ck.it.bhk * R;
 #pragma unroll
-                for (int sb = 0; sb < SUB; ++sb) tma_load_3d(sQ + sb * 16384, &tmQ, sb * 64, w.i0 - qoff, w.bh, bar_q);
-            }
-            // tiles, each into its stage as soon as the MMA that read the stage's previous tile has completed
-            auto load_tiles = [&](int t_lo, int t_hi) {
-                for (int t = t_lo; t < t_hi; ++t) {
-                    const uint32_t gg = g + t;
-                    const bool win = t < w.n_win;
-                    const int y = win ? w.j_start + t * BN : (t - w.n_win) * BN;
-                    const uint32_t ks = gg % KST, vs = gg % VST;
-                    if (gg >= (uint32_t)KST) mbar_wait(bar_kf0 + 8 * ks, (gg / KST - 1) & 1u, 6);
-                    mbar_expect_tx(bar_k0 + 8 * ks, S::KVTILE);
-#pragma unroll
-                    for (int sb = 0; sb < SUB; ++sb)
-                        tma_load_3d(sK + ks * S::KVTILE + sb * 8192, win ? &tmK : &tmKc, sb * 64, y, w.bhk, bar_k0 + 8 * ks);
-                    if (gg >= (uint32_t)VST) mbar_wait(bar_vf0 + 8 * vs, (gg / VST - 1) & 1u, 8);
-                    mbar_expect_tx(bar_v0 + 8 * vs, S::KVTILE);
-#pragma unroll
-                    for (int sb = 0; sb < SUB; ++sb)
-                        tma_load_3d(sV + vs * S::KVTILE + sb * 8192, win ? &tmV : &tmVc, sb * 64, y, w.bhk, bar_v0 + 8 * vs);
-                }
-            };
-            if (lane == 0) load_tiles(0, w.n_win);
-            // the item's retained tiles also take tile numbers (counted after the window loads are on their way)
-            const int n_ret_tiles = (count_le(idx + (size_t)w.bhk * R, cnt[w.bhk], w.i_hi - W, lane) + BN - 1) / BN;
-            if (COMPACT && lane == 0) load_tiles(w.n_win, w.n_win + n_ret_tiles);
-            g += w.n_win + n_ret_tiles;
-        }
-    } else if (warp == 4) {
-        // ================================= MMA warp (lane 0 issues) =========================================
-        // The whole warp walks the loop and waits on the barriers; only the tcgen05 instructions are guarded by the lane
-        // test.  Descriptors and addresses are then computed in convergent code (the compiler can keep them in uniform
-        // registers), which roughly halves the issue cost of an MMA compared with a loop run by one lane alone.
-        constexpr uint32_t IDESC_S = instr_desc(BM, BN, false);
-        constexpr uint32_t IDESC_O = S::ONES ? instr_desc(BM, D + 16, true) : instr_desc(BM, D, true);
-        // descriptor words: lo = (address >> 4) | LBO field, hi = SBO field | version | swizzle mode
-        constexpr uint32_t HI = (1024u >> 4) | (1u << 14) | (2u << 29);
-        const uint32_t q_lo = (sQ >> 4) | (1u << 16), k_lo = (sK >> 4) | (1u << 16);
-        uint32_t g = 0, g_waited = 0;                          // tiles before this item; bar_g phases consumed
-        uint32_t k_par = 0, v_par = 0;                         // TMA barrier parities (bit per stage)
-        int it = 0;
-        // tiles of an item (whole warp: the count of visible list entries takes global loads)
-        auto item_tiles = [&](int item) {
-            if (item >= n_items) return 0;
-            const Item w = decode_item(item, n_qt, n_bh, Tlen, W, G, qoff);
-            return w.n_win + (count_le(idx + (size_t)w.bhk * R, cnt[w.bhk], w.i_hi - W, lane) + BN - 1) / BN;
+            for (int u = 0; u < 4; ++u) pos_k[u] = e0 + u * 32 + lane < n ? id[e0 + u * 32 + lane] : -1;
         };
-        int n_tiles_next = item_tiles(blockIdx.x);
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
-            const Item w = decode_item(item, n_qt, n_bh, Tlen, W, G, qoff);
-            const int n_tiles = n_tiles_next;
-            int ts = 0;                                        // S products of this item issued so far
-            // gathers issued before the top of tile gg have landed
-            auto need_g = [&](uint32_t gg) {
-                while (g_waited <= gg) { mbar_wait(bar_g0 + 8 * (g_waited & 1), (g_waited >> 1) & 1, 10); ++g_waited; }
-            };
-            auto mma_s = [&]() {                           // S of the item's tile ts
-                const uint32_t gg = g + ts, ks = gg % KST;
-                if (COMPACT || ts < w.n_win) { mbar_wait(bar_k0 + 8 * ks, (k_par >> ks) & 1u, 2); k_par ^= 1u << ks; }
-                else need_g(g + max(ts - (KST == 2 ? 1 : 2), 0));   // a gathered K tile: issued in tile ts - KST or in the item's prologue
-                tc_fence_after();
-                const uint32_t kb = k_lo + ks * (S::KVTILE >> 4);
-                const uint32_t dcol = tmem + (gg & 1) * BN;
-                ++ts;
+        auto load = [&](const Cursor& c, bool is_v, uint32_t dst, uint32_t bar, uint32_t gbar) {
+            const bool win = c.t < c.it.n_win;
+            if (!GATHER || win) {
                 if (lane == 0) {
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma(dcol, desc64(q_lo + (kk >> 2) * 1024 + (kk & 3) * 2, HI), desc64(kb + (kk >> 2) * 512 + (kk & 3) * 2, HI),
-                             IDESC_S, kk > 0);
-                    umma_commit(bar_s0 + 8 * (gg & 1));
-                    umma_commit(bar_kf0 + 8 * ks);             // the K stage is free once this S has completed
-                    if (ts == n_tiles) umma_commit(bar_qf);    // and so is Q after the item's last S
+                    mbar_expect_tx(bar, TILE);
+                    tma_load_3d(dst, is_v ? (win ? &tmV : &tmVc) : (win ? &tmK : &tmKc), 0, win ? c.it.j_start + c.t * BN : (c.t - c.it.n_win) * BN, c.it.bhk, bar);
                 }
-                __syncwarp();
-            };
-
-            mbar_wait(bar_q, it & 1, 1);
-            mma_s();                                           // tile 0 is always a window tile
-            if (n_tiles > 1) mma_s();
-            // the next item's tile count, fetched while the softmax of this item's first tile runs
-            n_tiles_next = item_tiles(item + gridDim.x);
-            {
-                for (int t = 0; t < n_tiles; ++t) {
-                    const uint32_t gg = g + t, vs = gg % VST;
-                    if (!COMPACT) need_g(gg);
-                    if (COMPACT || t < w.n_win) { mbar_wait(bar_v0 + 8 * vs, (v_par >> vs) & 1u, 4); v_par ^= 1u << vs; }
-                    // value operand: the second 64-column group of B is the next sub-tile (d = 128) or the block of
-                    // ones (d = 64, LBO = its distance from the value stage)
-                    const uint32_t va = sV + vs * S::KVTILE;
-                    const uint32_t vb = (va >> 4) | ((S::ONES ? ((base + S::OFF_ONES - va) >> 4) : (8192u >> 4)) << 16);
-                    if (t == 0 && it > 0) mbar_wait(bar_of, (it - 1) & 1, 13);   // the previous item's O has been read out
-                    mbar_wait(bar_p, gg & 1, 7);
-                    tc_fence_after();
-                    if (lane == 0) {
+            } else {                                           // 8 lanes per row copy its 16-byte pieces; rows past the list are zero
+                const __nv_bfloat16* src = (is_v ? vg : kg) + (size_t)c.it.bhk * args.Tlen * dg;
+                const int sub = lane & 7;
 #pragma unroll
-                        for (int kk = 0; kk < BN / 16; ++kk)
-                            umma_ts(tmem + O_COL, tmem + (gg & 1) * BN + kk * 8, desc64(vb + kk * 128, HI), IDESC_O, (t > 0 || kk > 0) ? 1u : 0u);
-                        umma_commit(bar_pv);
-                        umma_commit(bar_vf0 + 8 * vs);         // the V stage is free once PV has completed
-                    }
+                for (int ps = 0; ps < 32; ++ps) {
+                    const int row = ps * 4 + (lane >> 3), at = __shfl_sync(0xffffffffu, is_v ? pos_v[ps >> 3] : pos_k[ps >> 3], row & 31);
+                    const bool real = at >= 0 && sub * 8 < dg; // (columns past the head dimension are zero-filled)
+                    cp_async16(dst + row * 128 + ((sub ^ (row & 7)) << 4), src + (real ? (size_t)at * dg + sub * 8 : 0), real ? 16u : 0u);
+                }
+                cp_async_arrive(gbar);
+            }
+        };
+        auto load_k = [&]() {
+            const bool first = ck.t == 0;
+            if (first) {
+                // the item: this block's own, then whatever the last request brought; the next request goes out at once
+                int item = blockIdx.x;
+                if (ck.n > 0) {
+                    mbar_wait(bar_c, (ck.n - 1) & 1, 17);
+                    item = launch_aborted(&g_prefill_status) ? -1 : block_from(answer);   // (a lost launch ends)
+                    fence_proxy_async();                       // the answer has been read before the next one is written
                     __syncwarp();
-                    // S two tiles ahead, into the S buffer the softmax has just released
-                    if (ts < n_tiles) mma_s();
+                }
+                if (item >= 0 && lane == 0) ask_for_block(answer, bar_c);
+                const uint32_t b = ck.n & 1;
+                if (ck.n >= 2) mbar_wait(bar_qf + 8 * b, ((ck.n >> 1) - 1) & 1, 12);
+                if (item < 0) {
+                    ck.live = false;
+                    if (lane == 0) { slot(ck.n)->item = -1; mbar_arrive(bar_i + 8 * (ck.n & 3)); }
+                    return;
+                }
+                ck.it = item_of(args, item);
+                if (lane == 0) {
+                    mbar_expect_tx(bar_q + 8 * b, TILE);
+                    tma_load_3d(sQ + b * TILE, &tmQ, 0, ck.it.i0 - args.qoff, ck.it.bh, bar_q + 8 * b);
                 }
             }
-            g += n_tiles;
+            if (GATHER && ck.t >= ck.it.n_win) fetch_positions();   // (never tile 0)
+            const uint32_t s = ck.g % KST;
+            if (ck.g >= (uint32_t)KST) mbar_wait(bar_kf + 8 * s, (ck.g / KST - 1) & 1u, 6);
+            load(ck, false, sK + s * TILE, bar_k + 8 * s, bar_gk + 8 * s);
+            if (first) {                                       // tile 0 is a window tile; the list is looked up while it is on its way
+                const Info f = make_info(args, ck.it, idx + (size_t)ck.it.bhk * R, R > 0 ? cnt[ck.it.bhk] : 0, lane);
+                ck.it.n_tiles = f.n_tiles;
+                if (lane == 0) {
+                    volatile Info* o = slot(ck.n);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) { o->before[k] = f.before[k]; o->bits[k] = f.bits[k]; }
+                    o->n_tiles = f.n_tiles; o->item = ck.it.item;
+                    mbar_arrive(bar_i + 8 * (ck.n & 3));
+                }
+            }
+            ck.advance();
+        };
+        load_k();
+        for (;;) {
+            if (GATHER) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) pos_v[u] = pos_k[u];
+            }
+            if (ck.live) load_k();
+            if (cv.t == 0) {                                   // (written by this warp's lane 0: the key cursor is in or past this item)
+                __syncwarp();
+                const int item = slot(cv.n)->item;
+                if (item < 0) break;
+                cv.it = item_of(args, item);
+                cv.it.n_tiles = slot(cv.n)->n_tiles;
+            }
+            const uint32_t s = cv.g % VST;
+            if (cv.g >= (uint32_t)VST) mbar_wait(bar_vf + 8 * s, (cv.g / VST - 1) & 1u, 8);
+            load(cv, true, sV + s * TILE, bar_v + 8 * s, bar_gv + 8 * s);
+            cv.advance();
+        }
+        __syncwarp();
+    } else if (warp == 8) {
+        // ================================= MMA warp (lane 0 issues; the whole warp walks the loop) ==============
+        constexpr uint32_t IDESC_S = instr_desc(BM, BN, false), IDESC_O = instr_desc(BM, D, true);
+        const uint32_t q_lo = desc_lo(sQ, 16), k_lo = desc_lo(sK, 16), v_lo = desc_lo(sV, 16);
+        Cursor cs, cp;
+        uint32_t par = 0;                                      // GATHER: parities of bar_k (bits 0, 1), bar_gk (2, 3), bar_v (4, 5), bar_gv (6, 7)
+        auto landed = [&](uint32_t bar, uint32_t gbar, bool win, uint32_t s, uint32_t phase, int bit, int gbit, int code) {
+            if (!GATHER) { mbar_wait(bar + 8 * s, phase, code); return; }
+            const int at = (win ? bit : gbit) + (int)s;
+            mbar_wait((win ? bar : gbar) + 8 * s, (par >> at) & 1u, code);
+            par ^= 1u << at;
+            if (!win) fence_proxy_async();                     // the copies were generic-proxy writes
+        };
+        auto enter = [&](Cursor& c) {                          // the cursor's next item out of the ring
+            const int item = __shfl_sync(0xffffffffu, slot(c.n)->item, 0);
+            c.live = item >= 0;
+            if (!c.live) return;
+            c.it = item_of(args, item);
+            c.it.n_tiles = __shfl_sync(0xffffffffu, slot(c.n)->n_tiles, 0);
+        };
+        auto mma_s = [&]() {
+            const uint32_t s = cs.g % KST, b = cs.n & 1;
+            if (cs.t == 0) {
+                mbar_wait(bar_i + 8 * (cs.n & 3), (cs.n >> 2) & 1, 9);
+                enter(cs);
+                if (!cs.live) return;
+                mbar_wait(bar_q + 8 * b, (cs.n >> 1) & 1, 1);
+            }
+            landed(bar_k, bar_gk, cs.t < cs.it.n_win, s, (cs.g / KST) & 1u, 0, 2, 2);
+            if (cs.g > 0) mbar_wait(bar_sf, (cs.g - 1) & 1, 3);    // the previous tile's S is in registers
+            tc_fence_after();
+            if (lane == 0) {
+                const uint32_t qd = q_lo + b * (TILE >> 4), kd = k_lo + s * (TILE >> 4);
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk) umma(tmem + S_COL, desc64(qd + kk * 2, kDescHi), desc64(kd + kk * 2, kDescHi), IDESC_S, kk > 0);
+                umma_commit(bar_s);
+                umma_commit(bar_kf + 8 * s);
+                if (cs.t == cs.it.n_tiles - 1) umma_commit(bar_qf + 8 * b);
+            }
             __syncwarp();
+            cs.advance();
+        };
+        mma_s();
+        for (;;) {
+            if (cs.live) mma_s();
+            if (cp.t == 0) { enter(cp); if (!cp.live) break; }
+            const uint32_t s = cp.g % VST;
+            landed(bar_v, bar_gv, cp.t < cp.it.n_win, s, (cp.g / VST) & 1u, 4, 6, 4);
+            if (cp.t == 0 && cp.n > 0) mbar_wait(bar_of, (cp.n - 1) & 1, 13);   // the previous item's O has been read out
+            mbar_wait(bar_p, cp.g & 1, 7);
+            tc_fence_after();
+            if (lane == 0) {
+                const uint32_t vd = v_lo + s * (TILE >> 4);
+#pragma unroll
+                for (int kk = 0; kk < BN / 16; ++kk)
+                    umma_ts(tmem + O_COL, tmem + P_COL + kk * 8, desc64(vd + kk * 128, kDescHi), IDESC_O, (cp.t > 0 || kk > 0) ? 1u : 0u);
+                umma_commit(bar_pv);
+                umma_commit(bar_vf + 8 * s);
+            }
+            __syncwarp();
+            cp.advance();
         }
     } else {
         // =================================== softmax warps ==================================================
+        // Two threads per row: thread r of warps 0-3 takes columns [0, 64) of every tile, thread r of warps 4-7 columns [64, 128).
+        const int hf = warp >> 2, row = tid & 127, c0 = hf * 64;
         const float c2 = scale * 1.4426950408889634f;          // logits are handled in the log2 domain: x = s * c2
-        const uint32_t lane_base = ((uint32_t)(warp * 32)) << 16;   // this warp's TMEM lanes
-        const int g_row = tid >> 3, g_sub = tid & 7;           // gathers: 8 lanes per row, 16 rows per pass
-        uint32_t g = 0;                                        // tiles of the items before this one
-        int it = 0;
-        // the list length and the first 128 list entries of an item are fetched one item ahead, so that the visible
-        // counts at the start of an item wait for no load (entries past cnt are never used: the length guards them)
-        int pf_cnt = 0, pf_e[4] = {0, 0, 0, 0};
-        auto prefetch_list = [&](int item) {
-            if (item < n_items) {
-                const Item w = decode_item(item, n_qt, n_bh, Tlen, W, G, qoff);
-                pf_cnt = cnt[w.bhk];
+        const uint64_t c2_2 = pack2(c2, c2);
+        const uint32_t trow = tmem + (((uint32_t)((warp & 3) * 32)) << 16);   // this warp's TMEM lanes
+        const uint32_t s_col = trow + S_COL + c0, p_col = trow + P_COL + hf * 32, o_col = trow + O_COL + hf * 32;
+        float* x_mine = reinterpret_cast<float*>(smem_raw + S::OFF_X) + hf * BM + row;
+        const float* x_other = reinterpret_cast<float*>(smem_raw + S::OFF_X) + (hf ^ 1) * BM + row;
+        auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory"); };   // the two warps of these rows
+        uint32_t g = 0;
+        int n = 0;
+        // A row's output is read and stored while the next item's first tile is under way (its PV has then long completed).
+        float last_m = 0.f;
+        int last_row = -1;                                     // row of o and lse (-1: none)
+        auto epilogue = [&](int item_no) {
+            const float* lsum = reinterpret_cast<const float*>(smem_raw + S::OFF_L) + (item_no & 1) * 2 * BM + row;
+            const float l = lsum[0] + lsum[BM], inv = 1.f / l;
+            __nv_bfloat16* orow = og + (size_t)last_row * dg + hf * 32;   // 64 contiguous bytes of the row
 #pragma unroll
-                for (int u = 0; u < 4; ++u) pf_e[u] = u * 32 + lane < R ? idx[(size_t)w.bhk * R + u * 32 + lane] : 0x7fffffff;
-            }
-        };
-        prefetch_list(blockIdx.x);
-        PP_DECL;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
-            const Item w = decode_item(item, n_qt, n_bh, Tlen, W, G, qoff);
-            const int bh = w.bh, bhk = w.bhk, n_win = w.n_win, j_start = w.j_start;
-            const int32_t* id = idx + (size_t)bhk * R;
-            const int n_ret = pf_cnt;
-            const int i = w.i0 + tid;                          // this thread's query row
-            // retained entries visible to this row.  The rows of a warp are consecutive and the list is ascending, so
-            // nvis(row) = #{idx <= lim of lane 0} + #{idx in (lim of lane 0, lim of this lane]}: a ballot count plus a
-            // 31-bit map of the entries that fall between the warp's first and last limit.  No block barrier.
-            const int lim = min(i, Tlen - 1) - W;              // entry visible iff idx <= lim
-            const int lim_max = w.i_hi - W;
-            const int lim0 = __shfl_sync(0xffffffffu, lim, 0), lim31 = __shfl_sync(0xffffffffu, lim, 31);
-            int nvis = 0, nv_max = 0;                          // nv_max: entries visible to the tile's last row
-            {
-                uint32_t bits = 0;
-                for (int e0 = 0; e0 < n_ret; e0 += 128) {
-                    int e[4];
-                    if (e0 == 0) {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) e[u] = u * 32 + lane < n_ret ? pf_e[u] : 0x7fffffff;
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) e[u] = e0 + u * 32 + lane < n_ret ? id[e0 + u * 32 + lane] : 0x7fffffff;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        nvis += __popc(__ballot_sync(0xffffffffu, e[u] <= lim0));
-                        nv_max += __popc(__ballot_sync(0xffffffffu, e[u] <= lim_max));
-                        const bool in = e[u] > lim0 && e[u] <= lim31;
-                        bits |= __reduce_or_sync(0xffffffffu, in ? 1u << (e[u] - lim0 - 1) : 0u);
-                    }
-                    if (__shfl_sync(0xffffffffu, e[3], 31) > lim_max) break;   // nothing further is visible to any row
-                }
-                nvis += __popc(bits & ((1u << (lim - lim0)) - 1u));
-            }
-            const int n_tiles = n_win + (nv_max + BN - 1) / BN;
-            const int nvis_first = __shfl_sync(0xffffffffu, nvis, 0), nvis_last = __shfl_sync(0xffffffffu, nvis, 31);
-            prefetch_list(item + gridDim.x);
-            PP(0); PP_COUNT(14, 1); PP_COUNT(15, n_tiles);
-
-            // gather of one retained tile (t = its number within the item): 8 lanes per row copy its 16-byte chunks
-            // (coalesced reads, conflict-free swizzled writes); rows past the visible prefix are zero-filled
-            auto gather_rows = [&](int t, int (&rows4)[4]) {   // row positions of this thread's 4 rows of tile t
-#pragma unroll
-                for (int ps = 0; ps < 4; ++ps) {
-                    const int e = (t - n_win) * BN + ps * 16 + g_row;
-                    rows4[ps] = (t >= n_win && t < n_tiles && e < nv_max) ? id[e] : -1;
-                }
-            };
-            auto gather_issue = [&](int t, bool is_v, const int (&rows4)[4]) {
-                if (t >= n_win && t < n_tiles) {
-                    const uint32_t st = is_v ? ((g + t) % VST) : ((g + t) % KST);
-                    const uint32_t dst = (is_v ? sV : sK) + st * S::KVTILE;
-#pragma unroll
-                    for (int ps = 0; ps < 4; ++ps) {
-                        const int row = ps * 16 + g_row;
-                        const bool ok = rows4[ps] >= 0;
-                        const __nv_bfloat16* src = (is_v ? vg : kg) + ((size_t)bhk * Tlen + (ok ? rows4[ps] : 0)) * dg;
-#pragma unroll
-                        for (int c = g_sub; c < D / 8; c += 8) {
-                            const uint32_t off = (c >> 3) * 8192 + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-                            const bool real = ok && c * 8 < dg;    // columns past the head dimension are zero-filled
-                            cp_async16(dst + off, src + (real ? c * 8 : 0), real ? 16u : 0u);
-                        }
-                    }
-                }
-                cp_async_commit();
-            };
-            // prologue gathers: the first KST key tiles and VST value tiles, where those are retained tiles.  Their
-            // stages are free: every product of the previous item has completed (its last bar_s and bar_pv were awaited).
-            if (!COMPACT && n_win < KST) {
-                int rows4[4];
-                for (int t = 0; t < KST; ++t) { gather_rows(t, rows4); gather_issue(t, false, rows4); }
-                for (int t = 0; t < VST; ++t) { gather_rows(t, rows4); gather_issue(t, true, rows4); }
-            }
-            float m_run = -INFINITY, l_run = 0.f;              // running max (log2 domain) and sum (sum only if !ONES)
-            bool gathered = !COMPACT && n_win < KST;           // some gather of this item may be in flight (warp-uniform)
-
-            for (int t = 0; t < n_tiles; ++t) {
-                const uint32_t gg = g + t;
-                // row positions for this tile's two gathers, fetched first so their latency hides under the softmax
-                // (all of this tile's gather work sits behind warp-uniform tests: most tiles of a short list have none)
-                const bool k_gather = !COMPACT && t + KST >= n_win && t + KST < n_tiles;
-                const bool v_gather = !COMPACT && t > 0 && t + VST - 1 >= n_win && t + VST - 1 < n_tiles;
-                int rk[4], rv[4];
-                if (k_gather) gather_rows(t + KST, rk);
-                if (v_gather) gather_rows(t + VST - 1, rv);
-                if (!COMPACT) {
-                    // gathers issued before this point have landed (all of them, or all but the latest value tile)
-                    if (gathered) {
-                        if (VST == 3) cp_async_wait<1>(); else cp_async_wait<0>();
-                        fence_proxy_async();
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_g0 + 8 * (gg & 1));
-                }
-
-                // column range this row may see in the tile
-                int c_lo, c_hi;
-                if (t < n_win) {
-                    const int jt0 = j_start + t * BN;
-                    c_lo = max(i - W + 1, 0) - jt0;
-                    c_hi = i - jt0;
-                } else {
-                    c_lo = 0;
-                    c_hi = nvis - (t - n_win) * BN - 1;
-                }
-                // rows of a warp are consecutive and both bounds grow with the row: the bounds of its first and last row
-                // give the warp's union range (columns any row sees) and intersection range (columns every row sees).
-                // They follow from the warp's first row alone (no shuffles on the per-tile path).
-                int u_lo, u_hi, n_lo, n_hi;
-                if (t < n_win) {
-                    const int jt0 = j_start + t * BN, ia = i - lane, ib = ia + 31;
-                    u_lo = max(ia - W + 1, 0) - jt0; n_lo = max(ib - W + 1, 0) - jt0;
-                    n_hi = ia - jt0; u_hi = ib - jt0;
-                } else {
-                    u_lo = n_lo = 0;
-                    n_hi = nvis_first - (t - n_win) * BN - 1; u_hi = nvis_last - (t - n_win) * BN - 1;
-                }
-                bool act[2], full[2];
-                uint32_t vm[2];                                // per-thread validity bits of a partial chunk
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    const int lo = cb * 32, hi = lo + 31;
-                    act[cb] = lo <= u_hi && hi >= u_lo;
-                    full[cb] = lo >= n_lo && hi <= n_hi;
-                    const int a = min(max(c_lo - lo, 0), 32), b2 = min(max(c_hi - lo + 1, 0), 32);
-                    const uint32_t below_b = b2 >= 32 ? 0xffffffffu : ((1u << b2) - 1u);
-                    const uint32_t below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
-                    vm[cb] = b2 > a ? (below_b & ~below_a) : 0u;
-                }
-                if (STREAM && t >= n_win) {
-                    // the tile's 64 leave times go through a per-warp scratch (two coalesced loads), then every row tests
-                    // them against its own position; the chunks take the masked path
-                    int* slv = reinterpret_cast<int*>(smem_raw + S::OFF_LV) + warp * 64;
-                    const int e0 = (t - n_win) * BN;
-                    const int32_t* lvp = leave + (size_t)bhk * R;
-                    __syncwarp();                              // the previous tile's readers are done
-                    slv[lane] = e0 + lane < R ? lvp[e0 + lane] : 0;
-                    slv[32 + lane] = e0 + 32 + lane < R ? lvp[e0 + 32 + lane] : 0;
-                    __syncwarp();
-#pragma unroll
-                    for (int cb = 0; cb < 2; ++cb) {
-                        uint32_t m = 0;
-#pragma unroll
-                        for (int c = 0; c < 32; c += 4) {
-                            const int4 l4 = *reinterpret_cast<const int4*>(&slv[cb * 32 + c]);
-                            m |= (l4.x > i ? 1u : 0u) << c; m |= (l4.y > i ? 2u : 0u) << c;
-                            m |= (l4.z > i ? 4u : 0u) << c; m |= (l4.w > i ? 8u : 0u) << c;
-                        }
-                        vm[cb] &= m;
-                        full[cb] = false;
-                    }
-                }
-                PP(1);
-                mbar_wait(bar_s0 + 8 * (gg & 1), (gg >> 1) & 1, 3);   // S is in TMEM buffer gg & 1
-                tc_fence_after();
-                PP(2);
-                if (k_gather) { gather_issue(t + KST, false, rk); gathered = true; }   // its stage held this tile's K, which S has finished reading
-                else if (!COMPACT) cp_async_commit();
-                const uint32_t s_col = (gg & 1) * BN;
-                uint32_t r[2][32];
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb)
-                    if (act[cb]) tmem_ld32(tmem + lane_base + s_col + cb * 32, r[cb]);
+            for (int cb = 0; cb < 2; ++cb) {
+                uint32_t o[16], x[8];
+                tmem_ld16(o_col + cb * 16, o);
                 tmem_wait_ld();
-                PP(3);
-                float mr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // row max of the raw logits, 4 chains
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    if (!act[cb]) continue;
-                    if (full[cb]) {
-#pragma unroll
-                        for (int c = 0; c < 32; c += 2)
-                            mr[(c >> 1) & 3] = max3(mr[(c >> 1) & 3], __uint_as_float(r[cb][c]), __uint_as_float(r[cb][c + 1]));
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) {
-                            const float x = (vm[cb] & (1u << c)) ? __uint_as_float(r[cb][c]) : -INFINITY;
-                            r[cb][c] = __float_as_uint(x);
-                            mr[c & 3] = fmaxf(mr[c & 3], x);
-                        }
-                    }
-                }
-                const float m_tile = fmaxf(fmaxf(mr[0], mr[1]), fmaxf(mr[2], mr[3])) * c2;
-                // lazy rescale: the running max only moves when the new one is far above it (exp2 arguments stay <= 8)
-                float alpha = 1.f;
-                bool need = false;
-                if (m_run == -INFINITY) m_run = m_tile;         // nothing accumulated yet for this row: O row is 0
-                else if (m_tile > m_run + 8.f) { alpha = fast_exp2(m_run - m_tile); m_run = m_tile; need = true; }
-                if (__any_sync(0xffffffffu, need)) {
-                    // PV of the previous tile must be done before O is rescaled
-                    if (t > 0) { mbar_wait(bar_pv, (gg - 1) & 1, 4); tc_fence_after(); }
-#pragma unroll 1
-                    for (int cb = 0; cb < D / 32 + (S::ONES ? 1 : 0); ++cb) {   // with ONES the row-sum columns are rescaled too (rolled: rarely taken, and the loop is sensitive to its code size)
-                        uint32_t q4[32];
-                        tmem_ld32(tmem + lane_base + O_COL + cb * 32, q4);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) q4[c] = __float_as_uint(__uint_as_float(q4[c]) * alpha);
-                        tmem_st32(tmem + lane_base + O_COL + cb * 32, q4);
-                    }
-                    tmem_wait_st();
-                    l_run *= alpha;
-                }
-                const float neg_m = m_run == -INFINITY ? 0.f : -m_run;
-                PP(4);
-                const uint64_t c2_2 = pack2(c2, c2), neg_m2 = pack2(neg_m, neg_m);
-                float ls[4] = {0.f, 0.f, 0.f, 0.f};
-                uint32_t pk[32];                               // the row of P as 64 bf16, two per word
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    if (act[cb]) {
-#pragma unroll
-                        for (int c = 0; c < 32; c += 2) {
-                            // masked entries hold -inf: fma gives -inf and exp2(-inf) = 0
-                            float x0, x1;                      // two columns per packed fp32 instruction
-                            unpack2(fma2(pack2(__uint_as_float(r[cb][c]), __uint_as_float(r[cb][c + 1])), c2_2, neg_m2), x0, x1);
-                            const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
-                            if (!S::ONES) ls[(c >> 1) & 3] += p0 + p1;   // with ONES the tensor core sums the rounded probabilities
-                            __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-                            pk[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&h);
-                        }
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) pk[cb * 16 + c] = 0u;
-                    }
-                }
-                l_run += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-                PP(5);
-                // P goes back into TMEM, over the first 32 columns of the S buffer it was computed from (this thread has
-                // all of its row in registers), and feeds the PV product as the A operand: no trip through shared memory
-                tmem_st32(tmem + lane_base + s_col, pk);
-                tmem_wait_st();
-                tc_fence_before();                             // our TMEM accesses are ordered before the arrive
-                // PV of the previous tile has normally completed long ago.  Every phase of bar_pv is awaited in turn (a
-                // parity test is only meaningful for the current or the previous phase), and before the arrive: after
-                // it the barrier could run ahead of this thread.  At t = 0 the item's epilogue has awaited it.
-                PP(6);
-                if (t > 0) mbar_wait(bar_pv, (gg - 1) & 1, 4);
-                PP(7);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_p);
-                // value tile t+VST-1 goes into the stage of tile t-1's V, which that PV has finished reading
-                if (v_gather) { gather_issue(t + VST - 1, true, rv); gathered = true; }
-                else if (!COMPACT) cp_async_commit();
-            }
-            PP(1);
-            mbar_wait(bar_pv, (g + n_tiles - 1) & 1, 5);
-            tc_fence_after();
-            PP(8);
-
-            // ---- epilogue: O / l -> bf16, logsumexp ------------------------------------------------------
-            if (S::ONES) {                                     // the row sum is column D of the accumulator
-                uint32_t q1;
-                tmem_ld1(tmem + lane_base + O_COL + D, q1);
-                tmem_wait_ld();
-                l_run = __uint_as_float(q1);
-            }
-            const float inv = 1.f / l_run;
-            // a normalised row is D * 2 contiguous bytes of the output (whole 128-byte lines, and the rows of a warp are
-            // consecutive): each thread stores its own row with 16-byte stores, no staging in shared memory
-            __nv_bfloat16* orow = og + ((size_t)bh * (Tlen - qoff) + (i - qoff)) * dg;
-#pragma unroll
-            for (int sb = 0; sb < SUB; ++sb) {
-                uint32_t ow[32];                               // 64 columns of the row as bf16 pairs
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    uint32_t q4[32];
-                    tmem_ld32(tmem + lane_base + O_COL + sb * 64 + cb * 32, q4);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < 32; c += 2) {
-                        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(q4[c]) * inv, __uint_as_float(q4[c + 1]) * inv);
-                        ow[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&h);
-                    }
-                }
-                if (sb == SUB - 1) {
+                if (cb == 1) {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_of);        // the accumulator may take the next item
                 }
-                PP(9);
-                if (i < Tlen) {
 #pragma unroll
-                    for (int ch = 0; ch < 8; ++ch)
-                        if (sb * 64 + ch * 8 < dg)
-                            *reinterpret_cast<uint4*>(orow + sb * 64 + ch * 8) = make_uint4(ow[4 * ch], ow[4 * ch + 1], ow[4 * ch + 2], ow[4 * ch + 3]);
+                for (int c = 0; c < 8; ++c) {
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(o[2 * c]) * inv, __uint_as_float(o[2 * c + 1]) * inv);
+                    x[c] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+                if (last_row >= 0 && hf * 32 + cb * 16 < dg) {
+                    *reinterpret_cast<uint4*>(orow + cb * 16) = make_uint4(x[0], x[1], x[2], x[3]);
+                    *reinterpret_cast<uint4*>(orow + cb * 16 + 8) = make_uint4(x[4], x[5], x[6], x[7]);
                 }
             }
-            if (i < Tlen) lse[(size_t)bh * (Tlen - qoff) + (i - qoff)] = m_run * 0.6931471805599453f + logf(l_run);
-            g += n_tiles;
-            PP(11);
+            if (last_row >= 0 && hf == 0) lse[last_row] = last_m * 0.6931471805599453f + logf(l);
+        };
+        for (;; ++n) {
+            mbar_wait(bar_i + 8 * (n & 3), (n >> 2) & 1, 15);
+            const int item = __shfl_sync(0xffffffffu, slot(n)->item, 0);
+            if (item < 0) break;
+            const Item w = item_of(args, item);
+            const int W = args.W, Tlen = args.Tlen;
+            const int ia = w.i0 + (warp & 3) * 32, i = ia + lane;   // the warp's first query row, this thread's
+            int nvis, n_tiles;                                 // retained entries this row sees (a prefix of the list), tiles of the item
+            {
+                const volatile Info* f = slot(n);
+                const int x = min(i, Tlen - 1) - w.i0;
+                nvis = (int)(f->before[x >> 5] + __popc(f->bits[x >> 5] & ((1u << (x & 31)) - 1u)));
+                n_tiles = f->n_tiles;
+            }
+            n_tiles = __shfl_sync(0xffffffffu, n_tiles, 0);
+            const int nvis_first = __shfl_sync(0xffffffffu, nvis, 0), nvis_last = __shfl_sync(0xffffffffu, nvis, 31);
+            float m_run = -INFINITY;                           // reference (log2 domain), the same in both halves
+            uint64_t ls[2] = {0ull, 0ull};                     // sum of this half of the row, two packed pairs
+
+            for (int t = 0; t < n_tiles; ++t, ++g) {
+                // columns (of this half) the row may see in the tile, and (the bounds grow with the row, so the warp's first and
+                // last row give them) the columns any row and every row of the warp may see
+                int c_lo, c_hi, u_lo, u_hi, n_lo, n_hi;
+                if (t < w.n_win) {
+                    const int jt0 = w.j_start + t * BN + c0;
+                    c_lo = max(i - W + 1, 0) - jt0; c_hi = i - jt0;
+                    u_lo = max(ia - W + 1, 0) - jt0; n_lo = max(ia + 31 - W + 1, 0) - jt0;
+                    n_hi = ia - jt0; u_hi = ia + 31 - jt0;
+                } else {
+                    const int e0 = (t - w.n_win) * BN + c0;
+                    c_lo = u_lo = n_lo = 0;
+                    c_hi = nvis - e0 - 1; n_hi = nvis_first - e0 - 1; u_hi = nvis_last - e0 - 1;
+                }
+                const bool timed = STREAM && t >= w.n_win;
+                if (timed) {                                   // the leave times of this half of the tile go through a per-warp scratch
+                    int* slv = reinterpret_cast<int*>(smem_raw + S::OFF_LV) + warp * 64;
+                    const int e0 = (t - w.n_win) * BN + c0;
+                    const int32_t* lvp = leave + (size_t)w.bhk * R;
+                    __syncwarp();                              // the previous tile's readers are done
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) slv[u * 32 + lane] = e0 + u * 32 + lane < R ? lvp[e0 + u * 32 + lane] : 0;
+                    __syncwarp();
+                }
+                bool act[2], plain[2];
+#pragma unroll
+                for (int cb = 0; cb < 2; ++cb) {
+                    act[cb] = cb * 32 <= u_hi && cb * 32 + 31 >= u_lo;
+                    plain[cb] = cb * 32 >= n_lo && cb * 32 + 31 <= n_hi && !timed;
+                }
+                auto mask_of = [&](int cb) {                   // this row's columns of a chunk that needs a mask
+                    const int a = min(max(c_lo - cb * 32, 0), 32), b = min(max(c_hi - cb * 32 + 1, 0), 32);
+                    const uint32_t below_b = b >= 32 ? 0xffffffffu : ((1u << b) - 1u), below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
+                    uint32_t vm = b > a ? (below_b & ~below_a) : 0u;
+                    if (timed) {
+                        const int* slv = reinterpret_cast<const int*>(smem_raw + S::OFF_LV) + warp * 64 + cb * 32;
+                        uint32_t m = 0;
+#pragma unroll
+                        for (int c = 0; c < 32; c += 4) {
+                            const int4 l4 = *reinterpret_cast<const int4*>(slv + c);
+                            m |= (l4.x > i ? 1u : 0u) << c; m |= (l4.y > i ? 2u : 0u) << c;
+                            m |= (l4.z > i ? 4u : 0u) << c; m |= (l4.w > i ? 8u : 0u) << c;
+                        }
+                        vm &= m;
+                    }
+                    return vm;
+                };
+                auto apply = [&](uint32_t (&x)[32], uint32_t vm) {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) x[c] = (vm & (1u << c)) ? x[c] : 0xff800000u;   // -inf
+                };
+                float mr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                auto max_of = [&](const uint32_t (&x)[32]) {
+#pragma unroll
+                    for (int c = 0; c < 32; c += 2) mr[(c >> 1) & 3] = max3(mr[(c >> 1) & 3], __uint_as_float(x[c]), __uint_as_float(x[c + 1]));
+                };
+                mbar_wait(bar_s, g & 1, 5);
+                tc_fence_after();
+                // Chunk 0 passes through for the maximum and is fetched again after the exponentials of chunk 1 (32 logits at a time
+                // and the loop's state are what fits in the 96 registers there are).
+                uint32_t x[32], vm0 = 0xffffffffu;
+                if (act[0]) {
+                    tmem_ld32(s_col, x);
+                    tmem_wait_ld();
+                    if (!plain[0]) { vm0 = mask_of(0); apply(x, vm0); }
+                    max_of(x);
+                }
+                if (act[1]) {
+                    tmem_ld32(s_col + 32, x);
+                    tmem_wait_ld();
+                    if (!plain[1]) apply(x, mask_of(1));
+                    max_of(x);
+                }
+                float m_tile = fmaxf(fmaxf(mr[0], mr[1]), fmaxf(mr[2], mr[3])) * c2;
+                x_mine[(g & 1) * 2 * BM] = m_tile;
+                pair_sync();
+                m_tile = fmaxf(m_tile, x_other[(g & 1) * 2 * BM]);
+                // lazy rescale: the reference only moves when the maximum is far above it (exp2 arguments stay <= 8)
+                float alpha = 1.f;
+                bool need = false;
+                if (m_run == -INFINITY) m_run = m_tile;        // nothing accumulated yet for this row: its O is 0
+                else if (m_tile > m_run + 8.f) { alpha = fast_exp2(m_run - m_tile); m_run = m_tile; need = true; }
+                if (__any_sync(0xffffffffu, need)) {
+                    if (t > 0) {                               // PV of the previous tile must be done before O is rescaled
+                        mbar_wait(bar_pv, (g - 1) & 1, 10);
+                        tc_fence_after();
+#pragma unroll 1
+                        for (int cb = 0; cb < 2; ++cb) {       // (rolled, in small pieces: rarely taken, and S holds the registers)
+                            uint32_t q4[16];
+                            tmem_ld16(o_col + cb * 16, q4);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) q4[c] = __float_as_uint(__uint_as_float(q4[c]) * alpha);
+                            tmem_st16(o_col + cb * 16, q4);
+                        }
+                        tmem_wait_st();
+                    }
+                    const uint64_t a2 = pack2(alpha, alpha);
+                    ls[0] = mul2(ls[0], a2); ls[1] = mul2(ls[1], a2);
+                }
+                const float neg_m = m_run == -INFINITY ? 0.f : -m_run;
+                const uint64_t neg_m2 = pack2(neg_m, neg_m);
+                auto exps = [&](const uint32_t (&x)[32], uint32_t (&pk)[16]) {
+#pragma unroll
+                    for (int c = 0; c < 32; c += 2) {
+                        // masked entries hold -inf: fma gives -inf and exp2(-inf) = 0
+                        float x0, x1;                          // two columns per packed fp32 instruction
+                        unpack2(fma2(pack2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), c2_2, neg_m2), x0, x1);
+                        const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                        ls[(c >> 1) & 1] = add2(ls[(c >> 1) & 1], pack2(p0, p1));
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
+                        pk[c >> 1] = *reinterpret_cast<const uint32_t*>(&h);
+                    }
+                };
+                uint32_t pk[16];                               // 32 columns of the row of P, two per word
+                if (act[1]) exps(x, pk);
+                else
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) pk[c] = 0u;
+                if (act[0]) tmem_ld32(s_col, x);
+                // P(g) takes the place of P(g-1), whose product has normally completed long ago; every phase is awaited in turn
+                if (g > 0) { mbar_wait(bar_pv, (g - 1) & 1, 11); tc_fence_after(); }
+                tmem_st16(p_col + 16, pk);
+                if (t == 0 && n > 0) epilogue(n - 1);          // the previous item's
+                tmem_wait_ld();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_sf);            // S(g+1) may overwrite the buffer
+                if (act[0]) {
+                    if (!plain[0]) apply(x, vm0);
+                    exps(x, pk);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) pk[c] = 0u;
+                }
+                tmem_st16(p_col, pk);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_p);
+            }
+            float l0, l1;
+            unpack2(add2(ls[0], ls[1]), l0, l1);
+            // (read after the pair's next barrier; written again two items on)
+            reinterpret_cast<float*>(smem_raw + S::OFF_L)[(n & 1) * 2 * BM + hf * BM + row] = l0 + l1;
+            last_m = m_run;
+            last_row = i < Tlen ? w.bh * (Tlen - args.qoff) + (i - args.qoff) : -1;
         }
-        PP_FLUSH();
+        pair_sync();
+        mbar_wait(bar_pv, (g - 1) & 1, 14);
+        tc_fence_after();
+        epilogue(n - 1);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) tmem_dealloc(tmem, TMEM_COLS);
-}
-
-template <int D>
-int run(const Params& p, const void* q, const void* k, const void* v, const int32_t* idx, const int32_t* cnt, void* o,
-        float* lse, void* ws, size_t ws_bytes, cudaStream_t st, const int32_t* leave)
-{
-    CUtensorMap tq, tk, tv, tkc, tvc;
-    const int BHK = p.B * p.H, BH = BHK * p.G;                 // key/value heads, query heads
-    const int Tq = p.T - p.qoff;                               // query rows (the whole sequence unless a chunk is prefilled)
-    // head dimension in memory: D, or half of it (d = 32 runs the d = 64 kernel: the tensor maps' 64-column boxes reach past
-    // the 32 columns a row has and the copy engine fills the rest of every tile row with zeros, which change no product)
-    const int dg = p.d;
-    if (!make_map(&tq, q, BH, Tq, dg, BM) || !make_map(&tk, k, BHK, p.T, dg, BN) || !make_map(&tv, v, BHK, p.T, dg, BN)) return LTE_ERR_CUDA;
-    // with a workspace the retained rows are compacted first and every tile is a TMA box
-    const size_t half = prefill_compact_bytes(p) / 2;
-    const bool compact = ws != nullptr && half > 0 && ws_bytes >= 2 * half && ((uintptr_t)ws & 127u) == 0;
-    tkc = tk; tvc = tv;
-    if (compact) {
-        char* kc = (char*)ws; char* vc = kc + half;
-        if (int e = launch_prefill_compact(p, k, v, idx, cnt, kc, vc, st)) return e;
-        if (!make_map(&tkc, kc, BHK, p.R, dg, BN) || !make_map(&tvc, vc, BHK, p.R, dg, BN)) return LTE_ERR_CUDA;
-    }
-    static PerDeviceOnce attr;
-    if (int e = attr.run([] {
-            cudaError_t a = cudaFuncSetAttribute(prefill_tc_kernel<D, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
-            if (a == cudaSuccess) a = cudaFuncSetAttribute(prefill_tc_kernel<D, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
-            return a != cudaSuccess ? a : cudaFuncSetAttribute(prefill_tc_kernel<D, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
-        })) return e;
-    int sms = 0;
-    if (int e = device_sm_count(&sms)) return e;
-    const int slots = 2 * sms;                                 // resident CTAs: two per SM
-    const int n_qt = (Tq + BM - 1) / BM, n_items = n_qt * BH;
-    const int grid = n_items < slots ? n_items : slots;
-    if (leave != nullptr) {
-        if (!compact) return LTE_ERR_UNSUPPORTED;             // the streaming variant takes compacted rows only
-        return cuda_status(launch_pdl(prefill_tc_kernel<D, true, true>, dim3(grid), dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, tkc, tvc,
-                                      (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (__nv_bfloat16*)o, idx, cnt, leave, lse, p.T, p.W, p.R,
-                                      p.scale, n_qt, BH, p.G, p.qoff, dg));
-    }
-    if (compact)
-        return cuda_status(launch_pdl(prefill_tc_kernel<D, true, false>, dim3(grid), dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, tkc, tvc,
-                                      (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (__nv_bfloat16*)o, idx, cnt, leave, lse, p.T, p.W, p.R,
-                                      p.scale, n_qt, BH, p.G, p.qoff, dg));
-    return cuda_status(launch_pdl(prefill_tc_kernel<D, false, false>, dim3(grid), dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, tkc, tvc,
-                                  (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (__nv_bfloat16*)o, idx, cnt, leave, lse, p.T, p.W, p.R,
-                                  p.scale, n_qt, BH, p.G, p.qoff, dg));
+    if (warp == 8) tmem_dealloc(tmem, TMEM_COLS);
 }
 
 }  // namespace
 
-// leave: null, or the streaming reading's per-entry leave times (d = 64 or 128 with a workspace: the tiled kernels; otherwise
-// the row-by-row kernel)
+static int launch_d64(const Params& p, const void* q, const void* k, const void* v, const int32_t* idx, const int32_t* cnt, void* o,
+                      float* lse, void* ws, size_t ws_bytes, cudaStream_t st, const int32_t* leave)
+{
+    // with a workspace the retained rows are compacted first and every tile is a TMA box
+    const size_t half = prefill_compact_bytes(p) / 2;
+    const bool compact = ws != nullptr && half > 0 && ws_bytes >= 2 * half && ((uintptr_t)ws & 127u) == 0;
+    if (leave && !compact) return LTE_ERR_UNSUPPORTED;
+    CUtensorMap tq, tk, tv, tkc, tvc;
+    const int BHK = p.B * p.H, BH = BHK * p.G, Tq = p.T - p.qoff;   // key/value heads, query heads, query rows
+    if (!make_map(&tq, q, BH, Tq, p.d, BM) || !make_map(&tk, k, BHK, p.T, p.d, BN) || !make_map(&tv, v, BHK, p.T, p.d, BN)) return LTE_ERR_CUDA;
+    tkc = tk; tvc = tv;
+    if (compact) {
+        char* kc = (char*)ws; char* vc = kc + half;
+        if (int e = launch_prefill_compact(p, k, v, idx, cnt, kc, vc, st)) return e;
+        if (!make_map(&tkc, kc, BHK, p.R, p.d, BN) || !make_map(&tvc, vc, BHK, p.R, p.d, BN)) return LTE_ERR_CUDA;
+    }
+    static PerDeviceOnce attr;
+    if (int e = attr.run([] {
+            cudaError_t a = cudaFuncSetAttribute(prefill_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<false>::BYTES);
+            if (a == cudaSuccess) a = cudaFuncSetAttribute(prefill_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<false>::BYTES);
+            return a != cudaSuccess ? a : cudaFuncSetAttribute(prefill_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<true>::BYTES);
+        })) return e;
+    Args a;
+    a.n_qt = (Tq + BM - 1) / BM; a.n_bh = BH; a.n_items = a.n_qt * BH; a.Tlen = p.T; a.W = p.W; a.G = p.G; a.qoff = p.qoff;
+    auto go = [&](auto kern, int smem) {
+        return cuda_status(launch_pdl(kern, dim3(a.n_items), dim3(NTHREADS), smem, st, tq, tk, tv, tkc, tvc, a, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                                      idx, cnt, (__nv_bfloat16*)o, lse, leave, p.R, p.scale, p.d));
+    };
+    if (leave) return go(prefill_tc_kernel<false, true>, Smem<true>::BYTES);
+    return compact ? go(prefill_tc_kernel<false, false>, Smem<false>::BYTES) : go(prefill_tc_kernel<true, false>, Smem<false>::BYTES);
+}
+
+// leave: null, or the streaming reading's per-entry leave times (with a workspace the tiled kernels; otherwise the row-by-row
+// kernel)
 int launch_prefill_tc(const Params& p, const void* q, const void* k, const void* v, const int32_t* idx,
                       const int32_t* cnt, void* o, float* lse, void* ws, size_t ws_bytes, cudaStream_t st, const int32_t* leave)
 {
-    if (p.d == 64 || p.d == 32) {
-        const int e = run<64>(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
-        if (e != LTE_ERR_UNSUPPORTED || leave == nullptr) return e;
-    }
-    if (leave != nullptr) {
-        if (p.d == 128) {
-            const int e = launch_prefill_tc_long(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
-            if (e != LTE_ERR_UNSUPPORTED) return e;
-        }
-        return launch_prefill_simt(p, q, k, v, idx, cnt, o, lse, st, leave);
-    }
-    // d = 128: ten and more key tiles per item; one CTA per item under the hardware scheduler is faster there
-    if (p.d == 128) return launch_prefill_tc_long(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st);
-    return launch_prefill_simt(p, q, k, v, idx, cnt, o, lse, st);
+    int e = LTE_ERR_UNSUPPORTED;
+    if (p.d == 64 || p.d == 32) e = launch_d64(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
+    else if (p.d == 128) e = launch_prefill_tc_long(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
+    return e != LTE_ERR_UNSUPPORTED ? e : launch_prefill_simt(p, q, k, v, idx, cnt, o, lse, st, leave);
 }
-
-
-#ifdef LTE_PROFILE
-extern "C" int lte_pprof_read(unsigned long long* out, int clear)
-{
-    if (cudaMemcpyFromSymbol(out, g_pprof, sizeof(unsigned long long) * 16) != cudaSuccess) return -1;
-    if (clear) { unsigned long long z[16] = {}; cudaMemcpyToSymbol(g_pprof, z, sizeof(z)); }
-    return 0;
-}
-extern "C" int lte_pprof_cta_read(unsigned long long* out)
-{
-    return cudaMemcpyFromSymbol(out, g_pprof_cta, sizeof(unsigned long long) * 2048) == cudaSuccess ? 0 : -1;
-}
-#endif
 
 int prefill_status_fetch_and_clear()
 {
