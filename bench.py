@@ -869,7 +869,7 @@ def run_reference(args):
 
 
 TRAFFIC_SOURCES = {
-    "prefill_attn_C2": ["prefill_tc.cu", "prefill_tc_long.cu", "tc_common.cuh", "tma_util.cuh", "common.cuh"],
+    "prefill_attn_C2": ["prefill_tc.cu", "prefill_tc_long.cu", "tile_items.cuh", "tc_common.cuh", "tma_util.cuh", "common.cuh"],
     "decode_C4": ["decode_tc.cu", "tc_common.cuh", "tma_util.cuh", "common.cuh"],
 }
 

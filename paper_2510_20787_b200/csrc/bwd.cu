@@ -15,13 +15,12 @@
 namespace lte {
 
 int launch_bwd_dq_tc(const Params& p, const void* q, const void* k, const void* v, const void* o, const float* lse,
-                     const void* dO, const int32_t* idx, const int32_t* cnt, void* dq, float* delta, cudaStream_t st);
+                     const void* dO, const int32_t* idx, const int32_t* cnt, void* dq, float* delta, void* ret_ws, cudaStream_t st);
 
 size_t bwd_tc_ret_bytes(const Params& p);
 int launch_bwd_dkv_tc(const Params& p, const void* q, const void* k, const void* v, const float* lse, const void* dO,
                       const float* delta, const float* z, const int32_t* idx, const int32_t* cnt, const float* lambda,
-                      void* dk, void* dv, float* dk32, float* dv32, float* dz, void* ret_ws, bool f32out, bool merge_here,
-                      cudaStream_t st);
+                      void* dk, void* dv, float* dz, void* ret_ws, bool merge_here, cudaStream_t st);
 
 namespace {
 
@@ -562,7 +561,7 @@ int run(const Params& p, const void* q, const void* k, const void* v, const void
     const bool f32 = want_in && !p.stack;             // the stack's backward adds its input gradient to dk, dv in place
     dim3 grid((p.T + 3) / 4, p.B * p.H), gridq((p.T + 3) / 4, p.B * p.H * p.G);
     if constexpr (sizeof(T) == 2 && (D == 32 || D == 64 || D == 128)) {
-        const int e = launch_bwd_dq_tc(p, q, k, v, o, lse, dO, idx, cnt, dq, delta, st);
+        const int e = launch_bwd_dq_tc(p, q, k, v, o, lse, dO, idx, cnt, dq, delta, base + w.ret, st);
         if (e != LTE_OK) return e;
     } else {
         bwd_dq_kernel<T, D><<<gridq, 128, 0, st>>>((const T*)q, (const T*)k, (const T*)v, (const T*)o, (const T*)dO, lse,
@@ -571,8 +570,8 @@ int run(const Params& p, const void* q, const void* k, const void* v, const void
     if constexpr (sizeof(T) == 2 && (D == 32 || D == 64 || D == 128)) {
         // K = 5 or 7 with the single layer: the last pass (bwd_tail_kernel) also merges the retained shares and forms dz
         const bool tail_merges = !p.stack && (p.K == 5 || p.K == 7);
-        const int e = launch_bwd_dkv_tc(p, q, k, v, lse, dO, delta, z, idx, cnt, lambda, dk, dv, dk32, dv32, dz, base + w.ret,
-                                        false, !tail_merges, st);
+        const int e = launch_bwd_dkv_tc(p, q, k, v, lse, dO, delta, z, idx, cnt, lambda, dk, dv, dz, base + w.ret,
+                                        !tail_merges, st);
         if (e != LTE_OK) return e;
     } else if (f32) {
         bwd_dkv_kernel<T, D, true><<<grid, 128, 0, st>>>((const T*)q, (const T*)k, (const T*)v, (const T*)dO, lse, delta,

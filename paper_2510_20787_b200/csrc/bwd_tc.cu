@@ -1,25 +1,32 @@
-// Backward of the LTE prefill attention on the tcgen05 tensor cores (Section 3.1.2), bf16, d = 64 or 128.
+// Backward of the LTE prefill attention on the tcgen05 tensor cores (Section 3.1.2), bf16, d = 128, 64 and 32.
 //
-// Two kernels, both in gather form (no floating-point atomics, deterministic):
+// Two passes of one kernel, both in gather form (no floating-point atomics, deterministic).  A pass keeps 128 rows (operands
+// A1, A2) and walks tiles of BN rows (operands B1, B2):
+//            rows        A1, A2     tiles          B1, B2     X = A1 B1^T   Y = A2 B2^T    accumulated
+//   dq       queries     Q,  dO     keys           K, V       S             dP             dQ += dS K
+//   dkv      keys        K,  V      queries        Q, dO      S^T           dP^T           dK += dS^T Q,  dV += P^T dO
+// with P = exp2(S c2 - L2_i) (the forward's logsumexp fixes the normalisation) and dS = P (dP - delta_i) scale,
+// delta_i = <dO_i, O_i>.  dq rows see the window keys and then the retained list (rows gathered); dkv rows are the 128 keys of a
+// window tile, or 128 entries of the retained list (gathered once), whose tiles are the query blocks that can see them, of
+// every query head of the group.  dkv also takes Eq. 6's inner product <v_j, dV_j> = sum_i P_ij dP_ij on the way; window tiles write
+// dK, dV of their keys, list tiles write their share to scratch, which the last pass adds row by row (a fixed order).
 //
-// dq kernel   one CTA per 128-query tile, the same key/value tile walk as the forward kernel (window tiles by
-//             TMA, retained tiles gathered with cp.async).  Per 64-key tile:
-//               S = Q K^T and dP = dO V^T          tcgen05.mma into TMEM
-//               P = exp2(S c2 - L2_i),  dS = P (dP - delta_i) scale   by the thread owning row i (no online softmax:
-//               the forward's logsumexp fixes the normalisation), written as bf16 into swizzled shared memory
-//               dQ += dS K                          tcgen05.mma, K tile as the MN-major operand, accumulated in TMEM
-//             delta_i = <dO_i, O_i> is computed by the same thread at the start and also written out for the second kernel.
-//
-// dkv kernel  one CTA per 128-key tile: the contiguous keys of a window tile, or 128 entries of the retained list
-//             (their K/V rows gathered once).  It walks the 64-query blocks that can see those keys:
-//               S^T = K Q^T and dP^T = V dO^T       tcgen05.mma (keys on the M side)
-//               P^T, dS^T                           by the thread owning the key row; L2 and delta of the block's
-//                                                   64 queries are read from shared memory
-//               dV += P^T dO,  dK += dS^T Q         tcgen05.mma with the dO / Q block as MN-major operand
-//             and finishes with Eq. 6's inner product <v_j, dV_j> per key from the fp32 accumulators.  Window tiles
-//             write dK, dV of their keys; retained tiles write their far-query share to scratch, which a small merge
-//             kernel adds row by row (each key appears once in the list, so the sum order is fixed).
-#include "tc_common.cuh"
+// Bound by the exponentials and the operand reads of the products about equally (a 128 x 128 tile: 1,024 cycles of the exponential
+// unit; at d = 64 dkv 24 products of 50-60 cycles), so both have to run all the time:
+//   - One CTA per SM with 16 row warps (four threads per row, BN/4 columns each): what two CTAs of four warps had in flight, but
+//     with wide tiles, and all of tensor memory for one set of buffers: X, Y, P, dS, accumulators side by side.
+//   - X, Y of tile g+1 are computed while the row warps work on tile g (X, Y are free as soon as they are in registers) and the
+//     accumulation of tile g runs under tile g+1; the two kinds of product are issued by two warps (one warp issues a product
+//     every 54 cycles at best).  P and dS are TMEM A operands: no trip through shared memory.
+//   - Items are handed out dynamically, the longest (list tiles) first; a finished item's accumulators are read and stored
+//     under the next item's first tile.
+// One warp loads (TMA; cp.async for gathered rows).  dq forms delta at an item's start, each thread from its part of the row, and writes
+// it for the dkv pass, where another warp prepares the constants -L2, -delta scale of every tile.  Every wait is bounded.
+// Measured (B200, us for dq + dkv, against four warps a CTA, two CTAs an SM, items dealt out beforehand):
+//   128 heads x 2,048, d = 64, W = R = 64                 66 + 84   (was 74 + 96)
+//   128 heads of 4-head groups x 4,096, d = 64, W 768, R 512   252 + 280  (364 + 455)
+//   16 heads x 8,192, d = 128, W = R = 512                101 + 128  (185 + 195)
+#include "tile_items.cuh"
 
 namespace lte {
 
@@ -29,797 +36,596 @@ namespace {
 
 using namespace tc;
 __device__ __forceinline__ void bwait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_bwd_status); }
-__device__ __forceinline__ void group_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-constexpr int BM = 128, BN = 64, NTHREADS = 160, NST = 3;      // 3 stages for every streamed tile
+constexpr int BM = 128, NRW = 16;                              // rows per item, row warps
+constexpr int W_LOAD = NRW, W_XY = NRW + 1, W_ACC = NRW + 2, NTHREADS = (NRW + 4) * 32;   // the last warp prepares constants
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <int D> struct SmemQ {                                // dq kernel
-    static constexpr int SUB = D / 64;
-    // d = 128 runs one CTA per SM (shared memory), so tensor memory has room for two S / dP buffers: the products of tile
-    // t+1 are in flight while the row threads work on tile t, which needs a fourth key / value stage
-    static constexpr bool DB = D == 128;
-    static constexpr int NS = DB ? 4 : 3;
-    static constexpr int QTILE = BM * D * 2, KVTILE = BN * D * 2;
-    static constexpr int OFF_Q = 0, OFF_DO = QTILE, OFF_K = 2 * QTILE, OFF_V = OFF_K + NS * KVTILE;
-    static constexpr int OFF_DS = OFF_V + NS * KVTILE;         // [128][64] bf16
-    static constexpr int OFF_BAR = OFF_DS + BM * BN * 2;
-    static constexpr int OFF_IDX = OFF_BAR + 128;
-    static constexpr int BYTES = OFF_IDX + 512;
-    // d = 64:  S [0,64)  dP [64,128)  dQ [128,192);   d = 128:  S, dP of buffer b at 128 b, 128 b + 64;  dQ [256,384)
-    static constexpr uint32_t TMEM_COLS = DB ? 512 : 256;
+// Stages are what shared memory holds (192 KB of tiles, and O beside them).
+template <int D, bool DKV> struct Cfg {
+    static constexpr int BN = D == 128 && DKV ? 64 : 128;      // d = 128 dkv: two accumulators of 128 columns leave room for 64-wide tiles
+    static constexpr int AST = D == 128 ? 1 : 3, ATILE = BM * D * 2;
+    static constexpr int BST = D == 64 ? 3 : DKV ? 4 : 2, BTILE = BN * D * 2;
+    static constexpr int OFF_A = 0, OFF_B = AST * 2 * ATILE, OFF_O = OFF_B + BST * 2 * BTILE;   // dq: the item's O, for delta
+    static constexpr int OFF_BAR = OFF_O + (DKV ? 0 : ATILE);
+    static constexpr int OFF_INFO = OFF_BAR + 512;             // ring of eight items' Info, 64 bytes apart
+    static constexpr int OFF_C = OFF_INFO + 512;               // dkv: constants [2][2][128];  dq: lse [2][128]
+    static constexpr int OFF_DR = OFF_C + 2 * (DKV ? 2 : 1) * 128 * 4;   // dkv: the four parts of a row's <v, dV> [2][4][128]
+    static constexpr int BYTES = OFF_DR + (DKV ? 2 * 4 * 128 * 4 : 0);
+    // tensor memory
+    static constexpr uint32_t X = 0, Y = BN, DS = 2 * BN, P = DS + BN / 2, ACC0 = DKV ? P + BN / 2 : P, ACC1 = ACC0 + D;
+    static_assert(BYTES <= 232448, "shared memory");
+    static_assert((DKV ? ACC1 + D : ACC1) <= 512, "tensor memory");
 };
 
-template <int D>
-__global__ void __launch_bounds__(NTHREADS, D == 64 ? 2 : 1)
-bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
-                 const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmDQ,
-                 const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                 const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* __restrict__ vg,
-                 const __nv_bfloat16* __restrict__ og, const __nv_bfloat16* __restrict__ dog,
-                 const float* __restrict__ lse, const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt,
-                 __nv_bfloat16* __restrict__ dq, float* __restrict__ delta, int Tlen, int W, int R, float scale, int G, int dg)
+struct Args {
+    const __nv_bfloat16 *k, *v;
+    const float* lse;
+    float* delta;
+    const int32_t *idx, *cnt;
+    __nv_bfloat16 *dq, *dk, *dv;
+    float *dr_win, *dk_ret, *dv_ret, *dr_ret;
+    int n_rows, n_bh;                                          // dq: query tiles, query heads;  dkv: window tiles, key/value heads
+    int n_list;                                                // dkv: list tiles per head
+    int Tlen, W, R, G, dg;
+    float scale;
+};
+// dq: row x (0 .. 127) sees before[x / 32] list entries and those of bits[x / 32] below bit x % 32.  dkv: a, b = first query, blocks
+// per query head.  item = -1: there is none.
+struct Info { uint32_t before[4], bits[4]; int n_tiles, item, a, b; };
+
+struct Item {
+    int item, bh, bhk, row0, n_win, j_start, n_tiles;          // dq: query head, its key/value head, first query, window tiles and their first key
+    int list, a, b;                                            // dkv: bh = key/value head, row0 = first key or list entry, list tile or not
+};
+template <bool DKV, int BN> __device__ __forceinline__ Item item_of(const Args& g, int item)
 {
-    // dg = the head dimension in memory: D, or 32 for the d = 64 kernel on d = 32 data (the tensor maps then fill the upper
-    // half of every tile row with zeros on the way in and clip it on the way out; the gathers zero-fill the same columns)
-    using S = SmemQ<D>;
-    constexpr int SUB = S::SUB;
-    constexpr bool DB = S::DB;
-    constexpr int NS = S::NS;
-    constexpr uint32_t DP_COL = BN, DQ_COL = DB ? 4 * BN : 2 * BN;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const uint32_t base = smem_u32(smem_raw);
-    if ((base & 1023u) != 0) { if (threadIdx.x == 0) atomicExch(&g_bwd_status.code, 9); return; }
-    const uint32_t sQ = base + S::OFF_Q, sDO = base + S::OFF_DO, sK = base + S::OFF_K, sV = base + S::OFF_V;
-    const uint32_t sDS = base + S::OFF_DS;
-    const uint32_t bar_q = base + S::OFF_BAR, bar_k0 = bar_q + 8, bar_v0 = bar_q + 40, bar_s0 = bar_q + 72;   // 4, 4, 2 slots
-    const uint32_t bar_g0 = bar_q + 88, bar_p = bar_q + 104, bar_pv = bar_q + 112, tmem_slot = bar_q + 120;
-    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + S::OFF_BAR + 120);
-    volatile int* s_idx = reinterpret_cast<volatile int*>(smem_raw + S::OFF_IDX);
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.y, bhk = bh / G;                   // query head; its key/value head (grouped queries: G per head)
-    const int i0 = blockIdx.x * BM;
-    const int i_hi = min(i0 + BM - 1, Tlen - 1);
-    const int j_start = max(i0 - W + 1, 0);
-    const int n_win = (i_hi - j_start + 1 + BN - 1) / BN;
-    const int32_t* id = idx + (size_t)bhk * R;
-
-    if (tid == 0) {
-        mbar_init(bar_q, 1);
-#pragma unroll
-        for (int s2 = 0; s2 < NS; ++s2) { mbar_init(bar_k0 + 8 * s2, 1); mbar_init(bar_v0 + 8 * s2, 1); }
-        mbar_init(bar_s0, 1); mbar_init(bar_s0 + 8, 1);
-        mbar_init(bar_g0, 128); mbar_init(bar_g0 + 8, 128);
-        mbar_init(bar_p, 128); mbar_init(bar_pv, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    Item it;
+    it.item = item;
+    it.list = 0; it.a = it.b = 0; it.n_win = it.j_start = 0;
+    if (!DKV) {                                                // from the last query tile of every head down to the first
+        const int r = item / g.n_bh;
+        it.bh = item - r * g.n_bh;
+        it.bhk = it.bh / g.G;
+        it.row0 = (g.n_rows - 1 - r) * BM;
+        const int i_hi = min(it.row0 + BM - 1, g.Tlen - 1);
+        it.j_start = max(it.row0 - g.W + 1, 0);
+        it.n_win = (i_hi - it.j_start + BN) / BN;
+        it.n_tiles = it.n_win;                                 // until the item's Info is there
+    } else {                                                   // the list tiles first: they walk many more query blocks
+        it.list = item < g.n_list * g.n_bh;
+        const int x = it.list ? item : item - g.n_list * g.n_bh;
+        const int tile = x / g.n_bh;
+        it.bh = it.bhk = x - tile * g.n_bh;
+        it.row0 = tile * BM;
+        it.a = it.row0;
+        it.b = (min(g.Tlen - 1, it.row0 + BM - 1 + g.W - 1) - it.row0) / BN + 1;
+        it.n_tiles = it.b * g.G;                               // (window tile)
     }
-    if (warp == 4) tmem_alloc(tmem_slot, S::TMEM_COLS);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot_gen;
-    pdl_launch_dependents();
-    pdl_wait();                                                // everything above ran beside the previous kernel's tail (see launch_pdl)
-    const int n_ret = cnt[bhk];
-
-    if (warp == 4) {
-        // =================================== control warp (one lane) ========================================
-        int n_tiles = n_win;                                   // + the retained tiles, counted once the first loads are on their way
-        // The whole warp walks the loop and waits on the barriers; only the TMA / tcgen05 instructions are guarded by the
-        // lane test, so that addresses and descriptors are computed in convergent code (cheaper to issue).
-        const bool leader = lane == 0;
-        {
-            constexpr uint32_t IDESC_S = instr_desc(BM, BN, false);
-            constexpr uint32_t IDESC_Q = instr_desc(BM, D, true);
-            const uint32_t q_lo = desc_lo(sQ, 16), do_lo = desc_lo(sDO, 16), k_lo = desc_lo(sK, 16), v_lo = desc_lo(sV, 16);
-            const uint32_t ds_lo = desc_lo(sDS, 16), kmn_lo = desc_lo(sK, 8192);
-            uint32_t k_phase = 0, v_phase = 0, g_waited = 0;
-            auto tma_kv = [&](int t, bool is_v) {
-                const int st = t % NS;
-                const uint32_t dst = (is_v ? sV : sK) + st * S::KVTILE;
-                const uint32_t bar = (is_v ? bar_v0 : bar_k0) + 8 * st;
-                const int y = j_start + t * BN;
-                if (leader) {
-                    mbar_expect_tx(bar, S::KVTILE);
-#pragma unroll
-                    for (int sb = 0; sb < SUB; ++sb) tma_load_3d(dst + sb * 8192, is_v ? &tmV : &tmK, sb * 64, y, bhk, bar);
-                }
-            };
-            auto need_g = [&](uint32_t phase) {
-                while (g_waited <= phase) { bwait(bar_g0 + 8 * (g_waited & 1), (g_waited >> 1) & 1, 10); ++g_waited; }
-            };
-            auto wait_kv = [&](int t) {
-                if (t < n_win) {
-                    const int st = t % NS;
-                    bwait(bar_k0 + 8 * st, (k_phase >> st) & 1u, 2); k_phase ^= 1u << st;
-                    bwait(bar_v0 + 8 * st, (v_phase >> st) & 1u, 4); v_phase ^= 1u << st;
-                }
-            };
-            auto mma_s_dp = [&](int t) {
-                const uint32_t so = (uint32_t)(t % NS) * (S::KVTILE >> 4);
-                const uint32_t sbuf = DB ? (uint32_t)(t & 1) * (2 * BN) : 0u;
-                if (leader) {
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma(tmem + sbuf, desc64(q_lo + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                             desc64(k_lo + so + (kk >> 2) * 512 + (kk & 3) * 2, kDescHi), IDESC_S, kk > 0);
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma(tmem + sbuf + DP_COL, desc64(do_lo + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                             desc64(v_lo + so + (kk >> 2) * 512 + (kk & 3) * 2, kDescHi), IDESC_S, kk > 0);
-                    umma_commit(bar_s0 + (DB ? 8 * (t & 1) : 0));
-                }
-                __syncwarp();
-            };
-
-            // d = 64: the O tile rides along into the (still unused) dS buffer, for delta = <dO, O>
-            if (leader) {
-                mbar_expect_tx(bar_q, (D == 64 ? 3 : 2) * S::QTILE);
-#pragma unroll
-                for (int sb = 0; sb < SUB; ++sb) {
-                    tma_load_3d(sQ + sb * 16384, &tmQ, sb * 64, i0, bh, bar_q);
-                    tma_load_3d(sDO + sb * 16384, &tmDO, sb * 64, i0, bh, bar_q);
-                }
-                if (D == 64) tma_load_3d(sDS, &tmO, 0, i0, bh, bar_q);
-            }
-            for (int t = 0; t < NS && t < n_win; ++t) { tma_kv(t, false); tma_kv(t, true); }
-            {
-                // retained entries visible to the tile's last row (idx ascending => a prefix): read while the loads fly
-                int nv_max = 0;
-                const int lim = i_hi - W;
-                for (int e0 = 0; e0 < n_ret; e0 += 32) {
-                    const int e = e0 + lane < n_ret ? id[e0 + lane] : 0x7fffffff;
-                    const unsigned bal = __ballot_sync(0xffffffffu, e <= lim);
-                    nv_max += __popc(bal);
-                    if (bal != 0xffffffffu) break;
-                }
-                n_tiles = n_win + (nv_max + BN - 1) / BN;
-            }
-            bwait(bar_q, 0, 1);                                // (tile 0 is always a window tile: no gather to wait for)
-            wait_kv(0);
-            tc_fence_after();
-            mma_s_dp(0);
-            if (DB && n_tiles > 1) {                           // two buffers: tile 1 follows at once (prologue gathers: phase 0)
-                need_g(0);
-                wait_kv(1);
-                tc_fence_after();
-                mma_s_dp(1);
-            }
-            for (int t = 0; t < n_tiles; ++t) {
-                bwait(bar_p, t & 1, 7);                        // dS(t) is in shared memory; its S / dP buffer is free
-                tc_fence_after();
-                // one buffer: the next tile's S, dP first: the row threads wait for those, while dQ of this tile is only
-                // needed before the dS buffer is rewritten a tile later
-                if (!DB && t + 1 < n_tiles) {
-                    need_g(t + 1);
-                    wait_kv(t + 1);
-                    mma_s_dp(t + 1);
-                }
-                {
-                    const uint32_t kb = kmn_lo + (uint32_t)(t % NS) * (S::KVTILE >> 4);
-                    if (leader) {
-#pragma unroll
-                        for (int kk = 0; kk < BN / 16; ++kk)
-                            umma(tmem + DQ_COL, desc64(ds_lo + kk * 2, kDescHi), desc64(kb + kk * 128, kDescHi), IDESC_Q,
-                                 (t > 0 || kk > 0) ? 1u : 0u);
-                        umma_commit(bar_pv);
-                    }
-                    __syncwarp();
-                }
-                // two buffers: the row threads are already on tile t+1; S, dP of tile t+2 go into the buffer tile t has left.
-                // Its gathers were committed in tile t-1 and are covered by the arrival at the top of tile t+1.
-                if (DB && t + 2 < n_tiles) {
-                    need_g(t + 1);
-                    wait_kv(t + 2);
-                    tc_fence_after();
-                    mma_s_dp(t + 2);
-                }
-                // dQ(t-1) has completed (the softmax warps waited for it before producing dS(t)): its key stage and
-                // the value stage of tile t-1 can take window tile t-1+NS
-                if (t >= 1 && t - 1 + NS < n_win) { tma_kv(t - 1 + NS, false); tma_kv(t - 1 + NS, true); }
-            }
-        }
-    } else {
-        // =================================== softmax warps ==================================================
-        const int i = i0 + tid;
-        const int ic = min(i, Tlen - 1);
-        // delta_i = <dO_i, O_i>, L2_i = lse_i * log2(e).  d = 64: both rows are in shared memory (the TMA tiles of dO and
-        // O, 128-byte swizzle: chunk c of row r sits at chunk position c ^ (r & 7)); d = 128: from global memory.
-        float dl = 0.f;
-        const float L2 = lse[(size_t)bh * Tlen + ic] * kLog2e;
-        if (D == 64) {
-            bwait(bar_q, 0, 12);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const uint32_t off = tid * 128 + ((c ^ (tid & 7)) << 4);
-                uint32_t aw[4], bw[4];
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(aw[0]), "=r"(aw[1]), "=r"(aw[2]), "=r"(aw[3]) : "r"(sDS + off));
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(bw[0]), "=r"(bw[1]), "=r"(bw[2]), "=r"(bw[3]) : "r"(sDO + off));
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    dl = fmaf(__uint_as_float(aw[u] << 16), __uint_as_float(bw[u] << 16), dl);
-                    dl = fmaf(__uint_as_float(aw[u] & 0xffff0000u), __uint_as_float(bw[u] & 0xffff0000u), dl);
-                }
-            }
-        } else {
-            const uint4* orow = reinterpret_cast<const uint4*>(og + ((size_t)bh * Tlen + ic) * D);
-            const uint4* grow = reinterpret_cast<const uint4*>(dog + ((size_t)bh * Tlen + ic) * D);
-#pragma unroll 4
-            for (int c = 0; c < D / 8; ++c) {
-                const uint4 a = orow[c], b = grow[c];
-                const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    dl = fmaf(__uint_as_float(aw[u] << 16), __uint_as_float(bw[u] << 16), dl);
-                    dl = fmaf(__uint_as_float(aw[u] & 0xffff0000u), __uint_as_float(bw[u] & 0xffff0000u), dl);
-                }
-            }
-        }
-        if (i < Tlen) delta[(size_t)bh * Tlen + i] = dl;
-
-        // retained entries visible to this row: rows of a warp are consecutive and the list is ascending, so the count is
-        // #{idx <= lim of lane 0} plus the entries between the warp's first limit and this lane's (a 31-bit map)
-        const int lim = ic - W, lim_max = i_hi - W;
-        const int lim0 = __shfl_sync(0xffffffffu, lim, 0), lim31 = __shfl_sync(0xffffffffu, lim, 31);
-        int nvis = 0, nv_max = 0;
-        {
-            uint32_t bits = 0;
-            for (int e0 = 0; e0 < n_ret; e0 += 128) {
-                int e[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) e[u] = e0 + u * 32 + lane < n_ret ? id[e0 + u * 32 + lane] : 0x7fffffff;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    nvis += __popc(__ballot_sync(0xffffffffu, e[u] <= lim0));
-                    nv_max += __popc(__ballot_sync(0xffffffffu, e[u] <= lim_max));
-                    const bool in = e[u] > lim0 && e[u] <= lim31;
-                    bits |= __reduce_or_sync(0xffffffffu, in ? 1u << (e[u] - lim0 - 1) : 0u);
-                }
-                if (__shfl_sync(0xffffffffu, e[3], 31) > lim_max) break;
-            }
-            nvis += __popc(bits & ((1u << (lim - lim0)) - 1u));
-        }
-        const int n_tiles = n_win + (nv_max + BN - 1) / BN;
-
-        const int g_row = tid >> 3, g_sub = tid & 7;
-        auto gather_rows = [&](int t, int (&rows4)[4]) {
-#pragma unroll
-            for (int ps = 0; ps < 4; ++ps) {
-                const int e = (t - n_win) * BN + ps * 16 + g_row;
-                rows4[ps] = (t >= n_win && t < n_tiles && e < nv_max) ? id[e] : -1;
-            }
-        };
-        auto gather_issue = [&](int t, bool is_v, const int (&rows4)[4]) {
-            if (t >= n_win && t < n_tiles) {
-                const uint32_t dst = (is_v ? sV : sK) + (t % NS) * S::KVTILE;
-#pragma unroll
-                for (int ps = 0; ps < 4; ++ps) {
-                    const int row = ps * 16 + g_row;
-                    const bool ok = rows4[ps] >= 0;
-                    const __nv_bfloat16* src = (is_v ? vg : kg) + ((size_t)bhk * Tlen + (ok ? rows4[ps] : 0)) * dg;
-#pragma unroll
-                    for (int c = g_sub; c < D / 8; c += 8) {
-                        const uint32_t off = (c >> 3) * 8192 + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-                        const bool real = ok && c * 8 < dg;
-                        cp_async16(dst + off, src + (real ? c * 8 : 0), real ? 16u : 0u);
-                    }
-                }
-            }
-        };
-        {
-            int rows4[4];
-            for (int t = 0; t < NS; ++t) { gather_rows(t, rows4); gather_issue(t, false, rows4); gather_issue(t, true, rows4); }
-            cp_async_commit();
-            cp_async_commit();                                 // empty group: the wait at the top of tile 0 then covers the one above
-        }
-        const float c2 = scale * kLog2e;
-        const uint32_t lane_base = ((uint32_t)(warp * 32)) << 16;
-
-        for (int t = 0; t < n_tiles; ++t) {
-            int rn[4];
-            gather_rows(t - 1 + NS, rn);                       // retained tile that goes into the stage of tile t-1
-            cp_async_wait<1>();                                // every gather but the latest tile's has landed
-            fence_proxy_async();
-            mbar_arrive(bar_g0 + 8 * (t & 1));
-
-            int c_lo, c_hi;
-            if (t < n_win) {
-                const int jt0 = j_start + t * BN;
-                c_lo = max(i - W + 1, 0) - jt0;
-                c_hi = i - jt0;
-            } else {
-                c_lo = 0;
-                c_hi = nvis - (t - n_win) * BN - 1;
-            }
-            const int u_lo = __shfl_sync(0xffffffffu, c_lo, 0), u_hi = __shfl_sync(0xffffffffu, c_hi, 31);
-
-            bwait(bar_s0 + (DB ? 8 * (t & 1) : 0), DB ? (t >> 1) & 1 : t & 1, 3);   // S(t), dP(t) are in TMEM
-            tc_fence_after();
-            const uint32_t sbuf = DB ? (uint32_t)(t & 1) * (2 * BN) : 0u;
-            uint32_t pk[32];                                   // dS row as 64 bf16
-            const uint64_t c2_2 = pack2(c2, c2), nl2_2 = pack2(-L2, -L2), scale_2 = pack2(scale, scale), ndls_2 = pack2(-dl * scale, -dl * scale);
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                const bool act = cb * 32 <= u_hi && cb * 32 + 31 >= u_lo;
-                if (act) {
-                    uint32_t rs[32], rp[32];
-                    tmem_ld32(tmem + lane_base + sbuf + cb * 32, rs);
-                    tmem_ld32(tmem + lane_base + sbuf + DP_COL + cb * 32, rp);
-                    tmem_wait_ld();
-                    // validity bits of this row's 32 columns; the arithmetic runs on packed fp32 pairs
-                    const int a = min(max(c_lo - cb * 32, 0), 32), b2 = min(max(c_hi - cb * 32 + 1, 0), 32);
-                    const uint32_t below_b = b2 >= 32 ? 0xffffffffu : ((1u << b2) - 1u);
-                    const uint32_t below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
-                    const uint32_t vm = b2 > a ? (below_b & ~below_a) : 0u;
-#pragma unroll
-                    for (int c = 0; c < 32; c += 2) {
-                        float x0, x1, d0, d1;
-                        unpack2(fma2(pack2(__uint_as_float(rs[c]), __uint_as_float(rs[c + 1])), c2_2, nl2_2), x0, x1);
-                        const uint64_t g2 = fma2(pack2(__uint_as_float(rp[c]), __uint_as_float(rp[c + 1])), scale_2, ndls_2);   // (dP - delta) scale
-                        unpack2(mul2(pack2(fast_exp2(x0), fast_exp2(x1)), g2), d0, d1);
-                        __nv_bfloat162 h = __floats2bfloat162_rn((vm & (1u << c)) ? d0 : 0.f, (vm & (2u << c)) ? d1 : 0.f);
-                        pk[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&h);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) pk[cb * 16 + c] = 0u;
-                }
-            }
-            // dQ(t-1) must be done before dS is overwritten; its key stage (and the value stage) are then free
-            if (t > 0) { bwait(bar_pv, (t - 1) & 1, 4); tc_fence_after(); }
-            if (t > 0) { gather_issue(t - 1 + NS, false, rn); gather_issue(t - 1 + NS, true, rn); }
-            cp_async_commit();
-#pragma unroll
-            for (int ch = 0; ch < 8; ++ch) {
-                const uint32_t dst = sDS + tid * 128 + ((ch ^ (tid & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[4 * ch]), "r"(pk[4 * ch + 1]),
-                             "r"(pk[4 * ch + 2]), "r"(pk[4 * ch + 3]) : "memory");
-            }
-            fence_proxy_async();
-            tc_fence_before();
-            mbar_arrive(bar_p);
-        }
-        bwait(bar_pv, (n_tiles - 1) & 1, 5);
-        tc_fence_after();
-        // ---- epilogue: dQ (the softmax scale is already folded into dS) ------------------------------------
-        if (D == 64) {
-            // the rows go into the (now idle) dS buffer in the swizzled layout and leave as one tile store per warp
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                uint32_t q4[32];
-                tmem_ld32(tmem + lane_base + DQ_COL + cb * 32, q4);
-                tmem_wait_ld();
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    uint32_t w4[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(q4[g * 8 + 2 * u]), __uint_as_float(q4[g * 8 + 2 * u + 1]));
-                        w4[u] = *reinterpret_cast<uint32_t*>(&h);
-                    }
-                    const int ch = cb * 4 + g;
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sDS + tid * 128 + ((ch ^ (tid & 7)) << 4)),
-                                 "r"(w4[0]), "r"(w4[1]), "r"(w4[2]), "r"(w4[3]) : "memory");
-                }
-            }
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0 && i0 + warp * 32 < Tlen) {
-                tma_store_3d(&tmDQ, sDS + warp * 4096, 0, i0 + warp * 32, bh);
-                bulk_commit();
-                bulk_wait_read0();                             // the buffer is released with the CTA
-            }
-        } else {
-            __nv_bfloat16* qrow = dq + ((size_t)bh * Tlen + i) * D;
-#pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
-                uint32_t q4[32];
-                tmem_ld32(tmem + lane_base + DQ_COL + cb * 32, q4);
-                tmem_wait_ld();
-                if (i < Tlen) {
-#pragma unroll
-                    for (int c = 0; c < 32; c += 8) {
-                        uint32_t w4[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(q4[c + 2 * u]), __uint_as_float(q4[c + 2 * u + 1]));
-                            w4[u] = *reinterpret_cast<uint32_t*>(&h);
-                        }
-                        *reinterpret_cast<uint4*>(qrow + cb * 32 + c) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-                    }
-                }
-            }
-        }
+    return it;
+}
+template <int N> struct Tmem;                                  // N consecutive columns of the warp's lanes
+template <> struct Tmem<32> { static __device__ __forceinline__ void ld(uint32_t a, uint32_t (&r)[32]) { tmem_ld32(a, r); } };
+template <> struct Tmem<16> {
+    static __device__ __forceinline__ void ld(uint32_t a, uint32_t (&r)[16]) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                       "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(a) : "memory");
     }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 4) tmem_dealloc(tmem, S::TMEM_COLS);
+    static __device__ __forceinline__ void st(uint32_t a, const uint32_t (&r)[16]) {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                     ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+    }
+};
+template <> struct Tmem<8> {
+    static __device__ __forceinline__ void st(uint32_t a, const uint32_t (&r)[8]) {
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+    }
+};
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory"); }
+__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-
-// ================================================ dkv kernel =====================================================
-template <int D> struct SmemK {
-    static constexpr int SUB = D / 64;
-    // d = 128 runs one CTA per SM and has the TMEM columns for two S^T / dP^T buffers: block t+2's products are issued
-    // while the key threads work on block t+1, which takes one more stage of query blocks in flight
-    static constexpr bool DB = D == 128;
-    static constexpr int NSTK = DB ? 4 : 3;
-    static constexpr int KTILE = 128 * D * 2, QBLK = 64 * D * 2;
-    static constexpr int OFF_K = 0, OFF_V = KTILE, OFF_Q = 2 * KTILE, OFF_DO = OFF_Q + NSTK * QBLK;
-    static constexpr int OFF_PT = OFF_DO + NSTK * QBLK;        // [128][64] bf16
-    static constexpr int OFF_DST = OFF_PT + 128 * 64 * 2;      // [128][64] bf16
-    static constexpr int OFF_COL = OFF_DST + 128 * 64 * 2;     // L2[64], delta[64] of the current query block
-    static constexpr int OFF_BAR = OFF_COL + 512;
-    static constexpr int BYTES = OFF_BAR + 128;
-    // d = 64: S^T [0,64) dP^T [64,128) dV [128,192) dK [192,256); d = 128: S^T, dP^T of even blocks [0,128), of odd blocks
-    // [128,256), dV [256,384), dK [384,512)
-    static constexpr uint32_t TMEM_COLS = D == 64 ? 256 : 512;
-};
-
-template <int D, bool F32OUT>
-__global__ void __launch_bounds__(NTHREADS, D == 64 ? 2 : 1)
-bwd_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                  const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmDO,
-                  const __grid_constant__ CUtensorMap tmDK, const __grid_constant__ CUtensorMap tmDV,
-                  const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* __restrict__ vg,
-                  const float* __restrict__ lse, const float* __restrict__ delta, const int32_t* __restrict__ idx,
-                  const int32_t* __restrict__ cnt, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                  float* __restrict__ dk32, float* __restrict__ dv32, float* __restrict__ dr_win,
-                  float* __restrict__ dk_ret, float* __restrict__ dv_ret, float* __restrict__ dr_ret, int n_wt, int Tlen,
-                  int W, int R, float scale, int G, int dg)
+// Barriers (g = tile number, n = item number within the CTA):
+//   bar_a[b], bar_ga[b]  rows of item n are in buffer b = n % AST: by TMA / gathered (dkv list tiles; 32 arrivals by cp.async completion)
+//   bar_af[b]  (commit)  the item's last X, Y are complete                                                     phase n / AST
+//   bar_o, bar_od (16)   dq: O (TMA) and lse (32 arrivals by cp.async) of item n are in shared memory / have been read   phase n
+//   bar_b[s]             tile g is in stage s = g % BST                                                        phase g / BST
+//   bar_bf[s]  (commit)  the accumulation of the stage's tile is complete                                       phase g / BST
+//   bar_x  (commit) X, Y of tile g are in TMEM       bar_xf (16) they are in registers                           phase g
+//   bar_p  (16) P, dS of tile g are in TMEM and the accumulation of tile g-1 has been awaited   bar_acc (commit) it is complete   phase g
+//   bar_es[b] (4)  STAGED: the outputs of item n have left its A buffer                                           phase n / AST
+//   bar_of (16) the accumulators of item n have been read out                                                    phase n
+//   bar_i[n & 7]         Info of item n is in the ring                                                           phase n >> 3
+//   bar_cc[b], bar_cf[b] (16) dkv: the constants of tile g are in buffer b = g & 1 / have been read                phase g >> 1
+//   bar_c                the answer to the request for a block
+template <int D, bool DKV>
+__global__ void __launch_bounds__(NTHREADS, 1)
+bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB1,
+              const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmL1,
+              const __grid_constant__ CUtensorMap tmL2, const __grid_constant__ CUtensorMap tmS1, const __grid_constant__ CUtensorMap tmS2, const Args args)
 {
-    using S = SmemK<D>;
-    constexpr int SUB = S::SUB;
-    constexpr bool DB = S::DB;
-    constexpr int NSTK = S::NSTK;
-    constexpr uint32_t DP_COL = 64, DV_COL = DB ? 256 : 128, DK_COL = DV_COL + D;
+    using C = Cfg<D, DKV>;
+    constexpr int BN = C::BN, SUB = D / 64, CW = BN / 4, AST = C::AST, BST = C::BST, ATILE = C::ATILE, BTILE = C::BTILE;
+    constexpr bool STAGED = D == 64;                           // outputs leave through the item's A buffers as tiles
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if ((base & 1023u) != 0) { if (threadIdx.x == 0) atomicExch(&g_bwd_status.code, 9); return; }
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // the retained tiles walk many more query blocks than the window tiles: they take the lowest block numbers so
-    // that they start first and do not form the tail of the launch
-    const int n_rt = (int)gridDim.x - n_wt;
-    const int lin = blockIdx.y * gridDim.x + blockIdx.x, tot_ret = n_rt * (int)gridDim.y;
-    const bool is_ret = lin < tot_ret;
-    const int bh = is_ret ? lin / n_rt : (lin - tot_ret) / n_wt;
-    const int tile = is_ret ? lin % n_rt : (lin - tot_ret) % n_wt;
-    const uint32_t sK = base + S::OFF_K, sV = base + S::OFF_V, sQ = base + S::OFF_Q, sDO = base + S::OFF_DO;
-    const uint32_t sPT = base + S::OFF_PT, sDST = base + S::OFF_DST;
-    float* s_col = reinterpret_cast<float*>(smem_raw + S::OFF_COL);
-    const uint32_t bar_kv = base + S::OFF_BAR, bar_q0 = bar_kv + 8, bar_s0 = bar_kv + 40, bar_g = bar_kv + 56;
-    const uint32_t bar_p = bar_kv + 64, bar_pv = bar_kv + 72, tmem_slot = bar_kv + 80;
-    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + S::OFF_BAR + 80);
+    const uint32_t sA = base + C::OFF_A, sB = base + C::OFF_B, bars = base + C::OFF_BAR;
+    const uint32_t bar_a = bars, bar_ga = bars + 32, bar_af = bars + 64, bar_b = bars + 96, bar_bf = bars + 128, bar_i = bars + 160;   // 4 slots each, bar_i 8
+    const uint32_t bar_x = bars + 224, bar_xf = bars + 232, bar_p = bars + 240, bar_acc = bars + 248, bar_of = bars + 256, bar_c = bars + 264;
+    const uint32_t bar_cc = bars + 272, bar_cf = bars + 288, bar_o = bars + 304, bar_od = bars + 312, bar_es = bars + 320, tmem_slot = bars + 352, answer = bars + 368;   // bar_es 4
+    auto slot = [&](int n) { return reinterpret_cast<volatile Info*>(smem_raw + C::OFF_INFO + (n & 7) * 64); };
+    float* const consts = reinterpret_cast<float*>(smem_raw + C::OFF_C);
+    volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + C::OFF_BAR + 352);
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (so the compiler knows warp is uniform)
 
     if (tid == 0) {
-        mbar_init(bar_kv, 1);
 #pragma unroll
-        for (int s2 = 0; s2 < NSTK; ++s2) mbar_init(bar_q0 + 8 * s2, 1);
-        mbar_init(bar_s0, 1); mbar_init(bar_s0 + 8, 1); mbar_init(bar_g, 128); mbar_init(bar_p, 128); mbar_init(bar_pv, 1);
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_cc + 8 * s, 1); mbar_init(bar_cf + 8 * s, NRW); }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(bar_a + 8 * s, 1); mbar_init(bar_ga + 8 * s, 32); mbar_init(bar_af + 8 * s, 1);
+            mbar_init(bar_b + 8 * s, 1); mbar_init(bar_bf + 8 * s, 1); mbar_init(bar_es + 8 * s, 4);
+        }
+#pragma unroll
+        for (int s = 0; s < 8; ++s) mbar_init(bar_i + 8 * s, 1);
+        mbar_init(bar_x, 1); mbar_init(bar_xf, NRW); mbar_init(bar_p, NRW); mbar_init(bar_acc, 1); mbar_init(bar_of, NRW); mbar_init(bar_c, 1);
+        mbar_init(bar_o, 33); mbar_init(bar_od, NRW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 4) tmem_alloc(tmem_slot, S::TMEM_COLS);
+    if (warp == W_XY) tmem_alloc(tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot_gen;
     pdl_launch_dependents();
     pdl_wait();                                                // everything above ran beside the previous kernel's tail (see launch_pdl)
-    const int n_ret = cnt[bh];
-    const int32_t* id = idx + (size_t)bh * R;
-    const int j0 = is_ret ? 0 : tile * 128;                    // window tile: first key
-    const int e0 = is_ret ? tile * 128 : 0;                    // retained tile: first list entry
-    if (is_ret && e0 >= n_ret) {                               // nothing retained in this slice of the list
-        if (warp == 4) tmem_dealloc(tmem, S::TMEM_COLS);
-        return;
-    }
 
-    // query blocks that can see the tile
-    int ib_start, n_blk;
-    if (!is_ret) {
-        ib_start = j0;
-        const int i_end = min(Tlen - 1, j0 + 127 + W - 1);
-        n_blk = (i_end - ib_start) / 64 + 1;
-    } else {
-        const int first = id[e0] + W;                          // the oldest entry's first far query
-        ib_start = (first / 64) * 64;
-        n_blk = first <= Tlen - 1 ? (Tlen - 1 - ib_start) / 64 + 1 : 0;
-    }
-    // grouped queries: the G query heads of this key/value head walk the same query blocks one after the other and
-    // accumulate into the same dK, dV; walk step t is block t % n_pos of query head bh G + t / n_pos
-    const int n_pos = n_blk;
-    n_blk *= G;
+    // the n-th item out of the ring (whole warp); false: there is none
+    auto enter = [&](int n, Item& it) {
+        bwait(bar_i + 8 * (n & 7), (n >> 3) & 1, 9);
+        const int item = __shfl_sync(0xffffffffu, slot(n)->item, 0);
+        if (item < 0) return false;
+        it = item_of<DKV, BN>(args, item);
+        it.n_tiles = __shfl_sync(0xffffffffu, slot(n)->n_tiles, 0);
+        if (DKV) { it.a = __shfl_sync(0xffffffffu, slot(n)->a, 0); it.b = __shfl_sync(0xffffffffu, slot(n)->b, 0); }
+        return true;
+    };
 
-    if (warp == 4) {
-        // (the whole warp walks the loop and waits; only the TMA / tcgen05 instructions are guarded by the lane test)
-        const bool leader = lane == 0;
-        if (n_blk > 0) {
-            constexpr uint32_t IDESC_S = instr_desc(128, 64, false);
-            constexpr uint32_t IDESC_O = instr_desc(128, D, true);
-            const uint32_t k_lo = desc_lo(sK, 16), v_lo = desc_lo(sV, 16), q_lo = desc_lo(sQ, 16), do_lo = desc_lo(sDO, 16);
-            const uint32_t pt_lo = desc_lo(sPT, 16), dst_lo = desc_lo(sDST, 16);
-            const uint32_t qmn_lo = desc_lo(sQ, 8192), domn_lo = desc_lo(sDO, 8192);
-            uint32_t q_phase = 0;
-            auto tma_blk = [&](int t) {
-                const int st = t % NSTK;
-                const uint32_t bar = bar_q0 + 8 * st;
-                const int y = ib_start + (t % n_pos) * 64, bhq = bh * G + t / n_pos;
-                if (leader) {
-                    mbar_expect_tx(bar, 2 * S::QBLK);
+    if (warp == W_LOAD) {
+        // ================================= load warp (lane 0 issues the TMA loads) ==============================
+        // gathers the k and v rows at pos (-1: zeros): 8 lanes per row copy their 16-byte pieces
+        auto gather = [&](uint32_t dst1, uint32_t dst2, int bhk, const int (&pos)[4], uint32_t bar) {
+            const size_t head = (size_t)bhk * args.Tlen * args.dg;
+            const int sub = lane & 7;
 #pragma unroll
-                    for (int sb = 0; sb < SUB; ++sb) {
-                        tma_load_3d(sQ + st * S::QBLK + sb * 8192, &tmQ, sb * 64, y, bhq, bar);
-                        tma_load_3d(sDO + st * S::QBLK + sb * 8192, &tmDO, sb * 64, y, bhq, bar);
-                    }
-                }
-            };
-            auto wait_blk = [&](int t) {
-                const int st = t % NSTK;
-                bwait(bar_q0 + 8 * st, (q_phase >> st) & 1u, 2); q_phase ^= 1u << st;
-            };
-            auto mma_s_dp = [&](int t) {
-                const uint32_t so = (uint32_t)(t % NSTK) * (S::QBLK >> 4);
-                const uint32_t tb = tmem + (DB ? (uint32_t)(t & 1) * 128u : 0u);
-                if (leader) {
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma(tb, desc64(k_lo + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                             desc64(q_lo + so + (kk >> 2) * 512 + (kk & 3) * 2, kDescHi), IDESC_S, kk > 0);
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma(tb + DP_COL, desc64(v_lo + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                             desc64(do_lo + so + (kk >> 2) * 512 + (kk & 3) * 2, kDescHi), IDESC_S, kk > 0);
-                    umma_commit(DB ? bar_s0 + 8 * (t & 1) : bar_s0);
-                }
-                __syncwarp();
-            };
-            if (!is_ret && leader) {
-                mbar_expect_tx(bar_kv, 2 * S::KTILE);
+            for (int ps = 0; ps < 32; ++ps) {
+                const int row = ps * 4 + (lane >> 3), at = __shfl_sync(0xffffffffu, pos[ps >> 3], row & 31);
 #pragma unroll
                 for (int sb = 0; sb < SUB; ++sb) {
-                    tma_load_3d(sK + sb * 16384, &tmK, sb * 64, j0, bh, bar_kv);
-                    tma_load_3d(sV + sb * 16384, &tmV, sb * 64, j0, bh, bar_kv);
+                    const int c = sb * 8 + sub;
+                    const bool real = at >= 0 && c * 8 < args.dg;   // (columns past the head dimension are zero-filled)
+                    const size_t off = real ? head + (size_t)at * args.dg + c * 8 : 0;
+                    const uint32_t to = sb * 16384 + row * 128 + ((sub ^ (row & 7)) << 4);
+                    cp_async16(dst1 + to, args.k + off, real ? 16u : 0u);
+                    cp_async16(dst2 + to, args.v + off, real ? 16u : 0u);
                 }
             }
-            for (int t = 0; t < NSTK && t < n_blk; ++t) tma_blk(t);
-            if (!is_ret) bwait(bar_kv, 0, 1); else bwait(bar_g, 0, 10);   // the tile's own K/V rows are in shared memory
-            wait_blk(0);
-            tc_fence_after();
-            mma_s_dp(0);
-            if (DB && n_blk > 1) { wait_blk(1); mma_s_dp(1); }
-            for (int t = 0; t < n_blk; ++t) {
-                bwait(bar_p, t & 1, 7);                        // P^T(t), dS^T(t) are in shared memory
-                tc_fence_after();
-                // one buffer: the next block's S^T, dP^T first (the key threads wait for those, while dV, dK of this block
-                // are only needed before the operand buffers are rewritten a block later); two buffers: the next block's
-                // products are already there, so dV, dK go first and block t+2's products take the buffer of block t,
-                // which the key threads have read out
-                if (!DB && t + 1 < n_blk) { wait_blk(t + 1); mma_s_dp(t + 1); }
-                {
-                    const uint32_t so = (uint32_t)(t % NSTK) * (S::QBLK >> 4);
-                    if (leader) {
+            cp_async_arrive(bar);
+        };
+        uint32_t g = 0;
+        ItemQueue queue(answer, bar_c, lane);
+        for (int n = 0;; ++n) {
+            Item it;
+            int pos[4] = {-1, -1, -1, -1};                     // dkv list tiles: the positions of their rows
+            for (bool own = n == 0;; own = false) {
+                it.item = own ? (int)blockIdx.x : queue.take(17, &g_bwd_status);
+                if (it.item < 0) break;
+                it = item_of<DKV, BN>(args, it.item);
+                if (!it.list) break;
+                const int n_ret = args.cnt[it.bhk];
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            umma(tmem + DV_COL, desc64(pt_lo + kk * 2, kDescHi), desc64(domn_lo + so + kk * 128, kDescHi), IDESC_O,
-                                 (t > 0 || kk > 0) ? 1u : 0u);
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            umma(tmem + DK_COL, desc64(dst_lo + kk * 2, kDescHi), desc64(qmn_lo + so + kk * 128, kDescHi), IDESC_O,
-                                 (t > 0 || kk > 0) ? 1u : 0u);
-                        umma_commit(bar_pv);
-                    }
-                    __syncwarp();
+                for (int u = 0; u < 4; ++u) {
+                    const int e = it.row0 + u * 32 + lane, at = e < args.R ? args.idx[(size_t)it.bhk * args.R + e] : -1;
+                    pos[u] = e < n_ret ? at : -1;
                 }
-                if (DB && t + 2 < n_blk) { wait_blk(t + 2); mma_s_dp(t + 2); }
-                // the accumulations of block t-1 have completed (the key threads waited for them before producing
-                // block t's operands): its stage can take block t-1+NSTK
-                if (t >= 1 && t - 1 + NSTK < n_blk) tma_blk(t - 1 + NSTK);
+                if (it.row0 < n_ret) break;
+                queue.ask();                                   // nothing is retained in this part of the list
+            }
+            const bool brief = it.item >= 0 && !DKV && it.n_win <= 2;   // (the answer is wanted soon)
+            if (brief) queue.ask();
+            volatile Info* o = slot(n);
+            auto publish = [&]() {
+                if (lane == 0) {
+                    o->item = it.item; o->n_tiles = it.n_tiles; o->a = it.a; o->b = it.b;
+                    mbar_arrive(bar_i + 8 * (n & 7));
+                }
+            };
+            const uint32_t ab = n % AST, a1 = sA + ab * 2 * ATILE, a2 = a1 + ATILE;
+            if (n >= AST) bwait(bar_af + 8 * ab, (n / AST - 1) & 1, 12);
+            if (it.item < 0) { publish(); break; }
+            if (STAGED && n >= AST) bwait(bar_es + 8 * ab, (n / AST - 1) & 1, 22);   // the item's outputs have left the buffer
+            if (!DKV && n >= 1) bwait(bar_od, (n - 1) & 1, 19);   // (O and lse of the item before have been read)
+            if (!it.list) {
+                if (lane == 0) {
+                    mbar_expect_tx(bar_a + 8 * ab, 2 * ATILE);
+#pragma unroll
+                    for (int sb = 0; sb < SUB; ++sb) {
+                        tma_load_3d(a1 + sb * 16384, &tmA1, sb * 64, it.row0, it.bh, bar_a + 8 * ab);
+                        tma_load_3d(a2 + sb * 16384, &tmA2, sb * 64, it.row0, it.bh, bar_a + 8 * ab);
+                    }
+                    if (!DKV) {
+                        mbar_expect_tx(bar_o, ATILE);
+#pragma unroll
+                        for (int sb = 0; sb < SUB; ++sb) tma_load_3d(base + C::OFF_O + sb * 16384, &tmO, sb * 64, it.row0, it.bh, bar_o);
+                    }
+                }
+                if (!DKV) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int r = u * 32 + lane;
+                        cp_async4(base + C::OFF_C + (n & 1) * 512 + r * 4, args.lse + (size_t)it.bh * args.Tlen + min(it.row0 + r, args.Tlen - 1));
+                    }
+                    cp_async_arrive(bar_o);
+                }
+            } else {
+                gather(a1, a2, it.bhk, pos, bar_ga + 8 * ab);
+                // queries from the oldest entry's first far query on (at least one block, whose columns the masks then take out)
+                const int first = min(__shfl_sync(0xffffffffu, pos[0], 0) + args.W, args.Tlen - 1);
+                it.a = first / BN * BN;
+                it.b = (args.Tlen - 1 - it.a) / BN + 1;
+                it.n_tiles = it.b * args.G;
+            }
+            if (DKV) publish();
+            int blk = 0, h = DKV ? it.bh * args.G : it.bhk;    // dkv: block of the query head, query head
+            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+                const uint32_t s = g % BST, b1 = sB + s * 2 * BTILE, b2 = b1 + BTILE;
+                if (g >= (uint32_t)BST) bwait(bar_bf + 8 * s, (g / BST - 1) & 1u, 6);
+                if (lane == 0) {
+                    const bool list = !DKV && t >= it.n_win;
+                    const int y = DKV ? it.a + blk * BN : list ? (t - it.n_win) * BN : it.j_start + t * BN;
+                    mbar_expect_tx(bar_b + 8 * s, 2 * BTILE);
+#pragma unroll
+                    for (int sb = 0; sb < SUB; ++sb) {
+                        tma_load_3d(b1 + sb * BN * 128, list ? &tmL1 : &tmB1, sb * 64, y, h, bar_b + 8 * s);
+                        tma_load_3d(b2 + sb * BN * 128, list ? &tmL2 : &tmB2, sb * 64, y, h, bar_b + 8 * s);
+                    }
+                }
+                if (!DKV && t == 0) {                          // tile 0 is a window tile; the list is looked up while it is on its way
+                    const int last = min(it.row0 + BM - 1, args.Tlen - 1) - it.row0;
+                    const ListView f = view_list(args.idx + (size_t)it.bhk * args.R, args.cnt + it.bhk, args.R, it.row0 - args.W, last, lane);
+                    it.n_tiles = it.n_win + (f.all + BN - 1) / BN;
+                    if (lane == 0) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) { o->before[k] = f.before[k]; o->bits[k] = f.bits[k]; }
+                    }
+                    publish();
+                }
+                if (!brief && t == max(it.n_tiles - kAskTiles, 0)) queue.ask();
+                if (DKV && ++blk == it.b) { blk = 0; ++h; }
+            }
+        }
+        __syncwarp();
+    } else if (warp == W_XY) {
+        // ================================= X, Y products (lane 0 issues; the whole warp walks the loop) ==========
+        constexpr uint32_t IDESC = instr_desc(BM, BN, false);
+        const uint32_t a_lo = desc_lo(sA, 16), b_lo = desc_lo(sB, 16);
+        uint32_t g = 0, par_a = 0;                             // parities of bar_a (bits 0 .. 3), bar_ga (4 .. 7)
+        Item it;
+        for (int n = 0; enter(n, it); ++n) {
+            const uint32_t ab = n % AST, at = (it.list ? 4 : 0) + ab;
+            bwait((it.list ? bar_ga : bar_a) + 8 * ab, (par_a >> at) & 1u, 1);
+            par_a ^= 1u << at;
+            if (it.list) fence_proxy_async();                  // (gathered rows are generic-proxy writes)
+            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+                const uint32_t s = g % BST;
+                bwait(bar_b + 8 * s, (g / BST) & 1u, 2);
+                if (g > 0) bwait(bar_xf, (g - 1) & 1, 3);      // the previous tile's X, Y are in registers
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), b1 = b_lo + s * (2 * BTILE >> 4);
+#pragma unroll
+                    for (int xy = 0; xy < 2; ++xy)
+#pragma unroll
+                        for (int kk = 0; kk < D / 16; ++kk)
+                            umma(tmem + (xy ? C::Y : C::X), desc64(a1 + xy * (ATILE >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
+                                 desc64(b1 + xy * (BTILE >> 4) + (kk >> 2) * (BN * 8) + (kk & 3) * 2, kDescHi), IDESC, kk > 0);
+                    umma_commit(bar_x);
+                    if (t == it.n_tiles - 1) umma_commit(bar_af + 8 * ab);
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp == W_ACC) {
+        // ================================= accumulation ==========================================================
+        constexpr uint32_t IDESC = instr_desc(BM, D, true);
+        const uint32_t b_lo = desc_lo(sB, BN * 128);
+        uint32_t g = 0;
+        Item it;
+        for (int n = 0; enter(n, it); ++n) {
+            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+                const uint32_t s = g % BST;
+                if (t == 0 && n > 0) bwait(bar_of, (n - 1) & 1, 13);   // the previous item's accumulators have been read out
+                bwait(bar_p, g & 1, 7);
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t b1 = b_lo + s * (2 * BTILE >> 4);
+                    if (DKV) {
+#pragma unroll
+                        for (int kk = 0; kk < BN / 16; ++kk)
+                            umma_ts(tmem + C::ACC1, tmem + C::P + kk * 8, desc64(b1 + (BTILE >> 4) + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < BN / 16; ++kk)
+                        umma_ts(tmem + C::ACC0, tmem + C::DS + kk * 8, desc64(b1 + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+                    umma_commit(bar_acc);
+                    umma_commit(bar_bf + 8 * s);
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp >= NRW) {
+        // ================================= constants (dkv) =======================================================
+        // per tile: -L2 and -delta scale of its BN queries (queries past the end are masked by the rows)
+        Item it;
+        uint32_t g = 0;
+        for (int n = 0; DKV && enter(n, it); ++n) {
+            int i0 = it.a;
+            size_t head = (size_t)it.bh * args.G * args.Tlen;
+            for (int t = 0, blk = 0; t < it.n_tiles; ++t, ++g) {
+                float l[BN / 32], dl[BN / 32];
+#pragma unroll
+                for (int u = 0; u < BN / 32; ++u) {
+                    const int i = min(i0 + u * 32 + lane, args.Tlen - 1);
+                    l[u] = args.lse[head + i]; dl[u] = args.delta[head + i];
+                }
+                if (g >= 2) bwait(bar_cf + 8 * (g & 1), ((g >> 1) - 1) & 1, 14);
+                float* c = consts + (g & 1) * 256;
+#pragma unroll
+                for (int u = 0; u < BN / 32; ++u) { c[u * 32 + lane] = -l[u] * kLog2e; c[128 + u * 32 + lane] = -dl[u] * args.scale; }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_cc + 8 * (g & 1));
+                i0 += BN;
+                if (++blk == it.b) { blk = 0; i0 = it.a; head += args.Tlen; }
             }
         }
     } else {
-        // ==================================== key threads: thread r owns key row r ===========================
-        const int pos = is_ret ? (e0 + tid < n_ret ? id[e0 + tid] : -1) : (j0 + tid < Tlen ? j0 + tid : -1);
-        if (is_ret) {
-            // this tile's K / V rows, gathered once (zero rows past the end of the list)
-            const size_t rowoff = ((size_t)bh * Tlen + (pos >= 0 ? pos : 0)) * dg;   // dg: the head dimension in memory (see the dq kernel)
+        // ================================= row warps ==============================================================
+        // Four threads per row: thread `row` of warps 4 q .. 4 q + 3 takes columns [q CW, q CW + CW) of every tile.
+        const int quarter = warp & 3, q = warp >> 2, row = quarter * 32 + lane, c0 = q * CW;
+        const float c2 = args.scale * kLog2e;
+        const uint64_t c2_2 = pack2(c2, c2), scale_2 = pack2(args.scale, args.scale);
+        const uint32_t trow = tmem + (((uint32_t)(quarter * 32)) << 16);   // this warp's TMEM lanes
+        const int Tlen = args.Tlen, W = args.W, dg = args.dg;
+        uint32_t g = 0;
+        // The accumulators of a finished item: D/4 columns per thread, read and stored under the next item's first tile.
+        uint64_t l_dr = 0ull, dr2 = 0ull;                      // dkv: Eq. 6's <v_j, dV_j> = sum_i P_ij dP_ij over this thread's columns
+        int l_list = 0, l_bh = 0, l_row = -1, l_pos = -1;      // its kind, head, list entry or row, position (-1: none)
+        auto epilogue = [&](int n) {
+            constexpr int EC = D / 4;
+            const int e0 = q * EC;
+            const bool live = l_pos >= 0 && e0 < dg, tiles = STAGED && !l_list;
+            const size_t out = ((size_t)l_bh * (l_list ? args.R : Tlen) + l_row) * dg + e0;
+            const uint32_t stage = sA + (n % AST) * 2 * ATILE;
 #pragma unroll
-            for (int c = 0; c < D / 8; ++c) {
-                const uint32_t off = (c >> 3) * 16384 + tid * 128 + (((c & 7) ^ (tid & 7)) << 4);
-                const bool real = pos >= 0 && c * 8 < dg;
-                cp_async16(sK + off, kg + rowoff + (real ? c * 8 : 0), real ? 16u : 0u);
-                cp_async16(sV + off, vg + rowoff + (real ? c * 8 : 0), real ? 16u : 0u);
-            }
-            cp_async_commit();
-            cp_async_wait<0>();
-            fence_proxy_async();
-            mbar_arrive(bar_g);
-        }
-        const float c2 = scale * kLog2e;
-        const uint32_t lane_base = ((uint32_t)(warp * 32)) << 16;
-        // per-column constants of the next block, fetched one block ahead: thread c < 64 holds -L2, thread 64 + c
-        // -delta scale (the forms the fused multiply-adds below take).  The fetch returns the value as loaded and the
-        // factor is applied a block later, where it is stored: arithmetic placed right behind the load would hold the
-        // warp (which issues in order) for the whole latency of the load.
-        const float* col_src = tid < 64 ? lse : delta;
-        const float col_mul = tid < 64 ? -kLog2e : -scale;
-        auto col_fetch = [&](int t) -> float {
-            if (t >= n_blk) return 0.f;
-            const int i = ib_start + (t % n_pos) * 64 + (tid & 63);
-            if (i >= Tlen) return tid < 64 ? INFINITY : 0.f;                    // -L2 = -inf makes P = 0
-            const size_t bhq = (size_t)bh * G + t / n_pos;
-            return col_src[bhq * Tlen + i];
-        };
-        float col_next = col_fetch(0);
-
-        for (int t = 0; t < n_blk; ++t) {
-            group_sync();                                      // everyone is done with the previous block's constants
-            s_col[tid] = col_next * col_mul;
-            col_next = col_fetch(t + 1);
-            group_sync();
-            const int ib = ib_start + (t % n_pos) * 64;
-            int c_lo, c_hi;                                    // query columns of the block this key row may be seen by
-            if (pos < 0) { c_lo = 1 << 20; c_hi = -(1 << 20); }
-            else if (!is_ret) { c_lo = pos - ib; c_hi = min(pos + W - 1, Tlen - 1) - ib; }
-            else { c_lo = pos + W - ib; c_hi = Tlen - 1 - ib; }
-            const int u_lo = __reduce_min_sync(0xffffffffu, c_lo), u_hi = __reduce_max_sync(0xffffffffu, c_hi);
-
-            if (DB) bwait(bar_s0 + 8 * (t & 1), (t >> 1) & 1, 3);   // S^T(t), dP^T(t) are in TMEM
-            else bwait(bar_s0, t & 1, 3);
-            tc_fence_after();
-            const uint32_t tb = tmem + lane_base + (DB ? (uint32_t)(t & 1) * 128u : 0u);
-            uint32_t pp[32], pd[32];                           // P^T and dS^T rows as 64 bf16 each
-            const uint64_t c2_2 = pack2(c2, c2), scale_2 = pack2(scale, scale);
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                const bool act = cb * 32 <= u_hi && cb * 32 + 31 >= u_lo;
-                if (act) {
-                    uint32_t rs[32], rp[32];
-                    tmem_ld32(tb + cb * 32, rs);
-                    tmem_ld32(tb + DP_COL + cb * 32, rp);
-                    const int a = min(max(c_lo - cb * 32, 0), 32), b2 = min(max(c_hi - cb * 32 + 1, 0), 32);
-                    const uint32_t below_b = b2 >= 32 ? 0xffffffffu : ((1u << b2) - 1u);
-                    const uint32_t below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
-                    const uint32_t vm = b2 > a ? (below_b & ~below_a) : 0u;   // validity bits of this row's 32 columns
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < 32; c += 4) {
-                        const int col = cb * 32 + c;
-                        const float4 l4 = *reinterpret_cast<const float4*>(&s_col[col]);
-                        const float4 d4 = *reinterpret_cast<const float4*>(&s_col[64 + col]);
-                        // packed fp32 pairs: exponent arguments, (dP scale - delta scale), their product with P
-                        float x[4], p[4], ds[4];
-                        unpack2(fma2(pack2(__uint_as_float(rs[c]), __uint_as_float(rs[c + 1])), c2_2, pack2(l4.x, l4.y)), x[0], x[1]);
-                        unpack2(fma2(pack2(__uint_as_float(rs[c + 2]), __uint_as_float(rs[c + 3])), c2_2, pack2(l4.z, l4.w)), x[2], x[3]);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) p[u] = (vm & (1u << (c + u))) ? fast_exp2(x[u]) : 0.f;
-                        unpack2(mul2(pack2(p[0], p[1]), fma2(pack2(__uint_as_float(rp[c]), __uint_as_float(rp[c + 1])), scale_2, pack2(d4.x, d4.y))), ds[0], ds[1]);
-                        unpack2(mul2(pack2(p[2], p[3]), fma2(pack2(__uint_as_float(rp[c + 2]), __uint_as_float(rp[c + 3])), scale_2, pack2(d4.z, d4.w))), ds[2], ds[3]);
-                        __nv_bfloat162 h0 = __floats2bfloat162_rn(p[0], p[1]), h1 = __floats2bfloat162_rn(p[2], p[3]);
-                        __nv_bfloat162 g0 = __floats2bfloat162_rn(ds[0], ds[1]), g1 = __floats2bfloat162_rn(ds[2], ds[3]);
-                        pp[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&h0);
-                        pp[cb * 16 + (c >> 1) + 1] = *reinterpret_cast<uint32_t*>(&h1);
-                        pd[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&g0);
-                        pd[cb * 16 + (c >> 1) + 1] = *reinterpret_cast<uint32_t*>(&g1);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) { pp[cb * 16 + c] = 0u; pd[cb * 16 + c] = 0u; }
+            for (int a = DKV ? 1 : 0; a >= 0; --a) {           // dkv: dV (1), then dK (0);  dq: dQ
+                uint32_t x[EC];
+                Tmem<EC>::ld(trow + (a ? C::ACC1 : C::ACC0) + e0, x);
+                tmem_wait_ld();
+                if (a == 0) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_of);
                 }
-            }
-            if (t > 0) { bwait(bar_pv, (t - 1) & 1, 4); tc_fence_after(); }   // the MMAs reading the old operands are done
+                if (DKV && l_list) {
+                    float* dst = (a ? args.dv_ret : args.dk_ret) + out;
+                    if (live)
 #pragma unroll
-            for (int ch = 0; ch < 8; ++ch) {
-                const uint32_t off = tid * 128 + ((ch ^ (tid & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sPT + off), "r"(pp[4 * ch]), "r"(pp[4 * ch + 1]),
-                             "r"(pp[4 * ch + 2]), "r"(pp[4 * ch + 3]) : "memory");
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sDST + off), "r"(pd[4 * ch]), "r"(pd[4 * ch + 1]),
-                             "r"(pd[4 * ch + 2]), "r"(pd[4 * ch + 3]) : "memory");
-            }
-            fence_proxy_async();
-            tc_fence_before();
-            mbar_arrive(bar_p);
-        }
-        if (n_blk > 0) { bwait(bar_pv, (n_blk - 1) & 1, 5); tc_fence_after(); }
-
-        // ---- epilogue: dV, dK rows and Eq. 6's <v_j, dV_j> ------------------------------------------------------
-        float dr = 0.f;
-        const bool live = pos >= 0;
-        const size_t orow = is_ret ? ((size_t)bh * R + e0 + tid) * dg : ((size_t)bh * Tlen + (live ? pos : 0)) * dg;
+                        for (int c = 0; c < EC; c += 4)
+                            *reinterpret_cast<float4*>(dst + c) = make_float4(__uint_as_float(x[c]), __uint_as_float(x[c + 1]), __uint_as_float(x[c + 2]), __uint_as_float(x[c + 3]));
+                } else if constexpr (!STAGED) {
+                    // four lanes transpose their four 16-byte pieces, so that a store covers 64 bytes of 8 rows instead of 16 of 32
+                    uint32_t w[4][4];
 #pragma unroll
-        for (int half2 = 0; half2 < 2; ++half2) {              // 0: dV, 1: dK
+                    for (int c = 0; c < 4; ++c)
 #pragma unroll
-            for (int cb = 0; cb < D / 32; ++cb) {
-                uint32_t a4[32];
-                if (n_blk > 0) {
-                    tmem_ld32(tmem + lane_base + (half2 ? DK_COL : DV_COL) + cb * 32, a4);
-                    tmem_wait_ld();
-                } else {
+                        for (int e = 0; e < 4; ++e) w[c][e] = bf16x2(__uint_as_float(x[c * 8 + 2 * e]), __uint_as_float(x[c * 8 + 2 * e + 1]));
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) a4[c] = 0u;
-                }
-                if (half2 == 0) {
-                    // v row of this key from the swizzled tile in shared memory
+                    for (int m = 1; m <= 2; m <<= 1)
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const int ch = cb * 4 + g;             // 16-byte chunk index within the row
-                        const uint4 u = *reinterpret_cast<const uint4*>(smem_raw + S::OFF_V + (ch >> 3) * 16384 + tid * 128 +
-                                                                        (((ch & 7) ^ (tid & 7)) << 4));
-                        const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
+                        for (int c = 0; c < 4; ++c) {
+                            if (c & m) continue;
 #pragma unroll
-                        for (int x = 0; x < 4; ++x) {
-                            dr = fmaf(__uint_as_float(w4[x] << 16), __uint_as_float(a4[g * 8 + 2 * x]), dr);
-                            dr = fmaf(__uint_as_float(w4[x] & 0xffff0000u), __uint_as_float(a4[g * 8 + 2 * x + 1]), dr);
-                        }
-                    }
-                }
-                if (live && cb * 32 < dg && (is_ret || F32OUT || D != 64)) {
-                    if (is_ret || F32OUT) {
-                        float* dst = (is_ret ? (half2 ? dk_ret : dv_ret) : (half2 ? dk32 : dv32)) + orow + cb * 32;
-#pragma unroll
-                        for (int c = 0; c < 32; c += 4)
-                            *reinterpret_cast<float4*>(dst + c) = make_float4(__uint_as_float(a4[c]), __uint_as_float(a4[c + 1]),
-                                                                              __uint_as_float(a4[c + 2]), __uint_as_float(a4[c + 3]));
-                    } else if (D != 64) {
-                        __nv_bfloat16* dst = (half2 ? dk : dv) + orow + cb * 32;
-#pragma unroll
-                        for (int c = 0; c < 32; c += 8) {
-                            uint32_t w4[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(a4[c + 2 * u]), __uint_as_float(a4[c + 2 * u + 1]));
-                                w4[u] = *reinterpret_cast<uint32_t*>(&h);
+                            for (int e = 0; e < 4; ++e) {      // my piece for the partner: c ^ m if I am the lower lane, else c
+                                const bool up = (lane & m) != 0;
+                                const uint32_t r = __shfl_xor_sync(0xffffffffu, up ? w[c][e] : w[c ^ m][e], m);
+                                if (up) w[c][e] = r; else w[c ^ m][e] = r;
                             }
-                            *reinterpret_cast<uint4*>(dst + c) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
                         }
-                    }
-                }
-                if (D == 64 && !is_ret && !F32OUT) {
-                    // window tile, bf16 out: the rows go into the (now idle) P^T / dS^T operand buffers in the swizzled
-                    // layout and leave as one tile store per warp (a 128-byte store per thread stalls the load/store unit)
-                    const uint32_t buf = half2 ? sDST : sPT;
+                    __nv_bfloat16* dst = (DKV ? (a ? args.dv : args.dk) : args.dq);
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
+                    for (int c = 0; c < 4; ++c) {              // now piece lane & 3 of row (lane & ~3) + c
+                        const int r = l_row - lane + (lane & ~3) + c;
+                        if (r < Tlen) *reinterpret_cast<uint4*>(dst + ((size_t)l_bh * Tlen + r) * D + e0 + (lane & 3) * 8) = make_uint4(w[c][0], w[c][1], w[c][2], w[c][3]);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < EC; c += 8) {
                         uint32_t w4[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(a4[g * 8 + 2 * u]), __uint_as_float(a4[g * 8 + 2 * u + 1]));
-                            w4[u] = *reinterpret_cast<uint32_t*>(&h);
-                        }
-                        const int ch = cb * 4 + g;
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(buf + tid * 128 + ((ch ^ (tid & 7)) << 4)),
-                                     "r"(w4[0]), "r"(w4[1]), "r"(w4[2]), "r"(w4[3]) : "memory");
+                        for (int e = 0; e < 4; ++e) w4[e] = bf16x2(__uint_as_float(x[c + 2 * e]), __uint_as_float(x[c + 2 * e + 1]));
+                        const uint32_t to = stage + a * ATILE + row * 128 + ((((e0 + c) >> 3) ^ (row & 7)) << 4);   // (leave as tiles)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(to), "r"(w4[0]), "r"(w4[1]), "r"(w4[2]), "r"(w4[3]) : "memory");
                     }
                 }
             }
-        }
-        if (D == 64 && !is_ret && !F32OUT) {
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0 && j0 + warp * 32 < Tlen) {
-                tma_store_3d(&tmDV, sPT + warp * 4096, 0, j0 + warp * 32, bh);
-                tma_store_3d(&tmDK, sDST + warp * 4096, 0, j0 + warp * 32, bh);
-                bulk_commit();
-                bulk_wait_read0();                             // the buffers are released with the CTA
+            float* s = reinterpret_cast<float*>(smem_raw + C::OFF_DR) + (n & 1) * 512;
+            if (DKV) {                                         // the row's four parts meet (rewritten two items, so two barriers, on)
+                float d0, d1;
+                unpack2(l_dr, d0, d1);
+                s[q * 128 + row] = d0 + d1;
             }
+            if (tiles) fence_proxy_async();
+            if (DKV || STAGED) asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter) : "memory");
+            if (q != 0) return;
+            if (STAGED && lane == 0) {
+                const int r0 = l_row;                          // (lane 0: the first of the quarter's 32 rows)
+                if (tiles && r0 < Tlen) {
+                    tma_store_3d(&tmS1, stage + quarter * 4096, 0, r0, l_bh);
+                    if (DKV) tma_store_3d(&tmS2, stage + ATILE + quarter * 4096, 0, r0, l_bh);
+                    bulk_commit();
+                    bulk_wait_read0();
+                }
+                mbar_arrive(bar_es + 8 * (n % AST));
+            }
+            if (DKV && l_pos >= 0) {
+                const float sum = (s[row] + s[128 + row]) + (s[256 + row] + s[384 + row]);
+                if (l_list) args.dr_ret[(size_t)l_bh * args.R + l_row] = sum;
+                else args.dr_win[(size_t)l_bh * Tlen + l_row] = sum;
+            }
+        };
+        Item it;
+        int n = 0;
+        for (; enter(n, it); ++n) {
+            const int r_abs = it.row0 + row;                   // query, key, or list entry
+            int pos = r_abs, nvis = 0, key_lo = 0, key_hi = 0;
+            uint64_t nl2 = 0ull, ndls = 0ull;
+            if (DKV) {
+                if (it.list) pos = r_abs < args.cnt[it.bh] ? args.idx[(size_t)it.bh * args.R + r_abs] : -1;
+                else if (r_abs >= Tlen) pos = -1;
+                key_lo = it.list ? pos + W : pos;              // queries that see the key
+                key_hi = pos < 0 ? -1 - BN * it.b - it.a : min(it.list ? Tlen - 1 : pos + W - 1, Tlen - 1);
+            } else {
+                const volatile Info* f = slot(n);
+                const int x = min(r_abs, Tlen - 1) - it.row0;
+                nvis = (int)(f->before[x >> 5] + __popc(f->bits[x >> 5] & ((1u << (x & 31)) - 1u)));
+                // delta = <dO, O>: this thread's quarter of the channels, then the four parts (chunk c of row r is at c ^ (r & 7))
+                bwait(bar_a + 8 * (n % AST), (n / AST) & 1, 20);
+                bwait(bar_o, n & 1, 21);
+                const uint32_t so = base + C::OFF_O, sdo = sA + (n % AST) * 2 * ATILE + ATILE;
+                float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+                for (int u = 0; u < D / 32; ++u) {
+                    const int ch = q * (D / 32) + u;
+                    const uint32_t off = (ch >> 3) * 16384 + row * 128 + (((ch & 7) ^ (row & 7)) << 4);
+                    uint32_t aw[4], bw[4];
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(aw[0]), "=r"(aw[1]), "=r"(aw[2]), "=r"(aw[3]) : "r"(so + off));
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(bw[0]), "=r"(bw[1]), "=r"(bw[2]), "=r"(bw[3]) : "r"(sdo + off));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        d0 = fmaf(__uint_as_float(aw[e] << 16), __uint_as_float(bw[e] << 16), d0);
+                        d1 = fmaf(__uint_as_float(aw[e] & 0xffff0000u), __uint_as_float(bw[e] & 0xffff0000u), d1);
+                    }
+                }
+                auto part = [&](int k) {                       // part k replaces the first of the chunks that it was formed from
+                    const int ch = k * (D / 32);
+                    return reinterpret_cast<float*>(smem_raw + C::OFF_O + (ch >> 3) * 16384 + row * 128 + (((ch & 7) ^ (row & 7)) << 4));
+                };
+                *part(q) = d0 + d1;
+                const float nl = -consts[(n & 1) * 128 + row] * kLog2e;
+                asm volatile("bar.sync %0, 128;" ::"r"(5 + quarter) : "memory");
+                const float d = (*part(0) + *part(1)) + (*part(2) + *part(3));
+                fence_proxy_async();                           // (TMA writes the next item's O there)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_od);
+                if (q == 0 && r_abs < Tlen) args.delta[(size_t)it.bh * Tlen + r_abs] = d;
+                nl2 = pack2(nl, nl); ndls = pack2(-d * args.scale, -d * args.scale);
+            }
+            int i_blk = it.a + c0, blk = 0;                    // dkv: first query of this thread's columns, block of the query head
+            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+                // columns of this thread's part that the row may see
+                int c_lo, c_hi;
+                if (!DKV) {
+                    if (t < it.n_win) { const int j = it.j_start + t * BN + c0; c_lo = max(r_abs - W + 1, 0) - j; c_hi = r_abs - j; }
+                    else { c_lo = 0; c_hi = nvis - (t - it.n_win) * BN - c0 - 1; }
+                } else {
+                    c_lo = key_lo - i_blk; c_hi = key_hi - i_blk;
+                    i_blk += BN;
+                    if (++blk == it.b) { blk = 0; i_blk = it.a + c0; }
+                }
+                const int a = min(max(c_lo, 0), CW), b = min(max(c_hi + 1, 0), CW);
+                const uint32_t below_b = b >= 32 ? 0xffffffffu : ((1u << b) - 1u), below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
+                const uint32_t vm = below_b & ~below_a;
+                const bool some = __any_sync(0xffffffffu, vm != 0u), plain = __all_sync(0xffffffffu, a == 0 && b == CW);
+                uint32_t ds[CW / 2], pp[CW / 2];
+                const float* col = consts + (g & 1) * 256 + c0;
+                if (DKV) bwait(bar_cc + 8 * (g & 1), (g >> 1) & 1, 16);
+                bwait(bar_x, g & 1, 5);
+                tc_fence_after();
+                if (some) {
+                    uint32_t x[CW], y[CW];
+                    Tmem<CW>::ld(trow + C::X + c0, x);
+                    Tmem<CW>::ld(trow + C::Y + c0, y);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_xf);        // X, Y of tile g+1 may overwrite the buffers
+                    if (!plain) {
+#pragma unroll
+                        for (int c = 0; c < CW; ++c) x[c] = (vm & (1u << c)) ? x[c] : 0xff800000u;   // -inf: P = 0
+                    }
+#pragma unroll
+                    for (int c = 0; c < CW; c += 4) {          // packed fp32 pairs
+                        uint64_t nl_a = nl2, nl_b = nl2, nd_a = ndls, nd_b = ndls;
+                        if (DKV) {
+                            const float4 l4 = *reinterpret_cast<const float4*>(col + c), d4 = *reinterpret_cast<const float4*>(col + 128 + c);
+                            nl_a = pack2(l4.x, l4.y); nl_b = pack2(l4.z, l4.w); nd_a = pack2(d4.x, d4.y); nd_b = pack2(d4.z, d4.w);
+                        }
+                        float e[4], s[4];
+                        unpack2(fma2(pack2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), c2_2, nl_a), e[0], e[1]);
+                        unpack2(fma2(pack2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), c2_2, nl_b), e[2], e[3]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) e[u] = fast_exp2(e[u]);
+                        if (DKV) {
+                            dr2 = fma2(pack2(e[0], e[1]), pack2(__uint_as_float(y[c]), __uint_as_float(y[c + 1])), dr2);
+                            dr2 = fma2(pack2(e[2], e[3]), pack2(__uint_as_float(y[c + 2]), __uint_as_float(y[c + 3])), dr2);
+                        }
+                        unpack2(mul2(pack2(e[0], e[1]), fma2(pack2(__uint_as_float(y[c]), __uint_as_float(y[c + 1])), scale_2, nd_a)), s[0], s[1]);
+                        unpack2(mul2(pack2(e[2], e[3]), fma2(pack2(__uint_as_float(y[c + 2]), __uint_as_float(y[c + 3])), scale_2, nd_b)), s[2], s[3]);
+                        ds[c / 2] = bf16x2(s[0], s[1]); ds[c / 2 + 1] = bf16x2(s[2], s[3]);
+                        if (DKV) { pp[c / 2] = bf16x2(e[0], e[1]); pp[c / 2 + 1] = bf16x2(e[2], e[3]); }
+                    }
+                } else {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_xf);
+#pragma unroll
+                    for (int c = 0; c < CW / 2; ++c) { ds[c] = 0u; pp[c] = 0u; }
+                }
+                // P(g), dS(g) take the place of tile g-1's, whose accumulation has normally completed; every phase is awaited in turn
+                if (g > 0) { bwait(bar_acc, (g - 1) & 1, 11); tc_fence_after(); }
+                if (t == 0 && n > 0) epilogue(n - 1);
+                Tmem<CW / 2>::st(trow + C::DS + c0 / 2, ds);
+                if (DKV) Tmem<CW / 2>::st(trow + C::P + c0 / 2, pp);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(bar_p); if (DKV) mbar_arrive(bar_cf + 8 * (g & 1)); }
+            }
+            l_list = it.list; l_bh = it.bh; l_row = r_abs;
+            l_dr = dr2; dr2 = 0ull;
+            l_pos = DKV ? pos : r_abs < Tlen ? r_abs : -1;
         }
-        if (live) {
-            if (is_ret) dr_ret[(size_t)bh * R + e0 + tid] = dr;
-            else dr_win[(size_t)bh * Tlen + pos] = dr;
+        if (n > 0) {
+            bwait(bar_acc, (g - 1) & 1, 18);
+            tc_fence_after();
+            epilogue(n - 1);
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) tmem_dealloc(tmem, S::TMEM_COLS);
+    if (warp == W_XY) tmem_dealloc(tmem, 512);
 }
 
 // Far-query share of the retained keys added onto their rows (each key appears once in the list: fixed order).
-template <bool F32OUT>
 __global__ void bwd_merge_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt,
                                  const float* __restrict__ dk_ret, const float* __restrict__ dv_ret,
                                  const float* __restrict__ dr_ret, __nv_bfloat16* __restrict__ dk,
-                                 __nv_bfloat16* __restrict__ dv, float* __restrict__ dk32, float* __restrict__ dv32,
-                                 float* __restrict__ dr_win, int Tlen, int R, int D)
+                                 __nv_bfloat16* __restrict__ dv, float* __restrict__ dr_win, int Tlen, int R, int D)
 {
     pdl_launch_dependents();
     pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
@@ -828,11 +634,8 @@ __global__ void bwd_merge_kernel(const int32_t* __restrict__ idx, const int32_t*
     const int j = idx[(size_t)bh * R + e];
     const size_t src = ((size_t)bh * R + e) * D, dst = ((size_t)bh * Tlen + j) * D;
     for (int c = threadIdx.x; c < D; c += blockDim.x) {
-        if (F32OUT) { dk32[dst + c] += dk_ret[src + c]; dv32[dst + c] += dv_ret[src + c]; }
-        else {
-            dk[dst + c] = __float2bfloat16_rn(__bfloat162float(dk[dst + c]) + dk_ret[src + c]);
-            dv[dst + c] = __float2bfloat16_rn(__bfloat162float(dv[dst + c]) + dv_ret[src + c]);
-        }
+        dk[dst + c] = __float2bfloat16_rn(__bfloat162float(dk[dst + c]) + dk_ret[src + c]);
+        dv[dst + c] = __float2bfloat16_rn(__bfloat162float(dv[dst + c]) + dv_ret[src + c]);
     }
     if (threadIdx.x == 0) dr_win[(size_t)bh * Tlen + j] += dr_ret[(size_t)bh * R + e];
 }
@@ -857,85 +660,81 @@ __global__ void bwd_dz_kernel(float* __restrict__ dz, const float* __restrict__ 
     dz[(size_t)bh * Tlen + j] = g;
 }
 
-}  // namespace
-
-// dq (and delta) on the tensor cores.  Returns LTE_OK or an error; the caller runs the remaining stages.
-int launch_bwd_dq_tc(const Params& p, const void* q, const void* k, const void* v, const void* o, const float* lse,
-                     const void* dO, const int32_t* idx, const int32_t* cnt, void* dq, float* delta, cudaStream_t st)
+template <int D, bool DKV> int launch_pass(const CUtensorMap& a1, const CUtensorMap& a2, const CUtensorMap& b1, const CUtensorMap& b2, const CUtensorMap& o,
+                                           const CUtensorMap& l1, const CUtensorMap& l2, const CUtensorMap& s1, const CUtensorMap& s2, const Args& a, int items, cudaStream_t st)
 {
-    const int BHK = p.B * p.H, BH = BHK * p.G;                 // key/value heads, query heads
-    CUtensorMap tq, tdo, to, tdq, tk, tv;
-    if (!make_map(&tq, q, BH, p.T, p.d, BM) || !make_map(&tdo, dO, BH, p.T, p.d, BM) || !make_map(&to, o, BH, p.T, p.d, BM) ||
-        !make_map(&tdq, dq, BH, p.T, p.d, 32) ||
-        !make_map(&tk, k, BHK, p.T, p.d, BN) || !make_map(&tv, v, BHK, p.T, p.d, BN))
-        return LTE_ERR_CUDA;
-    dim3 grid((p.T + BM - 1) / BM, BH);
-#define LTE_GO(D)                                                                                                  \
-    do {                                                                                                           \
-        static PerDeviceOnce attr;                                                                                 \
-        if (int e = attr.run([] { return cudaFuncSetAttribute(bwd_dq_tc_kernel<D>,                                 \
-                cudaFuncAttributeMaxDynamicSharedMemorySize, SmemQ<D>::BYTES); })) return e;                       \
-        launch_pdl(bwd_dq_tc_kernel<D>, grid, dim3(NTHREADS), SmemQ<D>::BYTES, st,                            \
-            tq, tdo, to, tdq, tk, tv, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)o,        \
-            (const __nv_bfloat16*)dO, lse, idx, cnt, (__nv_bfloat16*)dq, delta, p.T, p.W, p.R, p.scale, p.G, p.d); \
-    } while (0)
-    if (p.d == 64 || p.d == 32) LTE_GO(64); else if (p.d == 128) LTE_GO(128); else return LTE_ERR_UNSUPPORTED;
-#undef LTE_GO
-    return cuda_status(cudaGetLastError());
+    using C = Cfg<D, DKV>;
+    static PerDeviceOnce attr;
+    if (int e = attr.run([] { return cudaFuncSetAttribute(bwd_tc_kernel<D, DKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::BYTES); })) return e;
+    return cuda_status(launch_pdl(bwd_tc_kernel<D, DKV>, dim3(items), dim3(NTHREADS), C::BYTES, st, a1, a2, b1, b2, o, l1, l2, s1, s2, a));
 }
 
-// dk, dv, dz on the tensor cores.  `ret_ws` holds dk_ret, dv_ret [B,H,R,d] and dr_ret [B,H,R] (fp32).
+}  // namespace
+
 size_t bwd_tc_ret_bytes(const Params& p)
 {
     const size_t n = (size_t)p.B * p.H * (p.R > 0 ? p.R : 1);
     return ((2 * n * p.d + n) * 4 + 255) / 256 * 256;
 }
 
+// dq (and delta) on the tensor cores.  Returns LTE_OK or an error; the caller runs the remaining stages.  `ret_ws` (the dkv pass's
+// scratch, not in use yet) takes the retained rows of k and v in list order, so that list tiles are TMA boxes.
+int launch_bwd_dq_tc(const Params& p, const void* q, const void* k, const void* v, const void* o, const float* lse,
+                     const void* dO, const int32_t* idx, const int32_t* cnt, void* dq, float* delta, void* ret_ws, cudaStream_t st)
+{
+    const int BHK = p.B * p.H, BH = BHK * p.G;                 // key/value heads, query heads
+    CUtensorMap tq, tdo, tk, tv, to, tdq, tlk, tlv;
+    constexpr int bn = Cfg<64, false>::BN;
+    static_assert(bn == Cfg<128, false>::BN, "");
+    if (!make_map(&tq, q, BH, p.T, p.d, BM) || !make_map(&tdo, dO, BH, p.T, p.d, BM) || !make_map(&to, o, BH, p.T, p.d, BM) ||
+        !make_map(&tdq, dq, BH, p.T, p.d, 32) || !make_map(&tk, k, BHK, p.T, p.d, bn) || !make_map(&tv, v, BHK, p.T, p.d, bn)) return LTE_ERR_CUDA;
+    tlk = tk; tlv = tv;
+    if (p.R > 0) {
+        char* kc = (char*)ret_ws; char* vc = kc + (size_t)BHK * p.R * p.d * 4;   // (each of the two fp32 tensors has room for a bf16 one)
+        if (int e = launch_prefill_compact(p, k, v, idx, cnt, kc, vc, st)) return e;
+        if (!make_map(&tlk, kc, BHK, p.R, p.d, bn) || !make_map(&tlv, vc, BHK, p.R, p.d, bn)) return LTE_ERR_CUDA;
+    }
+    Args a = {};
+    a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
+    a.lse = lse; a.delta = delta; a.idx = idx; a.cnt = cnt; a.dq = (__nv_bfloat16*)dq;
+    a.n_rows = (p.T + BM - 1) / BM; a.n_bh = BH;
+    a.Tlen = p.T; a.W = p.W; a.R = p.R; a.G = p.G; a.dg = p.d; a.scale = p.scale;
+    const int items = a.n_rows * BH;
+    if (p.d == 64 || p.d == 32) return launch_pass<64, false>(tq, tdo, tk, tv, to, tlk, tlv, tdq, tdq, a, items, st);
+    return p.d == 128 ? launch_pass<128, false>(tq, tdo, tk, tv, to, tlk, tlv, tdq, tdq, a, items, st) : LTE_ERR_UNSUPPORTED;
+}
+
+// dk, dv, dz on the tensor cores.  `ret_ws` holds dk_ret, dv_ret [B,H,R,d] and dr_ret [B,H,R] (fp32).
 int launch_bwd_dkv_tc(const Params& p, const void* q, const void* k, const void* v, const float* lse, const void* dO,
                       const float* delta, const float* z, const int32_t* idx, const int32_t* cnt, const float* lambda,
-                      void* dk, void* dv, float* dk32, float* dv32, float* dz, void* ret_ws, bool f32out, bool merge_here,
-                      cudaStream_t st)
+                      void* dk, void* dv, float* dz, void* ret_ws, bool merge_here, cudaStream_t st)
 {
-    const int BH = p.B * p.H;
+    const int BH = p.B * p.H, bn = p.d == 128 ? Cfg<128, true>::BN : Cfg<64, true>::BN;
     CUtensorMap tk, tv, tq, tdo, tdk, tdv;
-    if (!make_map(&tk, k, BH, p.T, p.d, 128) || !make_map(&tv, v, BH, p.T, p.d, 128) ||
-        !make_map(&tq, q, BH * p.G, p.T, p.d, 64) || !make_map(&tdo, dO, BH * p.G, p.T, p.d, 64) ||
-        !make_map(&tdk, dk, BH, p.T, p.d, 32) || !make_map(&tdv, dv, BH, p.T, p.d, 32))
-        return LTE_ERR_CUDA;
+    if (!make_map(&tk, k, BH, p.T, p.d, BM) || !make_map(&tv, v, BH, p.T, p.d, BM) ||
+        !make_map(&tq, q, BH * p.G, p.T, p.d, bn) || !make_map(&tdo, dO, BH * p.G, p.T, p.d, bn) ||
+        !make_map(&tdk, dk, BH, p.T, p.d, 32) || !make_map(&tdv, dv, BH, p.T, p.d, 32)) return LTE_ERR_CUDA;
     const size_t n = (size_t)BH * (p.R > 0 ? p.R : 1);
     float* dk_ret = (float*)ret_ws;
     float* dv_ret = dk_ret + n * p.d;
     float* dr_ret = dv_ret + n * p.d;
-    const int n_wt = (p.T + 127) / 128, n_rt = (p.R + 127) / 128;
-    dim3 grid(n_wt + n_rt, BH);
-#define LTE_GO(D, F)                                                                                               \
-    do {                                                                                                           \
-        static PerDeviceOnce attr;                                                                                 \
-        if (int e = attr.run([] { return cudaFuncSetAttribute(bwd_dkv_tc_kernel<D, F>,                             \
-                cudaFuncAttributeMaxDynamicSharedMemorySize, SmemK<D>::BYTES); })) return e;                       \
-        launch_pdl(bwd_dkv_tc_kernel<D, F>, grid, dim3(NTHREADS), SmemK<D>::BYTES, st,                              \
-            tk, tv, tq, tdo, tdk, tdv, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, lse, delta, idx, cnt,     \
-            (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dk32, dv32, dz, dk_ret, dv_ret, dr_ret, n_wt, p.T, p.W, p.R,   \
-            p.scale, p.G, p.d);                                                                                    \
-    } while (0)
-    if (p.d == 64 || p.d == 32) { if (f32out) LTE_GO(64, true); else LTE_GO(64, false); }
-    else if (p.d == 128) { if (f32out) LTE_GO(128, true); else LTE_GO(128, false); }
-    else return LTE_ERR_UNSUPPORTED;
-#undef LTE_GO
+    Args a = {};
+    a.k = (const __nv_bfloat16*)k; a.v = (const __nv_bfloat16*)v;
+    a.lse = lse; a.delta = const_cast<float*>(delta); a.idx = idx; a.cnt = cnt;
+    a.dk = (__nv_bfloat16*)dk; a.dv = (__nv_bfloat16*)dv; a.dr_win = dz; a.dk_ret = dk_ret; a.dv_ret = dv_ret; a.dr_ret = dr_ret;
+    a.n_rows = (p.T + BM - 1) / BM; a.n_bh = BH; a.n_list = (p.R + BM - 1) / BM;
+    a.Tlen = p.T; a.W = p.W; a.R = p.R; a.G = p.G; a.dg = p.d; a.scale = p.scale;
+    const int items = (a.n_rows + a.n_list) * BH;
+    int e = LTE_ERR_UNSUPPORTED;
+    if (p.d == 64 || p.d == 32) e = launch_pass<64, true>(tk, tv, tq, tdo, tq, tq, tq, tdk, tdv, a, items, st);
+    else if (p.d == 128) e = launch_pass<128, true>(tk, tv, tq, tdo, tq, tq, tq, tdk, tdv, a, items, st);
     // merge_here = false: the caller's last pass adds the retained shares and turns dr into dz itself
-    if (!merge_here) return cuda_status(cudaGetLastError());
+    if (e || !merge_here) return e;
     if (p.R > 0) {
-        dim3 gm(p.R, BH);
-        if (f32out)
-            launch_pdl(bwd_merge_kernel<true>, gm, dim3(64), 0, st, idx, cnt, dk_ret, dv_ret, dr_ret, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv,
-                                                      dk32, dv32, dz, p.T, p.R, p.d);
-        else
-            launch_pdl(bwd_merge_kernel<false>, gm, dim3(64), 0, st, idx, cnt, dk_ret, dv_ret, dr_ret, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv,
-                                                       dk32, dv32, dz, p.T, p.R, p.d);
+        if (launch_pdl(bwd_merge_kernel, dim3(p.R, BH), dim3(64), 0, st, idx, cnt, dk_ret, dv_ret, dr_ret, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv,
+                       dz, p.T, p.R, p.d) != cudaSuccess) return LTE_ERR_CUDA;
     }
-    dim3 gz((p.T + 255) / 256, BH);
-    launch_pdl(bwd_dz_kernel, gz, dim3(256), 0, st, dz, z, lambda, p.H, p.T, p.half, p.zthr);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(bwd_dz_kernel, dim3((p.T + 255) / 256, BH), dim3(256), 0, st, dz, z, lambda, p.H, p.T, p.half, p.zthr));
 }
 
 int bwd_status_fetch_and_clear() { return status_fetch_and_clear(g_bwd_status); }

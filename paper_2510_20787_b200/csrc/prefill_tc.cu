@@ -29,7 +29,7 @@
 //
 // d = 32 runs the same kernel: the tensor maps describe 32-column rows with a 64-column box, the copy engine fills the upper
 // half of every tile row with zeros, and only the first 32 output columns are stored.
-#include "tc_common.cuh"
+#include "tile_items.cuh"
 
 namespace lte {
 
@@ -119,19 +119,6 @@ struct Cursor {
     bool live = true;
     __device__ __forceinline__ void advance() { ++g; if (++t == it.n_tiles) { t = 0; ++n; } }
 };
-// Asks for a block of this grid that has not started (the answer, 16 bytes, arrives on the barrier).
-__device__ __forceinline__ void ask_for_block(uint32_t answer, uint32_t bar) {
-    mbar_expect_tx(bar, 16);
-    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
-}
-__device__ __forceinline__ int block_from(uint32_t answer) {   // its index, or -1
-    uint32_t ok, x;
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tld.shared.b128 h, [%2];\n\tclusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, _, _, _}, h;\n\t}"
-                 : "=r"(ok), "=r"(x) : "r"(answer) : "memory");
-    return ok ? (int)x : -1;
-}
-
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
