@@ -1157,8 +1157,8 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
     if (p.stack) ps.K = 0;                               // the stack is scored outside the step (lte_cache_score)
     if (p.W + p.R > MAX_ROWS) return LTE_ERR_UNSUPPORTED;
     if (p.dtype == LTE_BF16) {
-        // one query head and a block of 256 rows that is a tcgen05 operand as it stands: 29 us at 2,048 heads, where the other
-        // kernel takes 35; everything else in bf16 goes through mma.sync
+        // one query head and a block of rows that is a tcgen05 operand as it stands: 27 us at 2,048 heads x 256 rows, where the
+        // other kernel takes 36 (4,096 x 128: 29 and 45; 16 x 256: 5.2 and 6.6); everything else in bf16 goes through mma.sync
         if (p.G <= 1 && cache_layout(p.d, p.W, p.R, p.dtype).swz) return launch_decode_tc(ps, cache, q1, k1, v1, o1, lse1, st);
         return launch_decode_mma(ps, cache, q1, k1, v1, o1, lse1, st);
     }

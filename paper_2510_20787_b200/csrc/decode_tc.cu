@@ -10,8 +10,17 @@
 //            MN-major operand: group 0 = rows 0..127, group 1 = rows 128..255), N = 16 (B row 0 = p[0..127],
 //            row 1 = p[128..255]), K = 128 keys; channel c is D[c][0] + D[64+c][1].
 // Persistent CTAs walk consecutive heads; a control lane issues the bulk copies (next head's keys as soon as this
-// head's logits are taken, next values after the PV chain) and every tcgen05.mma; the replacement decision, the
-// scorer tap sums and the write-back stay as in the ALU kernel.  Every wait is bounded.
+// head's logits are taken, next values after the PV chain, the logits and positions a head ahead) and every tcgen05.mma; the replacement
+// decision, the scorer tap sums and the write-back stay as in the ALU kernel.  Every wait is bounded.
+//
+// Bound by memory only as far as the chain of a head (copy, logits, softmax, output: some 4 us) is short enough for the CTAs that fit
+// on an SM to keep it busy.  So only rows that exist are copied, the worst pool entry and the maximum are found by warp-wide
+// reductions of one instruction, the next head's inputs are asked for under this head's output, and one barrier per head is left.
+// Measured (B200, a step in a CUDA graph, before -> now): 2,048 heads x 256 rows 30.6 -> 26.9 us (137 MB: 5.1 TB/s), 1,024 x 256
+// 16.3 -> 13.7, 4,096 x 128 56.0 -> 28.9, 16 x 256 5.7 -> 5.2.  Asking for the next head in L2 ahead: 31.2 -> 33.3; two stages of 128
+// rows each instead of five CTAs: 37.9.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace lte {
@@ -21,24 +30,46 @@ __device__ StatusWord g_decode_tc_status = LTE_STATUS_INIT;
 namespace {
 
 using namespace tc;
-constexpr int NC = 256;                    // compute threads: thread j owns cache row j
-constexpr int NTHR = NC + 32;              // + control warp
+// NC compute threads (thread j owns cache row j): 256, or 128 where there are no more rows.  Half the threads and half the shared memory
+// then let five CTAs share an SM instead of three, which counts because every head costs its CTA a chain of some 4 us.
+template <int NC> constexpr int kThreads = NC + 32;            // + control warp
+template <int NC> constexpr int kPerSm = NC == 256 ? 3 : 5;
 constexpr int D = 64;
 constexpr uint32_t TMEM_COLS = 64;         // S^T: [0,16) keys 0..127, [16,32) keys 128..255;  O halves: [32,48)
 
 __device__ __forceinline__ void dwait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_decode_tc_status); }
-__device__ __forceinline__ void csync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ float redux_max(float x) {
+    float y;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Loads that stay where they are written (the compiler would move them to their first use, behind the waits).
+__device__ __forceinline__ uint32_t load32(const void* p) {
+    uint32_t x;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+    return x;
+}
+__device__ __forceinline__ uint4 load128(const void* p) {
+    uint4 x;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p) : "memory");
+    return x;
+}
+__device__ __forceinline__ float2 bf16_pair(uint32_t x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)); }
+template <int NC> __device__ __forceinline__ void csync() { asm volatile("bar.sync 1, %0;" ::"n"(NC) : "memory"); }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-struct Plan { uint32_t off_v, off_tail, tail_bytes, off_q, off_p, off_bar, total; };
-__host__ __device__ inline Plan plan_of(const CacheLayout& L) {
+struct Plan { uint32_t off_v, off_k, off_tail, tail_bytes, off_q, off_p, off_bar, total; };
+template <int NC> __host__ __device__ inline Plan plan_of(const CacheLayout& L) {
     Plan P;
-    P.off_v = 32768;                                   // K block [256][64] bf16, then V block
-    P.off_q = 65536;                                   // B operand of the logits: [16][64] bf16 (2 KB)
+    // V block [NC][64] bf16, then K block: the output product reads 256 rows from the value block on (its upper half is used with
+    // NC = 256 only), which have to be there
+    P.off_v = 0;
+    P.off_k = NC * 128;
+    P.off_q = 2 * NC * 128;                            // B operand of the logits: [16][64] bf16 (2 KB)
     P.off_p = P.off_q + 2048;                          // B operand of the PV chain: [2][16][64] bf16 (4 KB)
     P.off_tail = P.off_p + 4096;                       // two tail buffers
     P.tail_bytes = (uint32_t)(L.stride - L.off_z);
@@ -47,30 +78,31 @@ __host__ __device__ inline Plan plan_of(const CacheLayout& L) {
     return P;
 }
 
-__global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restrict__ cache, CacheLayout L,
+template <int NC>
+__global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(unsigned char* __restrict__ cache, CacheLayout L,
                                                          const __nv_bfloat16* __restrict__ q1,
                                                          const __nv_bfloat16* __restrict__ k1,
                                                          const __nv_bfloat16* __restrict__ v1,
                                                          __nv_bfloat16* __restrict__ o1, float* __restrict__ lse1,
                                                          const float* __restrict__ cw, const float* __restrict__ cbias,
-                                                         int BH, int per_cta, int H, int W, int R, int sink, int K,
+                                                         int BH, int H, int W, int R, int sink, int K,
                                                          float zthr, float scale, int G)
 {
     extern __shared__ __align__(1024) unsigned char dsm[];
-    const Plan P = plan_of(L);
+    constexpr int NW = NC / 32, NTHR = kThreads<NC>, TAPS = (kMaxTaps + NW - 1) / NW;
+    const Plan P = plan_of<NC>(L);
     const uint32_t base = smem_u32(dsm);
     if ((base & 1023u) != 0) { if (threadIdx.x == 0) atomicExch(&g_decode_tc_status.code, 9); return; }
-    const uint32_t sK = base, sV = base + P.off_v, sT = base + P.off_tail, sQ = base + P.off_q, sP = base + P.off_p;
+    const uint32_t sK = base + P.off_k, sV = base + P.off_v, sT = base + P.off_tail, sQ = base + P.off_q, sP = base + P.off_p;
     const uint32_t bar_k = base + P.off_bar, bar_v = bar_k + 8, bar_t0 = bar_k + 16;     // bar_t0, bar_t0 + 8
     const uint32_t bar_q = bar_k + 32, bar_s = bar_k + 40, bar_p = bar_k + 48, bar_o = bar_k + 56, tmem_slot = bar_k + 64;
     volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(dsm + P.off_bar + 64);
-    __shared__ float s_part[8], s_sum[8], s_tap[kMaxTaps], s_o[128];
+    __shared__ float s_part[NW], s_sum[NW], s_tap[2][kMaxTaps], s_o[D];
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int rows = W + R, half = K / 2;
-    const int bh_begin = blockIdx.x * per_cta;
-    const int bh_end = min(bh_begin + per_cta, BH);
-    if (bh_begin >= bh_end) return;
+    const int bh_begin = (int)((long long)blockIdx.x * BH / gridDim.x), bh_end = (int)((long long)(blockIdx.x + 1) * BH / gridDim.x);
+    const uint32_t blk_bytes = rows * 128;                     // only the rows that there are
 
     if (tid == 0) {
         mbar_init(bar_k, 1); mbar_init(bar_v, 1); mbar_init(bar_t0, 1); mbar_init(bar_t0 + 8, 1);
@@ -80,7 +112,12 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
     // the two small B tiles start as zeros (only row 0 of the q tile and rows 0, 1 of the p tile are ever written)
     for (int e = tid; e < (2048 + 4096) / 16; e += NTHR)
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sQ + e * 16), "r"(0u) : "memory");
-    if (wid == 8) tmem_alloc(tmem_slot, TMEM_COLS);
+    // rows that there are not are zeros (their logits are masked, but the values enter the product with weight 0)
+    for (int e = tid + rows * 8; e < NC * 8; e += NTHR) {
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sK + e * 16), "r"(0u) : "memory");
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sV + e * 16), "r"(0u) : "memory");
+    }
+    if (wid == NW) tmem_alloc(tmem_slot, TMEM_COLS);
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -89,7 +126,7 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
     pdl_launch_dependents();
     pdl_wait();                                                // the previous step (or whatever wrote the cache and the inputs) has completed
 
-    if (wid == 8) {
+    if (wid == NW) {
         // ======================================== control lane ==================================================
         if (lane == 0) {
             constexpr uint32_t IDESC_S = instr_desc(128, 16, false);
@@ -97,64 +134,57 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
             const uint32_t k_lo = desc_lo(sK, 16), q_lo = desc_lo(sQ, 16), vmn_lo = desc_lo(sV, 16384), p_lo = desc_lo(sP, 16);
             const unsigned char* g0 = cache + L.header + (size_t)bh_begin * L.stride;
             bulk_load(sT, g0 + L.off_z, P.tail_bytes, bar_t0);
-            bulk_load(sK, g0 + L.off_k, 32768, bar_k);
-            bulk_load(sV, g0 + L.off_v, 32768, bar_v);
+            bulk_load(sK, g0 + L.off_k, blk_bytes, bar_k);
+            bulk_load(sV, g0 + L.off_v, blk_bytes, bar_v);
             for (int bh = bh_begin, it = 0; bh < bh_end; ++bh, ++it) {
                 const unsigned char* gnext = cache + L.header + (size_t)(bh + 1) * L.stride;
                 dwait(bar_k, it & 1, 1);
-                dwait(bar_q, it & 1, 2);                       // q of this head is in the B tile
+                dwait(bar_q, it & 1, 2);                       // q of this head is in the B tile (and the tail of the head before has been used)
+                if (bh + 1 < bh_end) bulk_load(sT + ((it & 1) ^ 1) * P.tail_bytes, gnext + L.off_z, P.tail_bytes, bar_t0 + 8 * ((it & 1) ^ 1));
                 tc_fence_after();
 #pragma unroll
-                for (int g = 0; g < 2; ++g)
+                for (int g = 0; g < NC / 128; ++g)
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
                         umma(tmem + g * 16, desc64(k_lo + g * 1024 + kk * 2, kDescHi), desc64(q_lo + kk * 2, kDescHi), IDESC_S, kk > 0);
                 umma_commit(bar_s);
                 dwait(bar_p, it & 1, 3);                       // p is in its B tile; the key block is no longer read by anyone
-                if (bh + 1 < bh_end) bulk_load(sK, gnext + L.off_k, 32768, bar_k);
+                if (bh + 1 < bh_end) bulk_load(sK, gnext + L.off_k, blk_bytes, bar_k);
                 dwait(bar_v, it & 1, 4);
                 tc_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk)                 // 128 keys per half, 16 per instruction
+                for (int kk = 0; kk < 8; ++kk)                 // 128 keys per half, 16 per instruction (NC = 128: the lower half only)
                     umma(tmem + 32, desc64(vmn_lo + kk * 128, kDescHi), desc64(p_lo + (kk >> 2) * 128 + (kk & 3) * 2, kDescHi),
                          IDESC_O, kk > 0);
                 umma_commit(bar_o);
                 if (bh + 1 < bh_end) {
                     dwait(bar_o, it & 1, 5);                   // the value block has been consumed
-                    bulk_load(sV, gnext + L.off_v, 32768, bar_v);
-                    bulk_load(sT + ((it & 1) ^ 1) * P.tail_bytes, gnext + L.off_z, P.tail_bytes, bar_t0 + 8 * ((it & 1) ^ 1));
+                    bulk_load(sV, gnext + L.off_v, blk_bytes, bar_v);
                 }
             }
         }
     } else {
         // ======================================== compute threads ===============================================
-        constexpr int CPL = D / 32;            // channels per lane in the warp-per-row pieces
+        // Warp-per-row pieces: a lane has channels 2 lane, 2 lane + 1.  The inputs of a head are fetched under the head before.
         const uint32_t lane_base = ((uint32_t)((wid & 3) * 32)) << 16;
-        float k1f[CPL], v1f[CPL], q1f[CPL], wk[2][CPL], wv[2][CPL], bias = 0.f, v1_mine = 0.f;
+        uint32_t k1r, v1r, q1r, wk[TAPS][2], wv[TAPS][2], bias = 0u;   // (converted where they are used: fetching them waits for nothing)
         uint4 kv_new = make_uint4(0, 0, 0, 0), q_chunk = make_uint4(0, 0, 0, 0);
+        uint32_t v1_pair = 0u;
+        auto pair = [&](const __nv_bfloat16* x) { return load32(x + 2 * lane); };
         auto fetch_inputs = [&](int bh) {
             const int h = bh % H;
+            k1r = pair(k1 + (size_t)bh * D); v1r = pair(v1 + (size_t)bh * D); q1r = pair(q1 + (size_t)bh * G * D);
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                k1f[c] = __bfloat162float(k1[(size_t)bh * D + lane + 32 * c]);
-                v1f[c] = __bfloat162float(v1[(size_t)bh * D + lane + 32 * c]);
-                q1f[c] = __bfloat162float(q1[(size_t)bh * G * D + lane + 32 * c]);
+            for (int u = 0; u < TAPS; ++u) {
+                const float* w = cw + ((size_t)h * K + wid + u * NW) * 2 * D + 2 * lane;   // (4-byte aligned)
+                if (wid + u * NW < K) { wk[u][0] = load32(w); wk[u][1] = load32(w + 1); wv[u][0] = load32(w + D); wv[u][1] = load32(w + D + 1); }
             }
-#pragma unroll
-            for (int u2 = 0; u2 < 2; ++u2) {
-                const int t = wid + u2 * 8;
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) {
-                    wk[u2][c] = t < K ? cw[((size_t)h * K + t) * 2 * D + lane + 32 * c] : 0.f;
-                    wv[u2][c] = t < K ? cw[((size_t)h * K + t) * 2 * D + D + lane + 32 * c] : 0.f;
-                }
-            }
-            bias = cbias ? cbias[h] : 0.f;
-            if (tid < D) v1_mine = __bfloat162float(v1[(size_t)bh * D + tid]);
-            if (tid < 8) q_chunk = *reinterpret_cast<const uint4*>(q1 + (size_t)bh * G * D + tid * 8);
+            if (cbias) bias = load32(cbias + h);
+            if (tid < D) v1_pair = load32(v1 + (size_t)bh * D + (tid & ~1));
+            if (tid < 8) q_chunk = load128(q1 + (size_t)bh * G * D + tid * 8);
             if (tid >= 64 && tid < 80) {
                 const int t2 = tid - 64;
-                kv_new = *reinterpret_cast<const uint4*>((t2 < 8 ? k1 : v1) + (size_t)bh * D + (t2 & 7) * 8);
+                kv_new = load128((t2 < 8 ? k1 : v1) + (size_t)bh * D + (t2 & 7) * 8);
             }
         };
         fetch_inputs(bh_begin);
@@ -179,70 +209,54 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
 
             // ---- pool decision, taken redundantly by every warp so that the row masks are known early -----------
             int dst = -1, cnt_new = cnt_old;
-            {
-                const int p = n - W;
-                if (p >= 0 && R > 0) {
-                    const float zp = zc[slot];
-                    const bool is_sink = p < sink;
-                    if (is_sink || zp > zthr) {
-                        if (cnt_old < R) { dst = cnt_old; cnt_new = cnt_old + 1; }
-                        else if (!is_sink) {
-                            // worst entry: lowest logit, the youngest among equals, never a sink entry
-                            float wz = INFINITY; int wpos = -1, wslot = -1;
-                            for (int m = lane; m < cnt_old; m += 32) {
-                                const int pos = pidx[m];
-                                const float zm = zc[W + m];
-                                if (pos >= sink && (zm < wz || (zm == wz && pos > wpos))) { wz = zm; wpos = pos; wslot = m; }
-                            }
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) {
-                                const float oz = __shfl_xor_sync(0xffffffffu, wz, o);
-                                const int op = __shfl_xor_sync(0xffffffffu, wpos, o);
-                                const int os = __shfl_xor_sync(0xffffffffu, wslot, o);
-                                if (os >= 0 && (wslot < 0 || oz < wz || (oz == wz && op > wpos))) { wz = oz; wpos = op; wslot = os; }
-                            }
-                            if (wslot >= 0 && zp > wz) dst = wslot;
-                        }
+            const int p = n - W;
+            const float zp = zc[slot];
+            if (p >= 0 && R > 0 && (p < sink || zp > zthr)) {
+                if (cnt_old < R) { dst = cnt_old; cnt_new = cnt_old + 1; }
+                else if (p >= sink) {
+                    // worst entry: lowest logit, the youngest among equals, never a sink entry
+                    uint32_t key = 0xffffffffu;
+                    int wpos = -1, wslot = -1;
+                    for (int m = lane; m < cnt_old; m += 32) {
+                        const int pos = pidx[m];
+                        const uint32_t k = order_key(zc[W + m] + 0.f);
+                        if (pos >= sink && (k < key || (k == key && pos > wpos))) { key = k; wpos = pos; wslot = m; }
                     }
+                    const uint32_t kmin = __reduce_min_sync(0xffffffffu, key);
+                    const int pmax = __reduce_max_sync(0xffffffffu, key == kmin ? wpos : -1);
+                    const unsigned who = __ballot_sync(0xffffffffu, key == kmin && wpos == pmax);
+                    wslot = __shfl_sync(0xffffffffu, wslot, __ffs(who) - 1);
+                    if (wslot >= 0 && order_key(zp + 0.f) > kmin) dst = wslot;
                 }
             }
             // ---- direct reads of the key / value blocks: scorer taps and the popped row ----------------------
             dwait(bar_k, it & 1, 7);
             dwait(bar_v, it & 1, 8);
+            const float2 k1f = bf16_pair(k1r), q1f = bf16_pair(q1r);
             const int jsc = K > 0 ? n - half : -1;   // K = 0: the scorer runs outside (lte_cache_score)
             if (jsc >= 0) {
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int t = wid + u * 8;
+                for (int u = 0; u < TAPS; ++u) {
+                    const int t = wid + u * NW;
                     if (t >= K) continue;
                     const int pos = jsc + t - half;
-                    float a = 0.f;
-                    if (pos == n) {
-#pragma unroll
-                        for (int c = 0; c < CPL; ++c) a += wk[u][c] * k1f[c] + wv[u][c] * v1f[c];
-                    } else if (pos >= 0) {
-                        const int rr = pos % W;
-#pragma unroll
-                        for (int c = 0; c < CPL; ++c) {
-                            const int ch = lane + 32 * c;          // channel -> swizzled element index within the row
-                            const int el = (((ch >> 3) ^ (rr & 7)) << 3) | (ch & 7);
-                            const float kx = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(dsm)[rr * D + el]);
-                            const float vx = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(dsm + P.off_v)[rr * D + el]);
-                            a += wk[u][c] * kx + wv[u][c] * vx;
-                        }
+                    float2 x = k1f, y = bf16_pair(v1r);
+                    if (pos != n) {                            // row of the ring (W >= K); channel -> swizzled place within the row
+                        const int back = slot - (n - pos), rr = back < 0 ? back + W : back;
+                        const int el = rr * D + ((((lane >> 2) ^ (rr & 7)) << 3) | ((2 * lane) & 7));
+                        x = bf16_pair(*reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(dsm + P.off_k) + el));
+                        y = bf16_pair(*reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(dsm + P.off_v) + el));
                     }
+                    float a = pos < 0 ? 0.f : __uint_as_float(wk[u][0]) * x.x + __uint_as_float(wk[u][1]) * x.y + __uint_as_float(wv[u][0]) * y.x + __uint_as_float(wv[u][1]) * y.y;
                     a = warp_sum(a);
-                    if (lane == 0) s_tap[t] = a;
+                    if (lane == 0) s_tap[tb][t] = a;
                 }
             }
             // the popped row doubles as the new pool entry: logical chunk c of row `slot`, kept in a register
             uint4 mv = make_uint4(0, 0, 0, 0);
             if (tid < 16)
-                mv = reinterpret_cast<const uint4*>(dsm + (tid < 8 ? 0 : P.off_v))[(size_t)slot * 8 + ((tid & 7) ^ (slot & 7))];
-            float s_new = 0.f;                                 // logit of the incoming token (every warp computes it)
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) s_new = fmaf(q1f[c], k1f[c], s_new);
-            s_new = warp_sum(s_new) * scale;
+                mv = reinterpret_cast<const uint4*>(dsm + (tid < 8 ? P.off_k : P.off_v))[(size_t)slot * 8 + ((tid & 7) ^ (slot & 7))];
+            const float s_new = warp_sum(q1f.x * k1f.x + q1f.y * k1f.y) * scale;   // logit of the incoming token (every warp computes it)
 
             // ---- logits from TMEM, masks, softmax --------------------------------------------------------------
             dwait(bar_s, it & 1, 9);
@@ -256,12 +270,12 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
             else if (row < W) ok = (n >= W) ? (row != slot || dst >= 0) : (row < n);
             else ok = (row - W) < cnt_old && (row - W) != dst;
             const float sl = ok ? __uint_as_float(sraw) * scale : -INFINITY;
-            float mx = warp_max(fmaxf(sl, s_new));
+            float mx = redux_max(fmaxf(sl, s_new));
             if (lane == 0) s_part[wid] = mx;
-            csync();
+            csync<NC>();
             mx = s_part[0];
 #pragma unroll
-            for (int w2 = 1; w2 < 8; ++w2) mx = fmaxf(mx, s_part[w2]);
+            for (int w2 = 1; w2 < NW; ++w2) mx = fmaxf(mx, s_part[w2]);
             // p rounded to bf16: the same rounded values enter the product and the normalisation
             const __nv_bfloat16 pb = __float2bfloat16_rn(__expf(sl - mx));
             {
@@ -274,24 +288,33 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
             fence_proxy_async();
             tc_fence_before();
             mbar_arrive(bar_p);
+            // what the rest of this head needs, and the next head's inputs
+            const uint4 kv = kv_new;
+            const float bias_now = __uint_as_float(bias), v_now = __uint_as_float(tid & 1 ? v1_pair & 0xffff0000u : v1_pair << 16);
+            if (bh + 1 < bh_end) fetch_inputs(bh + 1);
 
             // ---- output ----------------------------------------------------------------------------------------
             dwait(bar_o, it & 1, 10);
             tc_fence_after();
-            if (tid < 128) {
-                uint32_t oraw;
-                tmem_ld1(tmem + lane_base + 32 + (tid >> 6), oraw);   // lanes 0..63: column 0, lanes 64..127: column 1
-                tmem_wait_ld();
-                s_o[tid] = __uint_as_float(oraw);
-            }
-            tc_fence_before();
-            csync();
             const float p_new = __expf(s_new - mx);
             float sum = p_new;
 #pragma unroll
-            for (int w2 = 0; w2 < 8; ++w2) sum += s_sum[w2];
+            for (int w2 = 0; w2 < NW; ++w2) sum += s_sum[w2];
+            float o_mine = 0.f;
+            if (tid < NC / 2) {                                // lanes 0..63: column 0, and for rows 128..255 lanes 64..127: column 1
+                uint32_t oraw;
+                tmem_ld1(tmem + lane_base + 32 + (tid >> 6), oraw);
+                tmem_wait_ld();
+                o_mine = __uint_as_float(oraw);
+                if (NC == 256) {
+                    if (tid >= D) s_o[tid - D] = o_mine;
+                    asm volatile("bar.sync 2, 128;" ::: "memory");
+                    if (tid < D) o_mine += s_o[tid];
+                }
+            }
+            tc_fence_before();
             if (tid < D) {
-                const float o = s_o[tid] + s_o[64 + tid] + p_new * v1_mine;
+                const float o = o_mine + p_new * v_now;
                 o1[(size_t)bh * G * D + tid] = __float2bfloat16_rn(o / sum);
             }
             if (tid == 0) lse1[(size_t)bh * G] = mx + logf(sum);
@@ -308,27 +331,27 @@ __global__ void __launch_bounds__(NTHR) decode_tc_kernel(unsigned char* __restri
             }
             if (tid >= 64 && tid < 80) {
                 const int t2 = tid - 64;
-                (t2 < 8 ? Kw : Vw)[(size_t)slot * 8 + ((t2 & 7) ^ (slot & 7))] = kv_new;
+                (t2 < 8 ? Kw : Vw)[(size_t)slot * 8 + ((t2 & 7) ^ (slot & 7))] = kv;
             }
-            if (tid == 128) {
-                if (dst >= 0) { zw[W + dst] = zc[slot]; pw[dst] = n - W; }
+            if (tid == NC / 2 + 32) {                          // (a warp with nothing else to write)
+                if (dst >= 0) { zw[W + dst] = zp; pw[dst] = p; }
                 float znew = -INFINITY;
                 if (jsc >= 0) {
-                    znew = bias;
-                    for (int t = 0; t < K; ++t) znew += s_tap[t];
+                    znew = bias_now;
+                    for (int t = 0; t < K; ++t) znew += s_tap[tb][t];
                 }
                 zw[slot] = -INFINITY;
                 if (jsc >= 0) zw[jsc % W] = znew;
                 mw[0] = n + 1;
                 mw[1] = cnt_new;
             }
-            csync();                                           // shared scratch is reused by the next head
-            if (bh + 1 < bh_end) fetch_inputs(bh + 1);
+            // (shared scratch: s_part, s_sum, s_o are written again only after a barrier of the next head that every reader of this
+            // one has reached; the taps alternate between two sets)
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (wid == 8) tmem_dealloc(tmem, TMEM_COLS);
+    if (wid == NW) tmem_dealloc(tmem, TMEM_COLS);
 }
 
 }  // namespace
@@ -338,19 +361,23 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
     if (!L.swz || p.K > 16) return LTE_ERR_UNSUPPORTED;
-    const Plan P = plan_of(L);
-    static PerDeviceOnce attr;
-    if (int e = attr.run([] { return cudaFuncSetAttribute(decode_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024); })) return e;
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
-    if (P.total > 80 * 1024) return LTE_ERR_UNSUPPORTED;
     const int BH = p.B * p.H;
-    const int slots = 3 * n_sm;                                // three CTAs per SM
-    const int per_cta = (BH + slots - 1) / slots;
-    const int n_cta = (BH + per_cta - 1) / per_cta;
-    return cuda_status(launch_pdl(decode_tc_kernel, dim3(n_cta), dim3(NTHR), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
-                                                   (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1,
-                                                   p.w, p.bias, BH, per_cta, p.H, p.W, p.R, p.sink, p.K, p.zthr, p.scale, p.G));
+    auto go = [&](auto nc, auto kern, PerDeviceOnce& attr) {
+        constexpr int NC = decltype(nc)::value;
+        const Plan P = plan_of<NC>(L);
+        constexpr int most = 227 * 1024 / kPerSm<NC> - 2048;
+        if (int e = attr.run([=] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most); })) return e;
+        if (P.total > (uint32_t)most) return (int)LTE_ERR_UNSUPPORTED;
+        const int n_cta = BH < kPerSm<NC> * n_sm ? BH : kPerSm<NC> * n_sm;   // each takes an equal share of the heads (+- 1)
+        return cuda_status(launch_pdl(kern, dim3(n_cta), dim3(kThreads<NC>), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
+                                      (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, BH, p.H, p.W, p.R,
+                                      p.sink, p.K, p.zthr, p.scale, p.G));
+    };
+    static PerDeviceOnce attr256, attr128;
+    if (p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256>, attr256);
+    return go(std::integral_constant<int, 128>{}, decode_tc_kernel<128>, attr128);
 }
 
 int decode_tc_status_fetch_and_clear() { return status_fetch_and_clear(g_decode_tc_status); }
