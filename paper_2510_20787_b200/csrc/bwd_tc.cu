@@ -37,6 +37,8 @@ namespace {
 using namespace tc;
 __device__ __forceinline__ void bwait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_bwd_status); }
 
+__device__ __forceinline__ void bwait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni(bar, parity, code, &g_bwd_status); }
+
 constexpr int BM = 128, NRW = 16;                              // rows per item, row warps
 constexpr int W_LOAD = NRW, W_XY = NRW + 1, W_ACC = NRW + 2, NTHREADS = (NRW + 4) * 32;   // the last warp prepares constants
 constexpr float kLog2e = 1.4426950408889634f;
@@ -317,17 +319,17 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
         const uint32_t a_lo = desc_lo(sA, 16), b_lo = desc_lo(sB, 16);
         uint32_t g = 0, par_a = 0;                             // parities of bar_a (bits 0 .. 3), bar_ga (4 .. 7)
         Item it;
-        for (int n = 0; enter(n, it); ++n) {
+        for (int n = 0; uni(enter(n, it)); ++n) {
             const uint32_t ab = n % AST, at = (it.list ? 4 : 0) + ab;
-            bwait((it.list ? bar_ga : bar_a) + 8 * ab, (par_a >> at) & 1u, 1);
+            bwait_u((it.list ? bar_ga : bar_a) + 8 * ab, (par_a >> at) & 1u, 1);
             par_a ^= 1u << at;
-            if (it.list) fence_proxy_async();                  // (gathered rows are generic-proxy writes)
-            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+            if (uni(it.list)) fence_proxy_async();                  // (gathered rows are generic-proxy writes)
+            for (int t = 0; uni(t < it.n_tiles); ++t, ++g) {
                 const uint32_t s = g % BST;
-                bwait(bar_b + 8 * s, (g / BST) & 1u, 2);
-                if (g > 0) bwait(bar_xf, (g - 1) & 1, 3);      // the previous tile's X, Y are in registers
+                bwait_u(bar_b + 8 * s, (g / BST) & 1u, 2);
+                if (uni(g > 0)) bwait_u(bar_xf, (g - 1) & 1, 3);      // the previous tile's X, Y are in registers
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), b1 = b_lo + s * (2 * BTILE >> 4);
 #pragma unroll
                     for (int xy = 0; xy < 2; ++xy)
@@ -347,13 +349,13 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
         const uint32_t b_lo = desc_lo(sB, BN * 128);
         uint32_t g = 0;
         Item it;
-        for (int n = 0; enter(n, it); ++n) {
-            for (int t = 0; t < it.n_tiles; ++t, ++g) {
+        for (int n = 0; uni(enter(n, it)); ++n) {
+            for (int t = 0; uni(t < it.n_tiles); ++t, ++g) {
                 const uint32_t s = g % BST;
-                if (t == 0 && n > 0) bwait(bar_of, (n - 1) & 1, 13);   // the previous item's accumulators have been read out
-                bwait(bar_p, g & 1, 7);
+                if (uni(t == 0 && n > 0)) bwait_u(bar_of, (n - 1) & 1, 13);   // the previous item's accumulators have been read out
+                bwait_u(bar_p, g & 1, 7);
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t b1 = b_lo + s * (2 * BTILE >> 4);
                     if (DKV) {
 #pragma unroll

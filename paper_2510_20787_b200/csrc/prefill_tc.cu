@@ -40,6 +40,7 @@ namespace {
 constexpr int BM = 128, BN = 128, D = 64, NTHREADS = 320;         // warps 0-7 softmax, 8 products, 9 loads
 using namespace tc;
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_prefill_status); }
+__device__ __forceinline__ void mbar_wait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni(bar, parity, code, &g_prefill_status); }
 
 template <bool STREAM> struct Smem {
     static constexpr int TILE = 128 * D * 2;                  // [128][64] bf16: Q, K and V tiles alike
@@ -290,9 +291,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         Cursor cs, cp;
         uint32_t par = 0;                                      // GATHER: parities of bar_k (bits 0, 1), bar_gk (2, 3), bar_v (4, 5), bar_gv (6, 7)
         auto landed = [&](uint32_t bar, uint32_t gbar, bool win, uint32_t s, uint32_t phase, int bit, int gbit, int code) {
-            if (!GATHER) { mbar_wait(bar + 8 * s, phase, code); return; }
+            if (!GATHER) { mbar_wait_u(bar + 8 * s, phase, code); return; }
             const int at = (win ? bit : gbit) + (int)s;
-            mbar_wait((win ? bar : gbar) + 8 * s, (par >> at) & 1u, code);
+            mbar_wait_u((win ? bar : gbar) + 8 * s, (par >> at) & 1u, code);
             par ^= 1u << at;
             if (!win) fence_proxy_async();                     // the copies were generic-proxy writes
         };
@@ -305,16 +306,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         };
         auto mma_s = [&]() {
             const uint32_t s = cs.g % KST, b = cs.n & 1;
-            if (cs.t == 0) {
-                mbar_wait(bar_i + 8 * (cs.n & 3), (cs.n >> 2) & 1, 9);
+            if (uni(cs.t == 0)) {
+                mbar_wait_u(bar_i + 8 * (cs.n & 3), (cs.n >> 2) & 1, 9);
                 enter(cs);
-                if (!cs.live) return;
-                mbar_wait(bar_q + 8 * b, (cs.n >> 1) & 1, 1);
+                if (uni(!cs.live)) return;
+                mbar_wait_u(bar_q + 8 * b, (cs.n >> 1) & 1, 1);
             }
             landed(bar_k, bar_gk, cs.t < cs.it.n_win, s, (cs.g / KST) & 1u, 0, 2, 2);
-            if (cs.g > 0) mbar_wait(bar_sf, (cs.g - 1) & 1, 3);    // the previous tile's S is in registers
+            if (uni(cs.g > 0)) mbar_wait_u(bar_sf, (cs.g - 1) & 1, 3);    // the previous tile's S is in registers
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t qd = q_lo + b * (TILE >> 4), kd = k_lo + s * (TILE >> 4);
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) umma(tmem + S_COL, desc64(qd + kk * 2, kDescHi), desc64(kd + kk * 2, kDescHi), IDESC_S, kk > 0);
@@ -327,14 +328,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         };
         mma_s();
         for (;;) {
-            if (cs.live) mma_s();
-            if (cp.t == 0) { enter(cp); if (!cp.live) break; }
+            if (uni(cs.live)) mma_s();
+            if (uni(cp.t == 0)) { enter(cp); if (uni(!cp.live)) break; }
             const uint32_t s = cp.g % VST;
             landed(bar_v, bar_gv, cp.t < cp.it.n_win, s, (cp.g / VST) & 1u, 4, 6, 4);
-            if (cp.t == 0 && cp.n > 0) mbar_wait(bar_of, (cp.n - 1) & 1, 13);   // the previous item's O has been read out
-            mbar_wait(bar_p, cp.g & 1, 7);
+            if (uni(cp.t == 0 && cp.n > 0)) mbar_wait_u(bar_of, (cp.n - 1) & 1, 13);   // the previous item's O has been read out
+            mbar_wait_u(bar_p, cp.g & 1, 7);
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t vd = v_lo + s * (TILE >> 4);
 #pragma unroll
                 for (int kk = 0; kk < BN / 16; ++kk)
