@@ -113,6 +113,10 @@ int launch_prefill_tc_long(const Params& p, const void* q, const void* k, const 
 size_t prefill_compact_bytes(const Params& p);
 int launch_prefill_compact(const Params& p, const void* k, const void* v, const int32_t* idx, const int32_t* cnt, void* kc, void* vc,
                            cudaStream_t st);
+// d = 128, two query tiles sharing their key tiles; `half`: bytes of the compacted keys (and of the values) in ws.
+int launch_prefill_tc_pair(const Params& p, const void* q, const void* k, const void* v, const int32_t* idx, const int32_t* cnt, void* o,
+                           float* lse, void* ws, size_t half, cudaStream_t st);
+int prefill_pair_status_fetch_and_clear();
 int prefill_long_status_fetch_and_clear();
 int launch_cache_init(const Params& p, const void* k, const void* v, const float* z, const int32_t* idx,
                       const int32_t* cnt, void* cache, cudaStream_t st);

@@ -612,8 +612,8 @@ int launch_prefill_tc(const Params& p, const void* q, const void* k, const void*
 
 int prefill_status_fetch_and_clear()
 {
-    const int h = status_fetch_and_clear(g_prefill_status), h2 = prefill_long_status_fetch_and_clear();
-    return h != 0 ? h : h2;
+    const int h = status_fetch_and_clear(g_prefill_status), h2 = prefill_long_status_fetch_and_clear(), h3 = prefill_pair_status_fetch_and_clear();
+    return h != 0 ? h : h2 != 0 ? h2 : h3;
 }
 
 }  // namespace lte
