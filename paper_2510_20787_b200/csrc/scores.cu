@@ -51,6 +51,8 @@ __global__ void __launch_bounds__(NT) scores_kernel(const T* __restrict__ k, con
     const int h = bh % H;
     const int j0 = blockIdx.x * TJ;
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();                             // see launch_pdl: earlier kernels of the stream have completed
     for (int i = tid; i < K * 2 * D; i += NT) ws[i] = w[(size_t)h * K * 2 * D + i];
     __syncthreads();
 
@@ -363,8 +365,7 @@ int run(const Params& p, const void* k, const void* v, float* z, float* r, cudaS
 {
     constexpr int TJ = NT - (K - 1);
     dim3 grid((p.T + TJ - 1) / TJ, p.B * p.H);
-    scores_kernel<T, D, K><<<grid, NT, 0, st>>>((const T*)k, (const T*)v, p.w, p.bias, z, r, p.H, p.T);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(scores_kernel<T, D, K>, grid, dim3(NT), 0, st, (const T*)k, (const T*)v, p.w, p.bias, z, r, p.H, p.T));
 }
 
 template <typename T, int D, int K>
