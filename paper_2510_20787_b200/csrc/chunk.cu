@@ -19,7 +19,8 @@ __device__ StatusWord g_chunk_status = LTE_STATUS_INIT;   // report only; 31: th
 
 namespace {
 
-// one 16-byte piece of a cache row -> the same piece of a plain row (the swizzled layout permutes the pieces of a row)
+// one 16-byte piece of a cache row -> the same piece of a plain row (the swizzled layout permutes the pieces of a row); a row has
+// 1 << piece_shift pieces, and a block's threads walk them in order, four in flight each
 __device__ __forceinline__ int piece_src(const CacheLayout& L, int row, int c) { return L.swz ? (c ^ (row & 7)) : c; }
 
 constexpr int kRowsPerBlock = 128;
@@ -34,6 +35,8 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
                                     unsigned char* __restrict__ vlin, float* __restrict__ zsrc, int32_t* __restrict__ oldpos,
                                     int32_t* __restrict__ gate, int D, int W, int R, int n0, int R0, int Wn, int Tloc)
 {
+    pdl_launch_dependents();
+    pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
     const int bh = blockIdx.y;
     const unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
     const uint4* Kc = reinterpret_cast<const uint4*>(blk + L.off_k);
@@ -47,15 +50,18 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) gate[bh] = 1;
     const int cnt = meta[1];
-    const int pieces = D * (int)L.esz / 16;                    // 16-byte pieces per row
+    const int pb = piece_shift(L, D), pieces = 1 << pb;         // 16-byte pieces per row
     uint4* kd = reinterpret_cast<uint4*>(klin) + (size_t)bh * Tloc * pieces;
     uint4* vd = reinterpret_cast<uint4*>(vlin) + (size_t)bh * Tloc * pieces;
     const int rows = R0 + Wn, Tc = Tloc - rows;
     const uint4* kq = reinterpret_cast<const uint4*>(kc) + (size_t)bh * Tc * pieces;
     const uint4* vq = reinterpret_cast<const uint4*>(vc) + (size_t)bh * Tc * pieces;
     const int r_lo = blockIdx.x * kRowsPerBlock, r_hi = min(r_lo + kRowsPerBlock, Tloc);
-    for (int e = r_lo * pieces + threadIdx.x; e < r_hi * pieces; e += blockDim.x) {
-        const int r = e / pieces, c = e % pieces;
+    const int ring0 = Wn > 0 ? (n0 - Wn) % W : 0;              // slot of the ring's oldest token
+    auto slot_of = [&](int r) { const int s = ring0 + (r - R0); return s >= W ? s - W : s; };
+#pragma unroll 4
+    for (int e = (r_lo << pb) + threadIdx.x; e < (r_hi << pb); e += 256) {
+        const int r = e >> pb, c = e & (pieces - 1);
         uint4 kx = make_uint4(0, 0, 0, 0), vx = kx;
         if (r >= rows) {
             kx = kq[(size_t)(r - rows) * pieces + c];
@@ -63,7 +69,7 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
         } else {
             int src = -1;
             if (r < R0) { if (r < cnt) src = W + r; }
-            else src = (n0 - Wn + (r - R0)) % W;
+            else src = slot_of(r);
             if (src >= 0) {
                 const int cs = piece_src(L, src, c);
                 kx = Kc[(size_t)src * pieces + cs];
@@ -77,7 +83,7 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
     for (int r = threadIdx.x; r < rows; r += blockDim.x) {
         float zz = -INFINITY;
         if (r < R0) { if (r < cnt) zz = zc[W + r]; }
-        else zz = zc[(n0 - Wn + (r - R0)) % W];
+        else zz = zc[slot_of(r)];
         zsrc[(size_t)bh * (R + W) + r] = zz;
     }
     for (int r = threadIdx.x; r < R; r += blockDim.x) oldpos[(size_t)bh * R + r] = r < cnt ? pidx[r] : -1;
@@ -90,6 +96,8 @@ __global__ void chunk_merge_z_kernel(float* __restrict__ z, float* __restrict__ 
                                      const int32_t* __restrict__ oldpos, int R, int W, int n0, int R0, int Wn, int Tloc,
                                      int half, int sink)
 {
+    pdl_launch_dependents();
+    pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
     const int bh = blockIdx.y;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= Tloc) return;
@@ -114,7 +122,7 @@ __global__ void chunk_merge_z_kernel(float* __restrict__ z, float* __restrict__ 
     zrank[(size_t)bh * Tloc + r] = (pos >= 0 && pos < sink) ? INFINITY : zt;
 }
 
-// Block (part, (b,h)): the cache after the chunk, 128 of its key/value rows per part; part 0 also writes the logits, the
+// Block (part, (b,h)): the cache after the chunk, 128 of its key/value rows per part (those that change); part 0 also writes the logits, the
 // positions and the counters.  Ring <- the last min(n1, W) rows of the local sequence, pool <- the rows the
 // selection kept, with their logits and positions.  Reads only the scratch copies, so the old block can be overwritten.
 __global__ void chunk_commit_kernel(unsigned char* __restrict__ cache, CacheLayout L, const unsigned char* __restrict__ klin,
@@ -123,6 +131,8 @@ __global__ void chunk_commit_kernel(unsigned char* __restrict__ cache, CacheLayo
                                     const int32_t* __restrict__ oldpos, const int32_t* __restrict__ gate, int D, int W, int R,
                                     int n0, int n1, int R0, int Wn, int Tloc, int half)
 {
+    pdl_launch_dependents();
+    pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
     const int bh = blockIdx.y;
     if (gate[bh] == 0) return;                                 // this call's gather found another state: leave the cache alone
     unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
@@ -131,18 +141,22 @@ __global__ void chunk_commit_kernel(unsigned char* __restrict__ cache, CacheLayo
     float* zc = reinterpret_cast<float*>(blk + L.off_z);
     int32_t* pidx = reinterpret_cast<int32_t*>(blk + L.off_pidx);
     int32_t* meta = reinterpret_cast<int32_t*>(blk + L.off_meta);
-    const int pieces = D * (int)L.esz / 16;
+    const int pb = piece_shift(L, D), pieces = 1 << pb;
     const uint4* ks = reinterpret_cast<const uint4*>(klin) + (size_t)bh * Tloc * pieces;
     const uint4* vs = reinterpret_cast<const uint4*>(vlin) + (size_t)bh * Tloc * pieces;
     const float* zl = z + (size_t)bh * Tloc;
     const int Wnew = n1 < W ? n1 : W;
     const int cnt = R > 0 ? cntp[bh] : 0;
     const int a_lo = blockIdx.x * kRowsPerBlock, a_hi = min(a_lo + kRowsPerBlock, Wnew + cnt);
-    for (int e = a_lo * pieces + threadIdx.x; e < a_hi * pieces; e += blockDim.x) {
-        const int a = e / pieces, c = e % pieces;
+    const int ring0 = (n1 - Wnew) % W;                         // slot of the ring's oldest token
+#pragma unroll 4
+    for (int e = (a_lo << pb) + threadIdx.x; e < (a_hi << pb); e += 256) {
+        const int a = e >> pb, c = e & (pieces - 1);
         int r, row;
-        if (a < Wnew) { r = Tloc - Wnew + a; row = (n1 - Wnew + a) % W; }
+        if (a < Wnew) { r = Tloc - Wnew + a; row = ring0 + a; if (row >= W) row -= W; }
         else { r = idx[(size_t)bh * R + (a - Wnew)]; row = W + (a - Wnew); }
+        // a token that stays in the ring stays in its slot, an entry that keeps its pool slot is there: nothing to write
+        if (a < Wnew ? r < R0 + Wn : r < R0 && r == a - Wnew) continue;
         const int cd = piece_src(L, row, c);
         Kc[(size_t)row * pieces + cd] = ks[(size_t)r * pieces + c];
         Vc[(size_t)row * pieces + cd] = vs[(size_t)r * pieces + c];
@@ -278,17 +292,15 @@ int launch_chunk_gather(const Params& p, const void* cache, const void* k, const
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
     dim3 grid((p.T + kRowsPerBlock - 1) / kRowsPerBlock, p.B * p.H);
-    chunk_gather_kernel<<<grid, 256, 0, st>>>((const unsigned char*)cache, L, (const unsigned char*)k, (const unsigned char*)v,
-                                              (unsigned char*)klin, (unsigned char*)vlin, zsrc, oldpos, gate, p.d, p.W, p.R, n0, R0, Wn, p.T);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(chunk_gather_kernel, grid, dim3(256), 0, st, (const unsigned char*)cache, L, (const unsigned char*)k, (const unsigned char*)v,
+                                              (unsigned char*)klin, (unsigned char*)vlin, zsrc, oldpos, gate, p.d, p.W, p.R, n0, R0, Wn, p.T));
 }
 
 int launch_chunk_merge_z(const Params& p, float* z, float* zrank, const float* zsrc, const int32_t* oldpos, int n0, int R0, int Wn,
                          cudaStream_t st)
 {
     dim3 grid((p.T + 255) / 256, p.B * p.H);
-    chunk_merge_z_kernel<<<grid, 256, 0, st>>>(z, zrank, zsrc, oldpos, p.R, p.W, n0, R0, Wn, p.T, p.half, p.sink);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(chunk_merge_z_kernel, grid, dim3(256), 0, st, z, zrank, zsrc, oldpos, p.R, p.W, n0, R0, Wn, p.T, p.half, p.sink));
 }
 
 int launch_chunk_commit(const Params& p, void* cache, const void* klin, const void* vlin, const float* z, const int32_t* idx,
@@ -297,9 +309,8 @@ int launch_chunk_commit(const Params& p, void* cache, const void* klin, const vo
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
     dim3 grid((p.W + p.R + kRowsPerBlock - 1) / kRowsPerBlock, p.B * p.H);
-    chunk_commit_kernel<<<grid, 256, 0, st>>>((unsigned char*)cache, L, (const unsigned char*)klin, (const unsigned char*)vlin, z,
-                                                   idx, cnt, oldpos, gate, p.d, p.W, p.R, n0, n1, R0, Wn, p.T, p.half);
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(chunk_commit_kernel, grid, dim3(256), 0, st, (unsigned char*)cache, L, (const unsigned char*)klin, (const unsigned char*)vlin, z,
+                                                   idx, cnt, oldpos, gate, p.d, p.W, p.R, n0, n1, R0, Wn, p.T, p.half));
 }
 
 }  // namespace lte

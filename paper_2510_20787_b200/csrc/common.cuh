@@ -84,7 +84,7 @@ __host__ __device__ inline CacheLayout cache_layout(int d, int W, int R, int dty
 __host__ __device__ inline int cache_chunk_pos(const CacheLayout& L, int row, int c) { return L.swz ? (c ^ (row & 7)) : c; }
 
 // log2 of the 16-byte pieces of a key or value row
-inline int piece_shift(const CacheLayout& L, int d) { int n = 0; while ((16u << n) < (unsigned)d * L.esz) ++n; return n; }
+__host__ __device__ inline int piece_shift(const CacheLayout& L, int d) { int n = 0; while ((16u << n) < (unsigned)d * L.esz) ++n; return n; }
 
 // kernel launchers (one translation unit each)
 int launch_scores(const Params& p, const void* k, const void* v, float* z, float* r, cudaStream_t st);
