@@ -14,6 +14,8 @@
 
 namespace lte {
 
+__device__ StatusWord g_tail_status = LTE_STATUS_INIT;   // 0 = fine; otherwise the code of the wait that gave up
+
 int launch_bwd_dq_tc(const Params& p, const void* q, const void* k, const void* v, const void* o, const float* lse,
                      const void* dO, const int32_t* idx, const int32_t* cnt, void* dq, float* delta, void* ret_ws, cudaStream_t st);
 
@@ -319,8 +321,18 @@ __global__ void __launch_bounds__(256) bwd_finish_inplace_kernel(const float* __
 // and (FINISH) the scorer's input gradient sum_t dz[p - t + half] w[h,t,c] added onto the bf16 dk, dv rows in place.
 // The partials of the threads that own the same channels are added in a fixed order (a tree over the row slots
 // through shared memory).
+// The rows come by bulk copies into a ring of four stages of 4 KB of each tensor, three of which are under way while a thread works on
+// its four consecutive rows of one (whose taps overlap), and the first are asked for before the logit gradients are formed.
+// 8 x 16 heads x 2,048, d = 64 (201 MB, 31 us at the copy rate): 54 us, with each thread loading eight rows at a time into registers 64;
+// 16 x 8,192, d = 128: 50 and 53.  The rest is the grid (256 blocks on 148 SMs) and about 70 instructions per thread and row.
 __device__ __forceinline__ bool isv_of(int cg, int D) { return cg >= D / 4; }
+constexpr int TAIL_STAGES = 4, TAIL_PART = 4096, TAIL_U = 4;   // stages; bytes of a tensor in one; rows of a thread in one
+constexpr int TAIL_RING = TAIL_STAGES * 4 * TAIL_PART, TAIL_BARS = 128;
 constexpr int TAIL_MIN_ROWS = 256, TAIL_MAX_ROWS = 1024;   // rows per block are chosen per launch to fill whole waves
+__device__ __forceinline__ void bulk_rows(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 template <int D, int K, bool FINISH>
 __global__ void __launch_bounds__(256, 2)
 bwd_tail_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, const float* __restrict__ dr_win,
@@ -336,15 +348,37 @@ bwd_tail_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __rest
     constexpr int RPP = 256 / TPR;                  // positions per pass (row slots)
     constexpr int half = K / 2;
     const int NDZ = (rows + K - 1 + 3) & ~3;
-    extern __shared__ float sm[];
-    float* dzs = sm;                                // dz[p0-half .. p0+rows-1+half]
+    extern __shared__ __align__(128) unsigned char tail_smem[];   // ring, barriers, dz, list entries
+    float* dzs = reinterpret_cast<float*>(tail_smem + TAIL_RING + TAIL_BARS);                                // dz[p0-half .. p0+rows-1+half]
     int* ent = reinterpret_cast<int*>(dzs + NDZ);   // list entry of the same positions, or -1
-    float* red = dzs + 2 * NDZ;                     // [RPP/2][K][2D]
+    float* red = reinterpret_cast<float*>(tail_smem);   // [RPP/2][K][2D], once the ring has been read
+    constexpr int SR = RPP * TAIL_U;                // rows of a stage
+    static_assert(SR * D * 2 == TAIL_PART && (RPP / 2) * K * 2 * D * 4 <= TAIL_RING, "");
     const int h = blockIdx.y;
     const int b = blockIdx.x / nchunk, ch = blockIdx.x % nchunk;
     const int bh = b * H + h;
     const int p0 = ch * rows;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // the ring: stage s holds rows [s SR, s SR + SR) of k, v, dk, dv (FINISH; otherwise k, v)
+    const uint32_t ring = tc::smem_u32(tail_smem), bar_f = ring + TAIL_RING, bar_e = bar_f + 8 * TAIL_STAGES;
+    const int n_own = min(rows, Tlen - p0), n_st = (n_own + SR - 1) / SR;
+    auto fill = [&](int s) {                        // (one thread)
+        const int at = s % TAIL_STAGES, nr = min(SR, n_own - s * SR);
+        const size_t off = ((size_t)bh * Tlen + p0 + s * SR) * D;
+        const uint32_t bytes = (uint32_t)nr * D * 2, dst = ring + at * 4 * TAIL_PART, bar = bar_f + 8 * at;
+        tc::mbar_expect_tx(bar, (FINISH ? 4 : 2) * bytes);
+        bulk_rows(dst, k + off, bytes, bar);
+        bulk_rows(dst + TAIL_PART, v + off, bytes, bar);
+        if (FINISH) {
+            bulk_rows(dst + 2 * TAIL_PART, dk + off, bytes, bar);
+            bulk_rows(dst + 3 * TAIL_PART, dv + off, bytes, bar);
+        }
+    };
+    if (tid == 0) {
+        for (int s = 0; s < TAIL_STAGES; ++s) { tc::mbar_init(bar_f + 8 * s, 1); tc::mbar_init(bar_e + 8 * s, 8); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int s = 0; s < TAIL_STAGES && s < n_st; ++s) fill(s);
+    }
     for (int a = tid; a < rows + K - 1; a += 256) ent[a] = -1;
     __syncthreads();
     {
@@ -390,37 +424,52 @@ bwd_tail_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __rest
     uint64_t acc2[K][2];
 #pragma unroll
     for (int t = 0; t < K; ++t) acc2[t][0] = acc2[t][1] = pack2(0.f, 0.f);
-    // U rows per batch: all of a batch's loads are issued before any of its arithmetic (row indices are clamped so
-    // that every load is legal; rows past the end are skipped afterwards)
-    constexpr int U = 8;
-    for (int rb = r0; rb < rows; rb += RPP * U) {
-        uint2 ux[U], ug[U];
+    for (int st = 0; st < n_st; ++st) {
+        const int at = st % TAIL_STAGES, rb = st * SR + r0 * TAIL_U;   // four consecutive rows: their taps overlap
+        tc::mbar_wait_s(bar_f + 8 * at, (st / TAIL_STAGES) & 1, 1, &g_tail_status);
+        // this thread's four channels of its rows of the stage
+        const unsigned char* xs = tail_smem + at * 4 * TAIL_PART + (isv ? TAIL_PART : 0) + (r0 * TAIL_U * D + cc) * 2;
+        uint2 ux[TAIL_U], ug[TAIL_U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int p = min(p0 + rb + u * RPP, Tlen - 1);
-            const size_t a0 = ((size_t)bh * Tlen + p) * D + cc;
-            ux[u] = *reinterpret_cast<const uint2*>(src + a0);
-            ug[u] = make_uint2(0u, 0u);
-            if (FINISH || ent[min(rb + u * RPP, rows - 1) + half] >= 0) ug[u] = *reinterpret_cast<const uint2*>(gdst + a0);
+        for (int u = 0; u < TAIL_U; ++u) {
+            ux[u] = *reinterpret_cast<const uint2*>(xs + u * D * 2);
+            ug[u] = FINISH ? *reinterpret_cast<const uint2*>(xs + 2 * TAIL_PART + u * D * 2) : make_uint2(0u, 0u);
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(bar_e + 8 * at);
+        if (tid == 0 && st >= 1 && st - 1 + TAIL_STAGES < n_st) {   // the stage before is refilled once every warp has read it
+            tc::mbar_wait_s(bar_e + 8 * ((st - 1) % TAIL_STAGES), ((st - 1) / TAIL_STAGES) & 1, 2, &g_tail_status);
+            fill(st - 1 + TAIL_STAGES);
+        }
+        if (rb >= n_own) continue;
+        uint64_t gw[K + TAIL_U - 1];                // dz around the four rows, from row rb - half on, as pairs
+#pragma unroll
+        for (int e = 0; e < (K + TAIL_U - 1 + 3) / 4; ++e) {
+            const float4 d4 = *reinterpret_cast<const float4*>(dzs + rb + 4 * e);
+            const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (4 * e + x < K + TAIL_U - 1) gw[4 * e + x] = pack2(d[x], d[x]);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int rl = rb + u * RPP, p = p0 + rl;
-            if (rl >= rows || p >= Tlen) continue;
-            uint64_t g2[K];
+        for (int u = 0; u < TAIL_U; ++u) {
+            const int rl = rb + u, p = p0 + rl;
+            if (rl >= n_own) continue;
             const uint64_t x01 = pack2(__uint_as_float(ux[u].x << 16), __uint_as_float(ux[u].x & 0xffff0000u));
             const uint64_t x23 = pack2(__uint_as_float(ux[u].y << 16), __uint_as_float(ux[u].y & 0xffff0000u));
 #pragma unroll
-            for (int t = 0; t < K; ++t) { const float g = dzs[rl - t + 2 * half]; g2[t] = pack2(g, g); }   // dz[p - t + half]
-#pragma unroll
-            for (int t = 0; t < K; ++t) { acc2[t][0] = fma2(g2[t], x01, acc2[t][0]); acc2[t][1] = fma2(g2[t], x23, acc2[t][1]); }
+            for (int t = 0; t < K; ++t) {           // dz[p - t + half]
+                acc2[t][0] = fma2(gw[u - t + 2 * half], x01, acc2[t][0]);
+                acc2[t][1] = fma2(gw[u - t + 2 * half], x23, acc2[t][1]);
+            }
             const int er = ent[rl + half];                   // retained: its far-query share is added here
             if (FINISH || er >= 0) {
+                if (!FINISH) ug[u] = *reinterpret_cast<const uint2*>(gdst + ((size_t)bh * Tlen + p) * D + cc);
                 float gi[4] = {0.f, 0.f, 0.f, 0.f};
                 if (FINISH) {
                     uint64_t gi01 = pack2(0.f, 0.f), gi23 = gi01;
 #pragma unroll
-                    for (int t = 0; t < K; ++t) { gi01 = fma2(g2[t], wr2[t][0], gi01); gi23 = fma2(g2[t], wr2[t][1], gi23); }
+                    for (int t = 0; t < K; ++t) { gi01 = fma2(gw[u - t + 2 * half], wr2[t][0], gi01); gi23 = fma2(gw[u - t + 2 * half], wr2[t][1], gi23); }
                     unpack2(gi01, gi[0], gi[1]); unpack2(gi23, gi[2], gi[3]);
                 }
                 if (er >= 0) {
@@ -437,6 +486,7 @@ bwd_tail_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __rest
     float acc[K][4];
 #pragma unroll
     for (int t = 0; t < K; ++t) { unpack2(acc2[t][0], acc[t][0], acc[t][1]); unpack2(acc2[t][1], acc[t][2], acc[t][3]); }
+    __syncthreads();                                // the ring has been read
     // ---- add the partials of the row slots: slots [step, 2 step) hand their sums to slots [0, step) ---------
 #pragma unroll
     for (int step = RPP / 2; step >= 1; step >>= 1) {
@@ -498,7 +548,13 @@ int run_tail(const Params& p, const void* k, const void* v, const float* dr_win,
              const int32_t* idx, const int32_t* cnt, const float* ret_ws, void* dk, void* dv, float* part_w, float* part_b,
              bool finish, int nchunk, int rows, cudaStream_t st)
 {
-    const size_t sm = (size_t)(2 * ((rows + K - 1 + 3) & ~3) + (256 / (2 * D / 4) / 2) * K * 2 * D) * sizeof(float);
+    const size_t sm = TAIL_RING + TAIL_BARS + (size_t)2 * ((rows + K - 1 + 3) & ~3) * sizeof(float);
+    static PerDeviceOnce attr;
+    if (int e = attr.run([] {
+            constexpr int most = TAIL_RING + TAIL_BARS + 2 * (TAIL_MAX_ROWS + 32) * 4;
+            const cudaError_t a = cudaFuncSetAttribute(bwd_tail_kernel<D, K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            return a != cudaSuccess ? a : cudaFuncSetAttribute(bwd_tail_kernel<D, K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        })) return e;
     dim3 grid(p.B * nchunk, p.H);
     // the retained tiles' scratch: dk_ret, dv_ret [B,H,R,d], dr_ret [B,H,R] (layout of launch_bwd_dkv_tc)
     const size_t n = (size_t)p.B * p.H * (p.R > 0 ? p.R : 1);
@@ -636,5 +692,7 @@ int launch_bwd(const Params& p, const void* q, const void* k, const void* v, con
 #undef LTE_GO
     return LTE_ERR_UNSUPPORTED;
 }
+
+int bwd_tail_status_fetch_and_clear() { return status_fetch_and_clear(g_tail_status); }
 
 }  // namespace lte
