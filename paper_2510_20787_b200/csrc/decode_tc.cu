@@ -77,6 +77,8 @@ template <int NC> __host__ __device__ inline Plan plan_of(const CacheLayout& L) 
     P.total = P.off_bar + 128;
     return P;
 }
+// The most a plan takes: NC rows, of which one is the ring's and the others the pool's (a logit each, a position for those).
+template <int NC> constexpr int kMostSmem = 2 * NC * 128 + 2048 + 4096 + 2 * ((4 * NC + 4 * (NC - 1) + 16 + 255) / 256 * 256) + 128;
 
 template <int NC>
 __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(unsigned char* __restrict__ cache, CacheLayout L,
@@ -367,10 +369,12 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
     auto go = [&](auto nc, auto kern, PerDeviceOnce& attr) {
         constexpr int NC = decltype(nc)::value;
         const Plan P = plan_of<NC>(L);
-        constexpr int most = 227 * 1024 / kPerSm<NC> - 2048;
-        if (int e = attr.run([=] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most); })) return e;
-        if (P.total > (uint32_t)most) return (int)LTE_ERR_UNSUPPORTED;
-        const int n_cta = BH < kPerSm<NC> * n_sm ? BH : kPerSm<NC> * n_sm;   // each takes an equal share of the heads (+- 1)
+        if (int e = attr.run([=] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem<NC>); })) return e;
+        if (P.total > (uint32_t)kMostSmem<NC>) return (int)LTE_ERR_UNSUPPORTED;
+        // As many CTAs as are resident at once, each with an equal share of the heads (+- 1).  Pools of which W + 2 R > 444 have two
+        // longer tail buffers (logits and positions), and with 256 rows two CTAs then fit an SM in place of three.
+        const int fit = 227 * 1024 / (int)(P.total + 2048), slots = (fit < kPerSm<NC> ? fit : kPerSm<NC>) * n_sm;
+        const int n_cta = BH < slots ? BH : slots;
         return cuda_status(launch_pdl(kern, dim3(n_cta), dim3(kThreads<NC>), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
                                       (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, BH, p.H, p.W, p.R,
                                       p.sink, p.K, p.zthr, p.scale, p.G));

@@ -34,3 +34,13 @@ def test_decode_tc(B, H, W, R, K, sink, T0, steps):
     o64, l64, _, _ = orc.stream(x["q"], x["k"], x["v"], orc.scores(x["k"], x["v"], x["w"]), W, R, sink, n_from=T0)
     assert np.max(np.abs(o - o64)) <= 2e-2 and np.max(np.abs(lse - l64)) <= 2e-3
     assert lte.lte_device_status() == 0
+
+
+@pytest.mark.parametrize("B,H,W,R,K,sink,T0,steps", [
+    (1, 2, 60, 192, 7, 0, 400, 6),         # the longest tail with which three blocks share an SM
+    (1, 2, 64, 192, 7, 2, 400, 6),         # the first with which two do
+    (2, 2, 1, 255, 1, 4, 300, 6),          # the longest there is
+    (53, 16, 20, 236, 7, 1, 300, 3),       # ... nearly, with more heads than blocks
+])
+def test_decode_tc_long_pools(B, H, W, R, K, sink, T0, steps):
+    test_decode_tc(B, H, W, R, K, sink, T0, steps)
