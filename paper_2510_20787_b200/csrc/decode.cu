@@ -622,22 +622,23 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
 
 // State after a T-token prompt.  Bound by memory: every byte of the cache is written exactly once (the rows nothing fills,
 // the tail's padding and the header as zeros, so no fill pass comes before), every window and retained row is read once, in
-// 16-byte pieces.  Block (part, (b,h)) writes IROWS rows of the head's block with their logits; a block per head with two
-// divisions per element took 248 + 17 us for 256 heads of 1,280 rows (d = 64), this takes 28.
+// 16-byte pieces.  Block (b,h) x parts + part (one-dimensional: there may be more heads than a grid's second dimension takes) writes
+// IROWS rows of the head's block with their logits; a block per head with two divisions per element took 248 + 17 us for 256 heads of
+// 1,280 rows (d = 64), this takes 28.
 constexpr int IROWS = 64;
 __global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restrict__ cache, CacheLayout L, const uint4* __restrict__ k,
                                                          const uint4* __restrict__ v, const float* __restrict__ z,
                                                          const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, int Tlen,
-                                                         int pshift, int W, int R, int half)
+                                                         int pshift, int W, int R, int half, int parts)
 {
     __shared__ int s_pos[IROWS];                               // token of each row of this part, -1: none
     pdl_launch_dependents();
     pdl_wait();
-    const int bh = blockIdx.y, tid = threadIdx.x;
+    const int bh = blockIdx.x / parts, part = blockIdx.x - bh * parts, tid = threadIdx.x;
     unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
     const int n_ret = Tlen > 0 && R > 0 ? cnt[bh] : 0;
     const int lo = Tlen - W > 0 ? Tlen - W : 0;
-    const int row0 = blockIdx.x * IROWS, n_rows = min(IROWS, L.rows_alloc - row0);
+    const int row0 = part * IROWS, n_rows = min(IROWS, L.rows_alloc - row0);
     if (tid < n_rows) {
         const int a = row0 + tid;
         int pos = -1;
@@ -655,7 +656,7 @@ __global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restri
             if (a >= W) reinterpret_cast<int32_t*>(blk + L.off_pidx)[a - W] = pos < 0 ? 0 : pos;
         }
     }
-    if (blockIdx.x == 0) {                                     // counters and padding; the header
+    if (part == 0) {                                           // counters and padding; the header
         uint32_t* tail = reinterpret_cast<uint32_t*>(blk + L.off_meta);
         const int n_tail = (int)((L.stride - L.off_meta) / 4);
         for (int e = tid; e < n_tail; e += 256) tail[e] = e == 0 ? (uint32_t)Tlen : e == 1 ? (uint32_t)n_ret : 0u;
@@ -688,9 +689,9 @@ int launch_cache_init(const Params& p, const void* k, const void* v, const float
                       const int32_t* cnt, void* cache, cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    const dim3 grid((L.rows_alloc + IROWS - 1) / IROWS, p.B * p.H);
-    return cuda_status(launch_pdl(cache_init_kernel, grid, dim3(256), 0, st, (unsigned char*)cache, L, (const uint4*)k, (const uint4*)v, z,
-                                  idx, cnt, p.T, piece_shift(L, p.d), p.W, p.R, p.half));
+    const int parts = (L.rows_alloc + IROWS - 1) / IROWS;
+    return cuda_status(launch_pdl(cache_init_kernel, dim3(parts * p.B * p.H), dim3(256), 0, st, (unsigned char*)cache, L, (const uint4*)k, (const uint4*)v, z,
+                                  idx, cnt, p.T, piece_shift(L, p.d), p.W, p.R, p.half, parts));
 }
 
 // ---- lazy scoring of the ring for scorers that do not run inside the step (the three-layer stack) -------------------
@@ -708,18 +709,18 @@ constexpr int LROWS = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) ring_linearize_kernel(const unsigned char* __restrict__ cache, CacheLayout L, uint4* __restrict__ klin,
                                                              uint4* __restrict__ vlin, int pshift, int W, const float* __restrict__ rope_cos,
-                                                             const float* __restrict__ rope_sin, int rope_len)
+                                                             const float* __restrict__ rope_sin, int rope_len, int parts)
 {
     constexpr int EPV = V16<T>::N;
     pdl_launch_dependents();
     pdl_wait();
-    const int bh = blockIdx.y;
+    const int bh = blockIdx.x / parts, part = blockIdx.x - bh * parts;   // (one-dimensional, as in cache_init_kernel)
     const unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
     const uint4* Kc = reinterpret_cast<const uint4*>(blk + L.off_k);
     const uint4* Vc = reinterpret_cast<const uint4*>(blk + L.off_v);
     const int n = reinterpret_cast<const int32_t*>(blk + L.off_meta)[0];
     const int base = n > W ? n - W : 0, n_eff = n < W ? n : W;
-    const int r0 = blockIdx.x * LROWS, n_rows = min(LROWS, W - r0);
+    const int r0 = part * LROWS, n_rows = min(LROWS, W - r0);
     const int hshift = pshift - 1, hp = 1 << hshift;           // pieces of half a row
     const int slot0 = (base + r0) % W;
     for (int e = threadIdx.x; e < n_rows << hshift; e += 256) {
@@ -778,10 +779,10 @@ int launch_ring_linearize(const Params& p, const void* cache, void* klin, void* 
                           int rope_len, cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    const dim3 grid((p.W + LROWS - 1) / LROWS, p.B * p.H);
+    const int parts = (p.W + LROWS - 1) / LROWS;
     auto kern = p.dtype == LTE_BF16 ? ring_linearize_kernel<__nv_bfloat16> : ring_linearize_kernel<float>;
-    return cuda_status(launch_pdl(kern, grid, dim3(256), 0, st, (const unsigned char*)cache, L, (uint4*)klin, (uint4*)vlin, piece_shift(L, p.d),
-                                  p.W, rope_cos, rope_sin, rope_len));
+    return cuda_status(launch_pdl(kern, dim3(parts * p.B * p.H), dim3(256), 0, st, (const unsigned char*)cache, L, (uint4*)klin, (uint4*)vlin, piece_shift(L, p.d),
+                                  p.W, rope_cos, rope_sin, rope_len, parts));
 }
 
 int launch_ring_scatter_z(const Params& p, void* cache, const float* zlin, cudaStream_t st)

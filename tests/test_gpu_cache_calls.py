@@ -1,0 +1,40 @@
+"""lte_cache_init, lte_cache_score and lte_cache_score_unrope beyond their usual arguments: more heads than a grid's second dimension."""
+import pytest
+import torch
+
+from paper_2510_20787_b200 import lte
+
+pytestmark = pytest.mark.gpu
+
+
+def test_empty_cache_of_many_heads():
+    B, H, W, R = 4096, 17, 20, 4                               # 69,632 heads
+    s = lte.shape(B, H, 0, 32, W, R, lte.BF16)
+    c = lte.conv(torch.zeros((H, 7, 64), device="cuda"))
+    cache = torch.full((lte.lte_cache_bytes(s),), 255, dtype=torch.uint8, device="cuda")
+    lte.lte_cache_init(s, c, cache=cache)
+    blocks = cache[256:].view(B * H, -1)
+    n = 2 * (W + R) * 32 * 2                                   # keys and values, then logits, then the rest
+    logits = blocks[:, n:n + 4 * (W + R)].view(torch.float32)
+    assert bool((logits == -float("inf")).all())
+    assert not bool(cache[:256].any()) and not bool(blocks[:, :n].any()) and not bool(blocks[:, n + 4 * (W + R):].any())
+
+
+def test_ring_of_many_heads_is_scored():
+    B, H, d, W, R, T = 4096, 17, 32, 20, 4, 20
+    g = torch.Generator(device="cuda").manual_seed(1)
+    ch = [2 * d, d, d // 2, d // 4]
+    c = lte.conv_stack([torch.randn((H, ch[i + 1], 3, ch[i]), generator=g, device="cuda") * 0.1 for i in range(3)],
+                       torch.randn((H, ch[3]), generator=g, device="cuda"))
+    s = lte.shape(B, H, T, d, W, R, lte.BF16)
+    k, v = (torch.randn((B, H, T, d), generator=g, device="cuda").to(torch.bfloat16) for _ in "kv")
+    z = lte.lte_scores(s, c, k, v)
+    unscored = torch.full_like(z, -float("inf"))
+    idx, cnt = (torch.zeros(n, dtype=torch.int32, device="cuda") for n in ((B, H, R), (B, H)))
+    cache = lte.lte_cache_init(s, c, k, v, unscored, idx, cnt)
+    lte.lte_cache_score(s, c, cache)
+    n = 2 * (W + R) * d * 2
+    got = cache[256:].view(B * H, -1)[:, n:n + 4 * W].view(torch.float32).view(B, H, W)
+    assert torch.equal(got[:, :, :T - 6], z[:, :, :T - 6])     # the last six tokens' right context is not there yet
+    assert bool((got[:, :, T - 6:] == -float("inf")).all())
+    assert lte.lte_device_status() == 0
