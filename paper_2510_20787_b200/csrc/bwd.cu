@@ -560,14 +560,12 @@ int run_tail(const Params& p, const void* k, const void* v, const float* dr_win,
     const size_t n = (size_t)p.B * p.H * (p.R > 0 ? p.R : 1);
     const float* dk_ret = ret_ws; const float* dv_ret = dk_ret + n * D; const float* dr_ret = dv_ret + n * D;
     if (finish)
-        launch_pdl(bwd_tail_kernel<D, K, true>, grid, dim3(256), sm, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, dr_win, z,
+        return cuda_status(launch_pdl(bwd_tail_kernel<D, K, true>, grid, dim3(256), sm, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, dr_win, z,
                    lambda, idx, cnt, dk_ret, dv_ret, dr_ret, p.w, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, part_w, part_b, p.B, p.H,
-                   p.T, p.R, p.zthr, nchunk, rows);
-    else
-        launch_pdl(bwd_tail_kernel<D, K, false>, grid, dim3(256), sm, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, dr_win, z,
+                   p.T, p.R, p.zthr, nchunk, rows));
+    return cuda_status(launch_pdl(bwd_tail_kernel<D, K, false>, grid, dim3(256), sm, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, dr_win, z,
                    lambda, idx, cnt, dk_ret, dv_ret, dr_ret, p.w, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, part_w, part_b, p.B, p.H,
-                   p.T, p.R, p.zthr, nchunk, rows);
-    return cuda_status(cudaGetLastError());
+                   p.T, p.R, p.zthr, nchunk, rows));
 }
 
 struct WsPlan { size_t delta, dz, part_w, part_b, dk32, dv32, ret, total; int nchunk; };
@@ -652,8 +650,7 @@ int run(const Params& p, const void* q, const void* k, const void* v, const void
             const int e = p.K == 7 ? run_tail<D, 7>(p, k, v, dz, z, lambda, idx, cnt, rw, dk, dv, part_w, part_b, f32, nch, rows, st)
                                    : run_tail<D, 5>(p, k, v, dz, z, lambda, idx, cnt, rw, dk, dv, part_w, part_b, f32, nch, rows, st);
             if (e != LTE_OK) return e;
-            launch_pdl(bwd_conv_reduce_kernel, gr, dim3(256), 0, st, part_w, part_b, dw, dbias, p.B * nch, per_head);
-            return cuda_status(cudaGetLastError());
+            return cuda_status(launch_pdl(bwd_conv_reduce_kernel, gr, dim3(256), 0, st, part_w, part_b, dw, dbias, p.B * nch, per_head));
         }
     }
     dim3 gc(p.B * w.nchunk, p.H);

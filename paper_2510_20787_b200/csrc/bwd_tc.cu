@@ -738,8 +738,8 @@ int launch_bwd_dkv_tc(const Params& p, const void* q, const void* k, const void*
     // merge_here = false: the caller's last pass adds the retained shares and turns dr into dz itself
     if (e || !merge_here) return e;
     if (p.R > 0) {
-        if (launch_pdl(bwd_merge_kernel, dim3((p.R * p.d + 1023) / 1024, BH), dim3(256), 0, st, idx, cnt, dk_ret, dv_ret, dr_ret, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv,
-                       dz, p.T, p.R, p.d) != cudaSuccess) return LTE_ERR_CUDA;
+        if (int e2 = cuda_status(launch_pdl(bwd_merge_kernel, dim3((p.R * p.d + 1023) / 1024, BH), dim3(256), 0, st, idx, cnt, dk_ret, dv_ret, dr_ret,
+                                            (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dz, p.T, p.R, p.d))) return e2;
     }
     return cuda_status(launch_pdl(bwd_dz_kernel, dim3((p.T + 255) / 256, BH), dim3(256), 0, st, dz, z, lambda, p.H, p.T, p.half, p.zthr));
 }

@@ -145,7 +145,14 @@ int launch_bwd(const Params& p, const void* q, const void* k, const void* v, con
                void* dq, void* dk, void* dv, float* dw, float* dbias, uint32_t flags, void* ws,
                cudaStream_t st);
 
-inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? LTE_OK : LTE_ERR_CUDA; }
+// Status of a runtime call or launch.  The runtime keeps a failed launch's error until it is asked for: it is taken here, so that the
+// caller's next check of a launch of its own does not find it.
+inline int cuda_status(cudaError_t e)
+{
+    if (e == cudaSuccess) return LTE_OK;
+    (void)cudaGetLastError();
+    return LTE_ERR_CUDA;
+}
 
 // Device-side status of one kernel family (a __device__ variable per family, so one per device).
 //   code        sticky report for the host: 0, or the code of the first anomaly since lte_device_status() last read it

@@ -1185,18 +1185,16 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
         if (int e = attr.run([] { return cudaFuncSetAttribute(decode_attend_kernel<T, D>,                              \
                 cudaFuncAttributeMaxDynamicSharedMemorySize,                                                           \
                 (int)(sizeof(float) * ((size_t)ATT_Q * MAX_ROWS + (DT / 32) * ATT_Q * 128))); })) return e;            \
-        if (cudaLaunchKernelEx(&acfg, decode_attend_kernel<T, D>, (unsigned char*)cache, L, (const T*)q1, (T*)o1, lse1,        \
-                               p.W, p.G, p.scale, 0, (const T*)k1, (const T*)v1, p.w, p.bias, p.H, p.R, p.sink, ps.K,    \
-                               p.zthr) != cudaSuccess) return LTE_ERR_CUDA;                                             \
+        return cuda_status(cudaLaunchKernelEx(&acfg, decode_attend_kernel<T, D>, (unsigned char*)cache, L, (const T*)q1, (T*)o1, lse1, \
+                               p.W, p.G, p.scale, 0, (const T*)k1, (const T*)v1, p.w, p.bias, p.H, p.R, p.sink, ps.K, p.zthr)); \
     } while (0)
     switch (p.d) {
-        case 32: LTE_ATT(float, 32); break;
-        case 64: LTE_ATT(float, 64); break;
-        case 128: LTE_ATT(float, 128); break;
+        case 32: LTE_ATT(float, 32);
+        case 64: LTE_ATT(float, 64);
+        case 128: LTE_ATT(float, 128);
         default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_ATT
-    return cuda_status(cudaGetLastError());
 }
 
 }  // namespace lte

@@ -354,10 +354,8 @@ int run_tma(const Params& p, const void* k, const void* v, float* z, float* r, c
     if (n_flat > 0x7fffffffLL) return LTE_ERR_UNSUPPORTED;
     const int slots = n_sm * (D == 64 ? 2 : 1);
     const int n_cta = (int)(n_flat < slots ? n_flat : slots);
-    if (launch_pdl(scores_tc_kernel<D, K>, dim3(n_cta), dim3(NT + 64), C::BYTES, st, tk, tv, p.w, p.bias, z, r, p.H, p.T,
-                   (int)n_flat, dg) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(scores_tc_kernel<D, K>, dim3(n_cta), dim3(NT + 64), C::BYTES, st, tk, tv, p.w, p.bias, z, r, p.H, p.T,
+                                  (int)n_flat, dg));
 }
 
 template <typename T, int D, int K>

@@ -416,13 +416,11 @@ int run_stack_bwd(const Params& p, const void* k, const void* v, const float* dz
     static PerDeviceOnce attr;
     if (int e2 = attr.run([] { return cudaFuncSetAttribute(stack_bwd_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::BYTES); }))
         return e2;
-    if (launch_pdl(stack_bwd_kernel<T, D>, grid, dim3(SB_NT), L::BYTES, st, (const T*)k, (const T*)v, p.w, p.bias, dz, (T*)dk, (T*)dv,
-                   (float*)part, p.H, p.T, per, input_grad ? 1 : 0) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    if (launch_pdl(stack_bwd_reduce_kernel<D>, dim3((L::PART + 255) / 256, p.H), dim3(256), 0, st, (const float*)part, dw, dbias, p.B,
-                   p.H, chunks) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    return cuda_status(cudaGetLastError());
+    if (int e2 = cuda_status(launch_pdl(stack_bwd_kernel<T, D>, grid, dim3(SB_NT), L::BYTES, st, (const T*)k, (const T*)v, p.w, p.bias, dz,
+                                        (T*)dk, (T*)dv, (float*)part, p.H, p.T, per, input_grad ? 1 : 0)))
+        return e2;
+    return cuda_status(launch_pdl(stack_bwd_reduce_kernel<D>, dim3((L::PART + 255) / 256, p.H), dim3(256), 0, st, (const float*)part, dw,
+                                  dbias, p.B, p.H, chunks));
 }
 }  // namespace
 

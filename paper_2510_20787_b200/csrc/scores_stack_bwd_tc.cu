@@ -605,17 +605,15 @@ int launch_stack_bwd_tc(const Params& p, const void* k, const void* v, const flo
     if (int e = attr.run([] { return cudaFuncSetAttribute(stack_bwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BT_SMEM); })) return e;
     uint8_t* img = (uint8_t*)ws;
     float* part = (float*)((char*)ws + ((size_t)p.H * BI_HEAD + 255) / 256 * 256);
-    if (launch_pdl(stack_bwd_image_kernel, dim3(p.H, 32), dim3(256), 0, st, p.w, p.bias, img, p.H) != cudaSuccess) return LTE_ERR_CUDA;
+    if (int e = cuda_status(launch_pdl(stack_bwd_image_kernel, dim3(p.H, 32), dim3(256), 0, st, p.w, p.bias, img, p.H))) return e;
     const int chunks = bt_chunks(p);
     const int n_tiles = (p.T + BT_OWN - 1) / BT_OWN, per = (n_tiles + chunks - 1) / chunks;
-    if (launch_pdl(stack_bwd_tc_kernel, dim3(chunks, p.B * p.H), dim3(BT_THREADS), BT_SMEM, st, (const __nv_bfloat16*)k,
-                   (const __nv_bfloat16*)v, (const uint8_t*)img, dz, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, part, p.H, p.T, per,
-                   input_grad ? 1 : 0) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    if (launch_pdl(stack_bwd_tc_reduce_kernel, dim3((BPART + 255) / 256, p.H), dim3(256), 0, st, (const float*)part, dw, dbias,
-                   p.B, p.H, chunks) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    return cuda_status(cudaGetLastError());
+    if (int e = cuda_status(launch_pdl(stack_bwd_tc_kernel, dim3(chunks, p.B * p.H), dim3(BT_THREADS), BT_SMEM, st, (const __nv_bfloat16*)k,
+                                       (const __nv_bfloat16*)v, (const uint8_t*)img, dz, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, part, p.H,
+                                       p.T, per, input_grad ? 1 : 0)))
+        return e;
+    return cuda_status(launch_pdl(stack_bwd_tc_reduce_kernel, dim3((BPART + 255) / 256, p.H), dim3(256), 0, st, (const float*)part, dw,
+                                  dbias, p.B, p.H, chunks));
 }
 
 }  // namespace lte

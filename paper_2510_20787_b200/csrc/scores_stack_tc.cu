@@ -541,17 +541,15 @@ int launch_scores_stack_tc(const Params& p, const void* k, const void* v, float*
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
     const int BH = p.B * p.H;
-    if (launch_pdl(stack_image_kernel, dim3(p.H, 32), dim3(256), 0, st, p.w, p.bias, (uint8_t*)ws, p.H, p.d) != cudaSuccess) return LTE_ERR_CUDA;
+    if (int e = cuda_status(launch_pdl(stack_image_kernel, dim3(p.H, 32), dim3(256), 0, st, p.w, p.bias, (uint8_t*)ws, p.H, p.d))) return e;
     const int n_t = (p.T - ST_HALF + ST_VALID - 1) / ST_VALID;
     const long long n_flat = (long long)BH * n_t;
     if (n_flat > 0x7fffffffLL) return LTE_ERR_UNSUPPORTED;
     const int grid = (int)(n_flat < n_sm ? n_flat : n_sm);
     const int per = (int)((n_flat + grid - 1) / grid);
     const int n_cta = (int)((n_flat + per - 1) / per);
-    if (launch_pdl(scores_stack_tc_kernel, dim3(n_cta), dim3(ST_THREADS), ST_SMEM, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const uint8_t*)ws, z, r, p.B, p.H,
-                   p.T, n_t, (int)n_flat, per, p.d) != cudaSuccess)
-        return LTE_ERR_CUDA;
-    return cuda_status(cudaGetLastError());
+    return cuda_status(launch_pdl(scores_stack_tc_kernel, dim3(n_cta), dim3(ST_THREADS), ST_SMEM, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                                  (const uint8_t*)ws, z, r, p.B, p.H, p.T, n_t, (int)n_flat, per, p.d));
 }
 
 }  // namespace lte

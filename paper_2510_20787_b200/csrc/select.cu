@@ -427,12 +427,9 @@ int launch_select(const Params& p, const float* z, int32_t* idx, int32_t* cnt, i
         const int kpt = (N + nt - 1) / nt;
         const int BH = p.B * p.H;
 #define LTE_SEL(KPT) launch_pdl(select_reg_kernel<KPT>, dim3(BH), dim3(nt), 0, st, z, idx, cnt, ncand, p.T, p.W, p.R, p.sink, p.zthr)
-        if (kpt <= 64) {
-            if (kpt <= 1) LTE_SEL(1); else if (kpt <= 2) LTE_SEL(2); else if (kpt <= 4) LTE_SEL(4);
-            else if (kpt <= 8) LTE_SEL(8); else if (kpt <= 16) LTE_SEL(16); else if (kpt <= 32) LTE_SEL(32);
-            else LTE_SEL(64);
-            return cuda_status(cudaGetLastError());
-        }
+        if (kpt <= 64)
+            return cuda_status(kpt <= 1 ? LTE_SEL(1) : kpt <= 2 ? LTE_SEL(2) : kpt <= 4 ? LTE_SEL(4) : kpt <= 8 ? LTE_SEL(8) :
+                               kpt <= 16 ? LTE_SEL(16) : kpt <= 32 ? LTE_SEL(32) : LTE_SEL(64));
 #undef LTE_SEL
     }
     const int threads = N <= 1024 ? 256 : (N <= 4096 ? 512 : 1024);

@@ -65,7 +65,7 @@ __global__ void stats_final_kernel(const float* __restrict__ part, const float* 
 int launch_sparsity_stats(const Params& p, const float* z, const float* lambda, float* count, float* penalty, float* part, float tau,
                           cudaStream_t st)
 {
-    if (launch_pdl(stats_partial_kernel, dim3(p.B * p.H), dim3(ST), 0, st, z, part, p.T, p.zthr, tau) != cudaSuccess) return LTE_ERR_CUDA;
+    if (int e = cuda_status(launch_pdl(stats_partial_kernel, dim3(p.B * p.H), dim3(ST), 0, st, z, part, p.T, p.zthr, tau))) return e;
     return cuda_status(launch_pdl(stats_final_kernel, dim3(1), dim3(256), (size_t)p.H * sizeof(float), st, part, lambda, count, penalty, p.B, p.H));
 }
 
