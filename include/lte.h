@@ -206,7 +206,8 @@ size_t lte_cache_bytes(const lte_shape* s);
  * State after a T-token prompt: ring <- last min(T,W) rows of k, v and their logits from z (the
  * last `half` prompt tokens are still unscored and are scored by the first decode steps), pool <-
  * rows idx[:cnt] of k, v with their logits.  T = 0 gives the empty cache (k, v, z, idx, cnt may
- * then be NULL).  Requires W >= K.
+ * then be NULL).  Requires W >= K.  k and v may start at any element (from a 16-byte boundary they
+ * are read faster).
  */
 int lte_cache_init(const lte_shape* s, const lte_conv* c, const void* k, const void* v,
                    const float* z, const int32_t* idx, const int32_t* cnt, void* cache, void* stream);

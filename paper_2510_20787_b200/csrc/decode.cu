@@ -626,8 +626,20 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
 // IROWS rows of the head's block with their logits; a block per head with two divisions per element took 248 + 17 us for 256 heads of
 // 1,280 rows (d = 64), this takes 28.
 constexpr int IROWS = 64;
-__global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restrict__ cache, CacheLayout L, const uint4* __restrict__ k,
-                                                         const uint4* __restrict__ v, const float* __restrict__ z,
+// The piece-th 16 bytes of a tensor, read in units of U (what the tensor is aligned to).
+template <typename U> __device__ __forceinline__ uint4 load_piece(const U* p, size_t piece)
+{
+    constexpr int N = 16 / (int)sizeof(U);
+    U x[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = p[piece * N + i];
+    uint4 r;
+    memcpy(&r, x, 16);
+    return r;
+}
+template <typename U>
+__global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restrict__ cache, CacheLayout L, const U* __restrict__ k,
+                                                         const U* __restrict__ v, const float* __restrict__ z,
                                                          const int32_t* __restrict__ idx, const int32_t* __restrict__ cnt, int Tlen,
                                                          int pshift, int W, int R, int half, int parts)
 {
@@ -672,8 +684,8 @@ __global__ void __launch_bounds__(256) cache_init_kernel(unsigned char* __restri
         const int r = e >> pshift, c = e & pmask, row = row0 + r, pos = s_pos[r];
         uint4 kx = make_uint4(0, 0, 0, 0), vx = kx;
         if (pos >= 0) {
-            kx = k[((src0 + pos) << pshift) + c];
-            vx = v[((src0 + pos) << pshift) + c];
+            kx = load_piece(k, ((src0 + pos) << pshift) + c);
+            vx = load_piece(v, ((src0 + pos) << pshift) + c);
         }
         const size_t d = ((size_t)row << pshift) + cache_chunk_pos(L, row, c);
         Kc[d] = kx;
@@ -690,8 +702,14 @@ int launch_cache_init(const Params& p, const void* k, const void* v, const float
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
     const int parts = (L.rows_alloc + IROWS - 1) / IROWS;
-    return cuda_status(launch_pdl(cache_init_kernel, dim3(parts * p.B * p.H), dim3(256), 0, st, (unsigned char*)cache, L, (const uint4*)k, (const uint4*)v, z,
-                                  idx, cnt, p.T, piece_shift(L, p.d), p.W, p.R, p.half, parts));
+    auto go = [&](auto unit) {
+        using U = decltype(unit);
+        return cuda_status(launch_pdl(cache_init_kernel<U>, dim3(parts * p.B * p.H), dim3(256), 0, st, (unsigned char*)cache, L, (const U*)k, (const U*)v,
+                                      z, idx, cnt, p.T, piece_shift(L, p.d), p.W, p.R, p.half, parts));
+    };
+    // views of k and v may start at any element; from there on their rows are whole pieces
+    if ((((uintptr_t)k | (uintptr_t)v) & 15u) == 0) return go(uint4());
+    return L.esz == 2 ? go(uint16_t()) : go(uint32_t());
 }
 
 // ---- lazy scoring of the ring for scorers that do not run inside the step (the three-layer stack) -------------------

@@ -33,7 +33,9 @@ int device_sm_count(int* n_sm)
 
 namespace {
 
-bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+bool aligned(const void* p, size_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; }
+bool aligned16(const void* p) { return aligned(p, 16); }
+size_t element_bytes(const lte_shape* s) { return s->dtype == LTE_BF16 ? 2 : 4; }
 
 int check_shape(const lte_shape* s, bool need_T)
 {
@@ -310,6 +312,7 @@ int lte_cache_init(const lte_shape* s, const lte_conv* c, const void* k, const v
     e = check_conv_or_stack(s, c); if (e) return e;
     if (!cache || !aligned16(cache)) return LTE_ERR_INVALID_ARG;
     if (s->T > 0 && (!k || !v || !z || !cnt || (s->R > 0 && !idx))) return LTE_ERR_INVALID_ARG;
+    if (!aligned(k, element_bytes(s)) || !aligned(v, element_bytes(s))) return LTE_ERR_INVALID_ARG;
     e = check_arch(); if (e) return e;
     return launch_cache_init(make_params(s, c), k, v, z, idx, cnt, cache, (cudaStream_t)stream);
 }

@@ -215,3 +215,13 @@ def test_streaming_chunk_host_side():
     assert L.lte_attn_prefill_chunk_ex(*args, lte.CHUNK_STREAMING, 256, need0, None) == -3   # the streaming scratch is larger
     big = lte.shape(1, 2, 64, 64, 16, 5000, lte.BF16)
     assert L.lte_attn_prefill_chunk_ex(ctypes.addressof(big), pc, 256, 0, 256, 256, 256, 256, 256, lte.CHUNK_STREAMING, 256, 1 << 40, None) == -2
+
+
+def test_cache_init_takes_whole_elements_only():
+    """k and v may start at any element, not inside one (validation fails before anything is launched)."""
+    L = lte.lib()
+    c = lte.LteConv(1, 5, 1, 256, 0)
+    for code, off in ((lte.F32, 2), (lte.BF16, 1)):
+        s = lte.shape(1, 2, 128, 32, 16, 8, code)
+        for k, v in ((4096 + off, 4096), (4096, 4096 + off)):
+            assert L.lte_cache_init(ctypes.addressof(s), ctypes.addressof(c), k, v, 4096, 4096, 4096, 4096, None) == -1

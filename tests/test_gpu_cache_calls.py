@@ -1,4 +1,5 @@
-"""lte_cache_init, lte_cache_score and lte_cache_score_unrope beyond their usual arguments: more heads than a grid's second dimension."""
+"""lte_cache_init, lte_cache_score and lte_cache_score_unrope beyond their usual arguments: more heads than a grid's second dimension,
+tensors that start between 16-byte boundaries."""
 import pytest
 import torch
 
@@ -38,3 +39,26 @@ def test_ring_of_many_heads_is_scored():
     assert torch.equal(got[:, :, :T - 6], z[:, :, :T - 6])     # the last six tokens' right context is not there yet
     assert bool((got[:, :, T - 6:] == -float("inf")).all())
     assert lte.lte_device_status() == 0
+
+
+def _at(t, offset):
+    """A contiguous copy of t that starts `offset` elements behind a 16-byte boundary."""
+    buf = torch.empty(t.numel() + 8, dtype=t.dtype, device=t.device)
+    out = buf[offset:offset + t.numel()].view(t.shape)
+    return out.copy_(t)
+
+
+@pytest.mark.parametrize("dtype,d,W,R,ok,ov", [
+    (lte.BF16, 64, 20, 12, 1, 0), (lte.BF16, 64, 130, 140, 0, 2), (lte.BF16, 32, 20, 12, 4, 7), (lte.BF16, 128, 20, 12, 3, 3),
+    (lte.F32, 32, 20, 12, 1, 0), (lte.F32, 64, 20, 0, 0, 3), (lte.F32, 128, 70, 12, 2, 1),
+])
+def test_cache_from_unaligned_tensors(dtype, d, W, R, ok, ov):
+    B, H, T = 2, 3, 300
+    g = torch.Generator(device="cuda").manual_seed(2)
+    k, v = (torch.randn((B, H, T, d), generator=g, device="cuda").to(torch.bfloat16 if dtype == lte.BF16 else torch.float32) for _ in "kv")
+    s = lte.shape(B, H, T, d, W, R, dtype)
+    c = lte.conv(torch.randn((H, 5, 2 * d), generator=g, device="cuda") * 0.1)
+    z = lte.lte_scores(s, c, k, v)
+    idx, cnt = lte.lte_select(s, z)
+    want = lte.lte_cache_init(s, c, k, v, z, idx, cnt)
+    assert torch.equal(lte.lte_cache_init(s, c, _at(k, ok), _at(v, ov), z, idx, cnt), want)
