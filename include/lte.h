@@ -253,7 +253,7 @@ int lte_cache_score(const lte_shape* s, const lte_conv* c, void* cache, void* ws
  * rotated ones.
  *   rope_cos, rope_sin   in  [rope_len, d/2] fp32 device: cos / sin of the angle of channel pair (c, c + d/2) at position p
  *                        (half-split pairing: (x1, x2) -> (x1 cos - x2 sin, x2 cos + x1 sin) is the embedding);
- *                        both NULL = lte_cache_score
+ *                        both NULL = lte_cache_score.  They may start at any element, e.g. be rows of a longer table
  *   rope_len             positions the tables cover; a ring token at a position >= rope_len keeps its rotated key and
  *                        lte_device_status() reports it
  * Errors: as lte_cache_score; INVALID_ARG for one NULL table or rope_len <= 0.

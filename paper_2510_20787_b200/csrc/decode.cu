@@ -724,6 +724,17 @@ int launch_cache_init(const Params& p, const void* k, const void* v, const float
 // byte is read and written once; blocks of LROWS rows (a block per head with two divisions per element took 154 us for 256
 // heads of 768 rows, d = 64, this takes 14).
 constexpr int LROWS = 64;
+// Four values of a table, which may start at any of its elements (`wide`: at a 16-byte boundary, like every row of it then).
+__device__ __forceinline__ void load4(const float* p, bool wide, float (&x)[4])
+{
+    if (wide) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = p[i];
+    }
+}
 template <typename T>
 __global__ void __launch_bounds__(256) ring_linearize_kernel(const unsigned char* __restrict__ cache, CacheLayout L, uint4* __restrict__ klin,
                                                              uint4* __restrict__ vlin, int pshift, int W, const float* __restrict__ rope_cos,
@@ -741,6 +752,7 @@ __global__ void __launch_bounds__(256) ring_linearize_kernel(const unsigned char
     const int r0 = part * LROWS, n_rows = min(LROWS, W - r0);
     const int hshift = pshift - 1, hp = 1 << hshift;           // pieces of half a row
     const int slot0 = (base + r0) % W;
+    const bool wide = ((reinterpret_cast<uintptr_t>(rope_cos) | reinterpret_cast<uintptr_t>(rope_sin)) & 15u) == 0;
     for (int e = threadIdx.x; e < n_rows << hshift; e += 256) {
         const int r = r0 + (e >> hshift), c = e & (hp - 1);
         uint4 k1 = make_uint4(0, 0, 0, 0), k2 = k1, v1 = k1, v2 = k1;
@@ -759,8 +771,8 @@ __global__ void __launch_bounds__(256) ring_linearize_kernel(const unsigned char
                     T o1[EPV], o2[EPV];
 #pragma unroll
                     for (int i = 0; i < EPV; i += 4) {
-                        const float4 co = *reinterpret_cast<const float4*>(rope_cos + tb + i), si = *reinterpret_cast<const float4*>(rope_sin + tb + i);
-                        const float cf[4] = {co.x, co.y, co.z, co.w}, sf[4] = {si.x, si.y, si.z, si.w};
+                        float cf[4], sf[4];
+                        load4(rope_cos + tb + i, wide, cf); load4(rope_sin + tb + i, wide, sf);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {          // inverse rotation: (x1, x2) -> (x1 cos + x2 sin, x2 cos - x1 sin)
                             o1[i + j] = from_f<T>(a[i + j] * cf[j] + b[i + j] * sf[j]);

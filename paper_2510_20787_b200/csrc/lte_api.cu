@@ -327,6 +327,7 @@ int lte_cache_score_unrope(const lte_shape* s, const lte_conv* c, void* cache, c
 {
     int e = check_shape(s, false); if (e) return e;
     if ((rope_cos == nullptr) != (rope_sin == nullptr) || (rope_cos && rope_len <= 0)) return LTE_ERR_INVALID_ARG;
+    if (!aligned(rope_cos, sizeof(float)) || !aligned(rope_sin, sizeof(float))) return LTE_ERR_INVALID_ARG;
     if (!c || !c->w || c->n_layers != 3) return LTE_ERR_UNSUPPORTED;       // the single layer is scored inside the step
     e = check_conv_or_stack(s, c); if (e) return e;
     if (!cache || !aligned16(cache)) return LTE_ERR_INVALID_ARG;

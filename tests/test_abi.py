@@ -225,3 +225,10 @@ def test_cache_init_takes_whole_elements_only():
         s = lte.shape(1, 2, 128, 32, 16, 8, code)
         for k, v in ((4096 + off, 4096), (4096, 4096 + off)):
             assert L.lte_cache_init(ctypes.addressof(s), ctypes.addressof(c), k, v, 4096, 4096, 4096, 4096, None) == -1
+
+
+def test_rotary_tables_are_whole_elements_only():
+    L = lte.lib()
+    s, c = lte.shape(4, 16, 0, 64, 128, 128, lte.BF16), lte.LteConv(3, 3, 2, 256, 0)
+    for co, si in ((4098, 4096), (4096, 4097)):
+        assert L.lte_cache_score_unrope(ctypes.addressof(s), ctypes.addressof(c), 4096, co, si, 100, 4096, 1 << 30, None) == -1

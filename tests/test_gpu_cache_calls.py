@@ -62,3 +62,23 @@ def test_cache_from_unaligned_tensors(dtype, d, W, R, ok, ov):
     idx, cnt = lte.lte_select(s, z)
     want = lte.lte_cache_init(s, c, k, v, z, idx, cnt)
     assert torch.equal(lte.lte_cache_init(s, c, _at(k, ok), _at(v, ov), z, idx, cnt), want)
+
+
+@pytest.mark.parametrize("dtype,d,W,oc,os", [(lte.BF16, 64, 70, 1, 0), (lte.BF16, 64, 300, 0, 2), (lte.BF16, 32, 20, 3, 1), (lte.F32, 64, 65, 2, 3), (lte.F32, 32, 20, 1, 1)])
+def test_unaligned_rotary_tables(dtype, d, W, oc, os):
+    B, H, R, T = 2, 2, 8, 2 * W + 5
+    g = torch.Generator(device="cuda").manual_seed(3)
+    ch = [2 * d, d, d // 2, d // 4]
+    c = lte.conv_stack([torch.randn((H, ch[i + 1], 3, ch[i]), generator=g, device="cuda") * 0.1 for i in range(3)],
+                       torch.randn((H, ch[3]), generator=g, device="cuda"))
+    s = lte.shape(B, H, T, d, W, R, dtype)
+    k, v = (torch.randn((B, H, T, d), generator=g, device="cuda").to(torch.bfloat16 if dtype == lte.BF16 else torch.float32) for _ in "kv")
+    z = torch.full((B, H, T), -float("inf"), device="cuda")    # nothing is scored yet
+    idx, cnt = lte.lte_select(s, z)
+    angle = torch.rand((T, d // 2), generator=g, device="cuda") * 6.0
+    cos, sin = angle.cos(), angle.sin()
+    caches = [lte.lte_cache_init(s, c, k, v, z, idx, cnt) for _ in range(3)]
+    lte.lte_cache_score_unrope(s, c, caches[0], cos, sin)
+    lte.lte_cache_score_unrope(s, c, caches[1], _at(cos, oc), _at(sin, os))
+    assert torch.equal(caches[0], caches[1]) and not torch.equal(caches[0], caches[2])
+    assert lte.lte_device_status() == 0
