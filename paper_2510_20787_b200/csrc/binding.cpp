@@ -21,10 +21,10 @@ struct PyFailure {};                                           // a Python excep
 
 [[noreturn]] void fail(PyObject* type, const char* text) { PyErr_SetString(type, text); throw PyFailure(); }
 
-// the C struct inside a ctypes object (which the caller holds during the call)
+// the C struct inside a ctypes object (which the caller holds during the call); never NULL: the callers read its sizes
 template <typename S> const S* c_struct(PyObject* o)
 {
-    if (o == Py_None) return nullptr;
+    if (o == Py_None) fail(PyExc_TypeError, "expected an LteShape and an LteConv, not None");
     Py_buffer b;
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw PyFailure();
     const void* p = b.buf;
@@ -266,7 +266,6 @@ LTE_FN(attn_bwd, 17)
 {
     const lte_shape* s = c_struct<lte_shape>(a[0]);
     const lte_conv* c = c_struct<lte_conv>(a[1]);
-    if (!s || !c) fail(PyExc_TypeError, "expected an LteShape and an LteConv");
     const at::Tensor &q = tensor(a[2]), &k = tensor(a[3]);
     const void *qp = ptr(a[2]), *kp = ptr(a[3]), *v = ptr(a[4]), *o = ptr(a[5]), *dO = ptr(a[7]);
     const float *lse = fptr(a[6]), *z = fptr(a[8]), *lam = fptr(a[11]);
