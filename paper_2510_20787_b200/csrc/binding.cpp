@@ -59,13 +59,20 @@ int32_t* iptr(PyObject* o) { return (int32_t*)ptr(o, at::kInt); }
 
 void* stream() { return (void*)c10::cuda::getCurrentCUDAStream().stream(); }
 
+// A new tensor where `like` is: the library's kernels work on it, so it has to be on a GPU.
+at::Tensor allocate(at::IntArrayRef size, at::ScalarType type, const at::Tensor& like)
+{
+    if (!like.is_cuda()) fail(PyExc_AssertionError, "tensors must be contiguous CUDA tensors");
+    return at::empty(size, like.options().dtype(type));
+}
+
 // An output: the tensor the caller brought, or a new one.
 class Out {
 public:
     Out(PyObject* given, at::IntArrayRef size, at::ScalarType type, const at::Tensor& like, bool checked = true) : given_(given)
     {
         if (given == Py_None) {
-            mine_ = at::empty(size, like.options().dtype(type));
+            mine_ = allocate(size, type, like);
             p_ = mine_.data_ptr();
         } else {
             p_ = checked ? ptr(given, type) : ptr(given);
@@ -88,7 +95,7 @@ public:
         if (given == Py_None) {
             n_ = need > at_least ? need : at_least;
             if (n_ == 0) return;
-            mine_ = at::empty({(int64_t)n_}, like.options().dtype(at::kByte));
+            mine_ = allocate({(int64_t)n_}, at::kByte, like);
             p_ = mine_.data_ptr();
         } else {
             p_ = ptr(given);

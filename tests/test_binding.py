@@ -3,6 +3,10 @@ import os
 import subprocess
 import sys
 
+import pytest
+
+from paper_2510_20787_b200 import lte
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
@@ -30,3 +34,10 @@ print("done")
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0 and r.stdout.strip() == "done", (r.returncode, r.stdout, r.stderr)
+
+
+def test_outputs_are_never_allocated_off_the_gpu():
+    """lte_select_rule is told where to allocate: on the host the library's kernels could not write them."""
+    s = lte.shape(1, 2, 64, 32, 8, 4, lte.F32)
+    with pytest.raises(AssertionError):
+        lte.lte_select_rule(s, lte.RULE_UNIFORM, device="cpu")
