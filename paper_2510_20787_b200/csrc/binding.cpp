@@ -110,12 +110,16 @@ private:
     size_t n_ = 0;
 };
 
-// the C call without the interpreter lock; a status other than LTE_OK becomes an LteError
+struct Unlocked {                                              // the interpreter lock given up for a scope, however that ends
+    PyThreadState* ts = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(ts); }
+};
+// the C call on the current stream, without the interpreter lock (torch is asked for the stream, and may throw, before that); a status
+// other than LTE_OK becomes an LteError
 template <typename F> void call(const char* fn, F&& f)
 {
-    PyThreadState* ts = PyEval_SaveThread();
-    const int status = f();
-    PyEval_RestoreThread(ts);
+    void* const st = stream();
+    const int status = [&] { Unlocked u; return f(st); }();
     if (status == LTE_OK) return;
     if (PyObject* e = PyObject_CallFunction(g_error, "si", fn, status)) {
         PyErr_SetObject(g_error, e);
@@ -155,7 +159,7 @@ LTE_FN(scores, 7)
     Scratch ws(a[6], a[6] == Py_None ? lte_workspace_bytes(LTE_OP_SCORES, s, c) : 0, k);
     const void *kp = ptr(a[2]), *vp = ptr(a[3]);
     float* r = fptr(a[5]);
-    call("lte_scores", [&] { return lte_scores(s, c, kp, vp, z.as<float>(), r, ws.p(), ws.n(), stream()); });
+    call("lte_scores", [&](void* st) { return lte_scores(s, c, kp, vp, z.as<float>(), r, ws.p(), ws.n(), st); });
     return z.result();
 }
 
@@ -169,8 +173,8 @@ LTE_FN(select_rule, 7)
     Out idx(a[3], {s->B, s->H, s->R}, at::kInt, like), cnt(a[4], {s->B, s->H}, at::kInt, like);
     const float* score = fptr(a[2]);
     int32_t* ncand = iptr(a[5]);
-    call(rule == LTE_RULE_LEARNED ? "lte_select" : "lte_select_rule", [&] {
-        return lte_select_rule(s, (int)rule, score, idx.as<int32_t>(), cnt.as<int32_t>(), ncand, nullptr, 0, stream()); });
+    call(rule == LTE_RULE_LEARNED ? "lte_select" : "lte_select_rule", [&](void* st) {
+        return lte_select_rule(s, (int)rule, score, idx.as<int32_t>(), cnt.as<int32_t>(), ncand, nullptr, 0, st); });
     return pack({idx.result(), cnt.result()});
 }
 
@@ -182,7 +186,7 @@ LTE_FN(attn_colsum, 7)
     const void *q = ptr(a[1]), *k = ptr(a[2]);
     const float* lse = fptr(a[3]);
     const int32_t *idx = iptr(a[4]), *cnt = iptr(a[5]);
-    call("lte_attn_colsum", [&] { return lte_attn_colsum(s, q, k, lse, idx, cnt, out.as<float>(), stream()); });
+    call("lte_attn_colsum", [&](void* st) { return lte_attn_colsum(s, q, k, lse, idx, cnt, out.as<float>(), st); });
     return out.result();
 }
 
@@ -195,7 +199,7 @@ LTE_FN(attn_prefill, 9)
     const int32_t *idx = iptr(a[4]), *cnt = iptr(a[5]);
     Out o(a[6], q.sizes(), q.scalar_type(), q, false), lse(a[7], {s->B, heads_q(s), s->T}, at::kFloat, q);
     Scratch ws(a[8], a[8] == Py_None ? lte_workspace_bytes(LTE_OP_PREFILL, s, nullptr) : 0, q);
-    call("lte_attn_prefill", [&] { return lte_attn_prefill(s, qp, k, v, idx, cnt, o.as<void>(), lse.as<float>(), ws.p(), ws.n(), stream()); });
+    call("lte_attn_prefill", [&](void* st) { return lte_attn_prefill(s, qp, k, v, idx, cnt, o.as<void>(), lse.as<float>(), ws.p(), ws.n(), st); });
     return pack({o.result(), lse.result()});
 }
 
@@ -208,7 +212,7 @@ LTE_FN(cache_init, 8)
     const float* z = (const float*)ptr(a[4]);
     const int32_t *idx = (const int32_t*)ptr(a[5]), *cnt = (const int32_t*)ptr(a[6]);
     void* cache = ptr(a[7]);
-    call("lte_cache_init", [&] { return lte_cache_init(s, c, k, v, z, idx, cnt, cache, stream()); });
+    call("lte_cache_init", [&](void* st) { return lte_cache_init(s, c, k, v, z, idx, cnt, cache, st); });
     return Py_NewRef(a[7]);
 }
 
@@ -221,7 +225,7 @@ LTE_FN(attn_decode, 8)
     void* cache = ptr(a[2]);
     const void *q1 = ptr(a[3]), *k1 = ptr(a[4]), *v1 = ptr(a[5]);
     Out o(a[6], q.sizes(), q.scalar_type(), q, false), lse(a[7], {s->B, heads_q(s)}, at::kFloat, q);
-    call("lte_attn_decode", [&] { return lte_attn_decode(s, c, cache, q1, k1, v1, o.as<void>(), lse.as<float>(), stream()); });
+    call("lte_attn_decode", [&](void* st) { return lte_attn_decode(s, c, cache, q1, k1, v1, o.as<void>(), lse.as<float>(), st); });
     return pack({o.result(), lse.result()});
 }
 
@@ -237,8 +241,8 @@ LTE_FN(attn_prefill_chunk, 11)
     const void *qp = ptr(a[4]), *k = ptr(a[5]), *v = ptr(a[6]);
     Out o(a[7], q.sizes(), q.scalar_type(), q, false), lse(a[8], {s->B, heads_q(s), s->T}, at::kFloat, q);
     Scratch ws(a[9], a[9] == Py_None ? lte_workspace_bytes((flags & LTE_CHUNK_STREAMING) ? LTE_OP_CHUNK_STREAM : LTE_OP_CHUNK, s, c) : 0, q, 256);
-    call("lte_attn_prefill_chunk", [&] {
-        return lte_attn_prefill_chunk_ex(s, c, cache, (int32_t)n_past, qp, k, v, o.as<void>(), lse.as<float>(), (uint32_t)flags, ws.p(), ws.n(), stream()); });
+    call("lte_attn_prefill_chunk", [&](void* st) {
+        return lte_attn_prefill_chunk_ex(s, c, cache, (int32_t)n_past, qp, k, v, o.as<void>(), lse.as<float>(), (uint32_t)flags, ws.p(), ws.n(), st); });
     return pack({o.result(), lse.result()});
 }
 
@@ -250,7 +254,7 @@ LTE_FN(sparsity_stats, 4)
     const float *zp = fptr(a[1]), *lam = fptr(a[2]);
     Out count(Py_None, {s->H}, at::kFloat, z), penalty(Py_None, {1}, at::kFloat, z);
     Scratch ws(a[3], a[3] == Py_None ? lte_workspace_bytes(LTE_OP_STATS, s, nullptr) : 0, z, 256);
-    call("lte_sparsity_stats", [&] { return lte_sparsity_stats(s, zp, lam, count.as<float>(), penalty.as<float>(), ws.p(), ws.n(), stream()); });
+    call("lte_sparsity_stats", [&](void* st) { return lte_sparsity_stats(s, zp, lam, count.as<float>(), penalty.as<float>(), ws.p(), ws.n(), st); });
     return pack({count.result(), penalty.result()});
 }
 
@@ -264,7 +268,7 @@ LTE_FN(cache_score, 6)
     const float *co = fptr(a[3]), *si = fptr(a[4]);
     const int32_t len = co ? (int32_t)THPVariable_Unpack(a[3]).size(0) : 0;
     Scratch ws(a[5], a[5] == Py_None ? lte_workspace_bytes(LTE_OP_DECODE, s, c) : 0, like, 256);
-    call(co ? "lte_cache_score_unrope" : "lte_cache_score", [&] { return lte_cache_score_unrope(s, c, cache, co, si, len, ws.p(), ws.n(), stream()); });
+    call(co ? "lte_cache_score_unrope" : "lte_cache_score", [&](void* st) { return lte_cache_score_unrope(s, c, cache, co, si, len, ws.p(), ws.n(), st); });
     Py_RETURN_NONE;
 }
 
@@ -294,14 +298,14 @@ LTE_FN(attn_bwd, 17)
     if (given ? outs[4] != Py_None : want_db) db.reset(new Out(outs[4], {db_size}, at::kFloat, q, false));
     float* dbp = db ? db->as<float>() : nullptr;
     if (a[16] == Py_True) {
-        call("lte_attn_bwd_static", [&] {
+        call("lte_attn_bwd_static", [&](void* st) {
             return lte_attn_bwd_static(s, c, qp, kp, v, o, lse, dO, z, idx, cnt, lam, dq.as<void>(), dk.as<void>(), dv.as<void>(), dw.as<float>(), dbp,
-                                       (uint32_t)flags, stream()); });
+                                       (uint32_t)flags, st); });
     } else {
         Scratch ws(a[14], a[14] == Py_None ? lte_workspace_bytes(LTE_OP_BWD, s, c) : 0, q, 16);
-        call("lte_attn_bwd", [&] {
+        call("lte_attn_bwd", [&](void* st) {
             return lte_attn_bwd(s, c, qp, kp, v, o, lse, dO, z, idx, cnt, lam, dq.as<void>(), dk.as<void>(), dv.as<void>(), dw.as<float>(), dbp,
-                                (uint32_t)flags, ws.p(), ws.n(), stream()); });
+                                (uint32_t)flags, ws.p(), ws.n(), st); });
     }
     return pack({dq.result(), dk.result(), dv.result(), dw.result(), db ? db->result() : Py_NewRef(Py_None)});
 }

@@ -41,3 +41,17 @@ def test_outputs_are_never_allocated_off_the_gpu():
     s = lte.shape(1, 2, 64, 32, 8, 4, lte.F32)
     with pytest.raises(AssertionError):
         lte.lte_select_rule(s, lte.RULE_UNIFORM, device="cpu")
+
+
+def test_an_exception_on_the_way_to_the_library_is_raised():
+    """Without a GPU torch has no current stream and throws; with one the library refuses the missing cache.  Either way Python sees an
+    exception (in a process of its own: thrown without the interpreter lock it ended the process)."""
+    code = """
+from paper_2510_20787_b200 import lte
+try:
+    lte._load().cache_init(lte.shape(1, 2, 0, 32, 5, 2, lte.F32), lte.LteConv(1, 5, 1, 256, 0), None, None, None, None, None, None)
+except RuntimeError:
+    print("done")
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "done", (r.returncode, r.stdout, r.stderr[-500:])
