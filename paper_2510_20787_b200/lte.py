@@ -236,6 +236,8 @@ def lte_cache_score(s, c, cache, ws=None):
 
 def lte_cache_score_unrope(s, c, cache, rope_cos, rope_sin, ws=None):
     """lte_cache_score for a cache that holds rotated keys: rope_cos, rope_sin [positions, d/2] fp32 on the device."""
+    if rope_cos is None or rope_sin is None:
+        raise TypeError("lte_cache_score_unrope needs both rotary tables")
     (_native or _load()).cache_score(s, c, cache, rope_cos, rope_sin, ws)
 
 

@@ -4,6 +4,7 @@ import subprocess
 import sys
 
 import pytest
+import torch
 
 from paper_2510_20787_b200 import lte
 
@@ -55,3 +56,11 @@ except RuntimeError:
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0 and r.stdout.strip() == "done", (r.returncode, r.stdout, r.stderr[-500:])
+
+
+def test_rotary_tables_are_required():
+    """lte_cache_score_unrope without its tables would score rotated keys as they are: lte_cache_score is the call for that."""
+    s, c, x = lte.shape(1, 2, 0, 32, 20, 2, lte.F32), lte.LteConv(3, 3, 2, 256, 0), torch.zeros(4)
+    for tables in ((None, None), (x, None), (None, x)):
+        with pytest.raises(TypeError):
+            lte.lte_cache_score_unrope(s, c, x, *tables)
