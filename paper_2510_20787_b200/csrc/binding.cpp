@@ -86,10 +86,11 @@ private:
     void* p_ = nullptr;
 };
 
-// Scratch: the tensor the caller brought, `need` bytes allocated here for None, nothing for False.
+// Scratch: the tensor the caller brought (its elements count as bytes; `bytes_only`: it has to consist of them), `need` bytes allocated
+// here for None, nothing for False.
 class Scratch {
 public:
-    Scratch(PyObject* given, size_t need, const at::Tensor& like, size_t at_least = 0)
+    Scratch(PyObject* given, size_t need, const at::Tensor& like, size_t at_least = 0, bool bytes_only = false)
     {
         if (given == Py_False) return;
         if (given == Py_None) {
@@ -98,8 +99,8 @@ public:
             mine_ = allocate({(int64_t)n_}, at::kByte, like);
             p_ = mine_.data_ptr();
         } else {
-            p_ = ptr(given);
-            n_ = THPVariable_Unpack(given).nbytes();
+            p_ = bytes_only ? ptr(given, at::kByte) : ptr(given);
+            n_ = (size_t)THPVariable_Unpack(given).numel();
         }
     }
     void* p() const { return p_; }
@@ -156,7 +157,7 @@ LTE_FN(scores, 7)
     const lte_conv* c = c_struct<lte_conv>(a[1]);
     const at::Tensor& k = tensor(a[2]);
     Out z(a[4], {s->B, s->H, s->T}, at::kFloat, k);
-    Scratch ws(a[6], a[6] == Py_None ? lte_workspace_bytes(LTE_OP_SCORES, s, c) : 0, k);
+    Scratch ws(a[6], a[6] == Py_None ? lte_workspace_bytes(LTE_OP_SCORES, s, c) : 0, k, 0, true);
     const void *kp = ptr(a[2]), *vp = ptr(a[3]);
     float* r = fptr(a[5]);
     call("lte_scores", [&](void* st) { return lte_scores(s, c, kp, vp, z.as<float>(), r, ws.p(), ws.n(), st); });
