@@ -27,15 +27,23 @@ def _newer(target, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _built_for(target, tag):
+    with open(target, "rb") as f:
+        return tag.encode() in f.read()
+
+
 def build_binding(force=False, verbose=False):
-    """The CPython module over ``liblte.so``: needs torch's headers and libraries, no CUDA compiler."""
-    src = os.path.join(CSRC, "binding.cpp")
-    if not force and not _newer(BINDING, [src, LIB, os.path.join(INCLUDE, "lte.h")]):
-        return BINDING
+    """The CPython module over ``liblte.so``: needs torch's headers and libraries, no CUDA compiler.  It uses torch's C++ interface, so it
+    carries the versions it was built for (torch's, Python's) as a string and is built again for others."""
     import torch
+    src = os.path.join(CSRC, "binding.cpp")
+    tag = "lte binding for torch %s, %s" % (torch.__version__, sys.implementation.cache_tag)
+    if not force and not _newer(BINDING, [src, LIB, os.path.join(INCLUDE, "lte.h")]) and _built_for(BINDING, tag):
+        return BINDING
     troot = os.path.dirname(torch.__file__)
     tmp = BINDING + ".tmp.%d" % os.getpid()
-    cmd = (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), src, "-o", tmp]
+    cmd = (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            '-DLTE_BUILT_FOR="%s"' % tag, src, "-o", tmp]
            + ["-I" + d for d in (INCLUDE, sysconfig.get_paths()["include"])]
            + ["-isystem" + d for d in (os.path.join(troot, "include"), os.path.join(troot, "include", "torch", "csrc", "api", "include"),
                                        os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"))]

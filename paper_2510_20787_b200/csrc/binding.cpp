@@ -327,4 +327,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__binding()
+{
+    PyObject* m = PyModule_Create(&module);
+    if (m) PyModule_AddStringConstant(m, "built_for", LTE_BUILT_FOR);
+    return m;
+}
