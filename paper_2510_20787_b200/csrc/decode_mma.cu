@@ -134,6 +134,8 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
     float* zc = reinterpret_cast<float*>(blk + L.off_z);
     int32_t* pidx = reinterpret_cast<int32_t*>(blk + L.off_pidx);
     int32_t* meta = reinterpret_cast<int32_t*>(blk + L.off_meta);
+    const bool shared_head = SPLIT > 1 && nsplit > 1;          // (uniform in the cluster)
+    if (shared_head) cluster.barrier_arrive();                 // (awaited before the first store into another block's shared memory)
     pdl_launch_dependents();
     pdl_wait();
 
@@ -335,6 +337,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
             if (2 * t + 1 < nq) *reinterpret_cast<float2*>(&s_acc[wid][2 * t + 1][ch]) = make_float2(acc[i][1], acc[i][3]);
         }
         __syncthreads();
+        if (shared_head && g0 == 0) cluster.barrier_wait();    // every block of the cluster has started: its shared memory is there
         const int per = nq * D / nsplit, par = (g0 / MQ) & 1;  // output elements each block of the cluster finishes
         for (int e = tid; e < nq * D; e += NT) {
             const int u = e / D, ch = e - u * D;
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
                 tot = fmaf(f, s_l[w2][u], tot);
                 o = fmaf(f, s_acc[w2][u][ch], o);
             }
-            if (SPLIT == 1 || nsplit == 1) {
+            if (!shared_head) {
                 o1[((size_t)bh * G + g0 + u) * D + ch] = __float2bfloat16_rn(o / tot);
                 if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m * 0.69314718055994530942f + logf(tot);
             } else {                                           // into the shared memory of the block that finishes this element
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
                 if (ch < nsplit) *reinterpret_cast<float2*>(cluster.map_shared_rank(&s_ml[par][rank][u][0], ch)) = make_float2(m, tot);
             }
         }
-        if (SPLIT > 1 && nsplit > 1) {
+        if (shared_head) {
             cluster.sync();                                    // all shares have arrived, and every row has been read
             for (int e = tid; e < per; e += NT) {
                 const int el = rank * per + e, u = el / D, ch = el - u * D;
