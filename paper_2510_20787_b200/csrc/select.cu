@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2) select_cluster_kernel(cons
     const int N = T - W > 0 ? T - W : 0;
     const int p0 = (rank * NT + tid) * KPT;
     if (tid == 0) s_list[kSelList] = 0u;
+    cluster.barrier_arrive();                              // (awaited before the first access to another block's shared memory)
     SELP(0);
     pdl_launch_dependents();
     pdl_wait();                                            // z comes from the previous kernel
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kClusterThreads, 2) select_cluster_kernel(cons
         for (int i = 0; i < KPT; ++i) key[i] = p0 + i < N ? select_key_from(__ldg(zz + p0 + i), p0 + i, sink, zthr) : 0u;
     }
     SELP(2);
+    cluster.barrier_wait();                                // every block of the cluster has started: its shared memory is there
 
     // Cluster-wide sums of NC per-thread counts; lane k < NC of every warp returns the k-th total.  A row of s_part and a
     // row of s_x are rewritten two calls later, when every warp (every block) has passed the barrier of the call in

@@ -22,7 +22,7 @@ def _kernels():
 KERNELS = {"%s:%s" % (f, name): body for f, name, body in _kernels()}
 
 
-@pytest.mark.parametrize("kernel", ["decode_mma.cu:decode_mma_kernel", "decode.cu:decode_attend_kernel"])
+@pytest.mark.parametrize("kernel", sorted(KERNELS))
 def test_cluster_has_started_before_remote_shared_memory(kernel):
     body = KERNELS[kernel]
     barrier = re.search(r"cluster\.(sync|barrier_wait)\s*\(", body)
