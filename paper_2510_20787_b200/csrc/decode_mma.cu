@@ -9,7 +9,9 @@
 // The products are mma.sync m16n8k16, not tcgen05: N = 8 query heads and 16 rows at a time need no shared memory at all.
 // The contraction index of a product may be permuted freely, so a lane's operand registers are the 16-byte pieces it loaded:
 //   logits   S^T[16 rows][8 queries] = K q^T:  lane (g, t) = (lane / 4, lane % 4) holds pieces t, t + 4, .. of rows g and g + 8
-//            as A and the same pieces of query g as B (products of bf16 values are exact, the scale is applied in fp32 after);
+//            as A and the same pieces of query g as B (products of bf16 values are exact, the scale is applied in fp32 after: to
+//            the distance from the reference, which is held unscaled, so that the largest logit's weight is exact however large
+//            it is and the scale's rounding does not grow with the logits);
 //   output   O^T[16 channels][8 queries] += V^T P^T:  lane (g, t) holds piece g (and g + 8) of rows 2t, 2t+1, 2t+8, 2t+9; a
 //            byte permute pairs two rows' words into A.  P comes out of the logits' registers through movmatrix, split
 //            into two bf16 terms, so that the weights keep 16 bits of mantissa.
@@ -31,7 +33,7 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int MQ = 8;                                          // query heads per pass
-constexpr float M_NONE = -1e30f;                                // a running maximum before the first row (finite: no inf - inf)
+constexpr float M_NONE = -1e30f;                                // a reference before the first row (finite: no inf - inf)
 // Resident warps per SM the registers are budgeted for (128 and 255 a thread), and warps per block at most.
 __host__ __device__ constexpr int warps_per_sm(int d) { return d == 128 ? 8 : 16; }
 __host__ __device__ constexpr int max_warps(int d) { return d == 128 ? 4 : 8; }
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
 
     const int mover = NT - 1 - tid;                            // threads that move rows (not the warps that write the output, where there are several)
     uint4 mv = make_uint4(0, 0, 0, 0), nw = mv;                // a piece of the popped row, of the incoming one
-    const float scale2 = scale * 1.44269504088896340736f;
+    const float scale2 = scale * 1.44269504088896340736f, jump = 8.f / scale2;   // jump: a factor of 2^8 between weights, unscaled
     for (int g0 = 0; g0 < G; g0 += MQ) {
         const int nq = min(MQ, G - g0);
         if (g0 > 0) {                                          // further query heads read the rows again
@@ -287,8 +289,8 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
             }
             // The reference m follows the maximum only when that has grown by 2^8 (weights stay below 2^8, in fp32): a vote per
             // span instead of a reduction over its rows.
-            const float x0 = fmaxf(c[0], c[2]) * scale2, x1 = fmaxf(c[1], c[3]) * scale2;
-            if (__any_sync(0xffffffffu, x0 > m0 + 8.f || x1 > m1 + 8.f)) {
+            const float x0 = fmaxf(c[0], c[2]), x1 = fmaxf(c[1], c[3]);
+            if (__any_sync(0xffffffffu, x0 > m0 + jump || x1 > m1 + jump)) {
                 float y0 = x0, y1 = x1;
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
@@ -296,14 +298,14 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
                     y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
                 }
                 y0 = fmaxf(y0, m0); y1 = fmaxf(y1, m1);
-                const float f0 = exp2_fast(m0 - y0), f1 = exp2_fast(m1 - y1);
+                const float f0 = exp2_fast((m0 - y0) * scale2), f1 = exp2_fast((m1 - y1) * scale2);
                 m0 = y0; m1 = y1;
                 l0 *= f0; l1 *= f1;
 #pragma unroll
                 for (int m = 0; m < MT; ++m) { acc[m][0] *= f0; acc[m][1] *= f1; acc[m][2] *= f0; acc[m][3] *= f1; }
             }
-            const float p0 = exp2_fast(fmaf(c[0], scale2, -m0)), p1 = exp2_fast(fmaf(c[1], scale2, -m1));
-            const float p2 = exp2_fast(fmaf(c[2], scale2, -m0)), p3 = exp2_fast(fmaf(c[3], scale2, -m1));
+            const float p0 = exp2_fast((c[0] - m0) * scale2), p1 = exp2_fast((c[1] - m1) * scale2);
+            const float p2 = exp2_fast((c[2] - m0) * scale2), p3 = exp2_fast((c[3] - m1) * scale2);
             l0 += p0 + p2; l1 += p1 + p3;
             const uint32_t hi0 = pack_bf16(p0, p1), hi1 = pack_bf16(p2, p3);
             const uint32_t lo0 = pack_bf16(p0 - __uint_as_float(hi0 << 16), p1 - __uint_as_float(hi0 & 0xffff0000u));
@@ -347,13 +349,13 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
             float tot = 0.f, o = 0.f;
 #pragma unroll
             for (int w2 = 0; w2 < NW; ++w2) {
-                const float f = exp2_fast(s_m[w2][u] - m);     // a warp without rows: 0
+                const float f = exp2_fast((s_m[w2][u] - m) * scale2);   // a warp without rows: 0
                 tot = fmaf(f, s_l[w2][u], tot);
                 o = fmaf(f, s_acc[w2][u][ch], o);
             }
             if (!shared_head) {
                 o1[((size_t)bh * G + g0 + u) * D + ch] = __float2bfloat16_rn(o / tot);
-                if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m * 0.69314718055994530942f + logf(tot);
+                if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m * scale + logf(tot);
             } else {                                           // into the shared memory of the block that finishes this element
                 const int own = e / per;
                 *cluster.map_shared_rank(&s_in[par][rank * per + (e - own * per)], own) = o;
@@ -373,12 +375,12 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
                 }
 #pragma unroll
                 for (int r2 = 0; r2 < SPLIT; ++r2) {
-                    const float f = exp2_fast(ml[r2].x - m);
+                    const float f = exp2_fast((ml[r2].x - m) * scale2);
                     tot = fmaf(f, ml[r2].y, tot);
                     if (r2 < nsplit) o = fmaf(f, s_in[par][r2 * per + e], o);
                 }
                 o1[((size_t)bh * G + g0 + u) * D + ch] = __float2bfloat16_rn(o / tot);
-                if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m * 0.69314718055994530942f + logf(tot);
+                if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m * scale + logf(tot);
             }
         }
     }

@@ -44,3 +44,34 @@ def test_decode_mma(d, W, R, G, K, sink, T0, steps):
     o64, l64, _, _ = orc.stream(q, rep(x["k"]), rep(x["v"]), rep(z64), W, R, sink, n_from=T0)
     assert np.max(np.abs(o - o64)) <= 2e-2 and np.max(np.abs(lse - l64)) <= 2e-3
     assert lte.lte_device_status() == 0
+
+
+@pytest.mark.parametrize("d,W,R,G", [(32, 20, 12, 1), (64, 300, 80, 1), (64, 100, 99, 4), (128, 250, 70, 9), (128, 768, 256, 1)])
+@pytest.mark.parametrize("size", [30.0, 1e9, 1e18])
+def test_decode_mma_large_logits(d, W, R, G, size):
+    """Logits of about `size`: o and lse stay finite and as close to 64 bits as sums in fp32 of exact products are."""
+    H, T0 = 2, W + 50
+    g = torch.Generator(device="cuda").manual_seed(int(size) % 97 + d)
+    n = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    s, c = lte.shape(1, H, T0, d, W, R, lte.BF16, group=G), lte.conv(n(H, 7, 2 * d) * 1e-3)
+    k, v, q1, k1, v1 = (t.to(torch.bfloat16) for t in (n(1, H, T0, d), n(1, H, T0, d), n(1, H * G, d) * size, n(1, H, d), n(1, H, d)))
+    z = lte.lte_scores(s, c, k, v)
+    idx, cnt = lte.lte_select(s, z)
+    cache = lte.lte_cache_init(s, c, k, v, z, idx, cnt)
+    o, lse = lte.lte_attn_decode(s, c, cache, q1, k1, v1)
+    for h in range(H):
+        # after the step: the window's rows, and what the pool holds (its positions stand behind the logits)
+        e, alloc = 2, 256 if d == 64 and W + R <= 256 else W + R
+        tail = cache[256:].view(H, -1)[h, 2 * alloc * d * e + 4 * (W + R):]
+        pool = tail[:4 * R].view(torch.int32)[:int(tail[4 * R + 4:4 * R + 8].view(torch.int32)[0])].long()
+        kr = torch.cat([k[0, h, pool], k[0, h, T0 - W + 1:], k1[:, h]]).double()
+        vr = torch.cat([v[0, h, pool], v[0, h, T0 - W + 1:], v1[:, h]]).double()
+        qh = q1[0, h * G:(h + 1) * G].double()
+        x = qh @ kr.T / d ** 0.5
+        l64 = torch.logsumexp(x, -1)
+        # fp32 sums of d exact products, the scale, the sum of weights, the logarithm, their sum
+        bound = 2.0 ** -24 * ((d + 2) * (qh.abs() @ kr.abs().T).amax(-1) / d ** 0.5 + 8)
+        assert bool(((lse[0, h * G:(h + 1) * G].double() - l64).abs() <= bound).all())
+        if size > 1e6:                                         # one weight is 1, the others 0
+            assert torch.equal(o[0, h * G:(h + 1) * G].double(), vr[x.argmax(-1)])
+    assert lte.lte_device_status() == 0
