@@ -32,3 +32,20 @@ def test_tiles(B, H, d, T, W, R, ws, growing):
     assert np.max(np.abs(o.float().cpu().numpy() - o64)) <= 2e-2
     assert np.max(np.abs(lse.cpu().numpy() - l64)) <= 2e-3 * max(1.0, float(np.max(np.abs(l64))))
     assert lte.lte_device_status() == 0
+
+
+@pytest.mark.parametrize("d,T,W,R,ws", [(64, 700, 200, 100, None), (64, 700, 200, 100, False), (32, 500, 60, 200, None), (64, 100, 128, 0, None)])
+def test_equal_values_come_out_as_they_are(d, T, W, R, ws):
+    """Where every value row is the same, so is every output: the weights' rounding to bf16 cancels against their sum, whatever the reference
+    of the exponentials is (the rest are sums in fp32, some 1e-6 of the value, which is itself a bf16 number)."""
+    B, H = 2, 3
+    cfg = synth.Config("equal", "bf16", B, H, d, T, W, R, 7, 0.1)
+    s = shape_of(cfg)
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    n = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    q, k = n(B, H, T, d).to(torch.bfloat16), (n(B, H, T, d) * torch.linspace(0.2, 3.0, T, device="cuda")[:, None]).to(torch.bfloat16)
+    v = n(B, H, 1, d).to(torch.bfloat16).expand(B, H, T, d).contiguous()
+    idx, cnt = lte.lte_select(s, n(B, H, T))
+    o, _ = lte.lte_attn_prefill(s, q, k, v, idx, cnt, ws=ws)
+    assert torch.equal(o, v)
+    assert lte.lte_device_status() == 0
