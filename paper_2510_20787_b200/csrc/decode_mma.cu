@@ -79,7 +79,9 @@ template <int D, bool SWZ> struct Group {                      // what a lane ho
     static constexpr int KP = D / 32, VB = D / 16, PITCH = D * 2;   // 16-byte key pieces and 4-byte value words per row
     uint4 k[2][KP];
     uint32_t v[4][VB];
-    // Rows past the end of a span repeat its last row: their weights are zero, their values finite.
+    // Rows past the end of a span repeat its last row with weight zero, and so do the row that leaves and the entry that is replaced
+    // in this step.  (Zero times an infinite value is NaN, but those two have been part of every step up to this one.  Clearing
+    // their values cost 2.5 % of a step with grouped queries.)
     __device__ __forceinline__ void load_k(const Rows& R, const Span& s, int g, int t) {
         const unsigned char* base = s.row >= 0 ? R.K + (size_t)s.row * PITCH : R.k1;
 #pragma unroll
