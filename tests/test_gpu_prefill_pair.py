@@ -50,3 +50,26 @@ def test_chunk_of_many_heads_agrees_with_few():
     (o, lse), (o1, lse1) = run(B), run(1)
     assert lte.lte_device_status() == 0
     assert float((o[:1].float() - o1.float()).abs().max()) <= 2e-2 and float((lse[:1] - lse1).abs().max()) <= 2e-3
+
+
+def test_pair_large_values_and_growing_logits():
+    """Weights are taken relative to a reference that follows the row's maximum within 2^8, so that values of 1e30 do not overflow on the
+    way to outputs of 1e30."""
+    B, H, T, d, W, R = 2, 16, 2500, 128, 300, 64                # 320 pairs of query tiles: two for every SM
+    s = lte.shape(B, H, T, d, W, R, lte.BF16)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    n = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    up = torch.ones(d, device="cuda") * torch.arange(T, device="cuda")[:, None] * 0.02   # q.k / sqrt(d) grows by 0.23 per key
+    q, k, v = torch.ones((B, H, T, d), device="cuda").to(torch.bfloat16), (n(B, H, T, d) * 0.1 + up).to(torch.bfloat16), (n(B, H, T, d) * 1e30).to(torch.bfloat16)
+    idx, cnt = lte.lte_select(s, n(B, H, T))
+    o, lse = lte.lte_attn_prefill(s, q, k, v, idx, cnt)
+    j, i = torch.arange(T, device="cuda")[None], torch.arange(T, device="cuda")[:, None]
+    for b, h in ((0, 0), (1, 15)):
+        sees = (j <= i) & (j > i - W)
+        sees[:, idx[b, h, :int(cnt[b, h])].long()] |= (j <= i - W)[:, idx[b, h, :int(cnt[b, h])].long()]
+        x = (q[b, h].double() @ k[b, h].double().T / d ** 0.5).masked_fill(~sees, -float("inf"))
+        o64 = torch.softmax(x, -1) @ v[b, h].double()
+        # weights rounded to bf16, and o: 2^-9 each
+        assert bool(((o[b, h].double() - o64).abs() <= 2.0 ** -8 * v[b, h].double().abs().max()).all())
+        assert bool(((lse[b, h].double() - torch.logsumexp(x, -1)).abs() <= 2e-3 * x[sees].abs().max()).all())
+    assert lte.lte_device_status() == 0
