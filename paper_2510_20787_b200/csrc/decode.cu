@@ -33,15 +33,15 @@ template <> __device__ __forceinline__ void unpack<float>(const uint4& u, float*
     f[0] = __uint_as_float(u.x); f[1] = __uint_as_float(u.y); f[2] = __uint_as_float(u.z); f[3] = __uint_as_float(u.w);
 }
 
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ cache, CacheLayout L,
-                                                    const T* __restrict__ q1, const T* __restrict__ k1,
-                                                    const T* __restrict__ v1, T* __restrict__ o1,
+                                                    const float* __restrict__ q1, const float* __restrict__ k1,
+                                                    const float* __restrict__ v1, float* __restrict__ o1,
                                                     float* __restrict__ lse1, const float* __restrict__ cw,
                                                     const float* __restrict__ cbias, int H, int W, int R, int sink,
-                                                    int K, float zthr, float scale, int G)
+                                                    int K, float zthr, float scale)
 {
-    constexpr int EPV = V16<T>::N;            // elements per 16-byte vector
+    constexpr int EPV = 4;                    // elements per 16-byte vector
     constexpr int LPR = D / EPV;              // lanes per row
     constexpr int RPP = DT / LPR;             // rows per pass of the whole block
     __shared__ float s_log[MAX_ROWS + 1];
@@ -66,8 +66,8 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
     // query segment of this thread (pre-scaled)
     float qf[EPV];
     {
-        uint4 u = *reinterpret_cast<const uint4*>(q1 + (size_t)bh * G * D + seg * EPV);
-        unpack<T>(u, qf);
+        uint4 u = *reinterpret_cast<const uint4*>(q1 + (size_t)bh * D + seg * EPV);
+        unpack<float>(u, qf);
 #pragma unroll
         for (int e = 0; e < EPV; ++e) qf[e] *= scale;
     }
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
         for (int c = 0; c < NCH; ++c) {
             const int row = r0 + c * RPP + rsub;
             float kf[EPV];
-            unpack<T>(kreg[c], kf);
+            unpack<float>(kreg[c], kf);
             float s = 0.f;
 #pragma unroll
             for (int e = 0; e < EPV; ++e) s = fmaf(qf[e], kf[e], s);
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
     // logit of the incoming token (row index `rows`)
     if (wid == 1) {
         float s = 0.f;
-        for (int c = lane; c < D; c += 32) s = fmaf(to_f(q1[(size_t)bh * G * D + c]) * scale, to_f(k1[(size_t)bh * D + c]), s);
+        for (int c = lane; c < D; c += 32) s = fmaf(q1[(size_t)bh * D + c] * scale, k1[(size_t)bh * D + c], s);
         s = warp_sum(s);
         if (lane == 0) s_log[rows] = s;
     }
@@ -163,11 +163,11 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
                 const float* wt = cw + ((size_t)h * K + t) * 2 * D;
                 if (pos == n) {
                     for (int c = lane; c < D; c += 32)
-                        a += wt[c] * to_f(k1[(size_t)bh * D + c]) + wt[D + c] * to_f(v1[(size_t)bh * D + c]);
+                        a += wt[c] * k1[(size_t)bh * D + c] + wt[D + c] * v1[(size_t)bh * D + c];
                 } else {
-                    const T* kr = reinterpret_cast<const T*>(blk + L.off_k) + (size_t)(pos % W) * D;
-                    const T* vr = reinterpret_cast<const T*>(blk + L.off_v) + (size_t)(pos % W) * D;
-                    for (int c = lane; c < D; c += 32) a += wt[c] * to_f(kr[c]) + wt[D + c] * to_f(vr[c]);
+                    const float* kr = reinterpret_cast<const float*>(blk + L.off_k) + (size_t)(pos % W) * D;
+                    const float* vr = reinterpret_cast<const float*>(blk + L.off_v) + (size_t)(pos % W) * D;
+                    for (int c = lane; c < D; c += 32) a += wt[c] * kr[c] + wt[D + c] * vr[c];
                 }
             }
             a = warp_sum(a);
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
             const float pr = row < rows ? s_log[row] : 0.f;
             if (pr != 0.f) {
                 float vf[EPV];
-                unpack<T>(vreg[c], vf);
+                unpack<float>(vreg[c], vf);
 #pragma unroll
                 for (int e = 0; e < EPV; ++e) acc[e] = fmaf(pr, vf[e], acc[e]);
             }
@@ -252,10 +252,10 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
         float o = 0.f;
 #pragma unroll
         for (int w2 = 0; w2 < DT / 32; ++w2) o += s_red[w2][tid];
-        o = fmaf(s_log[rows], to_f(v1[(size_t)bh * D + tid]), o);
-        o1[(size_t)bh * G * D + tid] = from_f<T>(o * inv);
+        o = fmaf(s_log[rows], v1[(size_t)bh * D + tid], o);
+        o1[(size_t)bh * D + tid] = o * inv;
     }
-    if (tid == 0) lse1[(size_t)bh * G] = mx + logf(sum);
+    if (tid == 0) lse1[bh] = mx + logf(sum);
 
     // ---- write-back ---------------------------------------------------------------------------
     uint4* Kw = reinterpret_cast<uint4*>(blk + L.off_k);
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(DT) decode_kernel(unsigned char* __restrict__ 
     if (dst >= 0 && tid < 2 * LPR) (tid < LPR ? Kw : Vw)[(size_t)(W + dst) * LPR + (tid % LPR)] = mv;
     if (tid >= 64 && tid < 64 + 2 * LPR) {
         const int t2 = tid - 64;
-        const T* src = (t2 < LPR ? k1 : v1) + (size_t)bh * D + (t2 % LPR) * EPV;
+        const float* src = (t2 < LPR ? k1 : v1) + (size_t)bh * D + (t2 % LPR) * EPV;
         (t2 < LPR ? Kw : Vw)[(size_t)slot * LPR + (t2 % LPR)] = *reinterpret_cast<const uint4*>(src);
     }
     if (tid == 0) {
@@ -328,15 +328,15 @@ __host__ __device__ inline BulkSmem bulk_smem_plan(const CacheLayout& L, int W, 
     return b;
 }
 
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restrict__ cache, CacheLayout L,
-                                                         const T* __restrict__ q1, const T* __restrict__ k1,
-                                                         const T* __restrict__ v1, T* __restrict__ o1,
+                                                         const float* __restrict__ q1, const float* __restrict__ k1,
+                                                         const float* __restrict__ v1, float* __restrict__ o1,
                                                          float* __restrict__ lse1, const float* __restrict__ cw,
                                                          const float* __restrict__ cbias, int BH, int per_cta, int H,
-                                                         int W, int R, int sink, int K, float zthr, float scale, int G)
+                                                         int W, int R, int sink, int K, float zthr, float scale)
 {
-    constexpr int EPV = V16<T>::N;
+    constexpr int EPV = 4;
     constexpr int LPR = D / EPV;
     constexpr int RPP = DT / LPR;
     constexpr int CPL = D / 32;                // channels per lane in the warp-per-row pieces
@@ -378,13 +378,13 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
     uint4 kv_new = make_uint4(0, 0, 0, 0);
     auto fetch_inputs = [&](int bh) {
         const int h = bh % H;
-        uint4 u = *reinterpret_cast<const uint4*>(q1 + (size_t)bh * G * D + seg * EPV);
-        unpack<T>(u, qf);
+        uint4 u = *reinterpret_cast<const uint4*>(q1 + (size_t)bh * D + seg * EPV);
+        unpack<float>(u, qf);
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
-            k1f[c] = to_f(k1[(size_t)bh * D + lane + 32 * c]);
-            v1f[c] = to_f(v1[(size_t)bh * D + lane + 32 * c]);
-            q1f[c] = to_f(q1[(size_t)bh * G * D + lane + 32 * c]);
+            k1f[c] = k1[(size_t)bh * D + lane + 32 * c];
+            v1f[c] = v1[(size_t)bh * D + lane + 32 * c];
+            q1f[c] = q1[(size_t)bh * D + lane + 32 * c];
         }
 #pragma unroll
         for (int u2 = 0; u2 < 2; ++u2) {
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
             }
         }
         bias = cbias ? cbias[h] : 0.f;
-        if (tid < D) v1_mine = to_f(v1[(size_t)bh * D + tid]);
+        if (tid < D) v1_mine = v1[(size_t)bh * D + tid];
         if (tid >= 64 && tid < 64 + 2 * LPR) {
             const int t2 = tid - 64;
             kv_new = *reinterpret_cast<const uint4*>((t2 < LPR ? k1 : v1) + (size_t)bh * D + (t2 % LPR) * EPV);
@@ -471,10 +471,10 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
 #pragma unroll
                     for (int c = 0; c < CPL; ++c) a += wk[u][c] * k1f[c] + wv[u][c] * v1f[c];
                 } else if (pos >= 0) {
-                    const T* kr = reinterpret_cast<const T*>(dsm) + (size_t)(pos % W) * D;
-                    const T* vr = reinterpret_cast<const T*>(dsm + P.off_v) + (size_t)(pos % W) * D;
+                    const float* kr = reinterpret_cast<const float*>(dsm) + (size_t)(pos % W) * D;
+                    const float* vr = reinterpret_cast<const float*>(dsm + P.off_v) + (size_t)(pos % W) * D;
 #pragma unroll
-                    for (int c = 0; c < CPL; ++c) a += wk[u][c] * to_f(kr[lane + 32 * c]) + wv[u][c] * to_f(vr[lane + 32 * c]);
+                    for (int c = 0; c < CPL; ++c) a += wk[u][c] * kr[lane + 32 * c] + wv[u][c] * vr[lane + 32 * c];
                 }
                 a = warp_sum(a);
                 if (lane == 0) s_tap[t] = a;
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
                 float s0 = 0.f, s1 = 0.f;
                 if (row < rows) {
                     float kf[EPV];
-                    unpack<T>(Kc[(size_t)row * LPR + seg], kf);
+                    unpack<float>(Kc[(size_t)row * LPR + seg], kf);
 #pragma unroll
                     for (int e = 0; e < EPV; e += 2) { s0 = fmaf(qf[e], kf[e], s0); s1 = fmaf(qf[e + 1], kf[e + 1], s1); }
                 }
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
                     const float pr = __expf(s_log[row] - mx);   // exp(-inf) = 0 for masked rows
                     if (pr != 0.f) {
                         float vf[EPV];
-                        unpack<T>(Vc[(size_t)row * LPR + seg], vf);
+                        unpack<float>(Vc[(size_t)row * LPR + seg], vf);
 #pragma unroll
                         for (int e = 0; e < EPV; ++e) acc[e] = fmaf(pr, vf[e], acc[e]);
                         if (seg == 0) lsum += pr;
@@ -586,9 +586,9 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
 #pragma unroll
             for (int w2 = 0; w2 < DT / 32; ++w2) o += s_red[w2][tid];
             o = fmaf(p_new, v1_mine, o);
-            o1[(size_t)bh * G * D + tid] = from_f<T>(o / sum);
+            o1[(size_t)bh * D + tid] = o / sum;
         }
-        if (tid == 0) lse1[(size_t)bh * G] = mx + logf(sum);
+        if (tid == 0) lse1[bh] = mx + logf(sum);
 
         // ---- write-back: only what changed goes to HBM -----------------------------------------------------
         uint4* Kw = reinterpret_cast<uint4*>(gblk + L.off_k);
@@ -827,20 +827,20 @@ int launch_ring_scatter_z(const Params& p, void* cache, const float* zlin, cudaS
 // then serves all G query heads over the updated block (the attend kernel below).
 // The update of one key/value head's block by the DTU threads of a thread block (every thread of the block calls it; it
 // ends with the block's writes issued, not yet ordered: the caller synchronises).
-template <typename T, int D, int DTU>
+template <int D, int DTU>
 __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ cache, const CacheLayout& L, int bh,
-                                                   const T* __restrict__ k1, const T* __restrict__ v1,
+                                                   const float* __restrict__ k1, const float* __restrict__ v1,
                                                    const float* __restrict__ cw, const float* __restrict__ cbias, int H,
                                                    int W, int R, int sink, int K, float zthr)
 {
-    constexpr int CPL = D / 32, NWU = DTU / 32, PIECES = D * (int)sizeof(T) / 16;
+    constexpr int CPL = D / 32, NWU = DTU / 32, PIECES = D / 4;
     __shared__ float s_tap[kMaxTaps];
     __shared__ float s_wz[NWU];
     __shared__ int s_wpos[NWU], s_wslot[NWU];
     const int h = bh % H, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
-    T* Kc = reinterpret_cast<T*>(blk + L.off_k);
-    T* Vc = reinterpret_cast<T*>(blk + L.off_v);
+    float* Kc = reinterpret_cast<float*>(blk + L.off_k);
+    float* Vc = reinterpret_cast<float*>(blk + L.off_v);
     float* zc = reinterpret_cast<float*>(blk + L.off_z);
     int32_t* pidx = reinterpret_cast<int32_t*>(blk + L.off_pidx);
     int32_t* meta = reinterpret_cast<int32_t*>(blk + L.off_meta);
@@ -894,8 +894,8 @@ __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ c
                     const int ch = lane + 32 * c;
                     const float wk = cw[((size_t)h * K + t) * 2 * D + ch], wv = cw[((size_t)h * K + t) * 2 * D + D + ch];
                     float kx, vx;
-                    if (pos == n) { kx = to_f(k1[(size_t)bh * D + ch]); vx = to_f(v1[(size_t)bh * D + ch]); }
-                    else { const int r = pos % W; kx = to_f(Kc[(size_t)r * D + ch]); vx = to_f(Vc[(size_t)r * D + ch]); }
+                    if (pos == n) { kx = k1[(size_t)bh * D + ch]; vx = v1[(size_t)bh * D + ch]; }
+                    else { const int r = pos % W; kx = Kc[(size_t)r * D + ch]; vx = Vc[(size_t)r * D + ch]; }
                     a += wk * kx + wv * vx;
                 }
             }
@@ -932,22 +932,22 @@ __device__ __forceinline__ void cache_update_block(unsigned char* __restrict__ c
     }
 }
 
-// The attend kernel: query heads g_first .. G-1 of a key/value head over its block (ring rows of the min(n, W) newest
+// The attend kernel: the G query heads of a key/value head over its block (ring rows of the min(n, W) newest
 // tokens, cnt pool rows), after the update.  One block (or a cluster of blocks) per key/value head, up to ATT_Q query heads
 // per pass.  Rows are spread as in the step kernels: LPR lanes share a row, each with one 16-byte piece of it, so a warp's
 // load covers whole consecutive rows; eight rows per thread are in flight.  Logits: partial dots per lane against the
 // lane's slice of every query, reduced over the LPR lanes by shuffles; block maxima and sums per query head; value rows
 // the same way, weighted per query head in registers, reduced over lanes sharing a slice and then over the warps.
 constexpr int ATT_Q = 4;
-template <typename T, int D>
+template <int D>
 __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __restrict__ cache, CacheLayout L,
-                                                           const T* __restrict__ q1, T* __restrict__ o1,
-                                                           float* __restrict__ lse1, int W, int G, float scale, int g_first,
-                                                           const T* __restrict__ k1, const T* __restrict__ v1,
+                                                           const float* __restrict__ q1, float* __restrict__ o1,
+                                                           float* __restrict__ lse1, int W, int G, float scale,
+                                                           const float* __restrict__ k1, const float* __restrict__ v1,
                                                            const float* __restrict__ cw, const float* __restrict__ cbias, int H,
                                                            int R, int sink, int K, float zthr)
 {
-    constexpr int EPV = V16<T>::N;                             // elements per 16-byte piece
+    constexpr int EPV = 4;                                     // elements per 16-byte piece
     constexpr int LPR = D / EPV;                               // lanes per row
     constexpr int RPP = DT / LPR;                              // rows per pass of the block
     constexpr int NW = DT / 32, UNR = 8;
@@ -961,15 +961,12 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
     const int nsplit = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int bh = blockIdx.x / nsplit, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int seg = tid % LPR, rsub = tid / LPR;
-    // the step's cache update first (k1 != NULL), by the head's (first) block: a handful of rows, then everybody reads the
-    // updated block
-    if (k1 != nullptr) {
-        if (rank == 0) {
-            cache_update_block<T, D, DT>(cache, L, bh, k1, v1, cw, cbias, H, W, R, sink, K, zthr);
-            __threadfence();
-        }
-        if (nsplit > 1) cluster.sync(); else __syncthreads();
+    // the step's cache update first, by the head's (first) block: a handful of rows, then everybody reads the updated block
+    if (rank == 0) {
+        cache_update_block<D, DT>(cache, L, bh, k1, v1, cw, cbias, H, W, R, sink, K, zthr);
+        __threadfence();
     }
+    if (nsplit > 1) cluster.sync(); else __syncthreads();
     const unsigned char* blk = cache + L.header + (size_t)bh * L.stride;
     const uint4* Kc = reinterpret_cast<const uint4*>(blk + L.off_k);
     const uint4* Vc = reinterpret_cast<const uint4*>(blk + L.off_v);
@@ -985,14 +982,14 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
         const int r = a_lo + a < n_ring ? a_lo + a : W + (a_lo + a - n_ring);
         return (size_t)r * LPR + seg;
     };
-    for (int g0 = g_first; g0 < G; g0 += ATT_Q) {
+    for (int g0 = 0; g0 < G; g0 += ATT_Q) {
         const int nq = G - g0 < ATT_Q ? G - g0 : ATT_Q;
         float qv[ATT_Q][EPV];                                  // this lane's slice of the pass's queries, pre-scaled
 #pragma unroll
         for (int u = 0; u < ATT_Q; ++u)
 #pragma unroll
             for (int e = 0; e < EPV; ++e)
-                qv[u][e] = u < nq ? to_f(q1[((size_t)bh * G + g0 + u) * D + seg * EPV + e]) * scale : 0.f;
+                qv[u][e] = u < nq ? q1[((size_t)bh * G + g0 + u) * D + seg * EPV + e] * scale : 0.f;
         // ---- logits ----
         float mx[ATT_Q];
 #pragma unroll
@@ -1008,7 +1005,7 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
 #pragma unroll
             for (int j = 0; j < UNR; ++j) {
                 float kf[EPV];
-                unpack<T>(raw[j], kf);
+                unpack<float>(raw[j], kf);
 #pragma unroll
                 for (int u = 0; u < ATT_Q; ++u) {
                     float s0 = 0.f, s1 = 0.f;
@@ -1086,7 +1083,7 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
             for (int j = 0; j < UNR; ++j) {
                 const int a = min(a0 + j * RPP + rsub, rows - 1);   // (rows past the end carry zero values)
                 float vf[EPV];
-                unpack<T>(raw[j], vf);
+                unpack<float>(raw[j], vf);
 #pragma unroll
                 for (int u = 0; u < ATT_Q; ++u) {
                     const float pj = s_log[(size_t)u * rows + a];
@@ -1127,7 +1124,7 @@ __global__ void __launch_bounds__(DT) decode_attend_kernel(unsigned char* __rest
                     tot = fmaf(f, *cluster.map_shared_rank(&s_sum[u], r2), tot);
                     acc2 = fmaf(f, *cluster.map_shared_rank(&s_fin[u][ch], r2), acc2);
                 }
-                o1[((size_t)bh * G + g0 + u) * D + ch] = from_f<T>(acc2 / tot);
+                o1[((size_t)bh * G + g0 + u) * D + ch] = acc2 / tot;
                 if (ch == 0) lse1[(size_t)bh * G + g0 + u] = m + logf(tot);
             }
         }
@@ -1148,33 +1145,33 @@ static int launch_decode_step(const Params& p, void* cache, const void* q1, cons
     const int BH = p.B * p.H;
     const int per_cta = bulk ? (BH + 3 * n_sm - 1) / (3 * n_sm) : 1;
     const int n_cta = bulk ? (BH + per_cta - 1) / per_cta : BH;
-#define LTE_BULK(T, D)                                                                                            \
-    do {                                                                                                          \
-        static PerDeviceOnce attr;                                                                                \
-        if (int e = attr.run([] { return cudaFuncSetAttribute(decode_bulk_kernel<T, D>,                           \
-                cudaFuncAttributeMaxDynamicSharedMemorySize, 73 * 1024); })) return e;                            \
-        decode_bulk_kernel<T, D><<<n_cta, DT, bulk_smem, st>>>((unsigned char*)cache, L, (const T*)q1,             \
-            (const T*)k1, (const T*)v1, (T*)o1, lse1, p.w, p.bias, BH, per_cta, p.H, p.W, p.R, p.sink, p.K,        \
-            p.zthr, p.scale, p.G);                                                                                     \
+#define LTE_BULK(D)                                                                                                   \
+    do {                                                                                                              \
+        static PerDeviceOnce attr;                                                                                    \
+        if (int e = attr.run([] { return cudaFuncSetAttribute(decode_bulk_kernel<D>,                                  \
+                cudaFuncAttributeMaxDynamicSharedMemorySize, 73 * 1024); })) return e;                                \
+        decode_bulk_kernel<D><<<n_cta, DT, bulk_smem, st>>>((unsigned char*)cache, L, (const float*)q1,               \
+            (const float*)k1, (const float*)v1, (float*)o1, lse1, p.w, p.bias, BH, per_cta, p.H, p.W, p.R, p.sink, p.K,\
+            p.zthr, p.scale);                                                                                         \
     } while (0)
     if (bulk) {
         switch (p.d) {
-            case 32: LTE_BULK(float, 32); break;
-            case 64: LTE_BULK(float, 64); break;
-            case 128: LTE_BULK(float, 128); break;
+            case 32: LTE_BULK(32); break;
+            case 64: LTE_BULK(64); break;
+            case 128: LTE_BULK(128); break;
             default: return LTE_ERR_UNSUPPORTED;
         }
         return cuda_status(cudaGetLastError());
     }
 #undef LTE_BULK
-#define LTE_GO(T, D)                                                                                              \
-    decode_kernel<T, D><<<p.B * p.H, DT, 0, st>>>((unsigned char*)cache, L, (const T*)q1, (const T*)k1, (const T*)v1, \
-                                                  (T*)o1, lse1, p.w, p.bias, p.H, p.W, p.R, p.sink, p.K, p.zthr,   \
-                                                  p.scale, p.G)
+#define LTE_GO(D)                                                                                                     \
+    decode_kernel<D><<<p.B * p.H, DT, 0, st>>>((unsigned char*)cache, L, (const float*)q1, (const float*)k1, (const float*)v1,\
+                                                  (float*)o1, lse1, p.w, p.bias, p.H, p.W, p.R, p.sink, p.K, p.zthr,  \
+                                                  p.scale)
     switch (p.d) {
-        case 32: LTE_GO(float, 32); break;
-        case 64: LTE_GO(float, 64); break;
-        case 128: LTE_GO(float, 128); break;
+        case 32: LTE_GO(32); break;
+        case 64: LTE_GO(64); break;
+        case 128: LTE_GO(128); break;
         default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_GO
@@ -1209,19 +1206,19 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
     aattr[0].id = cudaLaunchAttributeClusterDimension;
     aattr[0].val.clusterDim.x = nsplit; aattr[0].val.clusterDim.y = 1; aattr[0].val.clusterDim.z = 1;
     acfg.attrs = aattr; acfg.numAttrs = 1;
-#define LTE_ATT(T, D)                                                                                                  \
-    do {                                                                                                               \
-        static PerDeviceOnce attr;                                                                                     \
-        if (int e = attr.run([] { return cudaFuncSetAttribute(decode_attend_kernel<T, D>,                              \
-                cudaFuncAttributeMaxDynamicSharedMemorySize,                                                           \
-                (int)(sizeof(float) * ((size_t)ATT_Q * MAX_ROWS + (DT / 32) * ATT_Q * 128))); })) return e;            \
-        return cuda_status(cudaLaunchKernelEx(&acfg, decode_attend_kernel<T, D>, (unsigned char*)cache, L, (const T*)q1, (T*)o1, lse1, \
-                               p.W, p.G, p.scale, 0, (const T*)k1, (const T*)v1, p.w, p.bias, p.H, p.R, p.sink, ps.K, p.zthr)); \
+#define LTE_ATT(D)                                                                                                    \
+    do {                                                                                                              \
+        static PerDeviceOnce attr;                                                                                    \
+        if (int e = attr.run([] { return cudaFuncSetAttribute(decode_attend_kernel<D>,                                \
+                cudaFuncAttributeMaxDynamicSharedMemorySize,                                                          \
+                (int)(sizeof(float) * ((size_t)ATT_Q * MAX_ROWS + (DT / 32) * ATT_Q * 128))); })) return e;           \
+        return cuda_status(cudaLaunchKernelEx(&acfg, decode_attend_kernel<D>, (unsigned char*)cache, L, (const float*)q1, (float*)o1, lse1,\
+                               p.W, p.G, p.scale, (const float*)k1, (const float*)v1, p.w, p.bias, p.H, p.R, p.sink, ps.K, p.zthr));\
     } while (0)
     switch (p.d) {
-        case 32: LTE_ATT(float, 32);
-        case 64: LTE_ATT(float, 64);
-        case 128: LTE_ATT(float, 128);
+        case 32: LTE_ATT(32);
+        case 64: LTE_ATT(64);
+        case 128: LTE_ATT(128);
         default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_ATT

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                                                          __nv_bfloat16* __restrict__ o1, float* __restrict__ lse1,
                                                          const float* __restrict__ cw, const float* __restrict__ cbias,
                                                          int BH, int H, int W, int R, int sink, int K,
-                                                         float zthr, float scale, int G)
+                                                         float zthr, float scale)
 {
     extern __shared__ __align__(1024) unsigned char dsm[];
     constexpr int NW = NC / 32, NTHR = kThreads<NC>, TAPS = (kMaxTaps + NW - 1) / NW;
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
         auto pair = [&](const __nv_bfloat16* x) { return load32(x + 2 * lane); };
         auto fetch_inputs = [&](int bh) {
             const int h = bh % H;
-            k1r = pair(k1 + (size_t)bh * D); v1r = pair(v1 + (size_t)bh * D); q1r = pair(q1 + (size_t)bh * G * D);
+            k1r = pair(k1 + (size_t)bh * D); v1r = pair(v1 + (size_t)bh * D); q1r = pair(q1 + (size_t)bh * D);
 #pragma unroll
             for (int u = 0; u < TAPS; ++u) {
                 const float* w = cw + ((size_t)h * K + wid + u * NW) * 2 * D + 2 * lane;   // (4-byte aligned)
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
             }
             if (cbias) bias = load32(cbias + h);
             if (tid < D) v1_pair = load32(v1 + (size_t)bh * D + (tid & ~1));
-            if (tid < 8) q_chunk = load128(q1 + (size_t)bh * G * D + tid * 8);
+            if (tid < 8) q_chunk = load128(q1 + (size_t)bh * D + tid * 8);
             if (tid >= 64 && tid < 80) {
                 const int t2 = tid - 64;
                 kv_new = load128((t2 < 8 ? k1 : v1) + (size_t)bh * D + (t2 & 7) * 8);
@@ -317,9 +317,9 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
             tc_fence_before();
             if (tid < D) {
                 const float o = o_mine + p_new * v_now;
-                o1[(size_t)bh * G * D + tid] = __float2bfloat16_rn(o / sum);
+                o1[(size_t)bh * D + tid] = __float2bfloat16_rn(o / sum);
             }
-            if (tid == 0) lse1[(size_t)bh * G] = mx + logf(sum);
+            if (tid == 0) lse1[bh] = mx + logf(sum);
 
             // ---- write-back: only what changed goes to HBM (rows are stored swizzled) ----------------------------
             uint4* Kw = reinterpret_cast<uint4*>(gblk + L.off_k);
@@ -362,7 +362,7 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
                      cudaStream_t st)
 {
     const CacheLayout L = cache_layout(p.d, p.W, p.R, p.dtype);
-    if (!L.swz || p.K > 16) return LTE_ERR_UNSUPPORTED;
+    if (!L.swz || p.G > 1) return LTE_ERR_UNSUPPORTED;
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
     const int BH = p.B * p.H;
@@ -377,7 +377,7 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
         const int n_cta = BH < slots ? BH : slots;
         return cuda_status(launch_pdl(kern, dim3(n_cta), dim3(kThreads<NC>), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
                                       (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, BH, p.H, p.W, p.R,
-                                      p.sink, p.K, p.zthr, p.scale, p.G));
+                                      p.sink, p.K, p.zthr, p.scale));
     };
     static PerDeviceOnce attr256, attr128;
     if (p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256>, attr256);

@@ -1,7 +1,6 @@
-// Prefill attention on the 5th-generation tensor cores (Section 3.1.3), variant for long items: one CTA per
-// 128-query tile of one (b,h), used at d = 128, where a tile walks ten and more key tiles and the hardware's block
-// scheduler balances the load better than a static persistent schedule (and the registers a persistent loop
-// keeps alive are not free).  The tile loop is the one of the persistent kernel:
+// Prefill attention at d = 128 on the 5th-generation tensor cores (Section 3.1.3): one CTA per 128-query tile of one (b,h), for calls that
+// do not fill the chip with pairs of such tiles (prefill_tc_pair.cu; the line is in launch_prefill_tc_long), that bring no workspace, and
+// for the streaming reading of a chunk.
 //   S = Q K^T      tcgen05.mma (kind::f16, bf16 in, fp32 out) into one of two TMEM buffers
 //   softmax        thread r owns query row r = TMEM lane r; P written as bf16 back into TMEM over its S buffer
 //   O += P V       tcgen05.mma with P as the TMEM A operand and V as an MN-major shared-memory operand; lazy rescale
@@ -31,32 +30,26 @@ __device__ unsigned long long g_plprof[64];
 
 namespace {
 
-constexpr int BM = 128, BN = 64, NTHREADS = 192;
+constexpr int D = 128, BM = 128, BN = 64, NTHREADS = 192;
 using namespace tc;
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_prefill_long_status); }
 
-template <int D> struct Smem {
+struct Smem {
     static constexpr int SUB = D / 64;                        // 64-column (128-byte) sub-tiles per row
     static constexpr int KST = 3;                             // key stages
-    static constexpr int VST = D == 64 ? 3 : 2;               // value stages
+    static constexpr int VST = 2;                             // value stages
     static constexpr int QTILE = BM * D * 2;                  // [128][D] bf16
     static constexpr int KVTILE = BN * D * 2;                 // [64][D] bf16
     static constexpr int OFF_Q = 0;
     static constexpr int OFF_K = QTILE;
     static constexpr int OFF_V = OFF_K + KST * KVTILE;
-    static constexpr int OFF_P = OFF_V + VST * KVTILE;        // (P lives in TMEM; nothing here)
-    // d = 64: the row sums are taken by the tensor core as well: PV gets 16 extra B columns of ones, so column D of
-    // the accumulator is sum_j P_ij of exactly the (bf16-rounded) probabilities the product used.  The ones live in one
-    // more 64-column group, LBO away from the value tile.
-    static constexpr bool ONES = D == 64;
-    static constexpr int OFF_ONES = OFF_P;                    // [64][64] bf16 ones (8 KB), d = 64 only
-    static constexpr int OFF_BAR = OFF_ONES + (ONES ? BN * 128 : 0);   // mbarriers, tmem slot
+    static constexpr int OFF_BAR = OFF_V + VST * KVTILE;      // mbarriers, tmem slot (P lives in TMEM)
 #ifdef LTE_PROFILE
     static constexpr int BYTES = OFF_BAR + 768;
 #else
     static constexpr int BYTES = OFF_BAR + 256;
 #endif
-    static constexpr uint32_t TMEM_COLS = 256;                // S0: [0,64)  S1: [64,128)  O: [128, 128+D) (+16 row-sum columns)
+    static constexpr uint32_t TMEM_COLS = 256;                // S0: [0,64)  S1: [64,128)  O: [128, 256)
 };
 
 
@@ -74,7 +67,7 @@ template <int D> struct Smem {
 // S(t+1) and S(t+2) are computed while the softmax of tile t runs; loads run two to three tiles ahead.
 // STREAM (with compact): the list is every entry retained at some query of a chunk and entry e is gone from query leave[e] on
 // (the streaming reading of a chunk): retained tiles take one more mask, leave > query position.
-template <int D, bool compact, bool STREAM>
+template <bool compact, bool STREAM>
 __global__ void __launch_bounds__(NTHREADS, 2)
 prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
@@ -84,7 +77,7 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                   const int32_t* __restrict__ cnt, const int32_t* __restrict__ leave, __nv_bfloat16* __restrict__ o,
                   float* __restrict__ lse, int Tlen, int W, int R, float scale, int G, int qoff)
 {
-    using S = Smem<D>;
+    using S = Smem;
     constexpr int SUB = S::SUB, KST = S::KST, VST = S::VST;
     constexpr uint32_t TMEM_COLS = S::TMEM_COLS;
     constexpr uint32_t O_COL = 2 * BN;
@@ -141,7 +134,7 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     pdl_launch_dependents();
     pdl_wait();                                                // everything above ran beside the previous kernel's tail
     // Q and the first window tiles need nothing but the tile's coordinates: they are on their way before the list is looked at
-    const int n_early = min(n_win, Smem<D>::VST);
+    const int n_early = min(n_win, Smem::VST);
     if (warp == 5 && lane == 0) {
         mbar_expect_tx(bar_q, S::QTILE);
 #pragma unroll
@@ -214,17 +207,16 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             //      walks the loop and waits; only the tcgen05 instructions are guarded by the lane test, so that addresses
             //      and descriptors are computed in convergent code (cheaper to issue than from a loop run by one lane).
             constexpr uint32_t IDESC_S = instr_desc(BM, BN, false);
-            constexpr uint32_t IDESC_O = S::ONES ? instr_desc(BM, D + 16, true) : instr_desc(BM, D, true);
+            constexpr uint32_t IDESC_O = instr_desc(BM, D, true);
             // descriptor words: lo = (address >> 4) | LBO field, hi = SBO field | version | swizzle mode
             constexpr uint32_t HI = (1024u >> 4) | (1u << 14) | (2u << 29);
             const uint32_t q_lo = (sQ >> 4) | (1u << 16), k_lo = (sK >> 4) | (1u << 16);
-            // value operand: the second 64-column group of B is the next sub-tile (d = 128) or the block of ones
-            // (d = 64, LBO = its distance from the value stage)
+            // value operand: the second 64-column group of B is the next sub-tile
             uint32_t v_desc[VST];
 #pragma unroll
             for (int st = 0; st < VST; ++st) {
                 const uint32_t va = sV + st * S::KVTILE;
-                v_desc[st] = (va >> 4) | ((S::ONES ? ((base + S::OFF_ONES - va) >> 4) : (8192u >> 4)) << 16);
+                v_desc[st] = (va >> 4) | ((8192u >> 4) << 16);
             }
             uint32_t k_par = 0, v_par = 0, gk_par = 0, gv_par = 0;   // barrier parities, a bit per stage (TMA tiles; gathered tiles)
             int ks = 0, vs = 0;                                // stage of the next S / PV operand
@@ -288,11 +280,6 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     } else {
         // =================================== softmax warps ==================================================
         const int i = i0 + tid;                                // this thread's query row
-        if (S::ONES) {                                         // 8 KB of bf16 1.0: 64 bytes per thread
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(base + S::OFF_ONES + tid * 64 + u * 16), "r"(0x3F803F80u) : "memory");
-        }
         // retained entries visible to this row.  The rows of a warp are consecutive and the list is ascending, so
         // nvis(row) = #{idx <= lim of lane 0} + #{idx in (lim of lane 0, lim of this lane]}: a ballot count plus a
         // 31-bit map of the entries that fall between the warp's first and last limit.  No block barrier.
@@ -358,7 +345,7 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
         const float c2 = scale * 1.4426950408889634f;          // logits are handled in the log2 domain: x = s * c2
         const uint32_t lane_base = ((uint32_t)(warp * 32)) << 16;   // this warp's TMEM lanes
-        float m_run = -INFINITY, l_run = 0.f;                  // running max (log2 domain) and sum (sum only if !ONES)
+        float m_run = -INFINITY, l_run = 0.f;                  // running max (log2 domain) and sum
 
         PLM_INIT(tid == 0);
         PLM(0);
@@ -457,7 +444,7 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 // PV(t-1) must be done before O is rescaled
                 if (t > 0) { mbar_wait(((t - 1) & 1) ? bar_pv1 : bar_pv0, ((t - 1) >> 1) & 1, 4); tc_fence_after(); }
 #pragma unroll 1
-                for (int cb = 0; cb < D / 32 + (S::ONES ? 1 : 0); ++cb) {   // (rolled: rarely taken, and the softmax loop is sensitive to its code size)   // with ONES the row-sum columns are rescaled too
+                for (int cb = 0; cb < D / 32; ++cb) {          // (rolled: rarely taken, and the softmax loop is sensitive to its code size)
                     uint32_t q4[32];
                     tmem_ld32(tmem + lane_base + O_COL + cb * 32, q4);
                     tmem_wait_ld();
@@ -483,7 +470,7 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                         float a0, a1;
                         unpack2(fma2(pack2(__uint_as_float(r[cb][c]), __uint_as_float(r[cb][c + 1])), c2p, nmp), a0, a1);
                         const float p0 = fast_exp2(a0), p1 = fast_exp2(a1);
-                        if (!S::ONES) ls2[(c >> 1) & 1] = add2(ls2[(c >> 1) & 1], pack2(p0, p1));   // with ONES the tensor core sums the rounded probabilities
+                        ls2[(c >> 1) & 1] = add2(ls2[(c >> 1) & 1], pack2(p0, p1));
                         __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
                         pk[cb * 16 + (c >> 1)] = *reinterpret_cast<uint32_t*>(&h);
                     }
@@ -519,12 +506,6 @@ prefill_long_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         tc_fence_after();
 
         // ---- epilogue: O / l -> bf16, logsumexp ----------------------------------------------------------
-        if (S::ONES) {                                         // the row sum is column D of the accumulator
-            uint32_t q4[32];
-            tmem_ld32(tmem + lane_base + O_COL + D, q4);
-            tmem_wait_ld();
-            l_run = __uint_as_float(q4[0]);
-        }
         const float inv = 1.f / l_run;
         // the normalised rows go into the Q tile's buffer (idle: every product of the CTA has completed) in the swizzled
         // layout and leave as one tile store per warp and 64 columns (rows past the end are clipped by the tensor map;
@@ -588,7 +569,6 @@ __global__ void prefill_compact_kernel(const uint4* __restrict__ k, const uint4*
     }
 }
 
-template <int D>
 int run(const Params& p, const void* q, const void* k, const void* v, const int32_t* idx, const int32_t* cnt, void* o,
         float* lse, void* ws, size_t ws_bytes, cudaStream_t st, const int32_t* leave)
 {
@@ -609,22 +589,22 @@ int run(const Params& p, const void* q, const void* k, const void* v, const int3
     }
     static PerDeviceOnce attr;
     if (int e = attr.run([] {
-            cudaError_t a = cudaFuncSetAttribute(prefill_long_kernel<D, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
-            if (a == cudaSuccess) a = cudaFuncSetAttribute(prefill_long_kernel<D, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
-            return a != cudaSuccess ? a : cudaFuncSetAttribute(prefill_long_kernel<D, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::BYTES);
+            cudaError_t a = cudaFuncSetAttribute(prefill_long_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::BYTES);
+            if (a == cudaSuccess) a = cudaFuncSetAttribute(prefill_long_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::BYTES);
+            return a != cudaSuccess ? a : cudaFuncSetAttribute(prefill_long_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::BYTES);
         })) return e;
     dim3 grid((Tq + BM - 1) / BM, BH);
     if (leave != nullptr) {
         if (!compact) return LTE_ERR_UNSUPPORTED;             // the streaming variant takes compacted rows only
-        return cuda_status(launch_pdl(prefill_long_kernel<D, true, true>, grid, dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, to, tkc, tvc,
+        return cuda_status(launch_pdl(prefill_long_kernel<true, true>, grid, dim3(NTHREADS), Smem::BYTES, st, tq, tk, tv, to, tkc, tvc,
                                       (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, cnt, leave, (__nv_bfloat16*)o, lse, p.T, p.W, p.R,
                                       p.scale, p.G, p.qoff));
     }
     if (compact)
-        return cuda_status(launch_pdl(prefill_long_kernel<D, true, false>, grid, dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, to, tkc, tvc,
+        return cuda_status(launch_pdl(prefill_long_kernel<true, false>, grid, dim3(NTHREADS), Smem::BYTES, st, tq, tk, tv, to, tkc, tvc,
                                       (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, cnt, leave, (__nv_bfloat16*)o, lse, p.T, p.W, p.R,
                                       p.scale, p.G, p.qoff));
-    return cuda_status(launch_pdl(prefill_long_kernel<D, false, false>, grid, dim3(NTHREADS), Smem<D>::BYTES, st, tq, tk, tv, to, tkc, tvc,
+    return cuda_status(launch_pdl(prefill_long_kernel<false, false>, grid, dim3(NTHREADS), Smem::BYTES, st, tq, tk, tv, to, tkc, tvc,
                                   (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, cnt, leave, (__nv_bfloat16*)o, lse, p.T, p.W, p.R,
                                   p.scale, p.G, p.qoff));
 }
@@ -659,7 +639,7 @@ int launch_prefill_tc_long(const Params& p, const void* q, const void* k, const 
     if (!leave && ws != nullptr && half > 0 && ws_bytes >= 2 * half && ((uintptr_t)ws & 127u) == 0 &&
         (long long)((p.T - p.qoff + 255) / 256) * p.B * p.H * p.G >= 2 * n_sm)
         return launch_prefill_tc_pair(p, q, k, v, idx, cnt, o, lse, ws, half, st);
-    return run<128>(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
+    return run(p, q, k, v, idx, cnt, o, lse, ws, ws_bytes, st, leave);
 }
 
 #ifdef LTE_PROFILE
