@@ -81,39 +81,6 @@ __device__ __forceinline__ Item item_of(const Args& a, int item)
     it.n_tiles = it.n_win;                                     // until the item's Info is there
     return it;
 }
-// The item's Info from the head's ascending list id[0, n) (whole warp).
-__device__ __forceinline__ Info make_info(const Args& a, const Item& it, const int32_t* id, int n, int lane)
-{
-    Info f;
-    const int last = min(it.i0 + BM - 1, a.Tlen - 1) - it.i0, lim0 = it.i0 - a.W;   // rows 0 .. last see positions <= lim0 .. lim0 + last
-    int lo = 0, hi = lim0 + last < 0 ? 0 : n;                  // entries <= lim0: in [lo, hi]
-    while (lo < hi) {
-        const int step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step - 1;
-        const int c = __popc(__ballot_sync(0xffffffffu, at < hi && id[min(at, n - 1)] <= lim0));
-        lo += c * step;
-        if (step == 1) break;
-        hi = min(hi, lo + step - 1);
-    }
-    lo = min(lo, n);
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {                              // at most 127 entries lie in (lim0, lim0 + 127]
-        const int e = lo + u * 32 + lane, x = e < n && lim0 + last >= 0 ? id[e] - lim0 - 1 : BM;
-        const uint32_t bit = x >= 0 && x < last ? 1u << (x & 31) : 0u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] |= (x >> 5) == k ? bit : 0u;
-    }
-    uint32_t sum = (uint32_t)lo;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        f.bits[k] = __reduce_or_sync(0xffffffffu, w[k]);
-        f.before[k] = sum;
-        sum += __popc(f.bits[k]);
-    }
-    f.n_tiles = it.n_win + ((int)sum + BN - 1) / BN;
-    return f;
-}
-
 // Walks a CTA's tiles in order: tile t of its n-th item is tile g.
 struct Cursor {
     Item it;
@@ -201,6 +168,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // Keys run one tile ahead of values: K(g+1) is wanted at the start of softmax g, V(g) at its end.  The whole warp walks
         // the loop, lane 0 issues the copies.
         Cursor ck, cv;
+        ItemQueue queue(answer, bar_c, lane);
         int pos_k[4], pos_v[4];                                // GATHER: positions of the rows of the key cursor's tile, of the tile before it
         auto fetch_positions = [&]() {                         // (of a retained tile)
             const int e0 = (ck.t - ck.it.n_win) * BN, n = cnt[ck.it.bhk];
@@ -230,15 +198,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         auto load_k = [&]() {
             const bool first = ck.t == 0;
             if (first) {
-                // the item: this block's own, then whatever the last request brought; the next request goes out at once
-                int item = blockIdx.x;
-                if (ck.n > 0) {
-                    mbar_wait(bar_c, (ck.n - 1) & 1, 17);
-                    item = launch_aborted(&g_prefill_status) ? -1 : block_from(answer);   // (a lost launch ends)
-                    fence_proxy_async();                       // the answer has been read before the next one is written
-                    __syncwarp();
-                }
-                if (item >= 0 && lane == 0) ask_for_block(answer, bar_c);
+                // the item: this block's own, then whatever the last request brought
+                const int item = ck.n > 0 ? queue.take(17, &g_prefill_status) : (int)blockIdx.x;
                 const uint32_t b = ck.n & 1;
                 if (ck.n >= 2) mbar_wait(bar_qf + 8 * b, ((ck.n >> 1) - 1) & 1, 12);
                 if (item < 0) {
@@ -257,16 +218,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (ck.g >= (uint32_t)KST) mbar_wait(bar_kf + 8 * s, (ck.g / KST - 1) & 1u, 6);
             load(ck, false, sK + s * TILE, bar_k + 8 * s, bar_gk + 8 * s);
             if (first) {                                       // tile 0 is a window tile; the list is looked up while it is on its way
-                const Info f = make_info(args, ck.it, idx + (size_t)ck.it.bhk * R, R > 0 ? cnt[ck.it.bhk] : 0, lane);
-                ck.it.n_tiles = f.n_tiles;
+                const int last = min(ck.it.i0 + BM - 1, args.Tlen - 1) - ck.it.i0;   // rows 0 .. last see positions up to i0 - W .. i0 - W + last
+                const ListView f = view_list(idx + (size_t)ck.it.bhk * R, cnt + ck.it.bhk, R, ck.it.i0 - args.W, last, lane);
+                ck.it.n_tiles = ck.it.n_win + (f.all + BN - 1) / BN;
                 if (lane == 0) {
                     volatile Info* o = slot(ck.n);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) { o->before[k] = f.before[k]; o->bits[k] = f.bits[k]; }
-                    o->n_tiles = f.n_tiles; o->item = ck.it.item;
+                    o->n_tiles = ck.it.n_tiles; o->item = ck.it.item;
                     mbar_arrive(bar_i + 8 * (ck.n & 3));
                 }
             }
+            if (ck.t == max(ck.it.n_tiles - kAskTiles, 0)) queue.ask();
             ck.advance();
         };
         load_k();
