@@ -22,10 +22,11 @@
 //     under the next item's first tile.
 // One warp loads (TMA; cp.async for gathered rows).  dq forms delta at an item's start, each thread from its part of the row, and writes
 // it for the dkv pass, where another warp prepares the constants -L2, -delta scale of every tile.  Every wait is bounded.
-// Measured (B200, us for dq + dkv, against four warps a CTA, two CTAs an SM, items dealt out beforehand):
-//   128 heads x 2,048, d = 64, W = R = 64                 66 + 84   (was 74 + 96)
-//   128 heads of 4-head groups x 4,096, d = 64, W 768, R 512   252 + 280  (364 + 455)
-//   16 heads x 8,192, d = 128, W = R = 512                101 + 128  (185 + 195)
+// Measured (B200, us for dq + dkv, back to back in a CUDA graph, against four warps a CTA, two CTAs an SM, items dealt out beforehand; in
+// brackets: exponential unit, tensor pipe active):
+//   128 heads x 2,048, d = 64, W = R = 64                 60 + 78   (was 74 + 96)       dq 17 %, 30 %;  dkv 12 %, 30 %
+//   128 heads of 4-head groups x 4,096, d = 64, W 768, R 512   243 + 298  (364 + 455)    dq 41 %, 35 %;  dkv 38 %, 45 %
+//   16 heads x 8,192, d = 128, W = R = 512                101 + 107  (185 + 195)
 #include "tile_items.cuh"
 
 namespace lte {
@@ -314,7 +315,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
         }
         __syncwarp();
     } else if (warp == W_XY) {
-        // ================================= X, Y products (lane 0 issues; the whole warp walks the loop) ==========
+        // ================================= X, Y products (an elected thread issues; the whole warp walks the loop) =
         constexpr uint32_t IDESC = instr_desc(BM, BN, false);
         const uint32_t a_lo = desc_lo(sA, 16), b_lo = desc_lo(sB, 16);
         uint32_t g = 0, par_a = 0;                             // parities of bar_a (bits 0 .. 3), bar_ga (4 .. 7)

@@ -623,8 +623,8 @@ __global__ void __launch_bounds__(DT) decode_bulk_kernel(unsigned char* __restri
 // State after a T-token prompt.  Bound by memory: every byte of the cache is written exactly once (the rows nothing fills,
 // the tail's padding and the header as zeros, so no fill pass comes before), every window and retained row is read once, in
 // 16-byte pieces.  Block (b,h) x parts + part (one-dimensional: there may be more heads than a grid's second dimension takes) writes
-// IROWS rows of the head's block with their logits; a block per head with two divisions per element took 248 + 17 us for 256 heads of
-// 1,280 rows (d = 64), this takes 28.
+// IROWS rows of the head's block with their logits; a block per head with two divisions per element took 254 us for 256 heads of
+// 1,280 rows (d = 64), this takes 27.
 constexpr int IROWS = 64;
 // The piece-th 16 bytes of a tensor, read in units of U (what the tensor is aligned to).
 template <typename U> __device__ __forceinline__ uint4 load_piece(const U* p, size_t piece)
@@ -1185,8 +1185,8 @@ int launch_decode(const Params& p, void* cache, const void* q1, const void* k1, 
     if (p.stack) ps.K = 0;                               // the stack is scored outside the step (lte_cache_score)
     if (p.W + p.R > MAX_ROWS) return LTE_ERR_UNSUPPORTED;
     if (p.dtype == LTE_BF16) {
-        // one query head and a block of rows that is a tcgen05 operand as it stands: 27 us at 2,048 heads x 256 rows, where the
-        // other kernel takes 36 (4,096 x 128: 29 and 45; 16 x 256: 5.2 and 6.6); everything else in bf16 goes through mma.sync
+        // one query head and a block of rows that is a tcgen05 operand as it stands: 26.2 us at 2,048 heads x 256 rows, where the
+        // other kernel takes 35.3 (4,096 x 128: 27.7 and 43.5; 16 x 256: 4.4 and 6.1); everything else in bf16 goes through mma.sync
         if (p.G <= 1 && cache_layout(p.d, p.W, p.R, p.dtype).swz) return launch_decode_tc(ps, cache, q1, k1, v1, o1, lse1, st);
         return launch_decode_mma(ps, cache, q1, k1, v1, o1, lse1, st);
     }

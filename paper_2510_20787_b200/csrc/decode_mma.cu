@@ -17,14 +17,14 @@
 //            into two bf16 terms: 16 bits of mantissa, below what the output's rounding shows (o against 64 bits over 35,000 random
 //            steps: 1.53e-3, the same to four digits as with fp32 weights).
 //
-// Measured (B200, a step in a CUDA graph; before: a block per head on the fp32 ALUs):
-//   256 heads x 1,280 rows, four query heads each, d = 64    14.3 us (68 MB: 4.8 TB/s), before 26.7
-//   512 heads x 1,280 rows, d = 64                           29.1 us, before 40.1
-//   512 heads x 1,024 rows, d = 128                          39.9 us, before 60.6
-//   16 heads x 1,024 rows, d = 128                            6.4 us in clusters of 8, before 14.6; six of it are the chain launch,
+// Measured (B200, a step in a CUDA graph of steps, full pools; before: a block per head on the fp32 ALUs):
+//   256 heads x 1,280 rows, four query heads each, d = 64    17.7 us (84 MB: 4.8 TB/s), before 29.9; with 1,160 rows 15.4
+//   512 heads x 1,280 rows, d = 64                           34.0 us (4.9 TB/s), before 43.1
+//   512 heads x 1,024 rows, d = 128                          49.1 us (5.5 TB/s), before 63.6
+//   16 heads x 1,024 rows, d = 128                            7.5 us in clusters of 8, before 16.5; six of it are the chain launch,
 //                                                            counters, rows, combination, and stay when there are fewer rows
-// With row-by-row address arithmetic (600 instead of 130 instructions a span) the first line took 17.9 us; asking for the ring's
-// rows in L2 ahead of the grid dependency made the large shapes slower (30.3 and 45.2 us).
+// With row-by-row address arithmetic (600 instead of 130 instructions a span) the first line was a quarter slower; asking for the
+// ring's rows in L2 ahead of the grid dependency made the large shapes slower (4 and 13 %).
 #include <cooperative_groups.h>
 
 #include "common.cuh"

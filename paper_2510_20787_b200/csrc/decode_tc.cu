@@ -16,8 +16,8 @@
 // Bound by memory only as far as the chain of a head (copy, logits, softmax, output: some 4 us) is short enough for the CTAs that fit
 // on an SM to keep it busy.  So only rows that exist are copied, the worst pool entry and the maximum are found by warp-wide
 // reductions of one instruction, the next head's inputs are asked for under this head's output, and one barrier per head is left.
-// Measured (B200, a step in a CUDA graph, before -> now): 2,048 heads x 256 rows 30.6 -> 26.9 us (137 MB: 5.1 TB/s), 1,024 x 256
-// 16.3 -> 13.7, 4,096 x 128 56.0 -> 28.9, 16 x 256 5.7 -> 5.2.  Asking for the next head in L2 ahead: 31.2 -> 33.3; two stages of 128
+// Measured (B200, a step in a CUDA graph of steps, before -> now): 2,048 heads x 256 rows 29.1 -> 26.0 us (137 MB: 5.3 TB/s; 28.3 with
+// R = 196, of which two blocks fit an SM), 1,024 x 256 15.0 -> 12.8, 4,096 x 128 53.8 -> 27.6, 16 x 256 4.9 -> 4.4.  Asking for the next head in L2 ahead: 31.2 -> 33.3; two stages of 128
 // rows each instead of five CTAs: 37.9.
 #include <type_traits>
 

@@ -1,8 +1,9 @@
 // Prefill attention on the 5th-generation tensor cores for bf16, d = 64 and d = 32 (Section 3.1.3, "Cached prefilling and
 // decoding").
 //
-// Bound by the instruction stream of the softmax warps (no pipe is full: exponential unit 50 %, issue 46 %, tensor pipe 28 %),
-// so work is paid once per 128 keys, spread over 16 warps per SM, and nothing waits that need not:
+// Bound by the instruction stream of the softmax warps and the latencies between them (no pipe is full: with items of nine tiles issue
+// 60 %, exponential unit 55 %, tensor pipe 31 %; with items of four 55, 37, 27), so work is paid once per 128 keys, spread over 16
+// warps per SM, and nothing waits that need not:
 //   work      Two CTAs per SM; an item is a 128-query tile of one head.  Key/value tiles of 128 rows come by TMA, first the window
 //             span, then the head's retained rows that any of the item's rows may see (compacted beforehand where the caller
 //             brought a workspace; otherwise the load warp gathers them row by row into the same swizzled layout).  Eight softmax
@@ -22,12 +23,15 @@
 // and products of the next item run under the current one.  Every mbarrier wait is bounded; one that runs out records a
 // status word and the kernel still terminates.
 //
-// Measured (B200, the call with a workspace): 1,024 query heads x 4,096, W = 768, R = 512 half used: 1.43 ms (601 TFLOP/s), before
-// 2.10; 64 heads x 4,096, W = R = 128: 51 us, before 66.  The steps, at an eighth of the first shape: four warps with 64-key
-// tiles 275 us; one thread per row, 128-key tiles 242; two threads per row 223; dynamic items 203; O stored under the next item
-// 190.  Tried there and slower: rolled 32-column loops (214), column bounds carried from tile to tile and a vote in place of the
-// exchange of maxima (209), one thread per row with dynamic items (213), the two streams of an SM taking turns at the
-// exponential unit (328), a quarter of the exponentials as polynomials on the multiply-add pipe (207).
+// Measured (B200, the call with a workspace, back to back in a CUDA graph; before: four warps with 64-key tiles, items dealt out):
+//   1,024 query heads x 4,096, W = 768, R = 512 half used   1.67 ms (515 TFLOP/s), before 2.09
+//   32 x 4,096 of it                                       198 us (542), before 285
+//   64 heads x 4,096, W = R = 128                          54 us, before 62      128 x 2,048, W = R = 64   44 us, before 50
+// The steps, at an eighth of the first shape and with one sum per row: four warps with 64-key tiles 275 us; one thread per row, 128-key
+// tiles 242; two threads per row 223; dynamic items 203; O stored under the next item 190.  Tried there and slower: rolled
+// 32-column loops (214), column bounds carried from tile to tile and a vote in place of the exchange of maxima (209), one thread
+// per row with dynamic items (213), the two streams of an SM taking turns at the exponential unit (328), a quarter of the
+// exponentials as polynomials on the multiply-add pipe (207).
 //
 // d = 32 runs the same kernel: the tensor maps describe 32-column rows with a 64-column box, the copy engine fills the upper
 // half of every tile row with zeros, and only the first 32 output columns are stored.
@@ -253,7 +257,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         }
         __syncwarp();
     } else if (warp == 8) {
-        // ================================= MMA warp (lane 0 issues; the whole warp walks the loop) ==============
+        // ================================= MMA warp (an elected thread issues; the whole warp walks the loop) ====
         constexpr uint32_t IDESC_S = instr_desc(BM, BN, false), IDESC_O = instr_desc(BM, D, true);
         const uint32_t q_lo = desc_lo(sQ, 16), k_lo = desc_lo(sK, 16), v_lo = desc_lo(sV, 16);
         Cursor cs, cp;

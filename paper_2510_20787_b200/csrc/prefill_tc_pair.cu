@@ -14,10 +14,11 @@
 // factor of 2^8 of the values and the largest weights stay near 1), which is asked once the exponentials are done.  (kFar = 64 is not
 // faster: 364.0 and 363.6 us for the whole case of the first line below.)
 // Every mbarrier wait is bounded; a wait that runs out records a status word and the kernel still terminates.
-// Measured (B200, us, compaction included; before: a CTA per 128-query tile, two CTAs per SM, prefill_tc_long.cu):
-//   16 heads x 32,768, W = R = 512      257 (793 TFLOP/s), before 286
-//   16 heads x 8,192, W = R = 512       81, before 91        32 heads x 8,192, W = R = 64         64, before 70
-//   64 heads x 4,096, W = R = 128       73, before 83        256 heads x 2,000 in fours, W 300    168, before 190
+// Measured (B200, us, compaction included, back to back in a CUDA graph, where the clock moves by some 5 % from run to run; before: a CTA
+// per 128-query tile, two CTAs per SM, prefill_tc_long.cu):
+//   16 heads x 32,768, W = R = 512      254 - 276 (769 TFLOP/s), before 283 - 294
+//   16 heads x 8,192, W = R = 512       88 - 91, before 92 - 98    32 heads x 8,192, W = R = 64         63 - 68, before 70 - 72
+//   64 heads x 4,096, W = R = 128       72 - 77, before 82 - 86    256 heads x 2,000 in fours, W 300    166 - 176, before 188 - 192
 // What was slower in the first line: S of 128 keys with P in its place (264 to 271: the chain P, PV, S is exposed), two S buffers and
 // groups of warps taking turns at the tiles (283), a product warp whose control flow the compiler takes for divergent (276), one
 // commit per tile and plain arrivals for what it implies (269: stages come free too late for short items).
@@ -194,7 +195,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
         __syncwarp();
     } else if (warp >= W_MMA) {
-        // ================================= MMA warps (lane 0 issues; the whole warp walks the loop) ================
+        // ================================= MMA warps (an elected thread issues; the whole warp walks the loop) ======
         constexpr uint32_t IDESC_S = instr_desc(BM, BN, false), IDESC_O = instr_desc(BM, D, true);
         const int q = warp - W_MMA;
         const uint32_t q_lo = desc_lo(sQ + q * QTILE, 16), k_lo = desc_lo(sK, 16), v_lo = desc_lo(sV, TILE / 2);
