@@ -58,7 +58,7 @@ struct Smem {
 // lane doing both was the bottleneck: its dependent instruction stream took longer per tile than the softmax).
 // They meet on mbarriers:
 //   bar_s[b]  (commit)       S(t) is in TMEM buffer b = t & 1                     control -> softmax
-//   bar_p     (128 arrivals) P(t) is in shared memory, S buffer b is free         softmax -> control
+//   bar_p     (128 arrivals) P(t) is in TMEM, over the S buffer it came from       softmax -> control
 //   bar_pv[b] (commit)       PV(t) has completed, b = t & 1 (a barrier per parity: a waiter can then never find it two
 //                            phases ahead, so the softmax threads wait on it only where they need the product)   control -> softmax
 //   bar_gk[s], bar_gv[s] (128 arrivals, by cp.async completion) a gathered tile is in stage s   softmax -> control
