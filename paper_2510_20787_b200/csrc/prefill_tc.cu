@@ -45,8 +45,8 @@ namespace {
 
 constexpr int BM = 128, BN = 128, D = 64, NTHREADS = 320;         // warps 0-7 softmax, 8 products, 9 loads
 using namespace tc;
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_prefill_status); }
-__device__ __forceinline__ void mbar_wait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni(bar, parity, code, &g_prefill_status); }
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_call(bar, parity, code, &g_prefill_status); }
+__device__ __forceinline__ void mbar_wait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni_call(bar, parity, code, &g_prefill_status); }
 
 template <bool STREAM> struct Smem {
     static constexpr int TILE = 128 * D * 2;                  // [128][64] bf16: Q, K and V tiles alike

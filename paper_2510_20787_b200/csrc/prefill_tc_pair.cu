@@ -31,9 +31,9 @@ __device__ StatusWord g_prefill_pair_status = LTE_STATUS_INIT; // 0 = fine; othe
 namespace {
 
 using namespace tc;
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_s(bar, parity, code, &g_prefill_pair_status); }
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int code) { mbar_wait_call(bar, parity, code, &g_prefill_pair_status); }
 
-__device__ __forceinline__ void mbar_wait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni(bar, parity, code, &g_prefill_pair_status); }
+__device__ __forceinline__ void mbar_wait_u(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni_call(bar, parity, code, &g_prefill_pair_status); }
 
 constexpr int D = 128, BM = 128, BN = 64, ST = 5;              // query tile, key tile, stages (of K, and as many of V)
 constexpr int W_MMA = 16, W_LOAD = 18, NTHREADS = 19 * 32;     // 16 softmax warps, an MMA warp per query tile, a load warp

@@ -39,8 +39,12 @@ __device__ __forceinline__ void wait_gave_up(StatusWord* st, int code) {
     atomicCAS(&st->code, 0, code);                              // the first anomaly since the host last read the word stays
     atomicExch(&st->abort_grid, grid_id());
 }
+// The loops are rolled: unrolled by the compiler, a kernel's waits were up to a quarter of its instructions, and these kernels, whose
+// warps run different code on one SM, wait for instructions (backward 194 -> 189 us at 128 heads x 2,048, 654 -> 640 with the paper's
+// window and query groups).
 template <uint32_t LIMIT = kSpinLimit>
 __device__ __forceinline__ void mbar_wait_s(uint32_t bar, uint32_t parity, int code, StatusWord* st) {
+#pragma unroll 1
     for (uint32_t i = 0; i < LIMIT; ++i) {
         if (mbar_try_wait(bar, parity)) return;
         if ((i & 1023u) == 1023u && launch_aborted(st)) return;
@@ -58,11 +62,26 @@ __device__ __forceinline__ bool elect_one() {
 }
 template <uint32_t LIMIT = kSpinLimit>
 __device__ __forceinline__ void mbar_wait_uni(uint32_t bar, uint32_t parity, int code, StatusWord* st) {   // mbar_wait_s by a whole warp
+#pragma unroll 1
     for (uint32_t i = 0; i < LIMIT; ++i) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
         if ((i & 1023u) == 1023u && uni(launch_aborted(st))) return;
     }
     wait_gave_up(st, code);
+}
+// The same two waits with everything behind the first look at the barrier out of line, for kernels that have registers to spare across a
+// call (prefill at d = 128: 252 -> 245 us at 16 heads x 32,768, 168 -> 157 at 256 x 2,000; the backward kernels, which have not: 189 -> 205).
+template <uint32_t LIMIT> __device__ __noinline__ void mbar_wait_behind(uint32_t bar, uint32_t parity, int code, StatusWord* st) {
+    mbar_wait_s<LIMIT>(bar, parity, code, st);
+}
+template <uint32_t LIMIT> __device__ __noinline__ void mbar_wait_uni_behind(uint32_t bar, uint32_t parity, int code, StatusWord* st) {
+    mbar_wait_uni<LIMIT>(bar, parity, code, st);
+}
+__device__ __forceinline__ void mbar_wait_call(uint32_t bar, uint32_t parity, int code, StatusWord* st) {
+    if (!mbar_try_wait(bar, parity)) mbar_wait_behind<kSpinLimit>(bar, parity, code, st);
+}
+__device__ __forceinline__ void mbar_wait_uni_call(uint32_t bar, uint32_t parity, int code, StatusWord* st) {
+    if (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) mbar_wait_uni_behind<kSpinLimit>(bar, parity, code, st);
 }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
