@@ -90,11 +90,15 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
 }
 
 // Logits of the local sequence.  In: z = the scorer's output over the local sequence (wrong where the receptive field
-// reaches below row R0 + half, undefined for the pool rows).  Out: z = the logit of each row's token (the cache's own where
+// reaches below row R0 + half, undefined for rows before zfrom).  Out: z = the logit of each row's token (the cache's own where
 // it holds one), zrank = the same with sink tokens lifted to +inf, which is what the selection ranks by.
-__global__ void chunk_merge_z_kernel(float* __restrict__ z, float* __restrict__ zrank, const float* __restrict__ zsrc,
-                                     const int32_t* __restrict__ oldpos, int R, int W, int n0, int R0, int Wn, int Tloc,
-                                     int half, int sink)
+// zfrom > 0: the single-layer scorer left out the rows before zfrom, whose logits a cache normally holds (8 x 16 heads, 512 tokens on
+// W = 768, R = 512: 15 -> 5 us for the scorer); a ring token among them that has none is scored here, channel by channel.
+template <typename T>
+__global__ void chunk_merge_z_kernel(const T* __restrict__ klin, const T* __restrict__ vlin, const float* __restrict__ w, const float* __restrict__ bias,
+                                     float* __restrict__ z, float* __restrict__ zrank, const float* __restrict__ zsrc,
+                                     const int32_t* __restrict__ oldpos, int H, int D, int K, int R, int W, int n0, int R0, int Wn, int Tloc,
+                                     int half, int sink, int zfrom)
 {
     pdl_launch_dependents();
     pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
@@ -109,13 +113,24 @@ __global__ void chunk_merge_z_kernel(float* __restrict__ z, float* __restrict__ 
         if (pos < 0) zt = -INFINITY;
     } else {
         pos = n0 - Wn + (r - R0);
-        zt = z[(size_t)bh * Tloc + r];
-        if (r < R0 + Wn) {
-            const float zc = zsrc[(size_t)bh * (R + W) + r];
-            // a ring token keeps the logit the cache holds; one the cache has not scored yet is scored now, unless its
-            // left neighbours are no longer there (then it stays unscored, as in the decode step)
-            if (zc > -INFINITY) zt = zc;
-            else if (R0 > 0 && r < R0 + half) zt = -INFINITY;
+        zt = r < R0 + Wn ? zsrc[(size_t)bh * (R + W) + r] : -INFINITY;
+        // a ring token keeps the logit the cache holds; one the cache has not scored yet is scored now, unless its
+        // left neighbours are no longer there (then it stays unscored, as in the decode step)
+        if (!(zt > -INFINITY)) {
+            if (r < R0 + Wn && R0 > 0 && r < R0 + half) zt = -INFINITY;
+            else if (r >= zfrom) zt = z[(size_t)bh * Tloc + r];
+            else {                                             // (its right context is there: zfrom is half rows before the chunk)
+                const int h = bh % H;
+                zt = bias ? bias[h] : 0.f;
+                for (int t = 0; t < K; ++t) {
+                    const int rr = r - half + t;
+                    if (rr < 0) continue;                      // (R0 = 0: before position 0)
+                    const T* kr = klin + ((size_t)bh * Tloc + rr) * D;
+                    const T* vr = vlin + ((size_t)bh * Tloc + rr) * D;
+                    const float* wt = w + ((size_t)h * K + t) * 2 * D;
+                    for (int c = 0; c < D; ++c) zt = fmaf(to_f(kr[c]), wt[c], fmaf(to_f(vr[c]), wt[D + c], zt));
+                }
+            }
         }
     }
     z[(size_t)bh * Tloc + r] = zt;
@@ -296,11 +311,16 @@ int launch_chunk_gather(const Params& p, const void* cache, const void* k, const
                                               (unsigned char*)klin, (unsigned char*)vlin, zsrc, oldpos, gate, p.d, p.W, p.R, n0, R0, Wn, p.T));
 }
 
-int launch_chunk_merge_z(const Params& p, float* z, float* zrank, const float* zsrc, const int32_t* oldpos, int n0, int R0, int Wn,
-                         cudaStream_t st)
+int launch_chunk_merge_z(const Params& p, const void* klin, const void* vlin, float* z, float* zrank, const float* zsrc, const int32_t* oldpos,
+                         int n0, int R0, int Wn, cudaStream_t st)
 {
     dim3 grid((p.T + 255) / 256, p.B * p.H);
-    return cuda_status(launch_pdl(chunk_merge_z_kernel, grid, dim3(256), 0, st, z, zrank, zsrc, oldpos, p.R, p.W, n0, R0, Wn, p.T, p.half, p.sink));
+    auto go = [&](auto kern, auto* k, auto* v) {
+        return cuda_status(launch_pdl(kern, grid, dim3(256), 0, st, k, v, p.w, p.bias, z, zrank, zsrc, oldpos, p.H, p.d, p.K, p.R, p.W, n0, R0, Wn, p.T, p.half,
+                                      p.sink, p.zfrom));
+    };
+    if (p.dtype == LTE_BF16) return go(chunk_merge_z_kernel<__nv_bfloat16>, (const __nv_bfloat16*)klin, (const __nv_bfloat16*)vlin);
+    return go(chunk_merge_z_kernel<float>, (const float*)klin, (const float*)vlin);
 }
 
 int launch_chunk_commit(const Params& p, void* cache, const void* klin, const void* vlin, const float* z, const int32_t* idx,

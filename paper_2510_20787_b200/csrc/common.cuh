@@ -17,6 +17,7 @@ struct Params {                       // validated, host-resolved view of lte_sh
     int B, H, T, d, W, R, sink, K, half;
     int G;                            // query heads per key/value head (q, o, lse have H * G heads)
     int qoff;                         // prefill attention: q, o, lse hold the queries at positions qoff .. T-1 only (chunked prefill; else 0)
+    int zfrom;                        // single-layer scorer: rows before zfrom need no logit (chunked prefill: the cache holds theirs; else 0)
     int stack;                        // 1: the three-layer scorer stack (w, bias packed as lte.h describes; K = 13, half = 6)
     float zthr;                       // logit(tau): keep iff z > zthr
     float scale;                      // softmax scale
@@ -125,7 +126,7 @@ int launch_ring_linearize(const Params& p, const void* cache, void* klin, void* 
 int launch_ring_scatter_z(const Params& p, void* cache, const float* zlin, cudaStream_t st);
 int launch_chunk_gather(const Params& p, const void* cache, const void* k, const void* v, void* klin, void* vlin, float* zsrc,
                         int32_t* oldpos, int32_t* gate, int n0, int R0, int Wn, cudaStream_t st);
-int launch_chunk_merge_z(const Params& p, float* z, float* zrank, const float* zsrc, const int32_t* oldpos, int n0, int R0, int Wn,
+int launch_chunk_merge_z(const Params& p, const void* klin, const void* vlin, float* z, float* zrank, const float* zsrc, const int32_t* oldpos, int n0, int R0, int Wn,
                          cudaStream_t st);
 int launch_chunk_commit(const Params& p, void* cache, const void* klin, const void* vlin, const float* z, const int32_t* idx,
                         const int32_t* cnt, const int32_t* oldpos, const int32_t* gate, int n0, int n1, int R0, int Wn,

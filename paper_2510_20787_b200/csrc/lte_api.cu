@@ -66,6 +66,7 @@ Params make_params(const lte_shape* s, const lte_conv* c)
     p.K = c ? c->kernel : 1; p.half = p.K / 2;
     p.stack = 0;
     p.qoff = 0;
+    p.zfrom = 0;
     if (c && c->n_layers == 3) { p.stack = 1; p.K = 13; p.half = 6; }   // the paper's stack: receptive field 13
     p.zthr = s->tau <= 0.f ? -INFINITY : (float)(log((double)s->tau) - log1p(-(double)s->tau));
     p.scale = s->softmax_scale > 0.f ? s->softmax_scale : (float)(1.0 / sqrt((double)s->d));
@@ -384,10 +385,12 @@ int lte_attn_prefill_chunk_ex(const lte_shape* s, const lte_conv* c, void* cache
         e = launch_scores_stack_tc(p, base + w.klin, base + w.vlin, z, nullptr, base + w.sub, w.att - w.sub, st);
         if (e == LTE_ERR_UNSUPPORTED) e = launch_scores_stack(p, base + w.klin, base + w.vlin, z, nullptr, st);
     } else {
+        // the ring's newest K/2 tokens and the chunk; a cache holds the logits of older ones (where it does not, the merge scores them)
+        p.zfrom = qoff > p.half ? qoff - p.half : 0;
         e = launch_scores(p, base + w.klin, base + w.vlin, z, nullptr, st);
     }
     if (e) return e;
-    e = launch_chunk_merge_z(p, z, zrank, zsrc, oldpos, n_past, R0, Wn, st); if (e) return e;
+    e = launch_chunk_merge_z(p, base + w.klin, base + w.vlin, z, zrank, zsrc, oldpos, n_past, R0, Wn, st); if (e) return e;
     if (streaming) {
         // token by token: the pool every query sees is the streaming rule's at that query.  The entries that are in the
         // pool at some query, each with the query from which it is gone, feed the row-by-row attention kernel (the tiled

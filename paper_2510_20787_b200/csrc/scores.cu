@@ -39,7 +39,7 @@ template <> struct Vec16<float> {
 template <typename T, int D, int K>
 __global__ void __launch_bounds__(NT) scores_kernel(const T* __restrict__ k, const T* __restrict__ v,
                                                     const float* __restrict__ w, const float* __restrict__ bias,
-                                                    float* __restrict__ z, float* __restrict__ r, int H, int Tlen)
+                                                    float* __restrict__ z, float* __restrict__ r, int H, int Tlen, int t0)
 {
     constexpr int HALF = K / 2;
     constexpr int TJ = NT - (K - 1);
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(NT) scores_kernel(const T* __restrict__ k, con
 
     const int bh = blockIdx.y;
     const int h = bh % H;
-    const int j0 = blockIdx.x * TJ;
+    const int j0 = (t0 + blockIdx.x) * TJ;  // (rows before tile t0 need no logit)
     const int tid = threadIdx.x;
     pdl_launch_dependents();
     pdl_wait();                             // see launch_pdl: earlier kernels of the stream have completed
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(NT + 64) scores_tc_kernel(const __grid_constan
                                                        const __grid_constant__ CUtensorMap tmV,
                                                        const float* __restrict__ w, const float* __restrict__ bias,
                                                        float* __restrict__ z, float* __restrict__ r, int H, int Tlen,
-                                                       int n_flat, int dg)
+                                                       int n_flat, int t0, int dg)
 {
     // dg = the head dimension in memory: D, or D / 2 = 32 for the d = 64 kernel on d = 32 data (the tensor maps then fill
     // the upper half of every tile row with zeros, and B carries zeros in the same columns)
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(NT + 64) scores_tc_kernel(const __grid_constan
     const uint32_t bar_ld0 = tile0 + C::OFF_BAR, bar_mma0 = bar_ld0 + 8 * NSTAGE, tmem_slot = bar_mma0 + 16;
     volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_BAR + 8 * NSTAGE + 16);
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int n_all = (Tlen + TJ - 1) / TJ;              // row tiles per head
+    const int n_all = (Tlen + TJ - 1) / TJ - t0;         // row tiles per head, from tile t0 on (rows before it need no logit)
     // this CTA's share of the flat list of (head, row tile) pairs: an even split, heads may change along the way
     const int f_begin = (int)(((long long)blockIdx.x * n_flat) / gridDim.x);
     const int f_end = (int)(((long long)(blockIdx.x + 1) * n_flat) / gridDim.x);
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(NT + 64) scores_tc_kernel(const __grid_constan
                 // the stage is free once the MMAs of the tile that used it have completed
                 if (i >= NSTAGE) mbar_wait_s(bar_mma0 + 8 * ((i - NSTAGE) & 1), ((i - NSTAGE) >> 1) & 1, 3, &g_scores_status);
                 const uint32_t dst = tile0 + (i % NSTAGE) * C::STAGE, bar = bar_ld0 + 8 * (i % NSTAGE);
-                const int y = ft * TJ - HALF;
+                const int y = (t0 + ft) * TJ - HALF;
                 mbar_expect_tx(bar, C::STAGE);
 #pragma unroll
                 for (int sb = 0; sb < SUB; ++sb) {
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(NT + 64) scores_tc_kernel(const __grid_constan
             }
             SPROF(4 * i + 2);
             group_sync();                                  // ys complete
-            const int j = ti * TJ + tid;
+            const int j = (t0 + ti) * TJ + tid;
             if (tid < TJ && j < Tlen) {
                 float zz;
                 if (j + HALF > Tlen - 1) {
@@ -349,21 +349,22 @@ int run_tma(const Params& p, const void* k, const void* v, float* z, float* r, c
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
     // one wave of CTAs (two per SM at d = 64, one at d = 128) shares the flat list of (head, row tile) pairs evenly
-    const int n_all = (p.T + TJ - 1) / TJ, BH = p.B * p.H;
+    const int t0 = p.zfrom / TJ, n_all = (p.T + TJ - 1) / TJ - t0, BH = p.B * p.H;
     const long long n_flat = (long long)n_all * BH;
     if (n_flat > 0x7fffffffLL) return LTE_ERR_UNSUPPORTED;
     const int slots = n_sm * (D == 64 ? 2 : 1);
     const int n_cta = (int)(n_flat < slots ? n_flat : slots);
     return cuda_status(launch_pdl(scores_tc_kernel<D, K>, dim3(n_cta), dim3(NT + 64), C::BYTES, st, tk, tv, p.w, p.bias, z, r, p.H, p.T,
-                                  (int)n_flat, dg));
+                                  (int)n_flat, t0, dg));
 }
 
 template <typename T, int D, int K>
 int run(const Params& p, const void* k, const void* v, float* z, float* r, cudaStream_t st)
 {
     constexpr int TJ = NT - (K - 1);
-    dim3 grid((p.T + TJ - 1) / TJ, p.B * p.H);
-    return cuda_status(launch_pdl(scores_kernel<T, D, K>, grid, dim3(NT), 0, st, (const T*)k, (const T*)v, p.w, p.bias, z, r, p.H, p.T));
+    const int t0 = p.zfrom / TJ;
+    dim3 grid((p.T + TJ - 1) / TJ - t0, p.B * p.H);
+    return cuda_status(launch_pdl(scores_kernel<T, D, K>, grid, dim3(NT), 0, st, (const T*)k, (const T*)v, p.w, p.bias, z, r, p.H, p.T, t0));
 }
 
 template <typename T, int D, int K>

@@ -217,3 +217,30 @@ def test_the_two_readings_differ_where_the_cap_binds_and_leave_the_same_cache():
     assert na == nb and all(np.array_equal(u, v) for u, v in zip(pa, pb))
     # the last query of the chunk sees the final pool under both readings
     assert np.max(np.abs(a[1][0][:, :, -1] - b[1][0][:, :, -1])) <= 2e-2
+
+
+@pytest.mark.parametrize("dtype,d,T0", [("bf16", 64, 300), ("f32", 32, 300), ("bf16", 128, 150), ("bf16", 64, 20)])
+def test_ring_tokens_without_a_logit_are_scored_by_the_chunk(dtype, d, T0):
+    """The scorer goes over the ring's last K/2 tokens and the chunk only; a cache may lack other logits (here: taken out of z before
+    lte_cache_init) and a chunk then scores those tokens too, as if the cache had had them."""
+    cfg = _cfg(dtype, d=d, W=140, R=64)
+    Tc, half = 200, cfg.K // 2
+    x = synth.make(cfg, 4, T=T0 + Tc)
+    c = lte.conv(torch.from_numpy(x["w"]).cuda(), torch.tensor([0.3, -0.2, 0.1], device="cuda"))
+    q, k, v = (dev(x[t], cfg.dtype) for t in "qkv")
+    code = lte.BF16 if dtype == "bf16" else lte.F32
+    s0, s1 = (lte.shape(cfg.B, cfg.H, n, d, cfg.W, cfg.R, code) for n in (T0, Tc))
+    kp, vp = (t[:, :, :T0].contiguous() for t in (k, v))
+    z = lte.lte_scores(s0, c, kp, vp)
+    idx, cnt = lte.lte_select(s0, z)
+    gaps = z.clone()
+    first = max(T0 - cfg.W, 0) + (half if T0 > cfg.W else 0)        # (tokens before it have lost their left neighbours)
+    gaps[:, :, [first, first + 1, (first + T0) // 2, T0 - half - 1]] = -float("inf")
+    out = []
+    for zz in (z, gaps):
+        cache = lte.lte_cache_init(s0, c, kp, vp, zz, idx, cnt)
+        o, lse = lte.lte_attn_prefill_chunk(s1, c, cache, T0, *(t[:, :, T0:].contiguous() for t in (q, k, v)))
+        out.append((o, lse, _read_pool(cache, cfg, cfg.B)))
+    assert lte.lte_device_status() == 0
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert out[0][2][1] == out[1][2][1] and all(np.array_equal(a, b) for a, b in zip(out[0][2][0], out[1][2][0]))
