@@ -115,7 +115,9 @@ template <int D, bool SWZ> struct Group {                      // what a lane ho
     }
 };
 
-template <int D, int NW, bool SWZ>
+// BACK: in every other step the spans come from the last to the first (see decode_turns; a variant of its own, since the sign of the
+// stride costs the other 3 %).
+template <int D, int NW, bool SWZ, bool BACK>
 __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kernel(
     unsigned char* __restrict__ cache, CacheLayout L, const __nv_bfloat16* __restrict__ q1, const __nv_bfloat16* __restrict__ k1,
     const __nv_bfloat16* __restrict__ v1, __nv_bfloat16* __restrict__ o1, float* __restrict__ lse1, const float* __restrict__ cw,
@@ -180,10 +182,12 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
     rows.n_ring = n < W ? n : W;
     rows.ring_spans = (rows.n_ring + 15) >> 4;
     rows.spans = rows.ring_spans + ((cnt_old + 15) >> 4) + 1;
-    const int step = NW * nsplit, first = wid * nsplit + rank;
+    const bool back = BACK && (n & 1);
+    const int step = back ? -NW * nsplit : NW * nsplit, first = back ? rows.spans - 1 - wid * nsplit - rank : wid * nsplit + rank;
+    auto has = [&](int i) { return BACK ? (unsigned)i < (unsigned)rows.spans : i < rows.spans; };
     Group<D, SWZ> buf[NBUF];
     const float zp = p >= 0 && R > 0 ? zc[slot] : 0.f;
-    if (first < rows.spans) { const Span sp = rows.span(first); buf[0].load_k(rows, sp, g, t); buf[0].load_v(rows, sp, g, t); }
+    if (has(first)) { const Span sp = rows.span(first); buf[0].load_k(rows, sp, g, t); buf[0].load_v(rows, sp, g, t); }
     const int jsc = K > 0 ? n - half : -1;                     // K = 0: the scorer runs outside (lte_cache_score)
     auto tap_rows = [&](int tap, float (&kx)[CPL], float (&vx)[CPL]) {   // channels lane, lane + 32, .. of the row under a tap
         const int pos = jsc + tap - half, r = pos < 0 ? 0 : pos % W;
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
     };
     float kx[CPL], vx[CPL];
     if (taps && jsc >= 0) tap_rows(wid, kx, vx);
-    if (NBUF == 2 && first + step < rows.spans) { const Span sp = rows.span(first + step); buf[NBUF - 1].load_k(rows, sp, g, t); buf[NBUF - 1].load_v(rows, sp, g, t); }
+    if (NBUF == 2 && has(first + step)) { const Span sp = rows.span(first + step); buf[NBUF - 1].load_k(rows, sp, g, t); buf[NBUF - 1].load_v(rows, sp, g, t); }
 
     // ---- what happens to the token leaving the window ------------------------------------------------------------
     int dst = -1, cnt_new = cnt_old;
@@ -264,7 +268,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
             load_q(g0);
 #pragma unroll
             for (int b = 0; b < NBUF; ++b)
-                if (first + b * step < rows.spans) { const Span sp = rows.span(first + b * step); buf[b].load_k(rows, sp, g, t); buf[b].load_v(rows, sp, g, t); }
+                if (has(first + b * step)) { const Span sp = rows.span(first + b * step); buf[b].load_k(rows, sp, g, t); buf[b].load_v(rows, sp, g, t); }
         }
         float acc[MT][4], m0 = M_NONE, m1 = M_NONE, l0 = 0.f, l1 = 0.f;
 #pragma unroll
@@ -275,7 +279,7 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
         // one span; its registers are refilled with the warp's span NBUF steps ahead as soon as a product has taken them
         auto compute = [&](Group<D, SWZ>& u, int i) {
             const Span cur = rows.span(i), nxt = rows.span(i + NBUF * step);
-            const bool more = i + NBUF * step < rows.spans;
+            const bool more = has(i + NBUF * step);
             // A product rounds its running sum towards zero, so every one starts from zero and the parts are added to the nearest
             // (NS sums side by side where the registers allow it: at d = 64 that costs 5 %).  With one running sum lse's error was 1.7
             // and 2.5 times what it is in plain fp32 (d = 64, 128; logits of 5), so it is 0.9 to 1.1 times.
@@ -336,9 +340,9 @@ __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kern
             }
             if (more) u.load_v(rows, nxt, g, t);
         };
-        for (int i = first; i < rows.spans; i += NBUF * step) {
+        for (int i = first; has(i); i += NBUF * step) {
             compute(buf[0], i);
-            if (NBUF == 2 && i + step < rows.spans) compute(buf[NBUF - 1], i + step);
+            if (NBUF == 2 && has(i + step)) compute(buf[NBUF - 1], i + step);
         }
         if (rank == 0 && g0 + MQ >= G && mover < 2 * PIECES) {  // (back by the time the write-back needs them)
             mv = reinterpret_cast<const uint4*>(mover < PIECES ? rows.K : rows.V)[(size_t)slot * PIECES + cache_chunk_pos(L, slot, mover % PIECES)];
@@ -435,6 +439,8 @@ int launch_decode_mma(const Params& p, void* cache, const void* q1, const void* 
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
     const int BH = p.B * p.H;
+    bool turn = false;
+    if (int e = decode_turns(p, &turn)) return e;
     const int warps = warps_per_sm(p.d) * n_sm, most = max_warps(p.d);
     int nw = 1, nsplit = 1;
     for (int c : {2, 3, 4, 8})
@@ -453,8 +459,9 @@ int launch_decode_mma(const Params& p, void* cache, const void* q1, const void* 
         return cudaLaunchKernelEx(&cfg, kern, (unsigned char*)cache, L, (const __nv_bfloat16*)q1, (const __nv_bfloat16*)k1,
                                   (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, p.H, p.W, p.R, p.sink, p.K, p.zthr, p.scale, p.G);
     };
-#define LTE_GO(D, S) (nw == 8 ? go(decode_mma_kernel<D, max_warps(D), S>) : nw == 4 ? go(decode_mma_kernel<D, 4, S>) : \
-                      nw == 3 ? go(decode_mma_kernel<D, 3, S>) : nw == 2 ? go(decode_mma_kernel<D, 2, S>) : go(decode_mma_kernel<D, 1, S>))
+#define LTE_GO2(D, S, T) (nw == 8 ? go(decode_mma_kernel<D, max_warps(D), S, T>) : nw == 4 ? go(decode_mma_kernel<D, 4, S, T>) : \
+                          nw == 3 ? go(decode_mma_kernel<D, 3, S, T>) : nw == 2 ? go(decode_mma_kernel<D, 2, S, T>) : go(decode_mma_kernel<D, 1, S, T>))
+#define LTE_GO(D, S) (turn ? LTE_GO2(D, S, true) : LTE_GO2(D, S, false))
     cudaError_t e;
     switch (p.d) {
         case 32: e = LTE_GO(32, false); break;
@@ -463,6 +470,7 @@ int launch_decode_mma(const Params& p, void* cache, const void* q1, const void* 
         default: return LTE_ERR_UNSUPPORTED;
     }
 #undef LTE_GO
+#undef LTE_GO2
     return cuda_status(e);
 }
 

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                                                          __nv_bfloat16* __restrict__ o1, float* __restrict__ lse1,
                                                          const float* __restrict__ cw, const float* __restrict__ cbias,
                                                          int BH, int H, int W, int R, int sink, int K,
-                                                         float zthr, float scale)
+                                                         float zthr, float scale, int turn)
 {
     extern __shared__ __align__(1024) unsigned char dsm[];
     constexpr int NW = NC / 32, NTHR = kThreads<NC>, TAPS = (kMaxTaps + NW - 1) / NW;
@@ -128,21 +128,27 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
     pdl_launch_dependents();
     pdl_wait();                                                // the previous step (or whatever wrote the cache and the inputs) has completed
 
+    // the block's heads, from the last to the first in every other step (see decode_turns; all threads read the counter before any of
+    // them can have come to its write-back, which lies behind barriers of the compute threads and behind the control lane's copies)
+    const int n_heads = bh_end - bh_begin;
+    const bool back = turn && (reinterpret_cast<const int32_t*>(cache + L.header + (size_t)bh_begin * L.stride + L.off_meta)[0] & 1) != 0;
+    auto head = [&](int it) { return back ? bh_end - 1 - it : bh_begin + it; };
+
     if (wid == NW) {
         // ======================================== control lane ==================================================
         if (lane == 0) {
             constexpr uint32_t IDESC_S = instr_desc(128, 16, false);
             constexpr uint32_t IDESC_O = instr_desc(128, 16, false, true);        // A (values) MN-major, B (p) K-major
             const uint32_t k_lo = desc_lo(sK, 16), q_lo = desc_lo(sQ, 16), vmn_lo = desc_lo(sV, 16384), p_lo = desc_lo(sP, 16);
-            const unsigned char* g0 = cache + L.header + (size_t)bh_begin * L.stride;
+            const unsigned char* g0 = cache + L.header + (size_t)head(0) * L.stride;
             bulk_load(sT, g0 + L.off_z, P.tail_bytes, bar_t0);
             bulk_load(sK, g0 + L.off_k, blk_bytes, bar_k);
             bulk_load(sV, g0 + L.off_v, blk_bytes, bar_v);
-            for (int bh = bh_begin, it = 0; bh < bh_end; ++bh, ++it) {
-                const unsigned char* gnext = cache + L.header + (size_t)(bh + 1) * L.stride;
+            for (int it = 0; it < n_heads; ++it) {
+                const unsigned char* gnext = cache + L.header + (size_t)head(it + 1) * L.stride;
                 dwait(bar_k, it & 1, 1);
                 dwait(bar_q, it & 1, 2);                       // q of this head is in the B tile (and the tail of the head before has been used)
-                if (bh + 1 < bh_end) bulk_load(sT + ((it & 1) ^ 1) * P.tail_bytes, gnext + L.off_z, P.tail_bytes, bar_t0 + 8 * ((it & 1) ^ 1));
+                if (it + 1 < n_heads) bulk_load(sT + ((it & 1) ^ 1) * P.tail_bytes, gnext + L.off_z, P.tail_bytes, bar_t0 + 8 * ((it & 1) ^ 1));
                 tc_fence_after();
 #pragma unroll
                 for (int g = 0; g < NC / 128; ++g)
@@ -151,7 +157,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                         umma(tmem + g * 16, desc64(k_lo + g * 1024 + kk * 2, kDescHi), desc64(q_lo + kk * 2, kDescHi), IDESC_S, kk > 0);
                 umma_commit(bar_s);
                 dwait(bar_p, it & 1, 3);                       // p is in its B tile; the key block is no longer read by anyone
-                if (bh + 1 < bh_end) bulk_load(sK, gnext + L.off_k, blk_bytes, bar_k);
+                if (it + 1 < n_heads) bulk_load(sK, gnext + L.off_k, blk_bytes, bar_k);
                 dwait(bar_v, it & 1, 4);
                 tc_fence_after();
 #pragma unroll
@@ -159,7 +165,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                     umma(tmem + 32, desc64(vmn_lo + kk * 128, kDescHi), desc64(p_lo + (kk >> 2) * 128 + (kk & 3) * 2, kDescHi),
                          IDESC_O, kk > 0);
                 umma_commit(bar_o);
-                if (bh + 1 < bh_end) {
+                if (it + 1 < n_heads) {
                     dwait(bar_o, it & 1, 5);                   // the value block has been consumed
                     bulk_load(sV, gnext + L.off_v, blk_bytes, bar_v);
                 }
@@ -189,10 +195,10 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                 kv_new = load128((t2 < 8 ? k1 : v1) + (size_t)bh * D + (t2 & 7) * 8);
             }
         };
-        fetch_inputs(bh_begin);
+        fetch_inputs(head(0));
 
-        for (int bh = bh_begin, it = 0; bh < bh_end; ++bh, ++it) {
-            const int tb = it & 1;
+        for (int it = 0; it < n_heads; ++it) {
+            const int bh = head(it), tb = it & 1;
             unsigned char* gblk = cache + L.header + (size_t)bh * L.stride;
             // q -> row 0 of the logits' B tile (row 0 of a swizzled tile is stored in order)
             if (tid < 8) {
@@ -293,7 +299,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
             // what the rest of this head needs, and the next head's inputs
             const uint4 kv = kv_new;
             const float bias_now = __uint_as_float(bias), v_now = __uint_as_float(tid & 1 ? v1_pair & 0xffff0000u : v1_pair << 16);
-            if (bh + 1 < bh_end) fetch_inputs(bh + 1);
+            if (it + 1 < n_heads) fetch_inputs(head(it + 1));
 
             // ---- output ----------------------------------------------------------------------------------------
             dwait(bar_o, it & 1, 10);
@@ -366,6 +372,8 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
     int n_sm = 0;
     if (int e = device_sm_count(&n_sm)) return e;
     const int BH = p.B * p.H;
+    bool turn = false;
+    if (int e = decode_turns(p, &turn)) return e;
     auto go = [&](auto nc, auto kern, PerDeviceOnce& attr) {
         constexpr int NC = decltype(nc)::value;
         const Plan P = plan_of<NC>(L);
@@ -377,7 +385,7 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
         const int n_cta = BH < slots ? BH : slots;
         return cuda_status(launch_pdl(kern, dim3(n_cta), dim3(kThreads<NC>), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
                                       (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, BH, p.H, p.W, p.R,
-                                      p.sink, p.K, p.zthr, p.scale));
+                                      p.sink, p.K, p.zthr, p.scale, (int)turn));
     };
     static PerDeviceOnce attr256, attr128;
     if (p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256>, attr256);

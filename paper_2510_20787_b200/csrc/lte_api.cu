@@ -31,6 +31,18 @@ int device_sm_count(int* n_sm)
     });
 }
 
+int decode_turns(const Params& p, bool* turn)
+{
+    static PerDevice<int> table;
+    int l2 = 0;
+    if (int e = table.get(&l2, [](int* out) {
+            int dev = 0;
+            return cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(out, cudaDevAttrL2CacheSize, dev) != cudaSuccess ? (int)LTE_ERR_CUDA : (int)LTE_OK;
+        })) return e;
+    *turn = (size_t)p.B * p.H * (p.W + p.R) * p.d * 4 > (size_t)l2 / 4 * 3;   // (bf16 keys and values)
+    return LTE_OK;
+}
+
 namespace {
 
 bool aligned(const void* p, size_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; }
