@@ -18,10 +18,17 @@
 //   - X, Y of tile g+1 are computed while the row warps work on tile g (X, Y are free as soon as they are in registers) and the
 //     accumulation of tile g runs under tile g+1; the two kinds of product are issued by two warps (one warp issues a product
 //     every 54 cycles at best).  P and dS are TMEM A operands: no trip through shared memory.
+//   - At d = 64 the halves of a tile's columns go their own way (X, Y of a half are issued when its eight row warps have the last
+//     tile's in registers, its share of the accumulation when its P, dS are there), so the products of one run under the
+//     exponentials of the other: dq + dkv and tail at the second shape below 570 -> 561, 64 x 3,000 with W = 300, R = 200 196 -> 192, the first
+//     190 -> 186.  At d = 128 a half would be 32 or 64 columns of products that read 256 of A.
 //   - Items are handed out dynamically, the longest (list tiles) first; a finished item's accumulators are read and stored
 //     under the next item's first tile.
 // One warp loads (TMA; cp.async for gathered rows).  dq forms delta at an item's start, each thread from its part of the row, and writes
 // it for the dkv pass, where another warp prepares the constants -L2, -delta scale of every tile.  Every wait is bounded.
+// Slower: two threads per row in place of four with the halves (64 columns each in two chunks: dkv 2 % at the second shape, 1 % faster at the
+// first), taking turns at the exponential unit, two of a scheduler's four row warps at a time (2 to 7 %), a barrier per half for the end
+// of the accumulation in place of one (1 %).
 // Measured (B200, us for dq + dkv, back to back in a CUDA graph, against four warps a CTA, two CTAs an SM, items dealt out beforehand; in
 // brackets: exponential unit, tensor pipe active):
 //   128 heads x 2,048, d = 64, W = R = 64                 60 + 78   (was 74 + 96)       dq 17 %, 30 %;  dkv 12 %, 30 %
@@ -47,6 +54,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 // Stages are what shared memory holds (192 KB of tiles, and O beside them).
 template <int D, bool DKV> struct Cfg {
     static constexpr int BN = D == 128 && DKV ? 64 : 128;      // d = 128 dkv: two accumulators of 128 columns leave room for 64-wide tiles
+    static constexpr int PARTS = D == 128 ? 1 : 2;             // halves of a tile's columns that go their own way
     static constexpr int AST = D == 128 ? 1 : 3, ATILE = BM * D * 2;
     static constexpr int BST = D == 64 ? 3 : DKV ? 4 : 2, BTILE = BN * D * 2;
     static constexpr int OFF_A = 0, OFF_B = AST * 2 * ATILE, OFF_O = OFF_B + BST * 2 * BTILE;   // dq: the item's O, for delta
@@ -139,8 +147,9 @@ __device__ __forceinline__ uint32_t bf16x2(float a, float b) {
 //   bar_o, bar_od (16)   dq: O (TMA) and lse (32 arrivals by cp.async) of item n are in shared memory / have been read   phase n
 //   bar_b[s]             tile g is in stage s = g % BST                                                        phase g / BST
 //   bar_bf[s]  (commit)  the accumulation of the stage's tile is complete                                       phase g / BST
-//   bar_x  (commit) X, Y of tile g are in TMEM       bar_xf (16) they are in registers                           phase g
-//   bar_p  (16) P, dS of tile g are in TMEM and the accumulation of tile g-1 has been awaited   bar_acc (commit) it is complete   phase g
+//   bar_x[h]  (commit) X, Y of part h of tile g are in TMEM      bar_xf[h] (row warps of the part) they are in registers   phase g
+//   bar_p[h]  (row warps of the part) its P, dS are in TMEM and the accumulation of tile g-1 has been awaited                  phase g
+//   bar_acc   (commit) the accumulation of tile g is complete                                                              phase g
 //   bar_es[b] (4)  STAGED: the outputs of item n have left its A buffer                                           phase n / AST
 //   bar_of (16) the accumulators of item n have been read out                                                    phase n
 //   bar_i[n & 7]         Info of item n is in the ring                                                           phase n >> 3
@@ -154,14 +163,15 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
 {
     using C = Cfg<D, DKV>;
     constexpr int BN = C::BN, SUB = D / 64, CW = BN / 4, AST = C::AST, BST = C::BST, ATILE = C::ATILE, BTILE = C::BTILE;
+    constexpr int PARTS = C::PARTS, PN = BN / PARTS, PW = NRW / PARTS;   // columns and row warps of a part
     constexpr bool STAGED = D == 64;                           // outputs leave through the item's A buffers as tiles
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     if ((base & 1023u) != 0) { if (threadIdx.x == 0) atomicExch(&g_bwd_status.code, 9); return; }
     const uint32_t sA = base + C::OFF_A, sB = base + C::OFF_B, bars = base + C::OFF_BAR;
     const uint32_t bar_a = bars, bar_ga = bars + 32, bar_af = bars + 64, bar_b = bars + 96, bar_bf = bars + 128, bar_i = bars + 160;   // 4 slots each, bar_i 8
-    const uint32_t bar_x = bars + 224, bar_xf = bars + 232, bar_p = bars + 240, bar_acc = bars + 248, bar_of = bars + 256, bar_c = bars + 264;
-    const uint32_t bar_cc = bars + 272, bar_cf = bars + 288, bar_o = bars + 304, bar_od = bars + 312, bar_es = bars + 320, tmem_slot = bars + 352, answer = bars + 368;   // bar_es 4
+    const uint32_t bar_x = bars + 224, bar_xf = bars + 376, bar_p = bars + 392, bar_acc = bars + 248, bar_of = bars + 256, bar_c = bars + 264;
+    const uint32_t bar_cc = bars + 272, bar_cf = bars + 288, bar_o = bars + 304, bar_od = bars + 312, bar_es = bars + 320, tmem_slot = bars + 352, answer = bars + 416;   // bar_es 4, bar_x, bar_xf, bar_p 2
     auto slot = [&](int n) { return reinterpret_cast<volatile Info*>(smem_raw + C::OFF_INFO + (n & 7) * 64); };
     float* const consts = reinterpret_cast<float*>(smem_raw + C::OFF_C);
     volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + C::OFF_BAR + 352);
@@ -171,13 +181,15 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
 #pragma unroll
         for (int s = 0; s < 2; ++s) { mbar_init(bar_cc + 8 * s, 1); mbar_init(bar_cf + 8 * s, NRW); }
 #pragma unroll
+        for (int s = 0; s < PARTS; ++s) { mbar_init(bar_x + 8 * s, 1); mbar_init(bar_xf + 8 * s, PW); mbar_init(bar_p + 8 * s, PW); }
+#pragma unroll
         for (int s = 0; s < 4; ++s) {
             mbar_init(bar_a + 8 * s, 1); mbar_init(bar_ga + 8 * s, 32); mbar_init(bar_af + 8 * s, 1);
             mbar_init(bar_b + 8 * s, 1); mbar_init(bar_bf + 8 * s, 1); mbar_init(bar_es + 8 * s, 4);
         }
 #pragma unroll
         for (int s = 0; s < 8; ++s) mbar_init(bar_i + 8 * s, 1);
-        mbar_init(bar_x, 1); mbar_init(bar_xf, NRW); mbar_init(bar_p, NRW); mbar_init(bar_acc, 1); mbar_init(bar_of, NRW); mbar_init(bar_c, 1);
+        mbar_init(bar_acc, 1); mbar_init(bar_of, NRW); mbar_init(bar_c, 1);
         mbar_init(bar_o, 33); mbar_init(bar_od, NRW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -316,7 +328,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
         __syncwarp();
     } else if (warp == W_XY) {
         // ================================= X, Y products (an elected thread issues; the whole warp walks the loop) =
-        constexpr uint32_t IDESC = instr_desc(BM, BN, false);
+        constexpr uint32_t IDESC = instr_desc(BM, PN, false);
         const uint32_t a_lo = desc_lo(sA, 16), b_lo = desc_lo(sB, 16);
         uint32_t g = 0, par_a = 0;                             // parities of bar_a (bits 0 .. 3), bar_ga (4 .. 7)
         Item it;
@@ -328,20 +340,23 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
             for (int t = 0; uni(t < it.n_tiles); ++t, ++g) {
                 const uint32_t s = g % BST;
                 bwait_u(bar_b + 8 * s, (g / BST) & 1u, 2);
-                if (uni(g > 0)) bwait_u(bar_xf, (g - 1) & 1, 3);      // the previous tile's X, Y are in registers
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), b1 = b_lo + s * (2 * BTILE >> 4);
 #pragma unroll
-                    for (int xy = 0; xy < 2; ++xy)
+                for (int h = 0; h < PARTS; ++h) {
+                    if (uni(g > 0)) bwait_u(bar_xf + 8 * h, (g - 1) & 1, 3);   // the previous tile's X, Y are in registers
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), b1 = b_lo + s * (2 * BTILE >> 4) + h * (PN * 8);
 #pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk)
-                            umma(tmem + (xy ? C::Y : C::X), desc64(a1 + xy * (ATILE >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                                 desc64(b1 + xy * (BTILE >> 4) + (kk >> 2) * (BN * 8) + (kk & 3) * 2, kDescHi), IDESC, kk > 0);
-                    umma_commit(bar_x);
-                    if (t == it.n_tiles - 1) umma_commit(bar_af + 8 * ab);
+                        for (int xy = 0; xy < 2; ++xy)
+#pragma unroll
+                            for (int kk = 0; kk < D / 16; ++kk)
+                                umma(tmem + (xy ? C::Y : C::X) + h * PN, desc64(a1 + xy * (ATILE >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
+                                     desc64(b1 + xy * (BTILE >> 4) + (kk >> 2) * (BN * 8) + (kk & 3) * 2, kDescHi), IDESC, kk > 0);
+                        umma_commit(bar_x + 8 * h);
+                        if (h == PARTS - 1 && t == it.n_tiles - 1) umma_commit(bar_af + 8 * ab);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
         }
     } else if (warp == W_ACC) {
@@ -354,22 +369,28 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
             for (int t = 0; uni(t < it.n_tiles); ++t, ++g) {
                 const uint32_t s = g % BST;
                 if (uni(t == 0 && n > 0)) bwait_u(bar_of, (n - 1) & 1, 13);   // the previous item's accumulators have been read out
-                bwait_u(bar_p, g & 1, 7);
-                tc_fence_after();
-                if (elect_one()) {
-                    const uint32_t b1 = b_lo + s * (2 * BTILE >> 4);
-                    if (DKV) {
 #pragma unroll
-                        for (int kk = 0; kk < BN / 16; ++kk)
-                            umma_ts(tmem + C::ACC1, tmem + C::P + kk * 8, desc64(b1 + (BTILE >> 4) + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+                for (int h = 0; h < PARTS; ++h) {
+                    constexpr int KP = PN / 16;
+                    bwait_u(bar_p + 8 * h, g & 1, 7);
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t b1 = b_lo + s * (2 * BTILE >> 4);
+                        if (DKV) {
+#pragma unroll
+                            for (int kk = h * KP; kk < h * KP + KP; ++kk)
+                                umma_ts(tmem + C::ACC1, tmem + C::P + kk * 8, desc64(b1 + (BTILE >> 4) + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+                        }
+#pragma unroll
+                        for (int kk = h * KP; kk < h * KP + KP; ++kk)
+                            umma_ts(tmem + C::ACC0, tmem + C::DS + kk * 8, desc64(b1 + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+                        if (h == PARTS - 1) {
+                            umma_commit(bar_acc);
+                            umma_commit(bar_bf + 8 * s);
+                        }
                     }
-#pragma unroll
-                    for (int kk = 0; kk < BN / 16; ++kk)
-                        umma_ts(tmem + C::ACC0, tmem + C::DS + kk * 8, desc64(b1 + kk * 128, kDescHi), IDESC, (t > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(bar_acc);
-                    umma_commit(bar_bf + 8 * s);
+                    __syncwarp();
                 }
-                __syncwarp();
             }
         }
     } else if (warp >= NRW) {
@@ -400,7 +421,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
     } else {
         // ================================= row warps ==============================================================
         // Four threads per row: thread `row` of warps 4 q .. 4 q + 3 takes columns [q CW, q CW + CW) of every tile.
-        const int quarter = warp & 3, q = warp >> 2, row = quarter * 32 + lane, c0 = q * CW;
+        const int quarter = warp & 3, q = warp >> 2, row = quarter * 32 + lane, c0 = q * CW, part8 = q / (4 / PARTS) * 8;
         const float c2 = args.scale * kLog2e;
         const uint64_t c2_2 = pack2(c2, c2), scale_2 = pack2(args.scale, args.scale);
         const uint32_t trow = tmem + (((uint32_t)(quarter * 32)) << 16);   // this warp's TMEM lanes
@@ -558,7 +579,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                 uint32_t ds[CW / 2], pp[CW / 2];
                 const float* col = consts + (g & 1) * 256 + c0;
                 if (DKV) bwait(bar_cc + 8 * (g & 1), (g >> 1) & 1, 16);
-                bwait(bar_x, g & 1, 5);
+                bwait(bar_x + part8, g & 1, 5);
                 tc_fence_after();
                 if (some) {
                     uint32_t x[CW], y[CW];
@@ -567,7 +588,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                     tmem_wait_ld();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_xf);        // X, Y of tile g+1 may overwrite the buffers
+                    if (lane == 0) mbar_arrive(bar_xf + part8);   // X, Y of tile g+1 may overwrite the buffers
                     if (!plain) {
 #pragma unroll
                         for (int c = 0; c < CW; ++c) x[c] = (vm & (1u << c)) ? x[c] : 0xff800000u;   // -inf: P = 0
@@ -595,7 +616,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                     }
                 } else {
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_xf);
+                    if (lane == 0) mbar_arrive(bar_xf + part8);
 #pragma unroll
                     for (int c = 0; c < CW / 2; ++c) { ds[c] = 0u; pp[c] = 0u; }
                 }
@@ -607,7 +628,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) { mbar_arrive(bar_p); if (DKV) mbar_arrive(bar_cf + 8 * (g & 1)); }
+                if (lane == 0) { mbar_arrive(bar_p + part8); if (DKV) mbar_arrive(bar_cf + 8 * (g & 1)); }
             }
             l_list = it.list; l_bh = it.bh; l_row = r_abs;
             l_dr = dr2; dr2 = 0ull;
