@@ -24,6 +24,9 @@
 //     190 -> 186.  At d = 128 a half would be 32 or 64 columns of products that read 256 of A.
 //   - Items are handed out dynamically, the longest (list tiles) first; a finished item's accumulators are read and stored
 //     under the next item's first tile.
+//   - dq at d = 128 has room for two 64 KB tiles, and dQ's product holds K: three stages of K and one of V (free once Y is computed, before
+//     the tile's exponentials) instead of two of both, 16 heads x 8,192 255 -> 246 for the call (at d = 64, with three stages of both, the
+//     barriers more cost 2 %).
 // One warp loads (TMA; cp.async for gathered rows).  dq forms delta at an item's start, each thread from its part of the row, and writes
 // it for the dkv pass, where another warp prepares the constants -L2, -delta scale of every tile.  Every wait is bounded.
 // Slower: two threads per row in place of four with the halves (64 columns each in two chunks: dkv 2 % at the second shape, 1 % faster at the
@@ -56,8 +59,9 @@ template <int D, bool DKV> struct Cfg {
     static constexpr int BN = D == 128 && DKV ? 64 : 128;      // d = 128 dkv: two accumulators of 128 columns leave room for 64-wide tiles
     static constexpr int PARTS = D == 128 ? 1 : 2;             // halves of a tile's columns that go their own way
     static constexpr int AST = D == 128 ? 1 : 3, ATILE = BM * D * 2;
-    static constexpr int BST = D == 64 ? 3 : DKV ? 4 : 2, BTILE = BN * D * 2;
-    static constexpr int OFF_A = 0, OFF_B = AST * 2 * ATILE, OFF_O = OFF_B + BST * 2 * BTILE;   // dq: the item's O, for delta
+    static constexpr bool SPLIT = D == 128 && !DKV;            // K (needed twice) and V (needed once) in stages of their own
+    static constexpr int BST = D == 128 && DKV ? 4 : 3, VST = 1, BTILE = BN * D * 2;   // stages of B1 and B2; SPLIT: of B1, of B2
+    static constexpr int OFF_A = 0, OFF_B = AST * 2 * ATILE, OFF_O = OFF_B + (SPLIT ? BST + VST : 2 * BST) * BTILE;   // dq: the item's O, for delta
     static constexpr int OFF_BAR = OFF_O + (DKV ? 0 : ATILE);
     static constexpr int OFF_INFO = OFF_BAR + 512;             // ring of eight items' Info, 64 bytes apart
     static constexpr int OFF_C = OFF_INFO + 512;               // dkv: constants [2][2][128];  dq: lse [2][128]
@@ -145,7 +149,8 @@ __device__ __forceinline__ uint32_t bf16x2(float a, float b) {
 //   bar_a[b], bar_ga[b]  rows of item n are in buffer b = n % AST: by TMA / gathered (dkv list tiles; 32 arrivals by cp.async completion)
 //   bar_af[b]  (commit)  the item's last X, Y are complete                                                     phase n / AST
 //   bar_o, bar_od (16)   dq: O (TMA) and lse (32 arrivals by cp.async) of item n are in shared memory / have been read   phase n
-//   bar_b[s]             tile g is in stage s = g % BST                                                        phase g / BST
+//   bar_b[s]             tile g (SPLIT: its K) is in stage s = g % BST                                          phase g / BST
+//   bar_v[s], bar_vf[s]  SPLIT: V of tile g is in stage s = g % VST / (commit) X, Y of the tile are complete      phase g / VST
 //   bar_bf[s]  (commit)  the accumulation of the stage's tile is complete                                       phase g / BST
 //   bar_x[h]  (commit) X, Y of part h of tile g are in TMEM      bar_xf[h] (row warps of the part) they are in registers   phase g
 //   bar_p[h]  (row warps of the part) its P, dS are in TMEM and the accumulation of tile g-1 has been awaited                  phase g
@@ -162,7 +167,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
               const __grid_constant__ CUtensorMap tmL2, const __grid_constant__ CUtensorMap tmS1, const __grid_constant__ CUtensorMap tmS2, const Args args)
 {
     using C = Cfg<D, DKV>;
-    constexpr int BN = C::BN, SUB = D / 64, CW = BN / 4, AST = C::AST, BST = C::BST, ATILE = C::ATILE, BTILE = C::BTILE;
+    constexpr int BN = C::BN, SUB = D / 64, CW = BN / 4, AST = C::AST, BST = C::BST, VST = C::VST, BPITCH = (C::SPLIT ? 1 : 2) * C::BTILE, ATILE = C::ATILE, BTILE = C::BTILE;
     constexpr int PARTS = C::PARTS, PN = BN / PARTS, PW = NRW / PARTS;   // columns and row warps of a part
     constexpr bool STAGED = D == 64;                           // outputs leave through the item's A buffers as tiles
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -171,7 +176,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
     const uint32_t sA = base + C::OFF_A, sB = base + C::OFF_B, bars = base + C::OFF_BAR;
     const uint32_t bar_a = bars, bar_ga = bars + 32, bar_af = bars + 64, bar_b = bars + 96, bar_bf = bars + 128, bar_i = bars + 160;   // 4 slots each, bar_i 8
     const uint32_t bar_x = bars + 224, bar_xf = bars + 376, bar_p = bars + 392, bar_acc = bars + 248, bar_of = bars + 256, bar_c = bars + 264;
-    const uint32_t bar_cc = bars + 272, bar_cf = bars + 288, bar_o = bars + 304, bar_od = bars + 312, bar_es = bars + 320, tmem_slot = bars + 352, answer = bars + 416;   // bar_es 4, bar_x, bar_xf, bar_p 2
+    const uint32_t bar_cc = bars + 272, bar_cf = bars + 288, bar_o = bars + 304, bar_od = bars + 312, bar_es = bars + 320, tmem_slot = bars + 352, answer = bars + 416, bar_v = bars + 432, bar_vf = bars + 464;   // bar_es, bar_v, bar_vf 4, bar_x, bar_xf, bar_p 2
     auto slot = [&](int n) { return reinterpret_cast<volatile Info*>(smem_raw + C::OFF_INFO + (n & 7) * 64); };
     float* const consts = reinterpret_cast<float*>(smem_raw + C::OFF_C);
     volatile uint32_t* tmem_slot_gen = reinterpret_cast<volatile uint32_t*>(smem_raw + C::OFF_BAR + 352);
@@ -186,6 +191,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
         for (int s = 0; s < 4; ++s) {
             mbar_init(bar_a + 8 * s, 1); mbar_init(bar_ga + 8 * s, 32); mbar_init(bar_af + 8 * s, 1);
             mbar_init(bar_b + 8 * s, 1); mbar_init(bar_bf + 8 * s, 1); mbar_init(bar_es + 8 * s, 4);
+            mbar_init(bar_v + 8 * s, 1); mbar_init(bar_vf + 8 * s, 1);
         }
 #pragma unroll
         for (int s = 0; s < 8; ++s) mbar_init(bar_i + 8 * s, 1);
@@ -299,17 +305,21 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
             if (DKV) publish();
             int blk = 0, h = DKV ? it.bh * args.G : it.bhk;    // dkv: block of the query head, query head
             for (int t = 0; t < it.n_tiles; ++t, ++g) {
-                const uint32_t s = g % BST, b1 = sB + s * 2 * BTILE, b2 = b1 + BTILE;
+                const uint32_t s = g % BST, sv = g % VST, b1 = sB + s * BPITCH, b2 = C::SPLIT ? sB + (BST + sv) * BTILE : b1 + BTILE;
+                const uint32_t bar2 = C::SPLIT ? bar_v + 8 * sv : bar_b + 8 * s;
+                const bool list = !DKV && t >= it.n_win;
+                const int y = DKV ? it.a + blk * BN : list ? (t - it.n_win) * BN : it.j_start + t * BN;
                 if (g >= (uint32_t)BST) bwait(bar_bf + 8 * s, (g / BST - 1) & 1u, 6);
                 if (lane == 0) {
-                    const bool list = !DKV && t >= it.n_win;
-                    const int y = DKV ? it.a + blk * BN : list ? (t - it.n_win) * BN : it.j_start + t * BN;
-                    mbar_expect_tx(bar_b + 8 * s, 2 * BTILE);
+                    mbar_expect_tx(bar_b + 8 * s, BPITCH);
 #pragma unroll
-                    for (int sb = 0; sb < SUB; ++sb) {
-                        tma_load_3d(b1 + sb * BN * 128, list ? &tmL1 : &tmB1, sb * 64, y, h, bar_b + 8 * s);
-                        tma_load_3d(b2 + sb * BN * 128, list ? &tmL2 : &tmB2, sb * 64, y, h, bar_b + 8 * s);
-                    }
+                    for (int sb = 0; sb < SUB; ++sb) tma_load_3d(b1 + sb * BN * 128, list ? &tmL1 : &tmB1, sb * 64, y, h, bar_b + 8 * s);
+                }
+                if (C::SPLIT && g >= (uint32_t)VST) bwait(bar_vf + 8 * sv, (g / VST - 1) & 1u, 24);
+                if (lane == 0) {
+                    if (C::SPLIT) mbar_expect_tx(bar2, BTILE);
+#pragma unroll
+                    for (int sb = 0; sb < SUB; ++sb) tma_load_3d(b2 + sb * BN * 128, list ? &tmL2 : &tmB2, sb * 64, y, h, bar2);
                 }
                 if (!DKV && t == 0) {                          // tile 0 is a window tile; the list is looked up while it is on its way
                     const int last = min(it.row0 + BM - 1, args.Tlen - 1) - it.row0;
@@ -344,15 +354,23 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                 for (int h = 0; h < PARTS; ++h) {
                     if (uni(g > 0)) bwait_u(bar_xf + 8 * h, (g - 1) & 1, 3);   // the previous tile's X, Y are in registers
                     tc_fence_after();
+                    const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), hb = h * (PN * 8), sv = g % VST;
+                    const uint32_t b1 = b_lo + s * (BPITCH >> 4), b2 = C::SPLIT ? b_lo + (BST + sv) * (BTILE >> 4) : b1 + (BTILE >> 4);
+                    auto product = [&](uint32_t d, uint32_t a, uint32_t b) {
+#pragma unroll
+                        for (int kk = 0; kk < D / 16; ++kk)
+                            umma(d + h * PN, desc64(a + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi), desc64(b + hb + (kk >> 2) * (BN * 8) + (kk & 3) * 2, kDescHi), IDESC, kk > 0);
+                    };
+                    if (C::SPLIT) {
+                        if (elect_one()) product(tmem + C::X, a1, b1);
+                        __syncwarp();
+                        if (h == 0) { bwait_u(bar_v + 8 * sv, (g / VST) & 1u, 25); tc_fence_after(); }
+                    }
                     if (elect_one()) {
-                        const uint32_t a1 = a_lo + ab * (2 * ATILE >> 4), b1 = b_lo + s * (2 * BTILE >> 4) + h * (PN * 8);
-#pragma unroll
-                        for (int xy = 0; xy < 2; ++xy)
-#pragma unroll
-                            for (int kk = 0; kk < D / 16; ++kk)
-                                umma(tmem + (xy ? C::Y : C::X) + h * PN, desc64(a1 + xy * (ATILE >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2, kDescHi),
-                                     desc64(b1 + xy * (BTILE >> 4) + (kk >> 2) * (BN * 8) + (kk & 3) * 2, kDescHi), IDESC, kk > 0);
+                        if (!C::SPLIT) product(tmem + C::X, a1, b1);
+                        product(tmem + C::Y, a1 + (ATILE >> 4), b2);
                         umma_commit(bar_x + 8 * h);
+                        if (C::SPLIT && h == PARTS - 1) umma_commit(bar_vf + 8 * sv);
                         if (h == PARTS - 1 && t == it.n_tiles - 1) umma_commit(bar_af + 8 * ab);
                     }
                     __syncwarp();
@@ -375,7 +393,7 @@ bwd_tc_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ 
                     bwait_u(bar_p + 8 * h, g & 1, 7);
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint32_t b1 = b_lo + s * (2 * BTILE >> 4);
+                        const uint32_t b1 = b_lo + s * (BPITCH >> 4);
                         if (DKV) {
 #pragma unroll
                             for (int kk = h * KP; kk < h * KP + KP; ++kk)
