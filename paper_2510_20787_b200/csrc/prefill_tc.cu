@@ -8,8 +8,9 @@
 //             span, then the head's retained rows that any of the item's rows may see (compacted beforehand where the caller
 //             brought a workspace; otherwise the load warp gathers them row by row into the same swizzled layout).  Four softmax
 //             warps (a thread per row), one warp issuing the products, one issuing the loads.
-//   S(g) = Q K^T    two buffers, and P(g) takes the place of S(g): S(g+2) is issued behind P V of tile g, so S(g+1) is there when a warp
-//             comes to it.  96 columns because two such buffers and O fill the 256 TMEM columns of a CTA: S [0,96), [96,192), O [192,256)
+//   S(g) = Q K^T    two buffers, and P(g) takes the place of S(g): S(g+2) is issued when P V of tile g is complete (products of different
+//             accumulators need not keep their order; the wait costs 0.3 % at the first shape below, nothing at the others), so S(g+1) is
+//             there when a warp comes to it.  96 columns because two such buffers and O fill the 256 TMEM columns of a CTA: S [0,96), [96,192), O [192,256)
 //   softmax   mask from positions.  A tile that all of the warp's rows see is taken whole (its 96 logits in registers, one vote); others
 //             go in chunks of 32 columns, which are skipped where no row sees any.  The reference is the maximum of the first columns
 //             seen and moves only for logits 2^8 above it (in an item's first tiles 2); exp2 with the scale folded in.  O is divided by
@@ -292,7 +293,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             landed(bar_k, bar_gk, ws.t < ws.n_win, ws.r, 0, 3, 2);
             ++ws.t;
             tc_fence_after();
-            const uint32_t s_tm = tmem + S_COL + (ws.g & 1) * BN;    // P of the tile two before, which lay there, is the operand of an earlier product
+            const uint32_t s_tm = tmem + S_COL + (ws.g & 1) * BN;    // P of the tile two before, which lay there, has been multiplied
             if (elect_one()) {
                 const uint32_t qd = q_lo + (ws.n & 1) * (QTILE >> 4), kd = k_lo + ws.r.s * (TILE >> 4);
 #pragma unroll
@@ -326,8 +327,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 umma_commit(bar_vf + 8 * wp.r.s);
             }
             __syncwarp();
+            if (uni(more)) {                                   // the next S but one takes the place of the P that this product reads
+                mbar_wait_u(bar_pv + 8 * (wp.g & 1), (wp.g >> 1) & 1, 3);
+                more = mma_s();
+            }
             ++wp.t; ++wp.g; wp.r.next<VST>();
-            if (uni(more)) more = mma_s();
         }
     } else {
         // =================================== softmax warps ==================================================
