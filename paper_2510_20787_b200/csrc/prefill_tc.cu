@@ -12,10 +12,11 @@
 //             accumulators need not keep their order; the wait costs 0.3 % at the first shape below, nothing at the others), so S(g+1) is
 //             there when a warp comes to it.  96 columns because two such buffers and O fill the 256 TMEM columns of a CTA: S [0,96), [96,192), O [192,256)
 //   softmax   mask from positions.  A tile that all of the warp's rows see is taken whole (its 96 logits in registers, one vote); others
-//             go in chunks of 32 columns, which are skipped where no row sees any.  The reference is the maximum of the first columns
-//             seen and moves only for logits 2^8 above it (in an item's first tiles 2); exp2 with the scale folded in.  O is divided by
-//             the sum of P, so that its rounding cancels as far as it is common to the row, and lse is the logarithm of the sum of the
-//             weights themselves (with the weights' sum alone O's error is 2 % larger, with P's alone lse's 1e-3).
+//             go in chunks of 32 columns, which are skipped where no row sees any, twice: for the tile's maximum and for the weights.  The
+//             reference is the maximum of the first tile seen and moves to a later tile's that is more than 2^2 above it (in an item's
+//             first tiles 2); exp2 with the scale folded in.  O is divided by the sum of P, so that its rounding cancels as far as it is
+//             common to the row, and lse is the logarithm of the sum of the weights themselves (with the weights' sum alone O's error is
+//             2 % larger, with P's alone lse's 1e-3).
 //   O += P V  P as the TMEM A operand, V as the MN-major shared-memory operand; O is read and stored under the next item's first tile
 // How many retained entries a row sees: the load warp finds an item's place in the list (a 32-way search) and hands out, one
 // item ahead, a bit map of the entries that fall between the limits of the item's first and last row.
@@ -24,10 +25,14 @@
 // status word and the kernel still terminates.
 //
 // Measured (B200, the call with a workspace, back to back in a CUDA graph; before: two threads per row, 128-key tiles, one S buffer):
-//   128 query heads x 4,096, W = 768, R = 512 half used     179 us (601 TFLOP/s), before 198 (192 with its waits out of line)
+//   128 query heads x 4,096, W = 768, R = 512 half used     176 us (611 TFLOP/s), before 198 (192 with its waits out of line)
 //   64 heads x 4,096, W = R = 128                          45 us, before 49     128 x 2,048, W = R = 64   36 us, before 44
 //   48 x 3,001, W = 300, R = 200                           38 us, before 44     64 x 4,096, W = 32, R = 16   34 us, before 42
-// O's error against 64 bits is 0.97 to 1.006 times what it was, lse's the same.
+// O's error against 64 bits, logits of N(0,1) rising by 0 to 1 per key, W = 64 to 768: 0.945 to 0.998 times what it was, 1.000 to 1.006 times
+// that of weights rounded beside each row's own maximum (tests/test_gpu_prefill_rounding.py).  Without the look at a partial tile's maximum, chunk
+// by chunk, a reference that moves within a tile and what is there of P rescaled (rounded a second time): 177 us here, 45, 36, 38, 34,
+// and O's error up to 1.04 times what it was.  The maximum in a pass of its own, all chunks fetched again: 183, 49, 40, 41, 36; partial tiles' chunks
+// all in registers, on one path with whole tiles: 190, 45, 36, 40, 33.
 // Tried and slower, the first line unless said otherwise: every tile in rolled chunks (192 us; the small windows 43 and 35), every tile
 // whole (183; 48 and 39), the next tile's logits fetched ahead (194), the maximum asked only behind the exponentials (193), tiles of 80
 // keys with the sum of P as sixteen columns more of the product (188), four CTAs per SM with one S buffer and 64-key tiles (181; 44 and 38),
@@ -56,7 +61,7 @@ constexpr int OFF_Q = 0, OFF_K = QST * QTILE, OFF_V = OFF_K + KST * TILE, OFF_BA
 constexpr int OFF_INFO = OFF_BAR + 320;                            // ring of four items' Info
 constexpr int OFF_LV = OFF_INFO + 4 * 64;                          // STREAM: the leave times of a retained tile, [4 warps][96]
 constexpr int smem_bytes(bool stream) { return OFF_LV + (stream ? 4 * BN * 4 : 0); }
-constexpr uint32_t TMEM_COLS = 256, S_COL = 0, O_COL = 2 * BN;     // two S buffers, P in the place of its S
+constexpr uint32_t TMEM_COLS = 256, S_COL = 0, O_COL = 2 * BN, P_AT = BN / 2;   // two S buffers, P in the second half of its S
 
 // An item: a 128-query tile of one (b,h).  Items are numbered from the last query tile of every head down to the first: later
 // tiles see more retained rows and cost more.  The grid has a block per item, but a block that has run out of work takes the
@@ -319,7 +324,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             mbar_wait_u(bar_p + 8 * (wp.g & 1), (wp.g >> 1) & 1u, 7);
             tc_fence_after();
             if (elect_one()) {
-                const uint32_t vd = v_lo + wp.r.s * (TILE >> 4), p_tm = tmem + S_COL + (wp.g & 1) * BN;
+                const uint32_t vd = v_lo + wp.r.s * (TILE >> 4), p_tm = tmem + S_COL + (wp.g & 1) * BN + P_AT;
 #pragma unroll
                 for (int kk = 0; kk < BN / 16; ++kk)
                     umma_ts(tmem + O_COL, p_tm + kk * 8, desc64(vd + kk * 128, kDescHi), IDESC_O, (wp.t > 0 || kk > 0) ? 1u : 0u);
@@ -411,11 +416,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     __syncwarp();
                 }
                 const uint32_t s_col = trow + S_COL + (g & 1) * BN;
-                // The reference is the maximum of the first columns that the row sees and only moves when a logit is far above it (exp2
-                // arguments stay <= 8; an item's first tiles follow closer: the nearer it is to the largest logit, the smaller P's rounding
-                // beside the large weights).  Then what has been added up is rescaled, P of this tile's first `done` chunks included.
-                auto follow = [&](float m_here, int done) {
-                    const bool up = m_here > m_run + (t < 2 ? 1.f : 8.f);
+                // The reference is the maximum of the first tile that the row sees and moves to a later tile's that is more than 2^2 above it (in
+                // an item's first tiles 2): the nearer it is to the largest logit, the smaller P's rounding beside the large weights, whose
+                // largest has none at the reference.  Then what has been added up is rescaled.
+                auto follow = [&](float m_here) {
+                    const bool up = m_here > m_run + (t < 2 ? 1.f : 2.f);
                     if (!__any_sync(0xffffffffu, up)) return;
                     const float alpha = up && m_run != -INFINITY ? fast_exp2(m_run - m_here) : 1.f;   // (1: nothing has been added up for this row)
                     if (up) m_run = m_here;
@@ -434,18 +439,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                             }
                         }
                         tmem_wait_st();
-#pragma unroll 1
-                        for (int c4 = 0; c4 < done; ++c4) {
-                            uint32_t q4[16];
-                            tmem_ld16(s_col + c4 * 16, q4);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(q4[c] << 16) * alpha, __uint_as_float(q4[c] & 0xffff0000u) * alpha);
-                                q4[c] = *reinterpret_cast<const uint32_t*>(&h);
-                            }
-                            tmem_st16(s_col + c4 * 16, q4);
-                        }
                         ls[0] = mul2(ls[0], pack2(alpha, alpha)); ls[1] = mul2(ls[1], pack2(alpha, alpha)); lr[0] *= alpha; lr[1] *= alpha;
                     }
                 };
@@ -479,53 +472,66 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         mr[((c >> 1) + 3) & 7] = max3(mr[((c >> 1) + 3) & 7], __uint_as_float(x1[c]), __uint_as_float(x1[c + 1]));
                         mr[((c >> 1) + 6) & 7] = max3(mr[((c >> 1) + 6) & 7], __uint_as_float(x2[c]), __uint_as_float(x2[c + 1]));
                     }
-                    follow(max3(max3(mr[0], mr[1], mr[2]), max3(mr[3], mr[4], mr[5]), fmaxf(mr[6], mr[7])) * c2, 0);
+                    follow(max3(max3(mr[0], mr[1], mr[2]), max3(mr[3], mr[4], mr[5]), fmaxf(mr[6], mr[7])) * c2);
                     const float neg_m = m_run == -INFINITY ? 0.f : -m_run;
                     const uint64_t neg_m2 = pack2(neg_m, neg_m);
                     weigh(x0, pk, neg_m2);
-                    tmem_st16(s_col, pk);                      // (over columns of S that have been taken)
+                    tmem_st16(s_col + P_AT, pk);               // (over columns of S that have been taken)
                     weigh(x1, pk, neg_m2);
-                    tmem_st16(s_col + 16, pk);
+                    tmem_st16(s_col + P_AT + 16, pk);
                     weigh(x2, pk, neg_m2);
-                    tmem_st16(s_col + 32, pk);
+                    tmem_st16(s_col + P_AT + 32, pk);
                 } else {
+                    // The chunks that any row sees: up to the last one for the maximum, then down again for the weights, the last one's logits
+                    // being there still and the others fetched again (P has the columns from P_AT on, so that on the way down it
+                    // lies over chunks that have been taken).
+                    uint32_t pk[16];
+                    const int first = max(u_lo, 0) & ~31, last = min(u_hi, BN - 1) & ~31;
+                    float mr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                    uint64_t neg_m2 = 0ull;
+                    int at = first;
+                    bool down = false;
 #pragma unroll 1
-                    for (int cb = 0; cb < CHUNKS; ++cb) {
-                        uint32_t pk[16];
-                        const int at = cb * 32;
-                        if (at <= u_hi && at + 31 >= u_lo) {
-                            uint32_t x[32];
-                            tmem_ld32(s_col + at, x);
-                            tmem_wait_ld();
-                            if (timed || at < n_lo || at + 31 > n_hi) {   // some row does not see all of it
-                                const int a = min(max(c_lo - at, 0), 32), b = min(max(c_hi - at + 1, 0), 32);
-                                const uint32_t below_b = b >= 32 ? 0xffffffffu : ((1u << b) - 1u), below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
-                                uint32_t vm = b > a ? (below_b & ~below_a) : 0u;
-                                if (timed) {
-                                    uint32_t m = 0;
+                    while (u_hi >= 0 && u_lo < BN) {
+                        uint32_t x[32];
+                        tmem_ld32(s_col + at, x);
+                        tmem_wait_ld();
+                        if (timed || at < n_lo || at + 31 > n_hi) {   // some row does not see all of it
+                            const int a = min(max(c_lo - at, 0), 32), b = min(max(c_hi - at + 1, 0), 32);
+                            const uint32_t below_b = b >= 32 ? 0xffffffffu : ((1u << b) - 1u), below_a = a >= 32 ? 0xffffffffu : ((1u << a) - 1u);
+                            uint32_t vm = b > a ? (below_b & ~below_a) : 0u;
+                            if (timed) {
+                                uint32_t m = 0;
 #pragma unroll
-                                    for (int c = 0; c < 32; c += 4) {
-                                        const int4 l4 = *reinterpret_cast<const int4*>(slv + at + c);
-                                        m |= (l4.x > i ? 1u : 0u) << c; m |= (l4.y > i ? 2u : 0u) << c;
-                                        m |= (l4.z > i ? 4u : 0u) << c; m |= (l4.w > i ? 8u : 0u) << c;
-                                    }
-                                    vm &= m;
+                                for (int c = 0; c < 32; c += 4) {
+                                    const int4 l4 = *reinterpret_cast<const int4*>(slv + at + c);
+                                    m |= (l4.x > i ? 1u : 0u) << c; m |= (l4.y > i ? 2u : 0u) << c;
+                                    m |= (l4.z > i ? 4u : 0u) << c; m |= (l4.w > i ? 8u : 0u) << c;
                                 }
-#pragma unroll
-                                for (int c = 0; c < 32; ++c) x[c] = (vm & (1u << c)) ? x[c] : 0xff800000u;   // -inf
+                                vm &= m;
                             }
-                            float mr[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) x[c] = (vm & (1u << c)) ? x[c] : 0xff800000u;   // -inf
+                        }
+                        if (!down) {
 #pragma unroll
                             for (int c = 0; c < 32; c += 2) mr[(c >> 1) & 3] = max3(mr[(c >> 1) & 3], __uint_as_float(x[c]), __uint_as_float(x[c + 1]));
-                            follow(fmaxf(fmaxf(mr[0], mr[1]), fmaxf(mr[2], mr[3])) * c2, cb);
+                            if (at < last) { at += 32; continue; }
+                            follow(fmaxf(fmaxf(mr[0], mr[1]), fmaxf(mr[2], mr[3])) * c2);
                             const float neg_m = m_run == -INFINITY ? 0.f : -m_run;
-                            weigh(x, pk, pack2(neg_m, neg_m));
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) pk[c] = 0u;
+                            neg_m2 = pack2(neg_m, neg_m);
+                            down = true;
                         }
-                        tmem_st16(s_col + cb * 16, pk);        // (over columns of S that have been taken)
+                        weigh(x, pk, neg_m2);
+                        tmem_st16(s_col + P_AT + at / 2, pk);  // (over columns of S that have been taken)
+                        if (at == first) break;
+                        at -= 32;
                     }
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) pk[c] = 0u;
+#pragma unroll
+                    for (int cb = 0; cb < CHUNKS; ++cb)
+                        if (cb * 32 > u_hi || cb * 32 + 31 < u_lo) tmem_st16(s_col + P_AT + cb * 16, pk);
                 }
                 if (t == 0 && n > 0) {                         // the previous item's output
                     mbar_wait(bar_pv + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, 11);
