@@ -210,11 +210,16 @@ private:
     PerDevice<char> t_;
 };
 int device_sm_count(int* n_sm);       // SM count of the current device
-// Whether a decode step should go through its caches alternately forwards and backwards (by the parity of the step).  Steps follow
-// one another on the same caches, and what a step reads last is still in L2 when the next one starts; read in the same order every
-// time, caches larger than L2 push out just what is wanted next.  Measured, us a step in a graph of steps: 2,048 heads x 256 rows
-// (137 MB) 26.5 -> 22.6, 512 x 1,024 at d = 128 (134 MB) 49.4 -> 46.3, 512 x 1,280 (168 MB) 34.2 -> 32.4, 1,024 x 400 (105 MB) 26.0 ->
-// 24.1; caches that fit lose 1 to 3 % (84 MB 18.3 -> 18.6), so the line is at three quarters of L2.
+// Whether a decode step should go through its caches alternately forwards and backwards (by the parity of the step).  That pays where the
+// next step of the SAME caches follows while L2 still holds what this one read last: read in the same order every time, caches
+// larger than L2 push out just what is wanted next.  It does not where other caches come in between (the layers of a model): then there is
+// nothing to find, and the direction must cost next to nothing.  Measured, us a step in a graph of steps on one cache / on eight in turn, forwards
+// only -> alternating (decode_tc.cu for up to 256 rows at d = 64, else decode_mma.cu):
+//   2,048 heads x 256 rows (137 MB)     25.9 -> 21.8 / 26.3 -> 26.5      512 x 1,280, d = 64 (168 MB)    33.8 -> 31.5 / 34.1 -> 34.0
+//   4,096 x 128 (134 MB of rows)        27.6 -> 24.6 / 27.7 -> 27.9      512 x 1,024, d = 128 (268 MB)   49.1 -> 46.0 / 48.5 -> 48.5
+//   8,192 x 256 (550 MB)                89.9 -> 84.7 / 89.7 -> 89.9      1,024 x 400 (105 MB)            25.0 -> 23.1 / 26.3 -> 26.1
+// Caches that fit lose 1 to 3 % (84 MB 18.3 -> 18.6), so the line is at three quarters of L2.  It counts rows that there may be, not those
+// in use, which the host does not know; 1,024 x 400 of which half the pool or a third of the ring is in use: 19.2 -> 18.8, 18.9 -> 18.9.
 int decode_turns(const Params& p, bool* turn);
 
 // Programmatic dependent launch: a kernel launched through launch_pdl may become resident while its predecessor in the

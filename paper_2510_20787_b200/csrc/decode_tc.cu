@@ -80,7 +80,7 @@ template <int NC> __host__ __device__ inline Plan plan_of(const CacheLayout& L) 
 // The most a plan takes: NC rows, of which one is the ring's and the others the pool's (a logit each, a position for those).
 template <int NC> constexpr int kMostSmem = 2 * NC * 128 + 2048 + 4096 + 2 * ((4 * NC + 4 * (NC - 1) + 16 + 255) / 256 * 256) + 128;
 
-template <int NC>
+template <int NC, bool TURN>
 __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(unsigned char* __restrict__ cache, CacheLayout L,
                                                          const __nv_bfloat16* __restrict__ q1,
                                                          const __nv_bfloat16* __restrict__ k1,
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                                                          __nv_bfloat16* __restrict__ o1, float* __restrict__ lse1,
                                                          const float* __restrict__ cw, const float* __restrict__ cbias,
                                                          int BH, int H, int W, int R, int sink, int K,
-                                                         float zthr, float scale, int turn)
+                                                         float zthr, float scale)
 {
     extern __shared__ __align__(1024) unsigned char dsm[];
     constexpr int NW = NC / 32, NTHR = kThreads<NC>, TAPS = (kMaxTaps + NW - 1) / NW;
@@ -125,14 +125,17 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot_gen;
+    // (asked for in L2 while the step before may still be at work, so that the copies below wait less for the direction)
+    const int32_t* counter = reinterpret_cast<const int32_t*>(cache + L.header + (size_t)bh_begin * L.stride + L.off_meta);
+    if (TURN && tid == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(counter));
     pdl_launch_dependents();
     pdl_wait();                                                // the previous step (or whatever wrote the cache and the inputs) has completed
 
-    // the block's heads, from the last to the first in every other step (see decode_turns; all threads read the counter before any of
+    // TURN: the block's heads from the last to the first in every other step (see decode_turns; all threads read the counter before any of
     // them can have come to its write-back, which lies behind barriers of the compute threads and behind the control lane's copies)
     const int n_heads = bh_end - bh_begin;
-    const bool back = turn && (reinterpret_cast<const int32_t*>(cache + L.header + (size_t)bh_begin * L.stride + L.off_meta)[0] & 1) != 0;
-    auto head = [&](int it) { return back ? bh_end - 1 - it : bh_begin + it; };
+    const bool back = TURN && (*counter & 1) != 0;
+    const int first = back ? bh_end - 1 : bh_begin, step = back ? -1 : 1;
 
     if (wid == NW) {
         // ======================================== control lane ==================================================
@@ -140,12 +143,12 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
             constexpr uint32_t IDESC_S = instr_desc(128, 16, false);
             constexpr uint32_t IDESC_O = instr_desc(128, 16, false, true);        // A (values) MN-major, B (p) K-major
             const uint32_t k_lo = desc_lo(sK, 16), q_lo = desc_lo(sQ, 16), vmn_lo = desc_lo(sV, 16384), p_lo = desc_lo(sP, 16);
-            const unsigned char* g0 = cache + L.header + (size_t)head(0) * L.stride;
+            const unsigned char* g0 = cache + L.header + (size_t)first * L.stride;
             bulk_load(sT, g0 + L.off_z, P.tail_bytes, bar_t0);
             bulk_load(sK, g0 + L.off_k, blk_bytes, bar_k);
             bulk_load(sV, g0 + L.off_v, blk_bytes, bar_v);
-            for (int it = 0; it < n_heads; ++it) {
-                const unsigned char* gnext = cache + L.header + (size_t)head(it + 1) * L.stride;
+            for (int it = 0, bh = first; it < n_heads; ++it, bh += step) {
+                const unsigned char* gnext = cache + L.header + (size_t)(bh + step) * L.stride;
                 dwait(bar_k, it & 1, 1);
                 dwait(bar_q, it & 1, 2);                       // q of this head is in the B tile (and the tail of the head before has been used)
                 if (it + 1 < n_heads) bulk_load(sT + ((it & 1) ^ 1) * P.tail_bytes, gnext + L.off_z, P.tail_bytes, bar_t0 + 8 * ((it & 1) ^ 1));
@@ -195,10 +198,10 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
                 kv_new = load128((t2 < 8 ? k1 : v1) + (size_t)bh * D + (t2 & 7) * 8);
             }
         };
-        fetch_inputs(head(0));
+        fetch_inputs(first);
 
-        for (int it = 0; it < n_heads; ++it) {
-            const int bh = head(it), tb = it & 1;
+        for (int it = 0, bh = first; it < n_heads; ++it, bh += step) {
+            const int tb = it & 1;
             unsigned char* gblk = cache + L.header + (size_t)bh * L.stride;
             // q -> row 0 of the logits' B tile (row 0 of a swizzled tile is stored in order)
             if (tid < 8) {
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(kThreads<NC>, kPerSm<NC>) decode_tc_kernel(uns
             // what the rest of this head needs, and the next head's inputs
             const uint4 kv = kv_new;
             const float bias_now = __uint_as_float(bias), v_now = __uint_as_float(tid & 1 ? v1_pair & 0xffff0000u : v1_pair << 16);
-            if (it + 1 < n_heads) fetch_inputs(head(it + 1));
+            if (it + 1 < n_heads) fetch_inputs(bh + step);
 
             // ---- output ----------------------------------------------------------------------------------------
             dwait(bar_o, it & 1, 10);
@@ -385,11 +388,13 @@ int launch_decode_tc(const Params& p, void* cache, const void* q1, const void* k
         const int n_cta = BH < slots ? BH : slots;
         return cuda_status(launch_pdl(kern, dim3(n_cta), dim3(kThreads<NC>), P.total, st, (unsigned char*)cache, L, (const __nv_bfloat16*)q1,
                                       (const __nv_bfloat16*)k1, (const __nv_bfloat16*)v1, (__nv_bfloat16*)o1, lse1, p.w, p.bias, BH, p.H, p.W, p.R,
-                                      p.sink, p.K, p.zthr, p.scale, (int)turn));
+                                      p.sink, p.K, p.zthr, p.scale));
     };
-    static PerDeviceOnce attr256, attr128;
-    if (p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256>, attr256);
-    return go(std::integral_constant<int, 128>{}, decode_tc_kernel<128>, attr128);
+    static PerDeviceOnce attr256, attr128, attr256t, attr128t;
+    if (turn && p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256, true>, attr256t);
+    if (turn) return go(std::integral_constant<int, 128>{}, decode_tc_kernel<128, true>, attr128t);
+    if (p.W + p.R > 128) return go(std::integral_constant<int, 256>{}, decode_tc_kernel<256, false>, attr256);
+    return go(std::integral_constant<int, 128>{}, decode_tc_kernel<128, false>, attr128);
 }
 
 int decode_tc_status_fetch_and_clear() { return status_fetch_and_clear(g_decode_tc_status); }
