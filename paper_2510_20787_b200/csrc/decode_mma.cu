@@ -116,7 +116,7 @@ template <int D, bool SWZ> struct Group {                      // what a lane ho
 };
 
 // BACK: in every other step the spans come from the last to the first (see decode_turns; a variant of its own, since the sign of the
-// stride costs the other 3 %).
+// stride costs up to 3 % of a step that takes its rows from L2, which is where `turn` is off).
 template <int D, int NW, bool SWZ, bool BACK>
 __global__ void __launch_bounds__(NW * 32, warps_per_sm(D) / NW) decode_mma_kernel(
     unsigned char* __restrict__ cache, CacheLayout L, const __nv_bfloat16* __restrict__ q1, const __nv_bfloat16* __restrict__ k1,
@@ -461,7 +461,8 @@ int launch_decode_mma(const Params& p, void* cache, const void* q1, const void* 
     };
 #define LTE_GO2(D, S, T) (nw == 8 ? go(decode_mma_kernel<D, max_warps(D), S, T>) : nw == 4 ? go(decode_mma_kernel<D, 4, S, T>) : \
                           nw == 3 ? go(decode_mma_kernel<D, 3, S, T>) : nw == 2 ? go(decode_mma_kernel<D, 2, S, T>) : go(decode_mma_kernel<D, 1, S, T>))
-#define LTE_GO(D, S) (turn ? LTE_GO2(D, S, true) : LTE_GO2(D, S, false))
+    // (256 swizzled rows pass the line of decode_turns from 1,400 heads on, which have a warp each)
+#define LTE_GO(D, S) (!turn ? LTE_GO2(D, S, false) : !S ? LTE_GO2(D, false, true) : nw == 1 ? go(decode_mma_kernel<D, 1, S, true>) : LTE_GO2(D, S, false))
     cudaError_t e;
     switch (p.d) {
         case 32: e = LTE_GO(32, false); break;

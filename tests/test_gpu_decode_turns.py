@@ -1,5 +1,6 @@
-"""GPU parity of decode steps over caches larger than three quarters of L2, which go through a block's heads forwards and backwards in turn, on
-sampled sequences."""
+"""GPU parity of decode steps over caches larger than three quarters of L2, which go through a block's heads or a head's rows forwards and
+backwards in turn, on sampled sequences: both kernels, one warp a head and several, clusters, more query heads than a pass takes, fewer spans of
+rows than warps, remainders of a span, rows swizzled and not, pools empty, growing and full."""
 import numpy as np
 import pytest
 import torch
@@ -14,6 +15,12 @@ pytestmark = pytest.mark.gpu
     (64, 64, 64, 1, 7, 0, 256, 16, 201, 5),        # the tensor-core step, 128 rows
     (64, 101, 120, 1, 7, 2, 150, 16, 300, 4),      # its variant of 256 rows
     (64, 128, 128, 1, 1, 0, 200, 8, 130, 4),       # blocks of three heads and of four
+    (64, 128, 101, 2, 7, 0, 128, 16, 300, 4),      # mma, swizzled rows
+    (32, 300, 100, 1, 5, 0, 128, 16, 421, 4),      # a warp a head
+    (64, 768, 512, 4, 7, 4, 32, 16, 1500, 4),      # several warps a head
+    (128, 401, 111, 1, 7, 0, 32, 16, 540, 4),
+    (64, 3000, 96, 1, 7, 0, 8, 16, 21, 4),         # a cluster of two, two spans of rows
+    (128, 2950, 1146, 9, 7, 3, 6, 8, 5300, 3),     # a cluster, two passes of query heads
 ])
 def test_decode_turns(d, W, R, G, K, sink, B, H, T0, steps):
     l2 = torch.cuda.get_device_properties(0).L2_cache_size
