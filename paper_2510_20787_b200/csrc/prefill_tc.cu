@@ -13,7 +13,7 @@
 //             there when a warp comes to it.  96 columns because two such buffers and O fill the 256 TMEM columns of a CTA: S [0,96), [96,192), O [192,256)
 //   softmax   mask from positions.  A tile that all of the warp's rows see is taken whole (its 96 logits in registers, one vote); others
 //             go in chunks of 32 columns, which are skipped where no row sees any, twice: for the tile's maximum and for the weights.  The
-//             reference is the maximum of the first tile seen and moves to a later tile's that is more than 2^2 above it (in an item's
+//             reference is the maximum of the first tile seen and moves to a later tile's that is more than 2^4 above it (in an item's
 //             first tiles 2); exp2 with the scale folded in.  O is divided by the sum of P, so that its rounding cancels as far as it is
 //             common to the row, and lse is the logarithm of the sum of the weights themselves (with the weights' sum alone O's error is
 //             2 % larger, with P's alone lse's 1e-3).
@@ -24,15 +24,18 @@
 // and products of the next item run under the current one.  Every mbarrier wait is bounded; one that runs out records a
 // status word and the kernel still terminates.
 //
-// Measured (B200, the call with a workspace, back to back in a CUDA graph; before: two threads per row, 128-key tiles, one S buffer):
-//   128 query heads x 4,096, W = 768, R = 512 half used     176 us (611 TFLOP/s), before 198 (192 with its waits out of line)
-//   64 heads x 4,096, W = R = 128                          45 us, before 49     128 x 2,048, W = R = 64   36 us, before 44
-//   48 x 3,001, W = 300, R = 200                           38 us, before 44     64 x 4,096, W = 32, R = 16   34 us, before 42
-// O's error against 64 bits, logits of N(0,1) rising by 0 to 1 per key, W = 64 to 768: 0.945 to 0.998 times what it was, 1.000 to 1.006 times
-// that of weights rounded beside each row's own maximum (tests/test_gpu_prefill_rounding.py).  Without the look at a partial tile's maximum, chunk
-// by chunk, a reference that moves within a tile and what is there of P rescaled (rounded a second time): 177 us here, 45, 36, 38, 34,
-// and O's error up to 1.04 times what it was.  The maximum in a pass of its own, all chunks fetched again: 183, 49, 40, 41, 36; partial tiles' chunks
-// all in registers, on one path with whole tiles: 190, 45, 36, 40, 33.
+// Measured (B200, the call with a workspace, back to back in a CUDA graph; before: two threads per row, 128-key tiles, one S buffer), logits of
+// N(0,1/64) / N(0,1) / N(0,4), which move the reference the more often the wider they are:
+//   128 query heads x 4,096, W = 768, R = 512 half used     176 / 181 / 191 us (611 TFLOP/s), before 196 / 196 / 199
+//   64 heads x 4,096, W = R = 128                          45 / 46 / 48 us, before 49 / 49 / 50
+//   128 x 2,048, W = R = 64                                37 / 37 / 38 us, before 44 / 44 / 47
+//   48 x 3,001, W = 300, R = 200                           39 / 40 / 41 us, before 44 / 44 / 45
+// O's error against 64 bits, logits of N(0,1) rising by 0 to 1 per key, W = 64 to 768: 0.962 to 0.9995 times what it was, 1.000 to 1.022 times
+// that of weights rounded beside each row's own maximum (tests/test_gpu_prefill_rounding.py).  A reference that follows from 2^2 on makes
+// that 0.945 to 0.998 and 1.006, the first line 176 / 194 / 202 us.  Without the look at a partial tile's maximum, chunk by chunk, with
+// a reference that moves within a tile from 2^8 on and what is there of P rescaled (rounded a second time): 177 / 188 / 188, 45 / 53 / 54,
+// 37 / 42 / 42, and O's error up to 1.04 times what it was.  The maximum in a pass of its own, all chunks fetched again: 183, 49, 40, 41;
+// partial tiles' chunks all in registers, on one path with whole tiles: 190, 45, 36, 40.
 // Tried and slower, the first line unless said otherwise: every tile in rolled chunks (192 us; the small windows 43 and 35), every tile
 // whole (183; 48 and 39), the next tile's logits fetched ahead (194), the maximum asked only behind the exponentials (193), tiles of 80
 // keys with the sum of P as sixteen columns more of the product (188), four CTAs per SM with one S buffer and 64-key tiles (181; 44 and 38),
@@ -416,11 +419,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     __syncwarp();
                 }
                 const uint32_t s_col = trow + S_COL + (g & 1) * BN;
-                // The reference is the maximum of the first tile that the row sees and moves to a later tile's that is more than 2^2 above it (in
+                // The reference is the maximum of the first tile that the row sees and moves to a later tile's that is more than 2^4 above it (in
                 // an item's first tiles 2): the nearer it is to the largest logit, the smaller P's rounding beside the large weights, whose
                 // largest has none at the reference.  Then what has been added up is rescaled.
                 auto follow = [&](float m_here) {
-                    const bool up = m_here > m_run + (t < 2 ? 1.f : 2.f);
+                    const bool up = m_here > m_run + (t < 2 ? 1.f : 4.f);
                     if (!__any_sync(0xffffffffu, up)) return;
                     const float alpha = up && m_run != -INFINITY ? fast_exp2(m_run - m_here) : 1.f;   // (1: nothing has been added up for this row)
                     if (up) m_run = m_here;

@@ -39,6 +39,7 @@ def test_rounding_of_the_weights(d, W, slope):
         best = (p @ v[0, h].double() / p.sum(-1, keepdim=True)).to(torch.bfloat16).double()
         err += float(((o[0, h].double() - exact) ** 2).mean())
         ideal += float(((best - exact) ** 2).mean())
-    # The reference stays within 2^2 of the maximum: where logits rise by less than that from one tile to the next it may be older than the
-    # largest weight, which then loses its exactness: some 0.5 % of the error at these slopes (the sampling of 768,000 errors is 0.1 %).
-    assert np.sqrt(err / ideal) <= 1.02, np.sqrt(err / ideal)
+    # The reference stays within 2^4 of the maximum: where logits rise by less than that from one tile to the next it may be older than the
+    # largest weight, which then loses its exactness.  That weight is a tenth to a quarter of its row at these slopes and a row in two to four has an
+    # older reference, so 1 to 2 % of the error (the sampling of 768,000 errors is 0.1 %).
+    assert np.sqrt(err / ideal) <= 1.03, np.sqrt(err / ideal)
