@@ -13,6 +13,8 @@
 // new cache (here).  Local row r stands for position pos(r) = old pool position (r < R0) or n0 - Wn + (r - R0).
 #include "common.cuh"
 
+#include <type_traits>
+
 namespace lte {
 
 __device__ StatusWord g_chunk_status = LTE_STATUS_INIT;   // report only; 31: the cache does not hold n_past tokens
@@ -89,50 +91,90 @@ __global__ void chunk_gather_kernel(const unsigned char* __restrict__ cache, Cac
     for (int r = threadIdx.x; r < R; r += blockDim.x) oldpos[(size_t)bh * R + r] = r < cnt ? pidx[r] : -1;
 }
 
+// The single-layer scorer's logits of up to four rows (r0 + the lowest bits of `todo`) by a whole warp: a lane has 2D / 32 channels of k or v,
+// coalesced, and sums them over the taps.  Lane b returns the logit of row r0 + b.  (Four at a time: one after the other 179 us in
+// the place of 132 below.)
+template <int N> struct alignas(N >= 4 ? 16 : N * 4) Words { uint32_t x[N]; };
+template <typename T, int D>
+__device__ __noinline__ float score_tokens(const T* klin, const T* vlin, const float* w, const float* bias, int h, int K, int half, int r0, unsigned todo)
+{
+    constexpr int C = 2 * D / 32, M = 4;
+    using Row = Words<C * (int)sizeof(T) / 4>;
+    const int lane = threadIdx.x & 31, c = (lane & 15) * C;
+    const T* rows = (lane < 16 ? klin : vlin) + c;
+    const float* wt = w + (size_t)h * K * 2 * D + (lane < 16 ? 0 : D) + c;
+    int at[M];
+    float a[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) { at[m] = todo != 0u ? __ffs(todo) - 1 : m > 0 ? at[m - 1] : 0; todo &= todo - 1u; a[m] = 0.f; }
+#pragma unroll 1
+    for (int t = 0; t < K; ++t) {
+        union { Row u; T x[C]; } row[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const int rr = r0 + at[m] - half + t;              // (rows before position 0 are zero)
+            row[m].u = Row{};
+            if (rr >= 0) row[m].u = *reinterpret_cast<const Row*>(rows + (size_t)rr * D);
+        }
+#pragma unroll
+        for (int e = 0; e < C; ++e) {
+            const float we = wt[(size_t)t * 2 * D + e];        // (w may start at any element)
+#pragma unroll
+            for (int m = 0; m < M; ++m) a[m] = fmaf(to_f(row[m].x[e]), we, a[m]);
+        }
+    }
+    float mine = 0.f;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const float s = warp_sum(a[m]) + (bias ? bias[h] : 0.f);
+        if (lane == at[m]) mine = s;
+    }
+    return mine;
+}
+
 // Logits of the local sequence.  In: z = the scorer's output over the local sequence (wrong where the receptive field
 // reaches below row R0 + half, undefined for rows before zfrom).  Out: z = the logit of each row's token (the cache's own where
 // it holds one), zrank = the same with sink tokens lifted to +inf, which is what the selection ranks by.
 // zfrom > 0: the single-layer scorer left out the rows before zfrom, whose logits a cache normally holds (8 x 16 heads, 512 tokens on
-// W = 768, R = 512: 15 -> 5 us for the scorer); a ring token among them that has none is scored here, channel by channel.
-template <typename T>
+// W = 768, R = 512: 15 -> 10 us for the scorer, the call 107 -> 100); ring tokens among them that have none are scored here.  With 1, 10 and 100 %
+// of the ring's logits missing that call takes 108, 114 and 132 us (scored by the scorer, 109, 109 and 95; by a thread each 128, 206 and 1,195).
+template <typename T, int D>
 __global__ void chunk_merge_z_kernel(const T* __restrict__ klin, const T* __restrict__ vlin, const float* __restrict__ w, const float* __restrict__ bias,
                                      float* __restrict__ z, float* __restrict__ zrank, const float* __restrict__ zsrc,
-                                     const int32_t* __restrict__ oldpos, int H, int D, int K, int R, int W, int n0, int R0, int Wn, int Tloc,
+                                     const int32_t* __restrict__ oldpos, int H, int K, int R, int W, int n0, int R0, int Wn, int Tloc,
                                      int half, int sink, int zfrom)
 {
     pdl_launch_dependents();
     pdl_wait();                                                // see launch_pdl: earlier kernels of the stream have completed
-    const int bh = blockIdx.y;
+    const int bh = blockIdx.y, lane = threadIdx.x & 31;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= Tloc) return;
-    float zt;
-    int pos;
+    float zt = -INFINITY;
+    int pos = -1;
+    bool gap = false;
     if (r < R0) {
         pos = oldpos[(size_t)bh * R + r];
         zt = zsrc[(size_t)bh * (R + W) + r];
         if (pos < 0) zt = -INFINITY;
-    } else {
+    } else if (r < Tloc) {
         pos = n0 - Wn + (r - R0);
-        zt = r < R0 + Wn ? zsrc[(size_t)bh * (R + W) + r] : -INFINITY;
+        if (r < R0 + Wn) zt = zsrc[(size_t)bh * (R + W) + r];
         // a ring token keeps the logit the cache holds; one the cache has not scored yet is scored now, unless its
         // left neighbours are no longer there (then it stays unscored, as in the decode step)
         if (!(zt > -INFINITY)) {
             if (r < R0 + Wn && R0 > 0 && r < R0 + half) zt = -INFINITY;
             else if (r >= zfrom) zt = z[(size_t)bh * Tloc + r];
-            else {                                             // (its right context is there: zfrom is half rows before the chunk)
-                const int h = bh % H;
-                zt = bias ? bias[h] : 0.f;
-                for (int t = 0; t < K; ++t) {
-                    const int rr = r - half + t;
-                    if (rr < 0) continue;                      // (R0 = 0: before position 0)
-                    const T* kr = klin + ((size_t)bh * Tloc + rr) * D;
-                    const T* vr = vlin + ((size_t)bh * Tloc + rr) * D;
-                    const float* wt = w + ((size_t)h * K + t) * 2 * D;
-                    for (int c = 0; c < D; ++c) zt = fmaf(to_f(kr[c]), wt[c], fmaf(to_f(vr[c]), wt[D + c], zt));
-                }
-            }
+            else gap = true;                                   // (its right context is there: zfrom is half rows before the chunk)
         }
     }
+    for (unsigned todo = __ballot_sync(0xffffffffu, gap); todo != 0u;) {
+        const float x = score_tokens<T, D>(klin + (size_t)bh * Tloc * D, vlin + (size_t)bh * Tloc * D, w, bias, bh % H, K, half, r - lane, todo);
+        unsigned rest = todo;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) rest &= rest - 1u;
+        if ((todo ^ rest) >> lane & 1u) zt = x;
+        todo = rest;
+    }
+    if (r >= Tloc) return;
     z[(size_t)bh * Tloc + r] = zt;
     zrank[(size_t)bh * Tloc + r] = (pos >= 0 && pos < sink) ? INFINITY : zt;
 }
@@ -316,11 +358,15 @@ int launch_chunk_merge_z(const Params& p, const void* klin, const void* vlin, fl
 {
     dim3 grid((p.T + 255) / 256, p.B * p.H);
     auto go = [&](auto kern, auto* k, auto* v) {
-        return cuda_status(launch_pdl(kern, grid, dim3(256), 0, st, k, v, p.w, p.bias, z, zrank, zsrc, oldpos, p.H, p.d, p.K, p.R, p.W, n0, R0, Wn, p.T, p.half,
+        return cuda_status(launch_pdl(kern, grid, dim3(256), 0, st, k, v, p.w, p.bias, z, zrank, zsrc, oldpos, p.H, p.K, p.R, p.W, n0, R0, Wn, p.T, p.half,
                                       p.sink, p.zfrom));
     };
-    if (p.dtype == LTE_BF16) return go(chunk_merge_z_kernel<__nv_bfloat16>, (const __nv_bfloat16*)klin, (const __nv_bfloat16*)vlin);
-    return go(chunk_merge_z_kernel<float>, (const float*)klin, (const float*)vlin);
+    auto by_d = [&](auto* k, auto* v) {
+        using T = std::remove_const_t<std::remove_pointer_t<decltype(k)>>;
+        return p.d == 32 ? go(chunk_merge_z_kernel<T, 32>, k, v) : p.d == 64 ? go(chunk_merge_z_kernel<T, 64>, k, v) : go(chunk_merge_z_kernel<T, 128>, k, v);
+    };
+    if (p.dtype == LTE_BF16) return by_d((const __nv_bfloat16*)klin, (const __nv_bfloat16*)vlin);
+    return by_d((const float*)klin, (const float*)vlin);
 }
 
 int launch_chunk_commit(const Params& p, void* cache, const void* klin, const void* vlin, const float* z, const int32_t* idx,
