@@ -16,7 +16,8 @@ pytestmark = pytest.mark.gpu
     (64, 101, 120, 1, 7, 2, 150, 16, 300, 4),      # its variant of 256 rows
     (64, 128, 128, 1, 1, 0, 200, 8, 130, 4),       # blocks of three heads and of four
     (64, 128, 101, 2, 7, 0, 128, 16, 300, 4),      # mma, swizzled rows
-    (32, 300, 100, 1, 5, 0, 128, 16, 421, 4),      # a warp a head
+    (32, 300, 100, 1, 5, 0, 128, 16, 421, 4),      # a warp a head, all heads at once: alternating
+    (32, 300, 100, 1, 5, 0, 160, 16, 421, 4),      # more heads than that: forwards only
     (64, 768, 512, 4, 7, 4, 32, 16, 1500, 4),      # several warps a head
     (128, 401, 111, 1, 7, 0, 32, 16, 540, 4),
     (64, 3000, 96, 1, 7, 0, 8, 16, 21, 4),         # a cluster of two, two spans of rows
