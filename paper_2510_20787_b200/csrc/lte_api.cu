@@ -47,6 +47,8 @@ namespace {
 
 bool aligned(const void* p, size_t n) { return reinterpret_cast<uintptr_t>(p) % n == 0; }
 bool aligned16(const void* p) { return aligned(p, 16); }
+// the tensor-core scorers (bf16) read their weights in 16-byte pieces
+bool scorer_reads(const lte_shape* s, const float* w) { return s->dtype != LTE_BF16 || aligned16(w); }
 size_t element_bytes(const lte_shape* s) { return s->dtype == LTE_BF16 ? 2 : 4; }
 
 int check_shape(const lte_shape* s, bool need_T)
@@ -253,7 +255,7 @@ int lte_scores(const lte_shape* s, const lte_conv* c, const void* k, const void*
         return launch_scores_stack(p, k, v, z, r_or_null, (cudaStream_t)stream);
     }
     e = check_conv(s, c); if (e) return e;
-    if (!k || !v || !z || !aligned16(k) || !aligned16(v)) return LTE_ERR_INVALID_ARG;
+    if (!k || !v || !z || !aligned16(k) || !aligned16(v) || !scorer_reads(s, c->w)) return LTE_ERR_INVALID_ARG;
     e = check_arch(); if (e) return e;
     return launch_scores(make_params(s, c), k, v, z, r_or_null, (cudaStream_t)stream);
 }
@@ -374,7 +376,7 @@ int lte_attn_prefill_chunk_ex(const lte_shape* s, const lte_conv* c, void* cache
     if (streaming && s->R > 4096) return LTE_ERR_UNSUPPORTED;
     e = check_conv_or_stack(s, c); if (e) return e;
     if (!cache || !q || !k || !v || !o || !lse || n_past < 0) return LTE_ERR_INVALID_ARG;
-    if (!aligned16(cache) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return LTE_ERR_INVALID_ARG;
+    if (!aligned16(cache) || !aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !scorer_reads(s, c->w)) return LTE_ERR_INVALID_ARG;
     const size_t G = s->group > 1 ? s->group : 1, bhq = (size_t)s->B * s->H * G;
     if ((double)bhq * ((double)s->R + s->W + s->T) * s->d > 2.0e10 || (double)n_past + s->T > 2.0e9) return LTE_ERR_UNSUPPORTED;
     const ChunkPlan w = chunk_plan(s, c, streaming);
