@@ -1,6 +1,6 @@
-"""GPU parity of the d = 64 / 32 prefill kernel at the edges of its 128 x 128 tiles: sequence, window and list lengths around a
-tile and around a half tile (two threads share a row), one tile per item, more items than blocks fit on the chip (blocks then
-take over the work of blocks that have not started), a row maximum that keeps growing (the accumulator is rescaled)."""
+"""GPU parity of the d = 64 / 32 prefill kernel around its items of 128 queries and at small shapes: sequence, window and list lengths around 128
+and 64, one tile per item, more items than blocks fit on the chip (blocks then take over the work of blocks that have not started), a row
+maximum that keeps growing (the accumulator is rescaled).  The edges of its 96-key tiles are in test_gpu_prefill_rows.py."""
 import numpy as np
 import pytest
 import torch
