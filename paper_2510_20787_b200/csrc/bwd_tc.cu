@@ -32,11 +32,11 @@
 // Slower: two threads per row in place of four with the halves (64 columns each in two chunks: dkv 2 % at the second shape, 1 % faster at the
 // first), taking turns at the exponential unit, two of a scheduler's four row warps at a time (2 to 7 %), a barrier per half for the end
 // of the accumulation in place of one (1 %).
-// Measured (B200, us for dq + dkv, back to back in a CUDA graph, against four warps a CTA, two CTAs an SM, items dealt out beforehand;
-// before the halves and the stages of K; on the right exponential unit, tensor pipe active, now):
-//   128 heads x 2,048, d = 64, W = R = 64                 60 + 78   (was 74 + 96)       dq 17 %, 31 %;  dkv 14 %, 33 %
-//   128 heads of 4-head groups x 4,096, d = 64, W 768, R 512   243 + 298  (364 + 455)    dq 42 %, 36 %;  dkv 41 %, 48 %
-//   16 heads x 8,192, d = 128, W = R = 512                101 + 107  (185 + 195)       dq 32 %, 56 %;  dkv 25 %, 58 %
+// Measured (B200, us for dq + dkv; four warps a CTA, two CTAs an SM, items dealt out beforehand; then one CTA of 16 row warps, both in a CUDA graph;
+// then with the halves and the stages of K, launches under ncu; exponential unit and tensor pipe active there):
+//   128 heads x 2,048, d = 64, W = R = 64                        74 + 96     60 + 78     62 + 77     dq 17 %, 31 %;  dkv 14 %, 33 %
+//   128 heads of 4-head groups x 4,096, d = 64, W 768, R 512   364 + 455   243 + 298   259 + 271     dq 42 %, 36 %;  dkv 41 %, 48 %
+//   16 heads x 8,192, d = 128, W = R = 512                     185 + 195   101 + 107    88 + 117     dq 32 %, 56 %;  dkv 25 %, 58 %
 #include "tile_items.cuh"
 
 namespace lte {

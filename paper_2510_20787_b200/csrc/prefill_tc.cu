@@ -2,7 +2,7 @@
 // decoding").
 //
 // Bound by the latencies of the softmax warps' chain (load, maximum, exponentials, store) and by their instructions (7 a weight, of which
-// the arithmetic is 4; with items of nine tiles issue 51 %, exponential unit 60 %, tensor pipe 31 %), so a row belongs to one thread, which
+// the arithmetic is 4; with items of ten window tiles and up to three of the list issue 51 %, exponential unit 60 %, tensor pipe 36 %), so a row belongs to one thread, which
 // waits for no other, and nothing waits that need not:
 //   work      Two CTAs per SM; an item is a 128-query tile of one head.  Key/value tiles of 96 rows come by TMA, first the window
 //             span, then the head's retained rows that any of the item's rows may see (compacted beforehand where the caller

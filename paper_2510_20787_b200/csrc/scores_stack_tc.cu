@@ -8,6 +8,10 @@
 // tensor core.  The pieces of a weight sit side by side along N (one MMA of N = 3 C_out covers hi, mid and lo at
 // once; the epilogue adds the three column blocks), so an input tile is read from shared memory once per K step.
 //
+// Products of different widths accumulate in the same columns of the second and third layer.  One thread issues them and the chip runs them in
+// that order (the logits agree with 64 bits to rounding wherever they have been compared), though only products of one shape are
+// promised to keep it.
+//
 // A layer is a sum over its three taps of a [128 rows x C_in] x [C_in x C_out] product whose A operand is the
 // previous layer's tile shifted down by 4, 2 or 0 rows.  Operands are kept in the unswizzled canonical layout (a
 // column of 16-byte chunks per 8 channels, rows 16 bytes apart), where a row shift is a 16-byte-aligned change of the
@@ -280,9 +284,9 @@ scores_stack_tc_kernel(const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16
                 }
                 // The resident weights change with the head, once every reader of the old ones is done with the previous tile; a
                 // head's first tile waits for the new ones.  The ends of the tiles are awaited two tiles late, where that does not hold
-                // up the loads above.  While this warp waits for the end of tile it-2, the others can get as far as the end of tile
-                // it+1, so the barrier is one of four by tile number: with fewer, a late waiter would take
-                // a later completion for the one it wants.
+                // up the loads above.  While this warp waits for the end of tile it-2, the others can get as far as the end of tile it (of tile
+                // it+1 only the keys' parts are there), so the barrier is one of four by tile number: with two, a late waiter would
+                // take the later completion for the one it wants.
                 if (it >= 2) swait(bar_ed4 + 8 * ((it - 2) & 3), ((it - 2) >> 2) & 1, 22);
                 if (more && wn.h != h_loaded) {
                     swait(bar_ed4 + 8 * (it & 3), (it >> 2) & 1, 23);
