@@ -122,16 +122,8 @@ template <bool DKV, int BN> __device__ __forceinline__ Item item_of(const Args& 
 template <int N> struct Tmem;                                  // N consecutive columns of the warp's lanes
 template <> struct Tmem<32> { static __device__ __forceinline__ void ld(uint32_t a, uint32_t (&r)[32]) { tmem_ld32(a, r); } };
 template <> struct Tmem<16> {
-    static __device__ __forceinline__ void ld(uint32_t a, uint32_t (&r)[16]) {
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-                       "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(a) : "memory");
-    }
-    static __device__ __forceinline__ void st(uint32_t a, const uint32_t (&r)[16]) {
-        asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                     ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-                       "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-    }
+    static __device__ __forceinline__ void ld(uint32_t a, uint32_t (&r)[16]) { tmem_ld16(a, r); }
+    static __device__ __forceinline__ void st(uint32_t a, const uint32_t (&r)[16]) { tmem_st16(a, r); }
 };
 template <> struct Tmem<8> {
     static __device__ __forceinline__ void st(uint32_t a, const uint32_t (&r)[8]) {

@@ -82,17 +82,6 @@ __device__ __forceinline__ Part part_of(const Args& a, const Item& it, int q, in
 }
 __device__ __forceinline__ bool takes(const Item& it, const Part& p, int t) { return t < it.n_win ? t >= p.w0 && t < p.w1 : t - it.n_win < p.nl; }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t a, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void tmem_st16(uint32_t a, const uint32_t (&r)[16]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                 ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-                   "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-
 // Barriers (n = item number within the CTA; g = tile number; a = tile number and e = item number counted over what the query tile takes
 // part in; b = a & 1):
 //   bar_k[s], bar_v[s]       K, V of tile g are in stage s = g % ST (TMA)          phase g / ST

@@ -69,41 +69,10 @@ __device__ __forceinline__ uint32_t mn_lo(uint32_t addr) { return (addr >> 4) | 
 constexpr int BG0 = 64 * 3 * 128, BG1 = 32 * 3 * 64, BG2 = 16 * 3 * 32;
 constexpr int BPART = BG0 + BG1 + BG2 + 16 + 64 + 32 + 16 + 1, BPART_PAD = (BPART + 31) & ~31;
 
-__device__ __forceinline__ bool try_wait_long(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void bwait(uint32_t bar, uint32_t parity, int code) {
-#pragma unroll 1
-    for (uint32_t i = 0; i < (1u << 20); ++i) {
-        if (try_wait_long(bar, parity)) return;
-        if ((i & 255u) == 255u && launch_aborted(&g_stack_bwd_status)) return;   // another wait of this launch has given up
-    }
-    wait_gave_up(&g_stack_bwd_status, code);
-}
-__device__ __forceinline__ void bwait_uni(uint32_t bar, uint32_t parity, int code) {   // by the whole warp, see mbar_wait_uni
-#pragma unroll 1
-    for (uint32_t i = 0; i < (1u << 20); ++i) {
-        if (__all_sync(0xffffffffu, try_wait_long(bar, parity))) return;
-        if ((i & 255u) == 255u && uni(launch_aborted(&g_stack_bwd_status))) return;
-    }
-    wait_gave_up(&g_stack_bwd_status, code);
-}
+__device__ __forceinline__ void bwait(uint32_t bar, uint32_t parity, int code) { mbar_wait_long(bar, parity, code, &g_stack_bwd_status); }
+__device__ __forceinline__ void bwait_uni(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni_long(bar, parity, code, &g_stack_bwd_status); }
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld16b(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -373,7 +342,7 @@ stack_bwd_tc_kernel(const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* _
             tc_fence_after();
             {
                 uint32_t a[16];
-                tmem_ld16b(tmem + lane_base + TC_F + part * 16, a);
+                tmem_ld16(tmem + lane_base + TC_F + part * 16, a);
                 tmem_wait_ld();
 #pragma unroll
                 for (int ch = 0; ch < 2; ++ch) {
@@ -460,7 +429,7 @@ stack_bwd_tc_kernel(const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* _
             tc_fence_after();
             {
                 uint32_t a[16];
-                tmem_ld16b(tmem + lane_base + TC_F + part * 16, a);
+                tmem_ld16(tmem + lane_base + TC_F + part * 16, a);
                 tmem_wait_ld();
 #pragma unroll
                 for (int ch = 0; ch < 2; ++ch) {
@@ -561,7 +530,7 @@ stack_bwd_tc_kernel(const __nv_bfloat16* __restrict__ kg, const __nv_bfloat16* _
         if (part > 0) {                                        // layer 2: 3 taps x 16 outputs, lanes 0..31; lane 32: bias gradient
             const int cb = part - 1;
             uint32_t a[16];
-            if (n_my > 0) { tmem_ld16b(tmem + lane_base + TC_W2 + cb * 16, a); tmem_wait_ld(); }
+            if (n_my > 0) { tmem_ld16(tmem + lane_base + TC_W2 + cb * 16, a); tmem_wait_ld(); }
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const float x = n_my > 0 ? __uint_as_float(a[e]) : 0.f;

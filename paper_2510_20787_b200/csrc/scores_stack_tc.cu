@@ -85,45 +85,11 @@ constexpr uint32_t D0_COL = 0, D1_COL = 384, D2_COL = 480, ST_TMEM = 512;
 // distance between the two 8-channel chunk columns of a K = 16 step
 constexpr uint32_t kDescHiFlat = (128u >> 4) | (1u << 14);
 
-// Bounded wait.  The phases of this kernel are long (thousands of cycles) and at any time most warps are waiting, so the
-// wait must not poll: try_wait is given a suspend-time hint and the thread sleeps in hardware until the phase
-// completes (polling warps kept the shared-memory pipeline busy and slowed the working warps several times over).
-__device__ __forceinline__ bool try_wait_long(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void swait(uint32_t bar, uint32_t parity, int code) {
-#pragma unroll 1
-    for (uint32_t i = 0; i < (1u << 20); ++i) {
-        if (try_wait_long(bar, parity)) return;
-        if ((i & 255u) == 255u && launch_aborted(&g_stack_tc_status)) return;   // another wait of this launch has given up
-    }
-    wait_gave_up(&g_stack_tc_status, code);
-}
-__device__ __forceinline__ void swait_uni(uint32_t bar, uint32_t parity, int code) {   // by the whole warp, see mbar_wait_uni
-#pragma unroll 1
-    for (uint32_t i = 0; i < (1u << 20); ++i) {
-        if (__all_sync(0xffffffffu, try_wait_long(bar, parity))) return;
-        if ((i & 255u) == 255u && uni(launch_aborted(&g_stack_tc_status))) return;
-    }
-    wait_gave_up(&g_stack_tc_status, code);
-}
+__device__ __forceinline__ void swait(uint32_t bar, uint32_t parity, int code) { mbar_wait_long(bar, parity, code, &g_stack_tc_status); }
+__device__ __forceinline__ void swait_uni(uint32_t bar, uint32_t parity, int code) { mbar_wait_uni_long(bar, parity, code, &g_stack_tc_status); }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr) : "memory");
 }
 // Swish with the fast exponential and division: their error (a few 1e-7 relative) is below that of the tensor core's
 // fp32 accumulation, which bounds the accuracy of the logits here (about 1e-5 absolute at |z| of a few units)
